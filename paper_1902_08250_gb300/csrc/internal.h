@@ -18,7 +18,7 @@ void lm_set_error(const char *fmt, ...);
 // tree: raise one (never lower it) so that trees built earlier, with larger
 // needs, still launch.  slot names the kernel in a small per-device cache.
 enum { LM_SMEM_NEAR_PW = 0, LM_SMEM_IMAGE_M2L = 1, LM_SMEM_CROSS_M2L = 2, LM_SMEM_NEAR_PW64 = 3,
-       LM_SMEM_IMAGE_M2L_A = 4, LM_SMEM_NEAR_PW64_A = 5, LM_SMEM_NEAR_PW_A = 6, LM_SMEM_SLOTS = 7 };
+       LM_SMEM_NEAR_PW64_A = 4, LM_SMEM_NEAR_PW_A = 5, LM_SMEM_SLOTS = 6 };
 cudaError_t lm_raise_smem(const void *func, int slot, int bytes);
 
 #define LM_CUDA(call)                                                                       \
@@ -240,6 +240,22 @@ void lm_phase_end(lm_tree_s *t, int ph, cudaStream_t st, int launches);
 void lm_profile_apply_start(lm_tree_s *t);
 void lm_profile_apply_stop(lm_tree_s *t);
 
+// translation tables (lmfmm_tables.cu)
+struct MediumD;
+struct M2LClass { // one M2L table: [2P+1][2P+1] at out, scaled by S_t(p) S_s(q)
+    int term;
+    double dx, dy;                    // target centre - source centre (free space); horizontal offset, image height h
+    double sc_t, sc_s;                // k2 w of the target's and the source's level
+    const double *scale_t, *scale_s;  // device: S(n), n = 0..P (free space)
+    zd *out;
+};
+lm_status lm_build_m2l_tables(const MediumD &md, int P, const std::vector<M2LClass> &cls, int *dflag, cudaStream_t st);
+struct ShiftJob { // M2M and L2L tables between a level of box width wc and its parent level; m2m or l2l may be null
+    double k, wc;
+    const double *sc_child, *sc_par;
+    zd *m2m, *l2l; // [4 child positions][2P+1][2P+1]
+};
+lm_status lm_build_shift_tables(int P, const std::vector<ShiftJob> &jobs, cudaStream_t st);
 // setup (lmfmm_setup.cu)
 lm_status lm_setup_tree(lm_tree_s *t, const double *x, const double *y, cudaStream_t st);
 lm_status lm_setup_tables(lm_tree_s *t, cudaStream_t st);

@@ -243,63 +243,6 @@ lm_status upload(lm_tree_s *t, T **dst, const std::vector<T> &src, cudaStream_t 
 
 } // namespace
 
-// ---------------------------------------------------------------------------
-// M2L tables of the adaptive lists.  A class is (term, target level lt, source
-// level ls, centre offsets in half widths of the finer level); its table is
-// scaled by S_lt(p) S_ls(q), S_l(n) = (k w_l / 2)^|n| / |n|!, so that it acts
-// on the scaled multipole of the source box and yields the scaled local
-// expansion of the target box.
-//   free term: A_pq = (i/4) H_{q-p}(k rho) e^{i (q-p) theta}, (rho, theta) the
-//              polar form of target centre - source centre (Rokhlin's translation);
-//   image terms: Lemma M2L with dx = x_t - x_s and h the image height.
-// ---------------------------------------------------------------------------
-__global__ void k_free_m2l_a(double k, int P, const double *cdx, const double *cdy, const int *clt,
-                             const int *cls, int ncls, const double *scales, zd *tab)
-{
-    const int np = 2 * P + 1;
-    const int ci = blockIdx.y;
-    if (ci >= ncls) return;
-    const double cx = cdx[ci], cy = cdy[ci];
-    const double rho = hypot(cx, cy), th = atan2(cy, cx);
-    const double *st = scales + (int64_t)clt[ci] * (P + 1), *ss = scales + (int64_t)cls[ci] * (P + 1);
-    zd *T = tab + (int64_t)ci * np * np;
-    for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < np * np; idx += gridDim.x * blockDim.x) {
-        const int p = idx / np - P, q = idx % np - P;
-        const int n = q - p, a = n < 0 ? -n : n;
-        double jv = jn(a, k * rho), yv = yn(a, k * rho);
-        if (n < 0 && (a & 1)) {
-            jv = -jv;
-            yv = -yv;
-        }
-        const double s = st[p < 0 ? -p : p] * ss[q < 0 ? -q : q];
-        const zd h = {-0.25 * yv * s, 0.25 * jv * s}; // (i/4)(J + iY) S_t S_s
-        const zd e = {cos(n * th), sin(n * th)};
-        T[idx] = h * e;
-    }
-}
-
-__global__ void __launch_bounds__(256) k_image_m2l_a(MediumD m, int P, const int *cterm, const double *cdx,
-                                                     const double *ch, const int *clt, const int *cls,
-                                                     int ncls, zd *tab, int *flag)
-{
-    const int ci = blockIdx.x;
-    if (ci >= ncls) return;
-    const int term = cterm[ci];
-    const int tau = (term == 2 || term == 4) ? 1 : -1;
-    const int vs = (term == 2 || term == 3) ? 1 : -1;
-    const int is = term == 1 ? 0 : (term == 2 ? 1 : 2);
-    auto sigf = [&](zd lam, zd *s2, zd *ss) {
-        zd sig[3];
-        densities(m, lam, s2, sig);
-        *ss = *s2;
-        return sig[is];
-    };
-    const double km = fmax(m.k1, fmax(m.k2, m.k3)), kmin = fmin(m.k1, fmin(m.k2, m.k3));
-    const double sct = m.k2 * ldexp(m.d, -clt[ci]), scs = m.k2 * ldexp(m.d, -cls[ci]);
-    m2l_table_body(sigf, km, kmin, m.k2, m.k2, P, sct, scs, tau, vs, cdx[ci], ch[ci], 0.0,
-                   tab + (int64_t)ci * (2 * P + 1) * (2 * P + 1), flag);
-}
-
 #define TRY_A(x)                    \
     do {                            \
         lm_status s_ = (x);         \
@@ -505,46 +448,16 @@ lm_status lm_setup_adaptive(lm_tree_s *t, const double *x, const double *y, cuda
             LM_CUDA(cudaMemcpyAsync(A.vslot, vslot.data(), vslot.size() * sizeof(int32_t), cudaMemcpyHostToDevice,
                                     st));
         }
-        const int nf = (int)fidx.size(), ni = (int)iidx.size();
-        int *dint;
-        double *ddbl, *dsc;
-        TRY_A(lm_dalloc(t, &dint, 3 * (size_t)ncls + 1));
-        TRY_A(lm_dalloc(t, &ddbl, 2 * (size_t)ncls + 1));
-        TRY_A(lm_dalloc(t, &dsc, (size_t)(t->L + 1) * (P + 1)));
-        std::vector<int> hint;
-        hint.insert(hint.end(), cterm.begin(), cterm.end());
-        hint.insert(hint.end(), clt.begin(), clt.end());
-        hint.insert(hint.end(), cls.begin(), cls.end());
-        std::vector<double> hdbl;
-        hdbl.insert(hdbl.end(), cdx.begin(), cdx.end());
-        hdbl.insert(hdbl.end(), cdy.begin(), cdy.end());
-        if (ncls > 0) {
-            LM_CUDA(cudaMemcpyAsync(dint, hint.data(), hint.size() * sizeof(int), cudaMemcpyHostToDevice, st));
-            LM_CUDA(cudaMemcpyAsync(ddbl, hdbl.data(), hdbl.size() * sizeof(double), cudaMemcpyHostToDevice, st));
-        }
-        for (int l = 0; l <= t->L; ++l)
-            LM_CUDA(cudaMemcpyAsync(dsc + (size_t)l * (P + 1), t->lev[l].scale, (P + 1) * sizeof(double),
-                                    cudaMemcpyDeviceToDevice, st));
+        // A class is (term, target level lt, source level ls, centre offsets in half widths of the
+        // finer level); its table is scaled by S_lt(p) S_ls(q), so that it acts on the scaled
+        // multipole of the source box and yields the scaled local expansion of the target box.
         if (md.deriv) // the free part does not depend on d: its tables stay zero
             LM_CUDA(cudaMemsetAsync(A.tab, 0, (size_t)std::max(1, ncls) * np * np * sizeof(zd), st));
-        if (nf > 0 && !md.deriv) {
-            dim3 g((np * np + 255) / 256, nf);
-            k_free_m2l_a<<<g, 256, 0, st>>>(t->med.k2, P, ddbl, ddbl + ncls, dint + ncls, dint + 2 * ncls, nf, dsc,
-                                            A.tab);
-        }
-        if (ni > 0) {
-            const size_t shm = (2 * TB_CHUNK * np + TB_CHUNK) * sizeof(zd);
-            LM_CUDA(lm_raise_smem((const void *)k_image_m2l_a, LM_SMEM_IMAGE_M2L_A, (int)shm));
-            k_image_m2l_a<<<ni, 256, shm, st>>>(md, P, dint + nf, ddbl + nf, ddbl + ncls + nf, dint + ncls + nf,
-                                                dint + 2 * ncls + nf, ni, A.tab + (size_t)nf * np * np, t->dflag);
-        }
-        LM_CUDA(cudaGetLastError());
-        LM_CUDA(cudaStreamSynchronize(st));
-        cudaFree(dint);
-        cudaFree(ddbl);
-        cudaFree(dsc);
-        t->bytes -= (3 * (size_t)ncls + 1) * sizeof(int) + (2 * (size_t)ncls + 1 + (size_t)(t->L + 1) * (P + 1)) *
-                                                               sizeof(double);
+        std::vector<M2LClass> tcls;
+        for (int j = 0; j < ncls; ++j)
+            tcls.push_back({cterm[j], cdx[j], cdy[j], md.k2 * ldexp(d, -clt[j]), md.k2 * ldexp(d, -cls[j]),
+                            t->lev[clt[j]].scale, t->lev[cls[j]].scale, A.tab + (size_t)j * np * np});
+        TRY_A(lm_build_m2l_tables(md, P, tcls, t->dflag, st));
     }
     // expansions and tree-order scratch
     TRY_A(lm_dalloc(t, &A.M, (size_t)nbox * np * LM_MAXV));
@@ -554,10 +467,6 @@ lm_status lm_setup_adaptive(lm_tree_s *t, const double *x, const double *y, cuda
     int hflag = 0;
     LM_CUDA(cudaMemcpyAsync(&hflag, t->dflag, sizeof(int), cudaMemcpyDeviceToHost, st));
     LM_CUDA(cudaStreamSynchronize(st));
-    if (hflag & 8) {
-        lm_set_error("build_tree: expansion order too large for the table builder");
-        return LM_ENOTSUP;
-    }
     if (hflag & 16) {
         lm_set_error("build_tree: a layered M2L table overflowed; lower p");
         return LM_ENOTSUP;

@@ -39,8 +39,6 @@ __global__ void k_scatter(const int32_t *key, int64_t n, const int64_t *start, i
 __global__ void k_leafsort(const int64_t *start, int64_t *idx, int *flag);
 __global__ void k_gather_pts(const double *x, const double *y, const int64_t *perm, int64_t n, double *xs,
                              double *ys);
-__global__ void k_shift_tables(double k, int P, double wc, const double *sc_child, const double *sc_par, zd *m2m,
-                               zd *l2l);
 __global__ void k_p2m64(LeafGeom g, int P, double k, const double *xs, const double *ys, const int64_t *ls,
                         const zd *qs, int64_t n, int nvec, zd *M);
 __global__ void k_m2m64(int64_t ncol, int64_t nbox, int P, int nvec, const zd *tabs, const zd *Mc, zd *Mp);
@@ -611,11 +609,13 @@ static lm_status cross_setup(lm_cross_s *c, const double *xs, const double *ys, 
         if (l < L) CTRY(calloc_dev(c, &lv.m2m, 4 * np * np));
         if (l > 0) CTRY(calloc_dev(c, &lv.l2l, 4 * np * np));
     }
+    std::vector<ShiftJob> jobs;
     for (int l = 0; l < L; ++l) {
         CrossLevel &par = c->lev[l], &ch = c->lev[l + 1];
-        k_shift_tables<<<gridc(4 * np * np, 128), 128, 0, st>>>(k1, P, ch.w, ch.sc_s, par.sc_s, par.m2m, nullptr);
-        k_shift_tables<<<gridc(4 * np * np, 128), 128, 0, st>>>(k2, P, ch.w, ch.sc_t, par.sc_t, nullptr, ch.l2l);
+        jobs.push_back({k1, ch.w, ch.sc_s, par.sc_s, par.m2m, nullptr});
+        jobs.push_back({k2, ch.w, ch.sc_t, par.sc_t, nullptr, ch.l2l});
     }
+    CTRY(lm_build_shift_tables(P, jobs, st));
 
     // V lists and classes (host): target-major, then term, then source box
     const size_t shm = (2 * 16 * np + 16) * sizeof(zd); // m2l_table_body's staging

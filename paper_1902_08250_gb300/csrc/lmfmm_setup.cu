@@ -365,103 +365,6 @@ __global__ void k_near_tail(MediumD m, double c, int nray, int order, zd *lam_o,
 }
 
 // ---------------------------------------------------------------------------
-// Translation tables (scaled; S_l(n) = (k w_l / 2)^|n| / |n|!):
-//  M2M (Lemma M2M, reading G3): M_p += sum_q M_q J_{p-q}(k r) e^{-i (p-q) theta},
-//     (r, theta) = child centre - parent centre; scaled by S_child(q)/S_parent(p).
-//  L2L (Lemma L2L, reading G3): L_p += sum_q L_q J_{p-q}(k r) e^{-i (p-q) theta},
-//     (r, theta) = parent centre - child centre; scaled by S_child(p)/S_parent(q).
-// ---------------------------------------------------------------------------
-__device__ double besj_int(int n, double x)
-{
-    int a = n < 0 ? -n : n;
-    double v = jn(a, x);
-    return (n < 0 && (a & 1)) ? -v : v;
-}
-
-__global__ void k_shift_tables(double k, int P, double wc, const double *sc_child,
-                               const double *sc_par, zd *m2m, zd *l2l)
-{
-    int np = 2 * P + 1;
-    int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= 4 * np * np) return;
-    int pos = idx / (np * np), p = (idx / np) % np - P, q = idx % np - P;
-    int dy = pos >> 1, dx = pos & 1;
-    // child centre - parent centre
-    double sx = (dx - 0.5) * wc, sy = -(dy - 0.5) * wc;
-    double r = hypot(sx, sy), th = atan2(sy, sx);
-    int n = p - q;
-    if (m2m) {
-        double j = besj_int(n, k * r);
-        double s = sc_child[q < 0 ? -q : q] / sc_par[p < 0 ? -p : p];
-        m2m[idx] = zd{j * cos(n * th) * s, -j * sin(n * th) * s};
-    }
-    if (l2l) {
-        // parent centre - child centre = -(sx, sy)
-        double th2 = atan2(-sy, -sx);
-        double j = besj_int(n, k * r);
-        double s = sc_child[p < 0 ? -p : p] / sc_par[q < 0 ? -q : q];
-        l2l[idx] = zd{j * cos(n * th2) * s, -j * sin(n * th2) * s};
-    }
-}
-
-// Free-space M2L (Rokhlin's translation): A_pq = (i/4) H_{q-p}(k rho) e^{i (q-p) theta},
-// c = target centre - source centre = (dc w, -dr w); scaled by S(p) S(q).
-__global__ void k_free_m2l(double k, int P, double w, const int *cdc, const int *cdr,
-                           const int *cidx, int ncls, const double *sc, zd *tab)
-{
-    int np = 2 * P + 1;
-    int ci = blockIdx.y;
-    if (ci >= ncls) return;
-    double cx = cdc[ci] * w, cy = -cdr[ci] * w;
-    double rho = hypot(cx, cy), th = atan2(cy, cx);
-    zd *T = tab + (int64_t)cidx[ci] * np * np;
-    for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < np * np;
-         idx += gridDim.x * blockDim.x) {
-        int p = idx / np - P, q = idx % np - P;
-        int n = q - p, a = n < 0 ? -n : n;
-        double jv = jn(a, k * rho), yv = yn(a, k * rho);
-        if (n < 0 && (a & 1)) {
-            jv = -jv;
-            yv = -yv;
-        }
-        double s = sc[p < 0 ? -p : p] * sc[q < 0 ? -q : q];
-        // (i/4)(J + iY) = (-Y/4) + i (J/4)
-        zd h = {-0.25 * yv * s, 0.25 * jv * s};
-        zd e = {cos(n * th), sin(n * th)};
-        T[idx] = h * e;
-    }
-}
-
-// Layered M2L (Lemma M2L, reading G2 for the phase i^{p-q}):
-//   A_pq = (i^{p-q}/4pi) Int Z_t^p Z_s^q e^{i lambda dx - s2 h} sigma_m / s2 d lambda,
-//   Z_t = (lambda + tau s2)/k2, Z_s = (lambda + vs s2)/k2,
-// scaled by S(p) S(q): the powers are formed as (Z sc/2)^|p| / |p|!.
-// Contour: trapezoid segment over [-c, c] (down on the right, up on the
-// left) at depth a = min(0.5, 1/|dx|), then steepest-descent rays from +-c.
-// One block per class; nodes staged in chunks through shared memory.
-
-__global__ void __launch_bounds__(256) k_image_m2l(MediumD m, int P, double w, double sc, const int *cterm,
-                                                   const int *cdc, const int *cdr, const int *cidx, int ncls,
-                                                   zd *tab, int *flag)
-{
-    const int ci = blockIdx.x;
-    if (ci >= ncls) return;
-    const int term = cterm[ci];
-    const int tau = (term == 2 || term == 4) ? 1 : -1;
-    const int vs = (term == 2 || term == 3) ? 1 : -1;
-    const int is = term == 1 ? 0 : (term == 2 ? 1 : 2);
-    auto sigf = [&](zd lam, zd *s2, zd *ss) {
-        zd sig[3];
-        densities(m, lam, s2, sig);
-        *ss = *s2;
-        return sig[is];
-    };
-    const double km = fmax(m.k1, fmax(m.k2, m.k3)), kmin = fmin(m.k1, fmin(m.k2, m.k3));
-    m2l_table_body(sigf, km, kmin, m.k2, m.k2, P, sc, sc, tau, vs, cdc[ci] * w, fabs((double)cdr[ci]) * w, 0.0,
-                   tab + (int64_t)cidx[ci] * (2 * P + 1) * (2 * P + 1), flag);
-}
-
-// ---------------------------------------------------------------------------
 // host orchestration
 // ---------------------------------------------------------------------------
 template <typename T>
@@ -662,14 +565,12 @@ lm_status lm_setup_levels(lm_tree_s *t, int L, bool boxes, cudaStream_t st)
         if (l < L) TRY(dalloc(t, &lv.m2m, 4 * np * np));
         if (l > 0) TRY(dalloc(t, &lv.l2l, 4 * np * np));
     }
-    for (int l = 0; l < L; ++l) {
-        // child level l+1 -> parent level l
-        Level &par = t->lev[l], &ch = t->lev[l + 1];
-        k_shift_tables<<<grid_for(4 * np * np, 128), 128, 0, st>>>(k, P, ch.w, ch.scale, par.scale,
-                                                                   par.m2m, ch.l2l);
+    std::vector<ShiftJob> jobs;
+    for (int l = 0; l < L; ++l) { // child level l+1 -> parent level l
+        const Level &par = t->lev[l], &ch = t->lev[l + 1];
+        jobs.push_back({k, ch.w, ch.scale, par.scale, par.m2m, ch.l2l});
     }
-    LM_CUDA(cudaGetLastError());
-    return LM_OK;
+    return lm_build_shift_tables(P, jobs, st);
 }
 
 // Near-field quadrature tables of the reflected direct terms (shared by both tree kinds)
@@ -751,6 +652,7 @@ lm_status lm_setup_tables(lm_tree_s *t, cudaStream_t st)
                {t->med.opt.top_alpha, t->med.opt.bottom_alpha}};
     TRY(lm_setup_levels(t, L, true, st));
     // lists and M2L classes
+    std::vector<M2LClass> tcls;
     for (int l = 0; l <= L; ++l) {
         Level &lv = t->lev[l];
         std::vector<std::tuple<int, int, int>> cls;
@@ -781,51 +683,19 @@ lm_status lm_setup_tables(lm_tree_s *t, cudaStream_t st)
         // tables
         int ncls = (int)cls.size();
         TRY(dalloc(t, &lv.tab, (size_t)std::max(1, ncls) * np * np));
-        std::vector<int> fdc, fdr, fidx, idc, idr, iterm, iidx;
-        for (int i = 0; i < ncls; ++i) {
-            if (lv.cls_term[i] == 0) {
-                fdc.push_back(lv.cls_dc[i]);
-                fdr.push_back(lv.cls_dr[i]);
-                fidx.push_back(i);
-            } else {
-                iterm.push_back(lv.cls_term[i]);
-                idc.push_back(lv.cls_dc[i]);
-                idr.push_back(lv.cls_dr[i]);
-                iidx.push_back(i);
-            }
-        }
-        int *dbuf;
-        int nf = (int)fdc.size(), ni = (int)idc.size();
-        TRY(dalloc(t, &dbuf, 3 * nf + 4 * ni + 1));
-        std::vector<int> hb;
-        hb.insert(hb.end(), fdc.begin(), fdc.end());
-        hb.insert(hb.end(), fdr.begin(), fdr.end());
-        hb.insert(hb.end(), fidx.begin(), fidx.end());
-        hb.insert(hb.end(), iterm.begin(), iterm.end());
-        hb.insert(hb.end(), idc.begin(), idc.end());
-        hb.insert(hb.end(), idr.begin(), idr.end());
-        hb.insert(hb.end(), iidx.begin(), iidx.end());
-        if (!hb.empty())
-            LM_CUDA(cudaMemcpyAsync(dbuf, hb.data(), hb.size() * sizeof(int), cudaMemcpyHostToDevice, st));
         if (md.deriv) // the free part does not depend on d: its tables stay zero
             LM_CUDA(cudaMemsetAsync(lv.tab, 0, (size_t)std::max(1, ncls) * np * np * sizeof(zd), st));
-        if (nf > 0 && !md.deriv) {
-            dim3 g(grid_for(np * np, 256), nf);
-            k_free_m2l<<<g, 256, 0, st>>>(k, P, lv.w, dbuf, dbuf + nf, dbuf + 2 * nf, nf, lv.scale, lv.tab);
-        }
-        if (ni > 0) {
-            size_t shm = (2 * TB_CHUNK * np + TB_CHUNK) * sizeof(zd);
-            LM_CUDA(lm_raise_smem((const void *)k_image_m2l, LM_SMEM_IMAGE_M2L, (int)shm));
-            k_image_m2l<<<ni, 256, shm, st>>>(md, P, lv.w, k * lv.w, dbuf + 3 * nf, dbuf + 3 * nf + ni,
-                                              dbuf + 3 * nf + 2 * ni, dbuf + 3 * nf + 3 * ni, ni, lv.tab,
-                                              t->dflag);
+        for (int i = 0; i < ncls; ++i) { // free space: target centre - source centre = (dc w, -dr w)
+            const double dy = lv.cls_term[i] == 0 ? -lv.cls_dr[i] * lv.w : fabs((double)lv.cls_dr[i]) * lv.w;
+            tcls.push_back({lv.cls_term[i], lv.cls_dc[i] * lv.w, dy, k * lv.w, k * lv.w, lv.scale, lv.scale,
+                            lv.tab + (size_t)i * np * np});
         }
         LM_CUDA(cudaGetLastError());
         LM_CUDA(cudaStreamSynchronize(st));
-        cudaFree(dbuf);
         cudaFree(dmap);
-        t->bytes -= (3 * nf + 4 * ni + 1) * sizeof(int) + smap.size() * sizeof(int32_t);
+        t->bytes -= smap.size() * sizeof(int32_t);
     }
+    TRY(lm_build_m2l_tables(md, P, tcls, t->dflag, st));
     // U list
     {
         const int64_t ncol = (int64_t)t->R << L, nrow = (int64_t)1 << L;
@@ -849,10 +719,6 @@ lm_status lm_setup_tables(lm_tree_s *t, cudaStream_t st)
     if (hflag & 4) {
         lm_set_error("build_tree: internal error, an interaction has no translation class");
         return LM_ECUDA;
-    }
-    if (hflag & 8) {
-        lm_set_error("build_tree: expansion order too large for the table builder");
-        return LM_ENOTSUP;
     }
     if (hflag & 16) {
         lm_set_error("build_tree: a layered M2L table overflowed; lower p");

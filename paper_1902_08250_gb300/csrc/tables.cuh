@@ -6,8 +6,19 @@
 
 // ---------------------------------------------------------------------------
 // Gauss-Legendre nodes on [-1, 1] by Newton's method on P_n (three-term
-// recurrence), initial guess cos(pi (i + 3/4) / (n + 1/2)).
+// recurrence), initial guess cos(pi (i + 3/4) / (n + 1/2)).  The recurrence's
+// 1/j come from a table: an FP64 division per step made the 24- to 192-point
+// rules of the near field a serial chain of 0.1 to 0.9 ms.
 // ---------------------------------------------------------------------------
+#define GL_MAXN 256
+struct InvTable {
+    double r[GL_MAXN + 1];
+    constexpr InvTable() : r()
+    {
+        for (int j = 1; j <= GL_MAXN; ++j) r[j] = 1.0 / j;
+    }
+};
+static __constant__ InvTable c_inv = InvTable();
 __device__ inline void gl_node(int n, int i, double *x, double *w)
 {
     double z = cos(M_PI * (i + 0.75) / (n + 0.5)), pp = 1.0;
@@ -16,16 +27,46 @@ __device__ inline void gl_node(int n, int i, double *x, double *w)
         for (int j = 1; j <= n; ++j) {
             double p3 = p2;
             p2 = p1;
-            p1 = ((2.0 * j - 1.0) * z * p2 - (j - 1.0) * p3) / j;
+            p1 = ((2.0 * j - 1.0) * z * p2 - (j - 1.0) * p3) * c_inv.r[j];
         }
         pp = n * (z * p1 - p2) / (z * z - 1.0);
         double dz = p1 / pp;
         z -= dz;
-        if (fabs(dz) < 1e-16) break;
+        if (fabs(dz) < 1e-15) break;
     }
     *x = -z; // ascending order
     *w = 2.0 / ((1.0 - z * z) * pp * pp);
 }
+// the 24-point rule of the table panels, formed at compile time by the same iteration
+#define TB_ORD 24
+struct GLTable {
+    double x[TB_ORD], w[TB_ORD];
+    constexpr GLTable() : x(), w()
+    {
+        for (int i = 0; i < TB_ORD; ++i) {
+            const double a = 3.14159265358979323846 * (i + 0.75) / (TB_ORD + 0.5);
+            double z = 0.0, f = 1.0; // cos(a) by its series: a starting value
+            for (int m = 0; m < 24; ++m) {
+                z += f;
+                f *= -a * a / ((2.0 * m + 1.0) * (2.0 * m + 2.0));
+            }
+            double pp = 1.0;
+            for (int it = 0; it < 12; ++it) {
+                double p1 = 1.0, p2 = 0.0;
+                for (int j = 1; j <= TB_ORD; ++j) {
+                    const double p3 = p2;
+                    p2 = p1;
+                    p1 = ((2.0 * j - 1.0) * z * p2 - (j - 1.0) * p3) / j;
+                }
+                pp = TB_ORD * (z * p1 - p2) / (z * z - 1.0);
+                z -= p1 / pp;
+            }
+            x[i] = -z;
+            w[i] = 2.0 / ((1.0 - z * z) * pp * pp);
+        }
+    }
+};
+static __constant__ GLTable c_gl = GLTable();
 
 // ---------------------------------------------------------------------------
 // Image densities (reading R1 of the paper's Example 4 for a middle-layer
@@ -105,13 +146,95 @@ __device__ inline void densities(const MediumD &m, zd lam, zd *s2o, zd sig[3])
     *s2o = s2;
 }
 
+// ---------------------------------------------------------------------------
+// Contour of one class's table integral over lambda: the trapezoid segment over
+// [-c, c] (down on the right, up on the left) at depth a = min(0.5, 1/|dx|) in
+// nflat + 2 panels a side, then steepest-descent rays from +-c in TPAN panels of
+// TB_ORD nodes on [0, tmax], geometrically graded: the first is at most 1 wide
+// (low orders vary on the scale of c near the start of the ray), later ones widen
+// by the ratio g (high orders peak near t = 2P / rho).  Uniform panels lost
+// accuracy for small boxes, where tmax ~ 1/rho is large.
+// ---------------------------------------------------------------------------
+struct TabContour {
+    double c, a, delta, flat, h0, g, cphi, sphi; // cphi, sphi: direction of the right ray
+    int nflat, tpan;
+    __host__ __device__ int nseg() const { return (nflat + 2) * TB_ORD; } // nodes of the right half segment
+    __host__ __device__ int ntail() const { return tpan * TB_ORD; }
+};
+__host__ __device__ inline TabContour tab_contour(double km, double kmin, int P, double dx, double h)
+{
+    TabContour C;
+    C.c = 1.5 * km + 1.0;
+    C.a = fmin(0.5, 1.0 / fmax(fabs(dx), 1e-3));
+    C.delta = fmin(0.25, 0.5 * kmin);
+    const double width = fmin(fmin(0.5, 2.0 * C.a), 1.5 / fmax(fabs(dx), 1e-3));
+    C.nflat = (int)ceil((C.c - 2.0 * C.delta) / width);
+    C.flat = (C.c - 2.0 * C.delta) / C.nflat;
+    const double rho = hypot(dx, h), tmax = 1.5 * (2.0 * P + 60.0) / rho;
+    C.tpan = P + 16 > 32 ? P + 16 : 32;
+    C.h0 = fmin(1.0, tmax / C.tpan);
+    C.g = 1.0;
+    if (C.h0 * C.tpan < tmax) { // solve h0 (g^TPAN - 1)/(g - 1) = tmax for g > 1 by bisection
+        double lo = 1.0, hi = 2.0;
+        while (C.h0 * (pow(hi, C.tpan) - 1.0) / (hi - 1.0) < tmax) hi *= 2.0;
+        for (int it = 0; it < 50; ++it) {
+            const double mid = 0.5 * (lo + hi);
+            if (C.h0 * (pow(mid, C.tpan) - 1.0) / (mid - 1.0) < tmax) lo = mid;
+            else hi = mid;
+        }
+        C.g = hi;
+    }
+    C.cphi = cos(atan2(dx, h));
+    C.sphi = sin(atan2(dx, h));
+    return C;
+}
+// node i of the half segment (i < nseg) or of the ray (i - nseg), side +1 or -1: lambda and its weight
+__device__ inline void tab_node(const TabContour &C, int i, int side, zd *lam, zd *dl)
+{
+    const int j = i % TB_ORD;
+    const double x = c_gl.x[j], gw = c_gl.w[j];
+    if (i < C.nseg()) {
+        const int pan = i / TB_ORD;
+        zd z0, z1;
+        if (pan == 0) {
+            z0 = {0.0, 0.0};
+            z1 = {C.delta, -C.a};
+        } else if (pan == C.nflat + 1) {
+            z0 = {C.c - C.delta, -C.a};
+            z1 = {C.c, 0.0};
+        } else {
+            z0 = {C.delta + (pan - 1) * C.flat, -C.a};
+            z1 = {C.delta + pan * C.flat, -C.a};
+        }
+        const zd dz = z1 - z0;
+        *lam = z0 + (0.5 * (x + 1.0)) * dz;
+        *dl = (0.5 * gw) * dz;
+        if (side < 0) *lam = -*lam; // mirrored through the origin; the orientation -c -> 0 keeps dl
+        return;
+    }
+    const int pan = (i - C.nseg()) / TB_ORD;
+    double t0, t1;
+    if (C.g == 1.0) {
+        t0 = C.h0 * pan;
+        t1 = C.h0 * (pan + 1);
+    } else {
+        const double gp = pow(C.g, pan);
+        t0 = C.h0 * (gp - 1.0) / (C.g - 1.0);
+        t1 = C.h0 * (gp * C.g - 1.0) / (C.g - 1.0);
+    }
+    const double t = t0 + 0.5 * (x + 1.0) * (t1 - t0), wt = 0.5 * gw * (t1 - t0);
+    const zd e = side > 0 ? zd{C.cphi, C.sphi} : zd{-C.cphi, C.sphi};
+    *lam = zd{side > 0 ? C.c : -C.c, 0.0} + t * e;
+    *dl = (side > 0 ? wt : -wt) * e; // the left ray runs from infinity to -c
+}
+
 #define TB_CHUNK 16
-// One class's table.  The integrand is sig(lambda) e^{i lambda dx - s2 ht - ss hs} / s2
+// One class's table of the cross-layer operator (the middle layer's own image terms need one
+// integral per order sum: lmfmm_tables.cu).  The integrand is sig(lambda) e^{i lambda dx - s2 ht - ss hs} / s2
 // with target Z_t = (lambda + tau s2)/k2 (scale sc = k2 w) and source
 // Z_s = (lambda + vs ss)/ks (scale scs = ks w), ss = sqrt(lambda^2 - ks^2); the
-// density functor sigf(lambda, &s2, &ss) returns sig.  ks = k2 (ss = s2) for
-// the middle layer's image terms; ks = k1 for the layer-1 sources of the
-// cross-layer operator.
+// density functor sigf(lambda, &s2, &ss) returns sig; ks = k1 for the layer-1
+// sources.
 template <class SigF>
 __device__ inline void m2l_table_body(SigF sigf, double km, double kmin, double k2, double ks, int P, double sc,
                                double scs, int tau, int vs, double dx, double ht, double hs, zd *tabout,
@@ -122,39 +245,10 @@ __device__ inline void m2l_table_body(SigF sigf, double km, double kmin, double 
     zd *ZT = (zd *)smem;                 // [TB_CHUNK][np]
     zd *ZS = ZT + TB_CHUNK * np;         // [TB_CHUNK][np]
     zd *BW = ZS + TB_CHUNK * np;         // [TB_CHUNK]
-    const double h = ht + hs;
-    double c = 1.5 * km + 1.0;
-    double a = fmin(0.5, 1.0 / fmax(fabs(dx), 1e-3));
-    double delta = fmin(0.25, 0.5 * kmin);
-    double width = fmin(fmin(0.5, 2.0 * a), 1.5 / fmax(fabs(dx), 1e-3));
-    int nflat = (int)ceil((c - 2.0 * delta) / width);
-    const int ORD = 24;
-    int nseg_half = (nflat + 2) * ORD;
-    double rho = hypot(dx, h);
-    double tmax = 1.5 * (2.0 * P + 60.0) / rho;
-    // Panels of ORD nodes on [0, tmax], geometrically graded: the first is at
-    // most 1 wide (low orders vary on the scale of c near the start of the ray),
-    // later ones widen by the ratio g (high orders peak near t = 2P / rho).
-    // Uniform panels lost accuracy for small boxes, where tmax ~ 1/rho is large.
-    const int TPAN = P + 16 > 32 ? P + 16 : 32;
-    const double h0 = fmin(1.0, tmax / TPAN);
-    double g = 1.0;
-    if (h0 * TPAN < tmax) { // solve h0 (g^TPAN - 1)/(g - 1) = tmax for g > 1 by bisection
-        double lo = 1.0, hi = 2.0;
-        while (h0 * (pow(hi, TPAN) - 1.0) / (hi - 1.0) < tmax) hi *= 2.0;
-        for (int it = 0; it < 100; ++it) {
-            const double mid = 0.5 * (lo + hi);
-            if (h0 * (pow(mid, TPAN) - 1.0) / (mid - 1.0) < tmax) lo = mid;
-            else hi = mid;
-        }
-        g = hi;
-    }
-    auto tpan = [&](int j) { return g == 1.0 ? h0 * j : h0 * (pow(g, j) - 1.0) / (g - 1.0); };
-    int ntail = TPAN * ORD;
-    int ntot = 2 * nseg_half + 2 * ntail;
-    double phi = atan2(dx, h);
-    zd er = {cos(phi), sin(phi)};       // right ray direction
-    zd el = {-cos(phi), sin(phi)};      // left ray direction: -e^{-i phi}
+    __shared__ TabContour C;
+    if (threadIdx.x == 0) C = tab_contour(km, kmin, P, dx, ht + hs);
+    __syncthreads();
+    const int nseg_half = C.nseg(), ntail = C.ntail(), ntot = 2 * nseg_half + 2 * ntail;
     // accumulators: each thread owns entries idx = tid + k*blockDim
     const int MAXE = (2 * LM_MAXP + 1) * (2 * LM_MAXP + 1);
     (void)MAXE;
@@ -174,46 +268,11 @@ __device__ inline void m2l_table_body(SigF sigf, double km, double kmin, double 
             zd lam = {0.0, 0.0}, dl = {0.0, 0.0};
             bool valid = i < ntot;
             if (valid) {
-                if (i < 2 * nseg_half) {
-                    int side = i < nseg_half ? 1 : -1;
-                    int ii = i % nseg_half, pan = ii / ORD, j = ii % ORD;
-                    double x, gw;
-                    gl_node(ORD, j, &x, &gw);
-                    zd z0, z1;
-                    double flat = (c - 2.0 * delta) / nflat;
-                    if (pan == 0) {
-                        z0 = {0.0, 0.0};
-                        z1 = {delta, -a};
-                    } else if (pan == nflat + 1) {
-                        z0 = {c - delta, -a};
-                        z1 = {c, 0.0};
-                    } else {
-                        z0 = {delta + (pan - 1) * flat, -a};
-                        z1 = {delta + pan * flat, -a};
-                    }
-                    zd dz = z1 - z0;
-                    lam = z0 + (0.5 * (x + 1.0)) * dz;
-                    dl = (0.5 * gw) * dz;
-                    if (side < 0) {
-                        // mirror through the origin; orientation -c -> 0 keeps dl
-                        lam = -lam;
-                    }
-                } else {
-                    int ii = i - 2 * nseg_half;
-                    int side = ii < ntail ? 1 : -1;
-                    ii %= ntail;
-                    int pan = ii / ORD, j = ii % ORD;
-                    double x, gw;
-                    gl_node(ORD, j, &x, &gw);
-                    double t0 = tpan(pan), t1 = tpan(pan + 1);
-                    double t = t0 + 0.5 * (x + 1.0) * (t1 - t0), wt = 0.5 * gw * (t1 - t0);
-                    if (side > 0) {
-                        lam = zd{c, 0.0} + t * er;
-                        dl = wt * er;
-                    } else {
-                        lam = zd{-c, 0.0} + t * el;
-                        dl = -wt * el; // runs from -inf to -c
-                    }
+                if (i < 2 * nseg_half)
+                    tab_node(C, i % nseg_half, i < nseg_half ? 1 : -1, &lam, &dl);
+                else {
+                    const int ii = i - 2 * nseg_half;
+                    tab_node(C, nseg_half + ii % ntail, ii < ntail ? 1 : -1, &lam, &dl);
                 }
                 zd s2, ss;
                 const zd sg = sigf(lam, &s2, &ss);
