@@ -51,7 +51,7 @@ typedef enum {
 } lm_status;
 
 typedef enum {
-    LM_FP64 = 0, /* every step in IEEE double */
+    LM_FP64 = 0, /* FP64 tables and potentials; see lm_options.m2l_fp64 for the apply's arithmetic */
     LM_MIXED = 1 /* tables built in FP64 and rounded to FP32; expansions, M2L and
                     near field in FP32 with FP32 accumulation; p in {4, 6, 8..14, 16,
                     18, 20, 24} */
@@ -89,12 +89,14 @@ typedef struct {
                         lists built by a dual traversal (see lm_build_tree).  Both precisions:
                         LM_MIXED trees run M2L between any two levels on the CUDA-core staged
                         contraction, the other steps on the box lists.  0 (default): uniform depth. */
-    int m2l_fp64;    /* LM_FP64 trees: 1 runs the M2L, M2M and L2L contractions in IEEE FP64;
-                        0 (default) runs them in double-float on the FP32 pipes -- each value a pair of
-                        FP32 numbers (48-bit significand), exact products by fma and
-                        error-free sums, densities scaled by a power of two per apply so
-                        the expansions stay inside FP32's exponent range; about 1e-14
-                        relative, and several times the FP64 pipe's rate on GB300. */
+    int m2l_fp64;    /* LM_FP64 trees: 1 runs every step of an apply in IEEE FP64; 0 (default) runs the
+                        expansions and the direct interactions in double-float on the FP32
+                        pipes -- each value a pair of FP32 numbers (48-bit significand), exact
+                        products by fma and error-free sums, densities scaled by a power of two
+                        per apply so the values stay inside FP32's exponent range; about 1e-14
+                        relative, and many times the FP64 pipe's rate on GB300.  Tables,
+                        quadratures and potentials are FP64 either way.  Trees whose leaves are
+                        wider than 140 / k2 take FP64 throughout. */
     int tensor_leaf; /* LM_MIXED uniform trees, p <= 14, applies of 5-16 vectors: the leaf step's
                         multiply-adds over the vectors (direct S2T pairs and L2T) on the tcgen05
                         tensor cores, the kernel values on the CUDA cores (FP16 hi/lo split of both

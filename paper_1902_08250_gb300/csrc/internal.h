@@ -113,10 +113,8 @@ struct Level {
     zd *m2m;         // [4][np][np]: child (level l+1) -> this level's box (l < L)
     zd *l2l;         // [4][np][np]: parent (level l-1) -> child at this level (l > 0)
     zd *M, *Lc;      // [nbox][np][LM_MAXV]
-    // FP64 form, double-float M2L: tables and multipoles as (re hi, re lo, im hi, im lo)
-    float4 *tabdf;   // [nclass][np][np]
-    float4 *tabdft;  // the same, each table transposed ([q][p])
-    float4 *Mdf;     // [nbox][np][LM_MAXV], scaled by 2^-qexp
+    // FP64 form in double-float: tables as (re hi, re lo, im hi, im lo), each transposed ([q][p])
+    float4 *tabdft;  // [nclass][np][np]
     float4 *m2mdf, *l2ldf; // [4][np][np] copies of m2m, l2l
     // mixed-precision copies (FP32, rounded from the FP64 tables)
     zf *tab32;       // [nclass][np][np]
@@ -157,11 +155,32 @@ struct AdaptTree {
     int32_t *vsrc = nullptr, *vslot = nullptr, *vterm = nullptr;
     zd *tab = nullptr;                                 // [nclass][np][np] scaled M2L tables
     zd *M = nullptr, *Lc = nullptr;                    // [nbox][np][LM_MAXV]
-    float4 *tabdf = nullptr, *tabdft = nullptr, *Mdf = nullptr; // double-float copies (as Level)
+    float4 *tabdft = nullptr;                          // double-float copy (as Level)
     // mixed form: FP32 copies of the tables and expansions, and per level the boxes with V entries
     zf *tab32 = nullptr, *M32 = nullptr, *L32 = nullptr;
     std::vector<int32_t *> m2l_tgt;
     std::vector<int64_t> m2l_ntgt;
+};
+
+// Double-float near field of the FP64 form (lmfmm_near_df.cu); coordinates scaled by k2/2
+struct NearTabDF {
+    bool ready;
+    double zmax, wmax;      // largest (k2 r / 2)^2 of a free pair; width of the widest leaf
+    float4 *node, *w, *w2;  // tail nodes [ray][node][2], weights [term][ray][node][2] (w2: see NearQuad::split)
+    float4 *seg, *segw;     // segment nodes [node][2], weights [term][node]
+    float4 *rel, *hgt;      // [n] offset from the leaf centre; y and y + d
+    float4 *q;              // [n][nvec] densities of the apply, scaled by 2^-qexp
+    float4 *node_g, *w_g, *w2_g, *segw_g; // target gradient: its tails and per-pair segment weights
+};
+// Double-float expansions of the FP64 form (lmfmm_exp_df.cu): the M and Lc arrays then hold float4
+// (re hi, re lo, im hi, im lo) scaled by 2^-qexp, [box][2p+1][nvec]
+struct ExpDF {
+    bool ready;
+    float2 *bes; // coefficients of the Bessel basis (BesselDF)
+    int N, nt;
+    void *lev;   // device M2LLevelDF[nlev]
+    int nlev;
+    int64_t nblk; // boxes of all levels
 };
 
 struct lm_tree_s {
@@ -220,7 +239,9 @@ struct lm_tree_s {
     bool adaptive;  // boxes refined where the points are (AdaptTree), FP64 only
     AdaptTree at;
     int *dflag;  // device error flag
-    bool m2l_df; // FP64 form: M2L contraction in double-float on the FP32 pipes
+    bool m2l_df; // FP64 form: expansions and direct interactions in double-float on the FP32 pipes
+    NearTabDF ndf;
+    ExpDF xdf;
     int *qexp;   // device: binary exponent of the largest |density| component of the apply
     int64_t bytes;
     // phase profiling
@@ -273,7 +294,15 @@ lm_status lm_run_apply(lm_tree_s *t, const zd *q, int nvec, zd *u, bool adjoint,
 size_t lm_near_pw64_smem(int nseg);
 lm_status lm_near_pw64_attr(size_t bytes);
 lm_status lm_setup_pwsrc(lm_tree_s *t, cudaStream_t st); // interface-leaf slots and coefficient buffer
-lm_status lm_setup_df(lm_tree_s *t, cudaStream_t st); // double-float tables and multipole buffers
+lm_status lm_setup_df(lm_tree_s *t, cudaStream_t st); // the FP64 form's double-float data
+lm_status lm_setup_near_df(lm_tree_s *t, cudaStream_t st); // double-float near field (lmfmm_near_df.cu)
+void lm_launch_q_df(lm_tree_s *t, int nv, cudaStream_t st);
+lm_status lm_launch_near_df(lm_tree_s *t, int nv, cudaStream_t st, int *launches);
+lm_status lm_launch_near_grad_df(lm_tree_s *t, int nvq, int v0, int nv, zd *u, zd *ux, zd *uy, cudaStream_t st);
+lm_status lm_launch_near64(lm_tree_s *t, int v0, int nv, zd *u, zd *ux, zd *uy, cudaStream_t st);
+bool lm_exp_df_fits(double k2, double wmax);                // double-float expansions (lmfmm_exp_df.cu)
+lm_status lm_setup_exp_df(lm_tree_s *t, cudaStream_t st);
+lm_status lm_run_df(lm_tree_s *t, const zd *q, int nvec, zd *u, bool adjoint, zd *ux, zd *uy, cudaStream_t st);
 lm_status lm_run_apply_grad(lm_tree_s *t, const zd *q, int nvec, zd *u, zd *ux, zd *uy, cudaStream_t st);
 // mixed precision (lmfmm_mixed.cu)
 lm_status lm_setup_mixed(lm_tree_s *t, cudaStream_t st);

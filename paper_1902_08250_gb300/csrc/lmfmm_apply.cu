@@ -2,42 +2,11 @@
 // evaluation) as device kernels, FP64 form.
 #include <algorithm>
 
+#include "df.cuh"
 #include "internal.h"
+#include "near64.cuh"
 
 static int gridn(int64_t n, int b) { return (int)((n + b - 1) / b); }
-
-// Box geometry of a launch: block i works on box id(i), whose centre and width
-// come from centre().
-struct GridLeaves { // uniform tree: leaf i of the leaf lattice
-    LeafGeom g;
-    __device__ int64_t id(int64_t i) const { return i; }
-    __device__ void centre(int64_t b, double *cx, double *cy, double *w) const
-    {
-        leaf_centre(g, b, cx, cy);
-        *w = g.w;
-    }
-};
-struct EdgeRowLeaves { // uniform tree: the leaves of the top row, then (nrow > 1) of the bottom row
-    LeafGeom g;
-    int64_t nrow;
-    __device__ int64_t id(int64_t i) const { return ((nrow == 1 || i < g.ncol) ? 0 : nrow - 1) * g.ncol + i % g.ncol; }
-    __device__ void centre(int64_t b, double *cx, double *cy, double *w) const
-    {
-        leaf_centre(g, b, cx, cy);
-        *w = g.w;
-    }
-};
-struct ListBoxes { // adaptive tree: box ids[i], centres and widths from arrays
-    const int32_t *ids;
-    const double *bx, *by, *bw;
-    __device__ int64_t id(int64_t i) const { return ids[i]; }
-    __device__ void centre(int64_t b, double *cx, double *cy, double *w) const
-    {
-        *cx = bx[b];
-        *cy = by[b];
-        *w = bw[b];
-    }
-};
 
 // q (input order, [nvec][n]) -> qs (tree order, [nvec][n]), optionally conjugated
 __global__ void k_permute_in(const zd *q, const int64_t *perm, int64_t n, int nvec, int conjugate,
@@ -236,60 +205,6 @@ __global__ void k_m2l64(int64_t nbox, int P, int nvec, const int64_t *vstart, co
     Lc[(b * np + p) * LM_MAXV + v] += acc;
 }
 
-// ---------------------------------------------------------------------------
-// M2L in double-float on the FP32 pipes (Dekker's representation: a value is
-// hi + lo, two FP32 numbers with |lo| <= ulp(hi)/2, 48 significand bits).  A
-// product is exact as p + e with p = hi*hi rounded and e = fma(hi, hi, -p),
-// plus the two cross terms; a sum is made exact by Knuth's TwoSum, whose
-// error joins the running low word.  The FP64 form keeps every other step in
-// IEEE FP64; GB300 issues FP32 at about 60 times its FP64 rate, so the
-// 48 FP32 instructions of a complex multiply-add cost less than its 4 DFMAs.
-// Multipoles are scaled by 2^-qexp (qexp: the binary exponent of the largest
-// density component of the apply), so that they stay inside FP32's exponent
-// range; tables are scaled (S_l) and of order one already.
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ float4 df_split(zd a)
-{
-    const float rh = __double2float_rn(a.re), ih = __double2float_rn(a.im);
-    return make_float4(rh, __double2float_rn(a.re - (double)rh), ih, __double2float_rn(a.im - (double)ih));
-}
-// (sh, sl) += (ah + al)(bh + bl)
-__device__ __forceinline__ void df_mac(float &sh, float &sl, float ah, float al, float bh, float bl)
-{
-    const float p = __fmul_rn(ah, bh);
-    float e = fmaf(ah, bh, -p);
-    e = fmaf(ah, bl, e);
-    e = fmaf(al, bh, e);
-    const float s = __fadd_rn(sh, p);
-    const float bb = __fsub_rn(s, sh);
-    const float err = __fadd_rn(__fsub_rn(sh, __fsub_rn(s, bb)), __fsub_rn(p, bb));
-    sh = s;
-    sl = __fadd_rn(sl, __fadd_rn(err, e));
-}
-// complex: acc += t m, each part a double-float (x, y) = real, (z, w) = imaginary
-__device__ __forceinline__ void dfc_mac(float4 &acc, const float4 t, const float4 m)
-{
-    df_mac(acc.x, acc.y, t.x, t.y, m.x, m.y);
-    df_mac(acc.x, acc.y, -t.z, -t.w, m.z, m.w);
-    df_mac(acc.z, acc.w, t.x, t.y, m.z, m.w);
-    df_mac(acc.z, acc.w, t.z, t.w, m.x, m.y);
-}
-
-__global__ void k_tab_df(const zd *tab, int64_t count, float4 *out)
-{
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i < count) out[i] = df_split(tab[i]);
-}
-// the same, each np x np table transposed ([q][p])
-__global__ void k_tab_df_t(const zd *tab, int64_t count, int np, float4 *out)
-{
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= count) return;
-    const int64_t slot = i / ((int64_t)np * np);
-    const int r = (int)(i % ((int64_t)np * np)), p = r / np, q = r % np;
-    out[slot * np * np + (int64_t)q * np + p] = df_split(tab[i]);
-}
-
 // largest |re|, |im| of the densities [nvec][n] -> its binary exponent, max-reduced into *qexp
 __global__ void k_qexp(const zd *qs, int64_t n, int nvec, int *qexp)
 {
@@ -305,229 +220,8 @@ __global__ void k_qexp(const zd *qs, int64_t n, int nvec, int *qexp)
         atomicMax(qexp, e);
     }
 }
-__device__ __forceinline__ int qexp_of(const int *qexp)
-{
-    const int e = *qexp;
-    return e < -1000 ? 0 : e; // all densities zero: no scaling
-}
-
-// multipoles of boxes b0 .. b0 + nb - 1 -> double-float, scaled by 2^-qexp
-__global__ void k_m_df(int64_t b0, int64_t nb, int P, int nvec, const zd *M, const int *qexp, float4 *Mdf)
-{
-    const int np = 2 * P + 1;
-    const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (idx >= nb * np * nvec) return;
-    const int v = idx % nvec;
-    const int64_t r = (b0 * np + idx / nvec) * LM_MAXV + v; // row (box, q), vector v
-    const int e = -qexp_of(qexp);
-    const zd a = M[r];
-    Mdf[r] = df_split(zd{ldexp(a.re, e), ldexp(a.im, e)});
-}
-
-// M2L over the V list, double-float: one thread per (target box, order p, vector).
-// TR: tables transposed ([q][p]).  With few vectors a warp spans 32 orders p of one
-// box, and the transposed rows make its table reads contiguous; with many vectors
-// a warp spans 2 orders, each thread reads its own row, and the row-major layout
-// keeps a thread's reads on few cache lines.
-template <bool TR>
-__global__ void __launch_bounds__(128) k_m2l_df(int64_t nbox, int P, int nvec, const int64_t *vstart,
-                                                const int32_t *vsrc, const int32_t *vslot, const float4 *tab,
-                                                const float4 *Mdf, const int *qexp, zd *Lc)
-{
-    const int np = 2 * P + 1;
-    const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (idx >= nbox * np * nvec) return;
-    const int v = idx % nvec;
-    const int p = (idx / nvec) % np;
-    const int64_t b = idx / (nvec * np);
-    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int64_t e = vstart[b]; e < vstart[b + 1]; ++e) {
-        const float4 *T = tab + (int64_t)vslot[e] * np * np + (TR ? p : (int64_t)p * np);
-        const int ts = TR ? np : 1;
-        const float4 *m = Mdf + (int64_t)vsrc[e] * np * LM_MAXV + v;
-        for (int q = 0; q < np; ++q) dfc_mac(acc, T[q * ts], m[q * LM_MAXV]);
-    }
-    const int ex = qexp_of(qexp);
-    zd &o = Lc[(b * np + p) * LM_MAXV + v];
-    o = o + zd{ldexp((double)acc.x + (double)acc.y, ex), ldexp((double)acc.z + (double)acc.w, ex)};
-}
-
-// M2M and L2L in double-float: one block per parent box.  The parent's children
-// (M2M: their multipoles, one child position at a time) or the parent's local
-// expansion (L2L) are converted once into shared memory, scaled by 2^-qexp;
-// each thread accumulates up to DF_MAXO outputs (order, vector).
-#define DF_THREADS 128
-#define DF_TR_NV 2 // applies of up to this many vectors read the transposed M2L tables
-#define DF_MAXO 13 // (2 * LM_MAXP + 1) * LM_MAXV / DF_THREADS, rounded up
-// threads of a double-float M2M / L2L block: 64 while its outputs (M2M: one box, L2L: four children)
-// fit, else DF_THREADS
-static int df_threads(int nout) { return nout <= 64 ? 64 : DF_THREADS; }
 // threads of an S2M block: the (order, vector) entries rounded up to warps, 64 to 256
 static int p2m_threads(int nent) { return std::max(64, std::min(256, (nent + 31) / 32 * 32)); }
-struct GridParents { // uniform tree: parent i of a level with ncol columns; children one level down
-    int64_t ncol;
-    __device__ int64_t parent(int64_t i) const { return i; }
-    __device__ int64_t child(int64_t b, int pos) const
-    {
-        const int64_t r = b / ncol, c = b % ncol;
-        return (2 * r + (pos >> 1)) * (2 * ncol) + 2 * c + (pos & 1);
-    }
-};
-struct ListParents { // adaptive tree: parent ids[i], children from the box links
-    const int32_t *ids, *kids;
-    __device__ int64_t parent(int64_t i) const { return ids[i]; }
-    __device__ int64_t child(int64_t b, int pos) const { return kids[4 * b + pos]; }
-};
-
-template <class Geo>
-__global__ void __launch_bounds__(DF_THREADS) k_m2m_df(Geo geo, int P, int nvec, const float4 *tabs, const zd *Mc,
-                                                       const int *qexp, zd *Mp)
-{
-    extern __shared__ float4 sm4[]; // [np][nvec]: one child's multipole
-    const int np = 2 * P + 1, nout = np * nvec;
-    const int64_t b = geo.parent(blockIdx.x);
-    const int e = qexp_of(qexp);
-    float4 acc[DF_MAXO];
-#pragma unroll
-    for (int k = 0; k < DF_MAXO; ++k) acc[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int pos = 0; pos < 4; ++pos) {
-        const int64_t ch = geo.child(b, pos);
-        __syncthreads();
-        for (int i = threadIdx.x; i < nout; i += blockDim.x) {
-            const zd a = Mc[(ch * np + i / nvec) * LM_MAXV + i % nvec];
-            sm4[i] = df_split(zd{ldexp(a.re, -e), ldexp(a.im, -e)});
-        }
-        __syncthreads();
-#pragma unroll
-        for (int k = 0; k < DF_MAXO; ++k) {
-            const int o = threadIdx.x + k * blockDim.x;
-            if (o < nout) {
-                const int p = o / nvec, v = o % nvec;
-                const float4 *T = tabs + ((int64_t)pos * np + p) * np;
-                for (int q = 0; q < np; ++q) dfc_mac(acc[k], T[q], sm4[q * nvec + v]);
-            }
-        }
-    }
-#pragma unroll
-    for (int k = 0; k < DF_MAXO; ++k) {
-        const int o = threadIdx.x + k * blockDim.x;
-        if (o < nout)
-            Mp[(b * np + o / nvec) * LM_MAXV + o % nvec] =
-                zd{ldexp((double)acc[k].x + (double)acc[k].y, e), ldexp((double)acc[k].z + (double)acc[k].w, e)};
-    }
-}
-
-template <class Geo>
-__global__ void __launch_bounds__(DF_THREADS) k_l2l_df(Geo geo, int P, int nvec, const float4 *tabs, const zd *Lp,
-                                                       const int *qexp, zd *Lc)
-{
-    extern __shared__ float4 sm4[]; // [np][nvec]: the parent's local expansion
-    const int np = 2 * P + 1, nout = np * nvec;
-    const int64_t b = geo.parent(blockIdx.x);
-    const int e = qexp_of(qexp);
-    for (int i = threadIdx.x; i < nout; i += blockDim.x) {
-        const zd a = Lp[(b * np + i / nvec) * LM_MAXV + i % nvec];
-        sm4[i] = df_split(zd{ldexp(a.re, -e), ldexp(a.im, -e)});
-    }
-    __syncthreads();
-    for (int o = threadIdx.x; o < 4 * nout; o += blockDim.x) {
-        const int pos = o / nout, r = o % nout, p = r / nvec, v = r % nvec;
-        const float4 *T = tabs + ((int64_t)pos * np + p) * np;
-        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int q = 0; q < np; ++q) dfc_mac(acc, T[q], sm4[q * nvec + v]);
-        Lc[(geo.child(b, pos) * np + p) * LM_MAXV + v] =
-            zd{ldexp((double)acc.x + (double)acc.y, e), ldexp((double)acc.z + (double)acc.w, e)};
-    }
-}
-
-// ---------------------------------------------------------------------------
-// Free-space kernel (i/4) H0^(1)(x) = (i/4)(J0(x) + i Y0(x)) of a near pair in
-// FP64.  For x <= 2 the ascending series (Abramowitz & Stegun 9.1.12, 9.1.13),
-// with z = x^2/4:
-//   J0 = sum_m (-z)^m / (m!)^2,
-//   Y0 = (2/pi) [(ln(x/2) + gamma) J0 - sum_{m>=1} H_m (-z)^m / (m!)^2],
-// H_m the harmonic numbers, gamma Euler's constant; 14 terms leave the first
-// omitted one below 2e-21 for z <= 1 (within 5e-16 of scipy's J0, Y0 on
-// (0, 2]).  Horner form: 28 FMAs and one log in place of the library's j0 and
-// y0 (1M FP64 strip: leaf kernel 72.0 -> 65.7 ms).  Larger x: j0, y0.
-// ---------------------------------------------------------------------------
-#define H0S_TERMS 14
-struct H0Series {
-    double cj[H0S_TERMS], cy[H0S_TERMS]; // (-1)^m / (m!)^2, -(-1)^m H_m / (m!)^2
-    constexpr H0Series() : cj(), cy()
-    {
-        double f = 1.0, h = 0.0; // 1/(m!)^2, H_m
-        for (int m = 0; m < H0S_TERMS; ++m) {
-            if (m > 0) {
-                f /= (double)m * (double)m;
-                h += 1.0 / m;
-            }
-            cj[m] = (m & 1) ? -f : f;
-            cy[m] = (m & 1) ? h * f : -h * f;
-        }
-    }
-};
-__constant__ H0Series c_h0s = H0Series();
-// J1 and Y1 for the target gradient (A&S 9.1.10, 9.1.11 with n = 1):
-//   J1 = (x/2) sum_m (-z)^m / (m! (m+1)!),
-//   Y1 = -2/(pi x) + (2/pi) ln(x/2) J1 - (x/(2 pi)) sum_m (-z)^m (psi(m+1) + psi(m+2)) / (m! (m+1)!),
-// psi(m+1) = H_m - gamma; within 5e-16 of scipy's J1, Y1 on (0, 2]
-struct H1Series {
-    double c[H0S_TERMS], e[H0S_TERMS]; // (-1)^m / (m! (m+1)!), (-1)^m (psi(m+1) + psi(m+2)) / (m! (m+1)!)
-    constexpr H1Series() : c(), e()
-    {
-        double f = 1.0, h = 0.0; // 1/(m! (m+1)!), H_m
-        for (int m = 0; m < H0S_TERMS; ++m) {
-            if (m > 0) {
-                f /= (double)m * (double)(m + 1);
-                h += 1.0 / m;
-            }
-            const double psi = (h - 0.57721566490153286061) + (h + 1.0 / (m + 1) - 0.57721566490153286061);
-            c[m] = (m & 1) ? -f : f;
-            e[m] = (m & 1) ? -psi * f : psi * f;
-        }
-    }
-};
-__constant__ H1Series c_h1s = H1Series();
-// (i/4) H0^(1)(x) and (i/4) H1^(1)(x) together (series for x <= 2, else the library's)
-__device__ __forceinline__ void h01_free64(double x, zd *h0, zd *h1)
-{
-    if (x > 2.0) {
-        *h0 = zd{-0.25 * y0(x), 0.25 * j0(x)};
-        *h1 = zd{-0.25 * y1(x), 0.25 * j1(x)};
-        return;
-    }
-    const double z = 0.25 * x * x;
-    double j = c_h0s.cj[H0S_TERMS - 1], sy = c_h0s.cy[H0S_TERMS - 1];
-    double a = c_h1s.c[H0S_TERMS - 1], b = c_h1s.e[H0S_TERMS - 1];
-#pragma unroll
-    for (int m = H0S_TERMS - 2; m >= 0; --m) {
-        j = fma(j, z, c_h0s.cj[m]);
-        sy = fma(sy, z, c_h0s.cy[m]);
-        a = fma(a, z, c_h1s.c[m]);
-        b = fma(b, z, c_h1s.e[m]);
-    }
-    const double tpi = 0.63661977236758134308, lg = log(0.5 * x);
-    const double yv0 = tpi * ((lg + 0.57721566490153286061) * j + sy);
-    const double jv1 = 0.5 * x * a;
-    const double yv1 = -tpi / x + tpi * lg * jv1 - 0.5 * tpi * 0.5 * x * b;
-    *h0 = zd{-0.25 * yv0, 0.25 * j};
-    *h1 = zd{-0.25 * yv1, 0.25 * jv1};
-}
-__device__ __forceinline__ zd h0_free64(double x)
-{
-    if (x > 2.0) return zd{-0.25 * y0(x), 0.25 * j0(x)};
-    const double z = 0.25 * x * x;
-    double j = c_h0s.cj[H0S_TERMS - 1], sy = c_h0s.cy[H0S_TERMS - 1];
-#pragma unroll
-    for (int m = H0S_TERMS - 2; m >= 0; --m) {
-        j = fma(j, z, c_h0s.cj[m]);
-        sy = fma(sy, z, c_h0s.cy[m]);
-    }
-    const double y = 0.63661977236758134308 * ((log(0.5 * x) + 0.57721566490153286061) * j + sy);
-    return zd{-0.25 * y, 0.25 * j};
-}
-
 // ---------------------------------------------------------------------------
 // Direct interaction of one reflected term (tt: term 1, bb: term 2) for a
 // pair at horizontal distance X and image height h, by the near-field
@@ -598,7 +292,7 @@ template <class Geo>
 __global__ void __launch_bounds__(LEAF64_THREADS)
     k_leaf64(Geo geo, int P, double k, double d, const double *xs, const double *ys, const int64_t *ls,
              const int64_t *ustart, const int32_t *usrc, const int32_t *uterm, NearQuadD nq, const zd *Lc,
-             const zd *qs, int64_t n, int nvec, int free_on, int pw, zd *us)
+             const zd *qs, int64_t n, int nvec, int free_on, int pw, int l2t, zd *us)
 {
     __shared__ int64_t fj0[LEAF64_UCHUNK]; // first tree position of each entry's source leaf
     __shared__ int fpre[LEAF64_UCHUNK + 1]; // running count of near sources before each entry
@@ -610,7 +304,7 @@ __global__ void __launch_bounds__(LEAF64_THREADS)
     const double sc = k * bw;
     const zd *Lb = Lc + b * np * LM_MAXV;
     const int64_t lo = ls[b], hi = ls[b + 1];
-    for (int64_t i = lo + threadIdx.x; i < hi; i += blockDim.x) {
+    for (int64_t i = lo + threadIdx.x; l2t && i < hi; i += blockDim.x) {
         const double xi = xs[i], yi = ys[i];
         zd acc[LM_MAXV];
         for (int v = 0; v < nvec; ++v) acc[v] = zd{0.0, 0.0};
@@ -880,7 +574,7 @@ template <class Geo>
 __global__ void __launch_bounds__(LEAF64_THREADS) k_leaf64_grad(Geo geo, int P, double k, double d, const double *xs, const double *ys,
                               const int64_t *ls, const int64_t *ustart, const int32_t *usrc,
                               const int32_t *uterm, NearQuadD nq, const zd *Lc, const zd *qs, int64_t n,
-                              int v0, int nv, int free_on, const int64_t *perm, zd *u, zd *ux, zd *uy)
+                              int v0, int nv, int free_on, int l2t, const int64_t *perm, zd *u, zd *ux, zd *uy)
 {
     const int64_t b = geo.id(blockIdx.x);
     double cx, cy, bw;
@@ -890,7 +584,7 @@ __global__ void __launch_bounds__(LEAF64_THREADS) k_leaf64_grad(Geo geo, int P, 
     __shared__ int64_t fj0[LEAF64_UCHUNK];
     __shared__ int fpre[LEAF64_UCHUNK + 1];
     __shared__ int fterm[LEAF64_UCHUNK];
-    for (int64_t i = ls[b] + threadIdx.x; i < ls[b + 1]; i += blockDim.x) {
+    for (int64_t i = ls[b] + threadIdx.x; l2t && i < ls[b + 1]; i += blockDim.x) {
         const double xi = xs[i], yi = ys[i];
         zd a[GV], dp[GV], dm[GV], gxa[GV], gya[GV]; // dp = (d/dx - i d/dy) u, dm = (d/dx + i d/dy) u
         for (int v = 0; v < GV; ++v) a[v] = dp[v] = dm[v] = zd{0.0, 0.0};
@@ -1016,12 +710,49 @@ static lm_status run_fp64(lm_tree_s *t, const zd *q, int nvec, zd *u, bool adjoi
 lm_status lm_run_apply(lm_tree_s *t, const zd *q, int nvec, zd *u, bool adjoint, cudaStream_t st)
 {
     if (t->precision == LM_MIXED) return lm_run_apply_mixed(t, q, nvec, u, adjoint, false, st);
+    if (t->m2l_df) return lm_run_df(t, q, nvec, u, adjoint, nullptr, nullptr, st);
     return run_fp64(t, q, nvec, u, adjoint, nullptr, nullptr, st);
 }
 
 lm_status lm_run_apply_grad(lm_tree_s *t, const zd *q, int nvec, zd *u, zd *ux, zd *uy, cudaStream_t st)
 {
+    if (t->m2l_df) return lm_run_df(t, q, nvec, u, false, ux, uy, st);
     return run_fp64(t, q, nvec, u, false, ux, uy, st);
+}
+
+// The near-field tables of a launch; the target gradient integrates its differentiated tails with
+// the longer rule
+static NearQuadD near_quad(const lm_tree_s *t, bool grad)
+{
+    const NearQuad &q = t->nq;
+    if (!grad)
+        return NearQuadD{q.nseg, q.nray, q.ntail, q.seg_lam, q.seg_s2, q.seg_w, q.tail_lam, q.tail_s2, q.tail_w,
+                         {q.rinf[0], q.rinf[1]}, q.hray, q.tail_w2, q.a_zero, 2.0 * t->med.d, nullptr, nullptr, {0.0, 0.0}};
+    return NearQuadD{q.nseg, q.nray, q.ntail_g, q.seg_lam, q.seg_s2, q.seg_w, q.tail_lam_g, q.tail_s2_g, q.tail_w_g,
+                     {q.rinf[0], q.rinf[1]}, q.hray, q.tail_w2_g, q.a_zero, 2.0 * t->med.d, q.seg_c, q.tail_c_g,
+                     {q.beta[0], q.beta[1]}};
+}
+
+// Direct interactions in FP64 beside double-float expansions (media whose segment coefficients do not
+// fit in shared memory): vectors v0 .. v0 + nv - 1 of t->qs, added to t->us or (ux set, nv <= 4) to u, ux, uy
+lm_status lm_launch_near64(lm_tree_s *t, int v0, int nv, zd *u, zd *ux, zd *uy, cudaStream_t st)
+{
+    const NearQuadD nq = near_quad(t, ux != nullptr);
+    const double k = t->med.k2, d = t->med.d;
+    const int free_on = t->med.opt.kernel == LM_KERNEL_G;
+    auto run = [&](auto geo, int64_t nleaf, const zd *Lc) {
+        if (ux)
+            k_leaf64_grad<<<(unsigned)nleaf, LEAF64_THREADS, 0, st>>>(geo, t->p, k, d, t->xs, t->ys, t->leaf_start, t->ustart,
+                                                                      t->usrc, t->uterm, nq, Lc, t->qs, t->n, v0, nv, free_on, 0,
+                                                                      t->perm, u, ux, uy);
+        else
+            k_leaf64<<<(unsigned)nleaf, LEAF64_THREADS, 0, st>>>(geo, t->p, k, d, t->xs, t->ys, t->leaf_start, t->ustart, t->usrc,
+                                                                 t->uterm, nq, Lc, t->qs, t->n, nv, free_on, 0, 0, t->us);
+    };
+    if (t->adaptive) run(ListBoxes{t->at.leaves, t->at.cx, t->at.cy, t->at.w}, t->at.nleaf, t->at.Lc);
+    else run(GridLeaves{LeafGeom{t->lev[t->L].ncol, t->x0, t->lev[t->L].w}}, t->lev[t->L].nbox, t->lev[t->L].Lc);
+    LM_CUDA(cudaGetLastError());
+    return LM_OK;
 }
 
 // FP64 driver of the adaptive tree: the same steps over the box lists of each level
@@ -1032,26 +763,14 @@ static lm_status run_fp64_adaptive(lm_tree_s *t, const zd *q, int nvec, zd *u, b
     const int L = t->L, P = t->p, np = 2 * P + 1;
     const int64_t n = t->n;
     const double k = t->med.k2;
-    NearQuadD nq{t->nq.nseg, t->nq.nray, t->nq.ntail, t->nq.seg_lam, t->nq.seg_s2,
-                 t->nq.seg_w, t->nq.tail_lam, t->nq.tail_s2, t->nq.tail_w, {t->nq.rinf[0], t->nq.rinf[1]}, t->nq.hray,
-                 t->nq.tail_w2, t->nq.a_zero, 2.0 * t->med.d, nullptr, nullptr, {0.0, 0.0}};
-    // the target gradient integrates its differentiated tails with the longer rule
-    const NearQuadD nqg{t->nq.nseg,     t->nq.nray,       t->nq.ntail_g,   t->nq.seg_lam,
-                        t->nq.seg_s2,   t->nq.seg_w,      t->nq.tail_lam_g, t->nq.tail_s2_g,
-                        t->nq.tail_w_g, {t->nq.rinf[0], t->nq.rinf[1]}, t->nq.hray,
-                        t->nq.tail_w2_g, t->nq.a_zero, 2.0 * t->med.d,
-                        t->nq.seg_c, t->nq.tail_c_g, {t->nq.beta[0], t->nq.beta[1]}};
+    const NearQuadD nq = near_quad(t, false), nqg = near_quad(t, true);
     const ListBoxes leaves{A.leaves, A.cx, A.cy, A.w}, pwl{A.pwleaves, A.cx, A.cy, A.w};
     const int free_on = t->med.opt.kernel == LM_KERNEL_G;
     for (int v0 = 0; v0 < nvec; v0 += LM_MAXV) {
         const int nv = std::min(LM_MAXV, nvec - v0);
         lm_phase_begin(t, PH_PERMUTE, st);
         k_permute_in<<<gridn(n, 256), 256, 0, st>>>(q + (int64_t)v0 * n, t->perm, n, nv, adjoint, t->qs);
-        if (t->m2l_df) {
-            LM_CUDA(cudaMemsetAsync(t->qexp, 0x80, sizeof(int), st)); // below any exponent
-            k_qexp<<<std::min(1024, gridn(n * nv, 256)), 256, 0, st>>>(t->qs, n, nv, t->qexp);
-        }
-        lm_phase_end(t, PH_PERMUTE, st, t->m2l_df ? 2 : 1);
+        lm_phase_end(t, PH_PERMUTE, st, 1);
         // step 2: S2M at every leaf, M2M up the levels
         lm_phase_begin(t, PH_S2M, st);
         const size_t shm = (P2M_CHUNK * np + P2M_CHUNK * LM_MAXV) * sizeof(zd);
@@ -1063,42 +782,23 @@ static lm_status run_fp64_adaptive(lm_tree_s *t, const zd *q, int nvec, zd *u, b
         for (int l = L - 1; l >= 0; --l) {
             const int64_t npar = A.nl_start[l + 1] - A.nl_start[l];
             if (npar == 0) continue;
-            if (t->m2l_df)
-                k_m2m_df<<<(unsigned)npar, df_threads(np * nv), np * nv * sizeof(float4), st>>>(
-                    ListParents{A.nonleaf + A.nl_start[l], A.child}, P, nv, t->lev[l].m2mdf, A.M, t->qexp, A.M);
-            else
-                k_m2m64a<<<gridn(npar * np * nv, 128), 128, 0, st>>>(npar, A.nonleaf + A.nl_start[l], A.child, P,
+            k_m2m64a<<<gridn(npar * np * nv, 128), 128, 0, st>>>(npar, A.nonleaf + A.nl_start[l], A.child, P,
                                                                      nv, t->lev[l].m2m, A.M);
             ++nl;
         }
         lm_phase_end(t, PH_M2M, st, nl);
-        if (t->m2l_df) {
-            lm_phase_begin(t, PH_M2L, st);
-            k_m_df<<<gridn(A.nbox * np * nv, 256), 256, 0, st>>>(0, A.nbox, P, nv, A.M, t->qexp, A.Mdf);
-            lm_phase_end(t, PH_M2L, st, 1);
-        }
         // step 3: level by level, L2L from the parent then M2L from the V list
         for (int l = 0; l <= L; ++l) {
             const int64_t b0 = A.lev_start[l], nb = A.lev_start[l + 1] - b0;
             lm_phase_begin(t, PH_L2L, st);
             if (l == 0)
                 LM_CUDA(cudaMemsetAsync(A.Lc, 0, nb * np * LM_MAXV * sizeof(zd), st));
-            else if (t->m2l_df) {
-                const int64_t npar = A.nl_start[l] - A.nl_start[l - 1]; // the parents of level l
-                k_l2l_df<<<(unsigned)npar, df_threads(4 * np * nv), np * nv * sizeof(float4), st>>>(
-                    ListParents{A.nonleaf + A.nl_start[l - 1], A.child}, P, nv, t->lev[l].l2ldf, A.Lc, t->qexp, A.Lc);
-            } else
+            else
                 k_l2l64a<<<gridn(nb * np * nv, 128), 128, 0, st>>>(b0, nb, A.parent, A.pos, P, nv, t->lev[l].l2l,
                                                                    A.Lc);
             lm_phase_end(t, PH_L2L, st, l > 0);
             lm_phase_begin(t, PH_M2L, st);
-            if (A.lev_nv[l] > 0 && t->m2l_df && nv <= DF_TR_NV)
-                k_m2l_df<true><<<gridn(nb * np * nv, 128), 128, 0, st>>>(
-                    nb, P, nv, A.vstart + b0, A.vsrc, A.vslot, A.tabdft, A.Mdf, t->qexp, A.Lc + b0 * np * LM_MAXV);
-            else if (A.lev_nv[l] > 0 && t->m2l_df)
-                k_m2l_df<false><<<gridn(nb * np * nv, 128), 128, 0, st>>>(
-                    nb, P, nv, A.vstart + b0, A.vsrc, A.vslot, A.tabdf, A.Mdf, t->qexp, A.Lc + b0 * np * LM_MAXV);
-            else if (A.lev_nv[l] > 0)
+            if (A.lev_nv[l] > 0)
                 k_m2l64<<<gridn(nb * np * nv, 128), 128, 0, st>>>(nb, P, nv, A.vstart + b0, A.vsrc, A.vslot, A.tab,
                                                                   A.M, A.Lc + b0 * np * LM_MAXV);
             lm_phase_end(t, PH_M2L, st, A.lev_nv[l] > 0);
@@ -1111,7 +811,7 @@ static lm_status run_fp64_adaptive(lm_tree_s *t, const zd *q, int nvec, zd *u, b
             for (int w0 = 0; w0 < nv; w0 += GV, ++ng)
                 k_leaf64_grad<<<(unsigned)A.nleaf, LEAF64_THREADS, 0, st>>>(
                     leaves, P, k, t->med.d, t->xs, t->ys, t->leaf_start, t->ustart, t->usrc, t->uterm, nqg, A.Lc,
-                    t->qs, n, w0, std::min(GV, nv - w0), free_on, t->perm, u ? u + off + (int64_t)w0 * n : nullptr,
+                    t->qs, n, w0, std::min(GV, nv - w0), free_on, 1, t->perm, u ? u + off + (int64_t)w0 * n : nullptr,
                     ux + off + (int64_t)w0 * n, uy + off + (int64_t)w0 * n);
             lm_phase_end(t, PH_LEAF, st, ng);
             LM_CUDA(cudaGetLastError());
@@ -1119,7 +819,7 @@ static lm_status run_fp64_adaptive(lm_tree_s *t, const zd *q, int nvec, zd *u, b
         }
         const int pw = t->near_pw64 ? 1 : 0;
         k_leaf64<<<(unsigned)A.nleaf, LEAF64_THREADS, 0, st>>>(leaves, P, k, t->med.d, t->xs, t->ys, t->leaf_start, t->ustart,
-                                                   t->usrc, t->uterm, nq, A.Lc, t->qs, n, nv, free_on, pw, t->us);
+                                                   t->usrc, t->uterm, nq, A.Lc, t->qs, n, nv, free_on, pw, 1, t->us);
         if (pw && A.npw > 0) {
             k_pw_src64<<<(unsigned)A.npw, 256, PW64_SRC_SMEM, st>>>(pwl, t->med.d, t->xs, t->ys, t->leaf_start,
                                                                     t->ustart, t->uterm, nq, t->qs, n, nv, t->pwC);
@@ -1144,24 +844,12 @@ static lm_status run_fp64(lm_tree_s *t, const zd *q, int nvec, zd *u, bool adjoi
     const int L = t->L, P = t->p, np = 2 * P + 1;
     const int64_t n = t->n;
     const double k = t->med.k2;
-    NearQuadD nq{t->nq.nseg, t->nq.nray, t->nq.ntail, t->nq.seg_lam, t->nq.seg_s2,
-                 t->nq.seg_w, t->nq.tail_lam, t->nq.tail_s2, t->nq.tail_w, {t->nq.rinf[0], t->nq.rinf[1]}, t->nq.hray,
-                 t->nq.tail_w2, t->nq.a_zero, 2.0 * t->med.d, nullptr, nullptr, {0.0, 0.0}};
-    // the target gradient integrates its differentiated tails with the longer rule
-    const NearQuadD nqg{t->nq.nseg,     t->nq.nray,       t->nq.ntail_g,   t->nq.seg_lam,
-                        t->nq.seg_s2,   t->nq.seg_w,      t->nq.tail_lam_g, t->nq.tail_s2_g,
-                        t->nq.tail_w_g, {t->nq.rinf[0], t->nq.rinf[1]}, t->nq.hray,
-                        t->nq.tail_w2_g, t->nq.a_zero, 2.0 * t->med.d,
-                        t->nq.seg_c, t->nq.tail_c_g, {t->nq.beta[0], t->nq.beta[1]}};
+    const NearQuadD nq = near_quad(t, false), nqg = near_quad(t, true);
     for (int v0 = 0; v0 < nvec; v0 += LM_MAXV) {
         const int nv = std::min(LM_MAXV, nvec - v0);
         lm_phase_begin(t, PH_PERMUTE, st);
         k_permute_in<<<gridn(n, 256), 256, 0, st>>>(q + (int64_t)v0 * n, t->perm, n, nv, adjoint, t->qs);
-        if (t->m2l_df) {
-            LM_CUDA(cudaMemsetAsync(t->qexp, 0x80, sizeof(int), st)); // below any exponent
-            k_qexp<<<std::min(1024, gridn(n * nv, 256)), 256, 0, st>>>(t->qs, n, nv, t->qexp);
-        }
-        lm_phase_end(t, PH_PERMUTE, st, t->m2l_df ? 2 : 1);
+        lm_phase_end(t, PH_PERMUTE, st, 1);
         // step 2: upward pass
         lm_phase_begin(t, PH_S2M, st);
         {
@@ -1176,22 +864,9 @@ static lm_status run_fp64(lm_tree_s *t, const zd *q, int nvec, zd *u, bool adjoi
         for (int l = L - 1; l >= 0; --l) {
             Level &lv = t->lev[l];
             int64_t tot = lv.nbox * np * nv;
-            if (t->m2l_df)
-                k_m2m_df<<<(unsigned)lv.nbox, df_threads(np * nv), np * nv * sizeof(float4), st>>>(
-                    GridParents{lv.ncol}, P, nv, lv.m2mdf, t->lev[l + 1].M, t->qexp, lv.M);
-            else
-                k_m2m64<<<gridn(tot, 128), 128, 0, st>>>(lv.ncol, lv.nbox, P, nv, lv.m2m, t->lev[l + 1].M, lv.M);
+            k_m2m64<<<gridn(tot, 128), 128, 0, st>>>(lv.ncol, lv.nbox, P, nv, lv.m2m, t->lev[l + 1].M, lv.M);
         }
         if (L > 0) lm_phase_end(t, PH_M2M, st, L);
-        if (t->m2l_df) {
-            lm_phase_begin(t, PH_M2L, st);
-            for (int l = 0; l <= L; ++l) {
-                Level &lv = t->lev[l];
-                k_m_df<<<gridn(lv.nbox * np * nv, 256), 256, 0, st>>>(0, lv.nbox, P, nv, lv.M, t->qexp, lv.Mdf);
-            }
-            lm_phase_end(t, PH_M2L, st, L + 1);
-        }
-
         // step 3: downward pass
         for (int l = 0; l <= L; ++l) {
             Level &lv = t->lev[l];
@@ -1199,21 +874,12 @@ static lm_status run_fp64(lm_tree_s *t, const zd *q, int nvec, zd *u, bool adjoi
             lm_phase_begin(t, PH_L2L, st);
             if (l == 0)
                 LM_CUDA(cudaMemsetAsync(lv.Lc, 0, lv.nbox * np * LM_MAXV * sizeof(zd), st));
-            else if (t->m2l_df)
-                k_l2l_df<<<(unsigned)t->lev[l - 1].nbox, df_threads(4 * np * nv), np * nv * sizeof(float4), st>>>(
-                    GridParents{t->lev[l - 1].ncol}, P, nv, lv.l2ldf, t->lev[l - 1].Lc, t->qexp, lv.Lc);
             else
                 k_l2l64<<<gridn(tot, 128), 128, 0, st>>>(lv.ncol, lv.nbox, P, nv, lv.l2l, t->lev[l - 1].Lc,
                                                          lv.Lc);
             lm_phase_end(t, PH_L2L, st, l > 0);
             lm_phase_begin(t, PH_M2L, st);
-            if (lv.nv > 0 && t->m2l_df && nv <= DF_TR_NV)
-                k_m2l_df<true><<<gridn(tot, 128), 128, 0, st>>>(lv.nbox, P, nv, lv.vstart, lv.vsrc, lv.vslot,
-                                                                lv.tabdft, lv.Mdf, t->qexp, lv.Lc);
-            else if (lv.nv > 0 && t->m2l_df)
-                k_m2l_df<false><<<gridn(tot, 128), 128, 0, st>>>(lv.nbox, P, nv, lv.vstart, lv.vsrc, lv.vslot,
-                                                                 lv.tabdf, lv.Mdf, t->qexp, lv.Lc);
-            else if (lv.nv > 0)
+            if (lv.nv > 0)
                 k_m2l64<<<gridn(tot, 128), 128, 0, st>>>(lv.nbox, P, nv, lv.vstart, lv.vsrc, lv.vslot, lv.tab,
                                                          lv.M, lv.Lc);
             lm_phase_end(t, PH_M2L, st, lv.nv > 0);
@@ -1229,7 +895,7 @@ static lm_status run_fp64(lm_tree_s *t, const zd *q, int nvec, zd *u, bool adjoi
             for (int w0 = 0; w0 < nv; w0 += GV, ++nl)
                 k_leaf64_grad<<<(unsigned)lv.nbox, LEAF64_THREADS, 0, st>>>(
                     GridLeaves{g}, P, k, t->med.d, t->xs, t->ys, t->leaf_start, t->ustart, t->usrc, t->uterm, nqg, lv.Lc,
-                    t->qs, n, w0, std::min(GV, nv - w0), free_on, t->perm,
+                    t->qs, n, w0, std::min(GV, nv - w0), free_on, 1, t->perm,
                     u ? u + off + (int64_t)w0 * n : nullptr, ux + off + (int64_t)w0 * n,
                     uy + off + (int64_t)w0 * n);
             lm_phase_end(t, PH_LEAF, st, nl);
@@ -1242,7 +908,7 @@ static lm_status run_fp64(lm_tree_s *t, const zd *q, int nvec, zd *u, bool adjoi
             const int pw = t->near_pw64 ? 1 : 0;
             k_leaf64<<<(unsigned)lv.nbox, LEAF64_THREADS, 0, st>>>(GridLeaves{g}, P, k, t->med.d, t->xs, t->ys, t->leaf_start,
                                                        t->ustart, t->usrc, t->uterm, nq, lv.Lc, t->qs, n,
-                                                       nv, free_on, pw, t->us);
+                                                       nv, free_on, pw, 1, t->us);
             if (pw) {
                 const unsigned npw = (unsigned)(lv.nrow == 1 ? lv.ncol : 2 * lv.ncol);
                 const EdgeRowLeaves er{g, lv.nrow};
@@ -1270,54 +936,24 @@ lm_status lm_near_pw64_attr(size_t bytes)
     return LM_OK;
 }
 
-// double-float copies of the M2L tables, multipole buffers and the exponent slot (FP64 form)
+// the double-float form's own data (FP64 form, unless opt.m2l_fp64 asks for IEEE FP64 throughout);
+// leaves t->m2l_df false where the form does not apply
 lm_status lm_setup_df(lm_tree_s *t, cudaStream_t st)
 {
     if (!t->m2l_df) return LM_OK;
-    const int np = 2 * t->p + 1;
-    LM_CUDA(cudaMalloc((void **)&t->qexp, sizeof(int)));
-    t->bytes += sizeof(int);
-    auto conv = [&](const zd *tab, int64_t ncls, float4 **out) -> lm_status {
-        const int64_t cnt = std::max<int64_t>(1, ncls) * np * np;
-        lm_status s = lm_dalloc(t, out, cnt);
-        if (s != LM_OK) return s;
-        k_tab_df<<<gridn(cnt, 256), 256, 0, st>>>(tab, cnt, *out);
+    double wmax = t->adaptive ? 0.0 : t->lev[t->L].w; // the widest leaf
+    if (t->adaptive)
+        for (int64_t b = 0; b < t->at.nbox; ++b)
+            if (t->at.hbox[4 * b + 3]) wmax = std::max(wmax, ldexp(t->med.d, -(int)t->at.hbox[4 * b]));
+    if (!lm_exp_df_fits(t->med.k2, wmax)) {
+        t->m2l_df = false;
         return LM_OK;
-    };
-    auto conv_t = [&](const zd *tab, int64_t ncls, float4 **out) -> lm_status {
-        const int64_t cnt = std::max<int64_t>(1, ncls) * np * np;
-        lm_status s = lm_dalloc(t, out, cnt);
-        if (s != LM_OK) return s;
-        k_tab_df_t<<<gridn(cnt, 256), 256, 0, st>>>(tab, cnt, np, *out);
-        return LM_OK;
-    };
-    for (Level &lv : t->lev) {
-        if (lv.m2m) {
-            lm_status s = conv(lv.m2m, 4, &lv.m2mdf); // 4 child positions
-            if (s != LM_OK) return s;
-        }
-        if (lv.l2l) {
-            lm_status s = conv(lv.l2l, 4, &lv.l2ldf);
-            if (s != LM_OK) return s;
-        }
     }
-    if (t->adaptive) {
-        lm_status s = conv(t->at.tab, (int64_t)t->at.cls_term.size(), &t->at.tabdf);
-        if (s == LM_OK) s = conv_t(t->at.tab, (int64_t)t->at.cls_term.size(), &t->at.tabdft);
-        if (s != LM_OK) return s;
-        s = lm_dalloc(t, &t->at.Mdf, (size_t)t->at.nbox * np * LM_MAXV);
-        if (s != LM_OK) return s;
-    } else {
-        for (Level &lv : t->lev) {
-            lm_status s = conv(lv.tab, (int64_t)lv.cls_term.size(), &lv.tabdf);
-            if (s == LM_OK) s = conv_t(lv.tab, (int64_t)lv.cls_term.size(), &lv.tabdft);
-            if (s != LM_OK) return s;
-            s = lm_dalloc(t, &lv.Mdf, (size_t)lv.nbox * np * LM_MAXV);
-            if (s != LM_OK) return s;
-        }
-    }
-    LM_CUDA(cudaGetLastError());
-    return LM_OK;
+    t->ndf.wmax = wmax;
+    lm_status s = lm_dalloc(t, &t->qexp, 1);
+    if (s == LM_OK) s = lm_setup_near_df(t, st);
+    if (s == LM_OK) s = lm_setup_exp_df(t, st);
+    return s;
 }
 
 // slots of the interface leaves (the blocks of k_pw_src64 / k_near_pw64) and their

@@ -777,12 +777,14 @@ void lm_free_tree_device(lm_tree_s *t)
     void *ptrs[] = {t->xs, t->ys, t->perm, t->leaf_start, t->ustart, t->usrc, t->uterm, t->qs, t->us,
                     t->dflag, t->qexp, t->pwidx, t->pwC, t->nq.seg_lam, t->nq.seg_s2, t->nq.seg_w, t->nq.tail_lam, t->nq.tail_s2,
                     t->nq.tail_w, t->nq.tail_lam_g, t->nq.tail_s2_g, t->nq.tail_w_g, t->nq.tail_w2,
-                    t->nq.tail_w2_g, t->nq.seg_c, t->nq.tail_c_g};
+                    t->nq.tail_w2_g, t->nq.seg_c, t->nq.tail_c_g, t->ndf.node, t->ndf.w, t->ndf.w2, t->ndf.seg,
+                    t->ndf.segw, t->ndf.rel, t->ndf.hgt, t->ndf.q, t->ndf.node_g, t->ndf.w_g, t->ndf.w2_g, t->ndf.segw_g,
+                    t->xdf.bes, t->xdf.lev};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     for (Level &lv : t->lev) {
         void *lp[] = {lv.vstart, lv.vsrc, lv.vslot, lv.vterm, lv.tab, lv.scale, lv.m2m, lv.l2l, lv.M, lv.Lc,
-                      lv.tabdf, lv.tabdft, lv.Mdf, lv.m2mdf, lv.l2ldf};
+                      lv.tabdft, lv.m2mdf, lv.l2ldf};
         for (void *p : lp)
             if (p) cudaFree(p);
     }

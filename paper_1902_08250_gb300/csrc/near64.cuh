@@ -1,0 +1,148 @@
+// near64.cuh -- device code shared by the FP64 form's kernels (lmfmm_apply.cu) and
+// their double-float near field (lmfmm_near_df.cu): box geometries, the density
+// exponent and the free-space kernel.
+#pragma once
+#include "internal.h"
+
+// Box geometry of a launch: block i works on box id(i), whose centre and width
+// come from centre().
+struct GridLeaves { // uniform tree: leaf i of the leaf lattice
+    LeafGeom g;
+    __device__ int64_t id(int64_t i) const { return i; }
+    __device__ void centre(int64_t b, double *cx, double *cy, double *w) const
+    {
+        leaf_centre(g, b, cx, cy);
+        *w = g.w;
+    }
+};
+struct EdgeRowLeaves { // uniform tree: the leaves of the top row, then (nrow > 1) of the bottom row
+    LeafGeom g;
+    int64_t nrow;
+    __device__ int64_t id(int64_t i) const { return ((nrow == 1 || i < g.ncol) ? 0 : nrow - 1) * g.ncol + i % g.ncol; }
+    __device__ void centre(int64_t b, double *cx, double *cy, double *w) const
+    {
+        leaf_centre(g, b, cx, cy);
+        *w = g.w;
+    }
+};
+struct ListBoxes { // adaptive tree: box ids[i], centres and widths from arrays
+    const int32_t *ids;
+    const double *bx, *by, *bw;
+    __device__ int64_t id(int64_t i) const { return ids[i]; }
+    __device__ void centre(int64_t b, double *cx, double *cy, double *w) const
+    {
+        *cx = bx[b];
+        *cy = by[b];
+        *w = bw[b];
+    }
+};
+
+struct GridParents { // uniform tree: parent i of a level with ncol columns; children one level down
+    int64_t ncol;
+    __device__ int64_t parent(int64_t i) const { return i; }
+    __device__ int64_t child(int64_t b, int pos) const
+    {
+        const int64_t r = b / ncol, c = b % ncol;
+        return (2 * r + (pos >> 1)) * (2 * ncol) + 2 * c + (pos & 1);
+    }
+};
+struct ListParents { // adaptive tree: parent ids[i], children from the box links
+    const int32_t *ids, *kids;
+    __device__ int64_t parent(int64_t i) const { return ids[i]; }
+    __device__ int64_t child(int64_t b, int pos) const { return kids[4 * b + pos]; }
+};
+
+
+__device__ __forceinline__ int qexp_of(const int *qexp)
+{
+    const int e = *qexp;
+    return e < -1000 ? 0 : e; // all densities zero: no scaling
+}
+
+// ---------------------------------------------------------------------------
+// Free-space kernel (i/4) H0^(1)(x) = (i/4)(J0(x) + i Y0(x)) of a near pair in
+// FP64.  For x <= 2 the ascending series (Abramowitz & Stegun 9.1.12, 9.1.13),
+// with z = x^2/4:
+//   J0 = sum_m (-z)^m / (m!)^2,
+//   Y0 = (2/pi) [(ln(x/2) + gamma) J0 - sum_{m>=1} H_m (-z)^m / (m!)^2],
+// H_m the harmonic numbers, gamma Euler's constant; 14 terms leave the first
+// omitted one below 2e-21 for z <= 1 (within 5e-16 of scipy's J0, Y0 on
+// (0, 2]).  Horner form: 28 FMAs and one log in place of the library's j0 and
+// y0 (1M FP64 strip: leaf kernel 72.0 -> 65.7 ms).  Larger x: j0, y0.
+// ---------------------------------------------------------------------------
+#define H0S_TERMS 14
+struct H0Series {
+    double cj[H0S_TERMS], cy[H0S_TERMS]; // (-1)^m / (m!)^2, -(-1)^m H_m / (m!)^2
+    constexpr H0Series() : cj(), cy()
+    {
+        double f = 1.0, h = 0.0; // 1/(m!)^2, H_m
+        for (int m = 0; m < H0S_TERMS; ++m) {
+            if (m > 0) {
+                f /= (double)m * (double)m;
+                h += 1.0 / m;
+            }
+            cj[m] = (m & 1) ? -f : f;
+            cy[m] = (m & 1) ? h * f : -h * f;
+        }
+    }
+};
+static __constant__ H0Series c_h0s = H0Series();
+// J1 and Y1 for the target gradient (A&S 9.1.10, 9.1.11 with n = 1):
+//   J1 = (x/2) sum_m (-z)^m / (m! (m+1)!),
+//   Y1 = -2/(pi x) + (2/pi) ln(x/2) J1 - (x/(2 pi)) sum_m (-z)^m (psi(m+1) + psi(m+2)) / (m! (m+1)!),
+// psi(m+1) = H_m - gamma; within 5e-16 of scipy's J1, Y1 on (0, 2]
+struct H1Series {
+    double c[H0S_TERMS], e[H0S_TERMS]; // (-1)^m / (m! (m+1)!), (-1)^m (psi(m+1) + psi(m+2)) / (m! (m+1)!)
+    constexpr H1Series() : c(), e()
+    {
+        double f = 1.0, h = 0.0; // 1/(m! (m+1)!), H_m
+        for (int m = 0; m < H0S_TERMS; ++m) {
+            if (m > 0) {
+                f /= (double)m * (double)(m + 1);
+                h += 1.0 / m;
+            }
+            const double psi = (h - 0.57721566490153286061) + (h + 1.0 / (m + 1) - 0.57721566490153286061);
+            c[m] = (m & 1) ? -f : f;
+            e[m] = (m & 1) ? -psi * f : psi * f;
+        }
+    }
+};
+static __constant__ H1Series c_h1s = H1Series();
+// (i/4) H0^(1)(x) and (i/4) H1^(1)(x) together (series for x <= 2, else the library's)
+__device__ __forceinline__ void h01_free64(double x, zd *h0, zd *h1)
+{
+    if (x > 2.0) {
+        *h0 = zd{-0.25 * y0(x), 0.25 * j0(x)};
+        *h1 = zd{-0.25 * y1(x), 0.25 * j1(x)};
+        return;
+    }
+    const double z = 0.25 * x * x;
+    double j = c_h0s.cj[H0S_TERMS - 1], sy = c_h0s.cy[H0S_TERMS - 1];
+    double a = c_h1s.c[H0S_TERMS - 1], b = c_h1s.e[H0S_TERMS - 1];
+#pragma unroll
+    for (int m = H0S_TERMS - 2; m >= 0; --m) {
+        j = fma(j, z, c_h0s.cj[m]);
+        sy = fma(sy, z, c_h0s.cy[m]);
+        a = fma(a, z, c_h1s.c[m]);
+        b = fma(b, z, c_h1s.e[m]);
+    }
+    const double tpi = 0.63661977236758134308, lg = log(0.5 * x);
+    const double yv0 = tpi * ((lg + 0.57721566490153286061) * j + sy);
+    const double jv1 = 0.5 * x * a;
+    const double yv1 = -tpi / x + tpi * lg * jv1 - 0.5 * tpi * 0.5 * x * b;
+    *h0 = zd{-0.25 * yv0, 0.25 * j};
+    *h1 = zd{-0.25 * yv1, 0.25 * jv1};
+}
+__device__ __forceinline__ zd h0_free64(double x)
+{
+    if (x > 2.0) return zd{-0.25 * y0(x), 0.25 * j0(x)};
+    const double z = 0.25 * x * x;
+    double j = c_h0s.cj[H0S_TERMS - 1], sy = c_h0s.cy[H0S_TERMS - 1];
+#pragma unroll
+    for (int m = H0S_TERMS - 2; m >= 0; --m) {
+        j = fma(j, z, c_h0s.cj[m]);
+        sy = fma(sy, z, c_h0s.cy[m]);
+    }
+    const double y = 0.63661977236758134308 * ((log(0.5 * x) + 0.57721566490153286061) * j + sy);
+    return zd{-0.25 * y, 0.25 * j};
+}
