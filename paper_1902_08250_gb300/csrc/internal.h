@@ -174,6 +174,19 @@ struct NearTabDF {
 };
 // Double-float expansions of the FP64 form (lmfmm_exp_df.cu): the M and Lc arrays then hold float4
 // (re hi, re lo, im hi, im lo) scaled by 2^-qexp, [box][2p+1][nvec]
+// Series and recurrence coefficients of the basis (device, double-floats): c[n] = 1/(n (n+1)), n = 1..N, at
+// [n]; then 1/(m (N+m)) and 1/(m (N+1+m)), m = 1..nt, at [N + m] and [N + nt + m]
+struct BesselDF {
+    const float2 *c;
+    int N, nt;
+};
+struct M2LLevelDF { // a level of the M2L launch over the V lists
+    int64_t box0;          // first block of the level in the launch
+    const int64_t *vstart;
+    const int32_t *vsrc, *vslot;
+    const float4 *tab, *M; // transposed tables, multipoles of the level
+    float4 *L;
+};
 struct ExpDF {
     bool ready;
     float2 *bes; // coefficients of the Bessel basis (BesselDF)
@@ -181,6 +194,23 @@ struct ExpDF {
     void *lev;   // device M2LLevelDF[nlev]
     int nlev;
     int64_t nblk; // boxes of all levels
+};
+
+// Tensor-core M2L of the FP64 form (lmfmm_oz.cu): its levels, and per vector form (1, 2, 4, 8, 16
+// slots) the device descriptors
+struct OzData {
+    struct Lv {
+        int l;
+        void *ents;
+        int32_t *e0;
+        unsigned char *A, *B;
+        uint32_t *tmax;
+    };
+    std::vector<Lv> lv;
+    uint32_t *mmax = nullptr;
+    void *desc[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
+    int64_t ntile[5] = {0, 0, 0, 0, 0};
+    int nsm = 0;
 };
 
 struct lm_tree_s {
@@ -242,6 +272,7 @@ struct lm_tree_s {
     bool m2l_df; // FP64 form: expansions and direct interactions in double-float on the FP32 pipes
     NearTabDF ndf;
     ExpDF xdf;
+    OzData oz;
     int *qexp;   // device: binary exponent of the largest |density| component of the apply
     int64_t bytes;
     // phase profiling
@@ -302,6 +333,20 @@ lm_status lm_launch_near_grad_df(lm_tree_s *t, int nvq, int v0, int nv, zd *u, z
 lm_status lm_launch_near64(lm_tree_s *t, int v0, int nv, zd *u, zd *ux, zd *uy, cudaStream_t st);
 bool lm_exp_df_fits(double k2, double wmax);                // double-float expansions (lmfmm_exp_df.cu)
 lm_status lm_setup_exp_df(lm_tree_s *t, cudaStream_t st);
+// parts of it for the cross-layer operator: basis coefficients, transposed tables, the steps on a lattice
+void lm_bessel_df(int P, double k, double wmax, std::vector<float> &h, int *N, int *nt);
+void lm_tab_df_t(const zd *tab, int64_t ncls, int np, float4 *out, cudaStream_t st);
+void lm_df_s2m(const BesselDF &B, const LeafGeom &g, int64_t nleaf, int P, double k, const float4 *rel, const int64_t *ls,
+               const float4 *q, int nv, float4 *M, cudaStream_t st);
+void lm_df_l2t(const BesselDF &B, const LeafGeom &g, int64_t nleaf, int P, double k, const float4 *rel, const int64_t *ls,
+               const float4 *L, int nv, const int *qexp, int64_t n, zd *us, cudaStream_t st);
+void lm_df_m2m(int64_t ncol, int64_t npar, int P, int nv, const float4 *tab, const float4 *Mc, float4 *Mp, cudaStream_t st);
+void lm_df_l2l(int64_t ncol, int64_t npar, int P, int nv, const float4 *tab, const float4 *Lp, float4 *Lc, cudaStream_t st);
+void lm_df_m2l(const M2LLevelDF *lev, int nlev, int64_t nblk, int P, int nv, cudaStream_t st);
+bool lm_oz_level(const lm_tree_s *t, int l); // tensor-core M2L of the FP64 form (lmfmm_oz.cu)
+lm_status lm_setup_oz(lm_tree_s *t, cudaStream_t st);
+lm_status lm_launch_m2l_oz(lm_tree_s *t, int nv, cudaStream_t st, int *launches);
+void lm_free_oz(lm_tree_s *t);
 lm_status lm_run_df(lm_tree_s *t, const zd *q, int nvec, zd *u, bool adjoint, zd *ux, zd *uy, cudaStream_t st);
 lm_status lm_run_apply_grad(lm_tree_s *t, const zd *q, int nvec, zd *u, zd *ux, zd *uy, cudaStream_t st);
 // mixed precision (lmfmm_mixed.cu)

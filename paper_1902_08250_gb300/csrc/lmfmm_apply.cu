@@ -952,6 +952,7 @@ lm_status lm_setup_df(lm_tree_s *t, cudaStream_t st)
     t->ndf.wmax = wmax;
     lm_status s = lm_dalloc(t, &t->qexp, 1);
     if (s == LM_OK) s = lm_setup_near_df(t, st);
+    if (s == LM_OK) s = lm_setup_oz(t, st);
     if (s == LM_OK) s = lm_setup_exp_df(t, st);
     return s;
 }

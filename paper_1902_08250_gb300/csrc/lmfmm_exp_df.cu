@@ -22,13 +22,6 @@
 
 static int gridn(int64_t n, int b) { return (int)((n + b - 1) / b); }
 
-// series and recurrence coefficients (device, double-floats): c[n] = 1/(n (n+1)), n = 1..N, at [n];
-// then 1/(m (N+m)) and 1/(m (N+1+m)), m = 1..nt, at [N + m] and [N + nt + m]
-struct BesselDF {
-    const float2 *c;
-    int N, nt;
-};
-
 // Z^n g_n, n = 0..P, of one point into row[0..P]; rel: offset from the box centre times k/2;
 // iw = 2/(k w)
 __device__ __forceinline__ void basis_row(const BesselDF &B, int P, float4 rel, df iw, float4 *row)
@@ -306,15 +299,7 @@ __global__ void __launch_bounds__(512) k_l2l_dx(Geo geo, int P, int nv, const fl
     }
 }
 
-// M2L over the V lists of every level in one launch: one block per target box, the
-// box's entries dealt out to G groups of threads; sets L
-struct M2LLevelDF {
-    int64_t box0;          // first block of the level in the launch
-    const int64_t *vstart;
-    const int32_t *vsrc, *vslot;
-    const float4 *tab, *M; // transposed tables, multipoles of the level
-    float4 *L;
-};
+// M2L over the V lists of every level in one launch: one block per target box; sets L.
 // The entries form GS interleaved subsets, each summed on its own, then added in order: a vector's
 // sums do not depend on how many vectors are applied or on how many threads share a box.  PAR: a group
 // of threads per subset (up to 2 vectors, whose threads would be too few), else a thread takes them all.
@@ -389,25 +374,37 @@ static int round32(int n) { return (n + 31) / 32 * 32; }
 #define XD_TMAX 2500.0
 bool lm_exp_df_fits(double k2, double wmax) { return 0.125 * k2 * k2 * wmax * wmax <= XD_TMAX; }
 
+void lm_bessel_df(int P, double k, double wmax, std::vector<float> &h, int *N, int *nt)
+{
+    const double tmax = 0.125 * k * k * wmax * wmax;
+    *N = std::max(P + 1, (int)ceil(tmax));
+    *nt = 1;
+    for (double v = tmax / (*N + 1); v > 1e-16; ++*nt) v *= tmax / ((*nt + 1.0) * (*N + *nt + 1.0));
+    h.assign(2 * (*N + 2 * *nt + 1), 0.f);
+    auto put = [&](int i, double v) {
+        h[2 * i] = (float)v;
+        h[2 * i + 1] = (float)(v - (double)(float)v);
+    };
+    for (int n = 1; n <= *N; ++n) put(n, 1.0 / ((double)n * (n + 1.0)));
+    for (int m = 1; m <= *nt; ++m) {
+        put(*N + m, 1.0 / ((double)m * (*N + m)));
+        put(*N + *nt + m, 1.0 / ((double)m * (*N + 1.0 + m)));
+    }
+}
+
+void lm_tab_df_t(const zd *tab, int64_t ncls, int np, float4 *out, cudaStream_t st)
+{
+    const int64_t cnt = ncls * np * np;
+    k_tab_df_t<<<gridn(cnt, 256), 256, 0, st>>>(tab, cnt, np, out);
+}
+
 // Bessel coefficients, transposed double-float tables, level descriptors; t->ndf.wmax is set
 lm_status lm_setup_exp_df(lm_tree_s *t, cudaStream_t st)
 {
     ExpDF &E = t->xdf;
     const int P = t->p, np = 2 * P + 1;
-    const double tmax = 0.125 * t->med.k2 * t->med.k2 * t->ndf.wmax * t->ndf.wmax;
-    E.N = std::max(P + 1, (int)ceil(tmax));
-    E.nt = 1;
-    for (double v = tmax / (E.N + 1); v > 1e-16; ++E.nt) v *= tmax / ((E.nt + 1.0) * (E.N + E.nt + 1.0));
-    std::vector<float> h(2 * (E.N + 2 * E.nt + 1), 0.f);
-    auto put = [&](int i, double v) {
-        h[2 * i] = (float)v;
-        h[2 * i + 1] = (float)(v - (double)(float)v);
-    };
-    for (int n = 1; n <= E.N; ++n) put(n, 1.0 / ((double)n * (n + 1.0)));
-    for (int m = 1; m <= E.nt; ++m) {
-        put(E.N + m, 1.0 / ((double)m * (E.N + m)));
-        put(E.N + E.nt + m, 1.0 / ((double)m * (E.N + 1.0 + m)));
-    }
+    std::vector<float> h;
+    lm_bessel_df(P, t->med.k2, t->ndf.wmax, h, &E.N, &E.nt);
     TRY_X(lm_dalloc(t, &E.bes, h.size() / 2));
     LM_CUDA(cudaMemcpyAsync(E.bes, h.data(), h.size() * sizeof(float), cudaMemcpyHostToDevice, st));
     auto conv = [&](const zd *tab, int64_t ncls, float4 **out) -> lm_status {
@@ -429,6 +426,7 @@ lm_status lm_setup_exp_df(lm_tree_s *t, cudaStream_t st)
         E.nblk = A.nbox;
     } else
         for (Level &lv : t->lev) {
+            if (lm_oz_level(t, lv.l)) continue; // on the tensor cores
             TRY_X(conv(lv.tab, (int64_t)lv.cls_term.size(), &lv.tabdft));
             lev.push_back({E.nblk, lv.vstart, lv.vsrc, lv.vslot, lv.tabdft, (const float4 *)lv.M, (float4 *)lv.Lc});
             E.nblk += lv.nbox;
@@ -444,59 +442,89 @@ lm_status lm_setup_exp_df(lm_tree_s *t, cudaStream_t st)
     return LM_OK;
 }
 
-template <int NV, class Geo>
-static void launch_s2m(lm_tree_s *t, Geo geo, int64_t nleaf, int nv, float4 *M, cudaStream_t st)
+template <class Geo>
+static void launch_s2m(const BesselDF &B, Geo geo, int64_t nleaf, int P, double k, const float4 *rel, const int64_t *ls,
+                       const float4 *q, int nv, float4 *M, cudaStream_t st)
 {
-    const ExpDF &E = t->xdf;
-    const size_t shm = (size_t)XD_PTS * (((t->p + 1) | 1) + nv) * sizeof(float4);
-    k_s2m_df<NV><<<(unsigned)nleaf, NV >= 4 ? 128 : 64, shm, st>>>(geo, t->p, t->med.k2, BesselDF{E.bes, E.N, E.nt}, t->ndf.rel,
-                                                                  t->leaf_start, t->ndf.q, nv, M);
+    const size_t shm = (size_t)XD_PTS * (((P + 1) | 1) + nv) * sizeof(float4);
+    NV_DISPATCH(nv, k_s2m_df<NV><<<(unsigned)nleaf, NV >= 4 ? 128 : 64, shm, st>>>(geo, P, k, B, rel, ls, q, nv, M))
 }
-// L2T of all nv vectors into t->us, or (GRAD) of vectors v0 .. v0 + nw - 1 into out
+// L2T of vectors v0 .. v0 + nw - 1 of the nvl in L
 template <bool GRAD, class Geo>
-static void launch_l2t(lm_tree_s *t, Geo geo, int64_t nleaf, const float4 *L, int nvl, int v0, int nw, const L2TOut &out,
-                       cudaStream_t st)
+static void launch_l2t(const BesselDF &B, Geo geo, int64_t nleaf, int P, double k, const float4 *rel, const int64_t *ls,
+                       const float4 *L, int nvl, int v0, int nw, const int *qexp, int64_t n, const L2TOut &out, cudaStream_t st)
 {
-    const ExpDF &E = t->xdf;
-    const int PB = t->p + (GRAD ? 1 : 0);
+    const int PB = P + (GRAD ? 1 : 0);
     const size_t shm = ((size_t)XD_PTS * ((PB + 1) | 1) + (GRAD ? 3 : 1) * (PB + 1) * nw * 2) * sizeof(float4);
-    k_l2t_df<GRAD><<<(unsigned)nleaf, nw > 2 || GRAD ? 128 : 64, shm, st>>>(geo, t->p, t->med.k2, BesselDF{E.bes, E.N, E.nt},
-                                                                                t->ndf.rel, t->leaf_start, L, nvl, v0, nw, t->qexp,
-                                                                                t->n, out);
+    k_l2t_df<GRAD><<<(unsigned)nleaf, nw > 2 || GRAD ? 128 : 64, shm, st>>>(geo, P, k, B, rel, ls, L, nvl, v0, nw, qexp, n, out);
+}
+// as many vectors at a time as the coefficients fit in 48 KB beside the basis; us: [nv][n], tree order
+template <class Geo>
+static int launch_l2t_all(const BesselDF &B, Geo geo, int64_t nleaf, int P, double k, const float4 *rel, const int64_t *ls,
+                          const float4 *L, int nv, const int *qexp, int64_t n, zd *us, cudaStream_t st)
+{
+    const int room = 48 * 1024 / 16 - XD_PTS * ((P + 1) | 1), step = std::max(1, std::min(nv, room / (2 * (P + 1))));
+    int k_ = 0;
+    for (int w0 = 0; w0 < nv; w0 += step, ++k_)
+        launch_l2t<false>(B, geo, nleaf, P, k, rel, ls, L, nv, w0, std::min(step, nv - w0), qexp, n,
+                          L2TOut{us + (int64_t)w0 * n, nullptr, nullptr, nullptr}, st);
+    return k_;
 }
 template <class Geo>
-static void launch_m2m(lm_tree_s *t, Geo geo, int64_t npar, int nv, const float4 *tab, const float4 *Mc, float4 *Mp, cudaStream_t st)
+static void launch_m2m(Geo geo, int64_t npar, int P, int nv, const float4 *tab, const float4 *Mc, float4 *Mp, cudaStream_t st)
 {
-    const int np = 2 * t->p + 1;
+    const int np = 2 * P + 1;
     NV_DISPATCH(nv, {
         constexpr int VPT = NV < 4 ? NV : 4;
         const int thr = NV <= 4 ? round32(4 * np) : round32(np * ((nv + 3) / 4));
         const size_t shm = NV <= 4 ? (size_t)3 * np * VPT * sizeof(float4) : 0;
-        k_m2m_dx<NV><<<(unsigned)npar, thr, shm, st>>>(geo, t->p, nv, tab, Mc, Mp);
+        k_m2m_dx<NV><<<(unsigned)npar, thr, shm, st>>>(geo, P, nv, tab, Mc, Mp);
     });
 }
 template <class Geo>
-static void launch_l2l(lm_tree_s *t, Geo geo, int64_t npar, int nv, const float4 *tab, const float4 *Lp, float4 *Lc, cudaStream_t st)
+static void launch_l2l(Geo geo, int64_t npar, int P, int nv, const float4 *tab, const float4 *Lp, float4 *Lc, cudaStream_t st)
 {
-    const int np = 2 * t->p + 1;
+    const int np = 2 * P + 1;
     NV_DISPATCH(nv, {
         const int thr = std::min(512, round32(4 * np * ((nv + 3) / 4)));
-        k_l2l_dx<NV><<<(unsigned)npar, thr, 0, st>>>(geo, t->p, nv, tab, Lp, Lc);
+        k_l2l_dx<NV><<<(unsigned)npar, thr, 0, st>>>(geo, P, nv, tab, Lp, Lc);
     });
 }
-static void launch_m2l(lm_tree_s *t, int nv, cudaStream_t st)
+static void launch_m2l(const M2LLevelDF *lev, int nlev, int64_t nblk, int P, int nv, cudaStream_t st)
 {
-    const ExpDF &E = t->xdf;
-    const int np = 2 * t->p + 1;
+    const int np = 2 * P + 1;
     // subsets of a box's entries: as many as threads of 512 for small trees, whose boxes leave SMs idle
-    const int GS = std::max(1, std::min(E.nblk < 1216 ? 12 : 3, 512 / np));
+    const int GS = std::max(1, std::min(nblk < 1216 ? 12 : 3, 512 / np));
     NV_DISPATCH(nv, {
         constexpr int VPT = NV < 4 ? NV : 4;
         constexpr bool PAR = NV <= 2;
         const int thr = round32(np * (PAR ? GS : (nv + VPT - 1) / VPT));
-        k_m2l_dx<NV, PAR><<<(unsigned)E.nblk, thr, PAR ? (size_t)(GS - 1) * np * VPT * sizeof(float4) : 0, st>>>(
-            (const M2LLevelDF *)E.lev, E.nlev, t->p, nv, GS);
+        k_m2l_dx<NV, PAR><<<(unsigned)nblk, thr, PAR ? (size_t)(GS - 1) * np * VPT * sizeof(float4) : 0, st>>>(lev, nlev, P, nv, GS);
     });
+}
+
+// The same for the cross-layer operator's two trees (lmfmm_cross.cu), whose levels share one lattice
+void lm_df_s2m(const BesselDF &B, const LeafGeom &g, int64_t nleaf, int P, double k, const float4 *rel, const int64_t *ls,
+               const float4 *q, int nv, float4 *M, cudaStream_t st)
+{
+    launch_s2m(B, GridLeaves{g}, nleaf, P, k, rel, ls, q, nv, M, st);
+}
+void lm_df_l2t(const BesselDF &B, const LeafGeom &g, int64_t nleaf, int P, double k, const float4 *rel, const int64_t *ls,
+               const float4 *L, int nv, const int *qexp, int64_t n, zd *us, cudaStream_t st)
+{
+    launch_l2t_all(B, GridLeaves{g}, nleaf, P, k, rel, ls, L, nv, qexp, n, us, st);
+}
+void lm_df_m2m(int64_t ncol, int64_t npar, int P, int nv, const float4 *tab, const float4 *Mc, float4 *Mp, cudaStream_t st)
+{
+    launch_m2m(GridParents{ncol}, npar, P, nv, tab, Mc, Mp, st);
+}
+void lm_df_l2l(int64_t ncol, int64_t npar, int P, int nv, const float4 *tab, const float4 *Lp, float4 *Lc, cudaStream_t st)
+{
+    launch_l2l(GridParents{ncol}, npar, P, nv, tab, Lp, Lc, st);
+}
+void lm_df_m2l(const M2LLevelDF *lev, int nlev, int64_t nblk, int P, int nv, cudaStream_t st)
+{
+    launch_m2l(lev, nlev, nblk, P, nv, st);
 }
 
 __global__ void k_permute_in(const zd *q, const int64_t *perm, int64_t n, int nvec, int conjugate, zd *qs);
@@ -514,6 +542,9 @@ lm_status lm_run_df(lm_tree_s *t, const zd *q, int nvec, zd *u, bool adjoint, zd
     const ListBoxes leaves{A.leaves, A.cx, A.cy, A.w};
     const GridLeaves gleaves{LeafGeom{t->lev[L].ncol, t->x0, t->lev[L].w}};
     const int64_t nleaf = ad ? A.nleaf : t->lev[L].nbox;
+    const BesselDF B{t->xdf.bes, t->xdf.N, t->xdf.nt};
+    const int P = t->p;
+    const double k2 = t->med.k2;
     auto Mof = [&](int l) { return (float4 *)(ad ? A.M : t->lev[l].M); };
     auto Lof = [&](int l) { return (float4 *)(ad ? A.Lc : t->lev[l].Lc); };
     for (int v0 = 0; v0 < nvec; v0 += LM_MAXV) {
@@ -526,30 +557,32 @@ lm_status lm_run_df(lm_tree_s *t, const zd *q, int nvec, zd *u, bool adjoint, zd
         lm_phase_end(t, PH_PERMUTE, st, 3);
         // step 2: S2M at every leaf, M2M up the levels
         lm_phase_begin(t, PH_S2M, st);
-        if (ad) NV_DISPATCH(nv, launch_s2m<NV>(t, leaves, nleaf, nv, Mof(L), st))
-        else NV_DISPATCH(nv, launch_s2m<NV>(t, gleaves, nleaf, nv, Mof(L), st))
+        if (ad) launch_s2m(B, leaves, nleaf, P, k2, t->ndf.rel, t->leaf_start, t->ndf.q, nv, Mof(L), st);
+        else launch_s2m(B, gleaves, nleaf, P, k2, t->ndf.rel, t->leaf_start, t->ndf.q, nv, Mof(L), st);
         lm_phase_end(t, PH_S2M, st, 1);
         if (L > 0) lm_phase_begin(t, PH_M2M, st);
         int nl = 0;
         for (int l = L - 1; l >= 0; --l) {
             const int64_t npar = ad ? A.nl_start[l + 1] - A.nl_start[l] : t->lev[l].nbox;
             if (npar == 0) continue;
-            if (ad) launch_m2m(t, ListParents{A.nonleaf + A.nl_start[l], A.child}, npar, nv, t->lev[l].m2mdf, Mof(0), Mof(0), st);
-            else launch_m2m(t, GridParents{t->lev[l].ncol}, npar, nv, t->lev[l].m2mdf, Mof(l + 1), Mof(l), st);
+            if (ad) launch_m2m(ListParents{A.nonleaf + A.nl_start[l], A.child}, npar, P, nv, t->lev[l].m2mdf, Mof(0), Mof(0), st);
+            else launch_m2m(GridParents{t->lev[l].ncol}, npar, P, nv, t->lev[l].m2mdf, Mof(l + 1), Mof(l), st);
             ++nl;
         }
         if (L > 0) lm_phase_end(t, PH_M2M, st, nl);
         // step 3: M2L of every level, then L2L down the levels
         lm_phase_begin(t, PH_M2L, st);
-        launch_m2l(t, nv, st);
-        lm_phase_end(t, PH_M2L, st, 1);
+        int km = 0;
+        TRY_X(lm_launch_m2l_oz(t, nv, st, &km));
+        if (t->xdf.nblk > 0) launch_m2l((const M2LLevelDF *)t->xdf.lev, t->xdf.nlev, t->xdf.nblk, P, nv, st);
+        lm_phase_end(t, PH_M2L, st, km + (t->xdf.nblk > 0));
         if (L > 0) lm_phase_begin(t, PH_L2L, st);
         nl = 0;
         for (int l = 1; l <= L; ++l) {
             const int64_t npar = ad ? A.nl_start[l] - A.nl_start[l - 1] : t->lev[l - 1].nbox;
             if (npar == 0) continue;
-            if (ad) launch_l2l(t, ListParents{A.nonleaf + A.nl_start[l - 1], A.child}, npar, nv, t->lev[l].l2ldf, Lof(0), Lof(0), st);
-            else launch_l2l(t, GridParents{t->lev[l - 1].ncol}, npar, nv, t->lev[l].l2ldf, Lof(l - 1), Lof(l), st);
+            if (ad) launch_l2l(ListParents{A.nonleaf + A.nl_start[l - 1], A.child}, npar, P, nv, t->lev[l].l2ldf, Lof(0), Lof(0), st);
+            else launch_l2l(GridParents{t->lev[l - 1].ncol}, npar, P, nv, t->lev[l].l2ldf, Lof(l - 1), Lof(l), st);
             ++nl;
         }
         if (L > 0) lm_phase_end(t, PH_L2L, st, nl);
@@ -561,8 +594,8 @@ lm_status lm_run_df(lm_tree_s *t, const zd *q, int nvec, zd *u, bool adjoint, zd
                 const int nw = std::min(4, nv - w0);
                 const int64_t off = (int64_t)(v0 + w0) * n;
                 const L2TOut out{u ? u + off : nullptr, ux + off, uy + off, t->perm};
-                if (ad) launch_l2t<true>(t, leaves, nleaf, Lof(L), nv, w0, nw, out, st);
-                else launch_l2t<true>(t, gleaves, nleaf, Lof(L), nv, w0, nw, out, st);
+                if (ad) launch_l2t<true>(B, leaves, nleaf, P, k2, t->ndf.rel, t->leaf_start, Lof(L), nv, w0, nw, t->qexp, n, out, st);
+                else launch_l2t<true>(B, gleaves, nleaf, P, k2, t->ndf.rel, t->leaf_start, Lof(L), nv, w0, nw, t->qexp, n, out, st);
                 if (t->ndf.ready) TRY_X(lm_launch_near_grad_df(t, nv, w0, nw, out.u, out.ux, out.uy, st));
                 else TRY_X(lm_launch_near64(t, w0, nw, out.u, out.ux, out.uy, st));
                 nnear += 2;
@@ -571,14 +604,8 @@ lm_status lm_run_df(lm_tree_s *t, const zd *q, int nvec, zd *u, bool adjoint, zd
             LM_CUDA(cudaGetLastError());
             continue;
         }
-        // as many vectors at a time as the coefficients fit in 48 KB beside the basis
-        const int room = 48 * 1024 / 16 - XD_PTS * ((t->p + 1) | 1), step = std::max(1, std::min(nv, room / (2 * (t->p + 1))));
-        for (int w0 = 0; w0 < nv; w0 += step, ++nnear) {
-            const int nw = std::min(step, nv - w0);
-            const L2TOut out{t->us + (int64_t)w0 * n, nullptr, nullptr, nullptr};
-            if (ad) launch_l2t<false>(t, leaves, nleaf, Lof(L), nv, w0, nw, out, st);
-            else launch_l2t<false>(t, gleaves, nleaf, Lof(L), nv, w0, nw, out, st);
-        }
+        nnear = ad ? launch_l2t_all(B, leaves, nleaf, P, k2, t->ndf.rel, t->leaf_start, Lof(L), nv, t->qexp, n, t->us, st)
+                   : launch_l2t_all(B, gleaves, nleaf, P, k2, t->ndf.rel, t->leaf_start, Lof(L), nv, t->qexp, n, t->us, st);
         int k = 1;
         if (t->ndf.ready) TRY_X(lm_launch_near_df(t, nv, st, &k));
         else TRY_X(lm_launch_near64(t, 0, nv, nullptr, nullptr, nullptr, st));

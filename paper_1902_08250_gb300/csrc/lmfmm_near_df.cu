@@ -29,49 +29,7 @@ __host__ __device__ constexpr int min_i(int a, int b) { return a < b ? a : b; }
 #define ND_SRC 64 // near sources a round
 // targets of a block's pass: 16, 8 where the sums take more registers
 __host__ __device__ constexpr int nd_tgt(int nv, bool grad) { return grad || nv == 16 ? 8 : 16; }
-#define ND_TINY 8.0779357e-28f // 2^-90
 
-// Series coefficients as double-floats (A&S 9.1.12, 9.1.13; H0Series of near64.cuh)
-struct H0DF {
-    float jh[H0S_TERMS], jl[H0S_TERMS], vh[H0S_TERMS], vl[H0S_TERMS];
-    constexpr H0DF() : jh(), jl(), vh(), vl()
-    {
-        const H0Series s = H0Series();
-        for (int m = 0; m < H0S_TERMS; ++m) {
-            jh[m] = df_hi(s.cj[m]);
-            jl[m] = df_lo(s.cj[m]);
-            vh[m] = df_hi(s.cy[m]);
-            vl[m] = df_lo(s.cy[m]);
-        }
-    }
-};
-static __constant__ H0DF c_h0df = H0DF();
-
-// (A, J) of a free pair at z = (k r / 2)^2.  The first D terms of both series in
-// double-float, the rest up to T in FP32: z^D / (D!)^2 < 2^-24 and z^T / (T!)^2 <
-// 2^-50 for z up to the instantiation's limit (1: D = 7, T = 12; 1/16: D = 4, T = 7).
-template <int D, int T>
-__device__ __forceinline__ void h0_df(const DfSmem &tab, df z, df *A, df *J)
-{
-    float fj = c_h0df.jh[T - 1], fv = c_h0df.vh[T - 1];
-#pragma unroll
-    for (int m = T - 2; m >= D; --m) {
-        fj = fmaf(fj, z.h, c_h0df.jh[m]);
-        fv = fmaf(fv, z.h, c_h0df.vh[m]);
-    }
-    df j = {fj, 0.f}, v = {fv, 0.f};
-#pragma unroll
-    for (int m = D - 1; m >= 0; --m) {
-        j = df_horner(df{c_h0df.jh[m], c_h0df.jl[m]}, z, j);
-        if (m >= 1) v = df_horner(df{c_h0df.vh[m], c_h0df.vl[m]}, z, v);
-    }
-    const df lz = df_add(df_log(tab, z), df{1.1544313f, -1.3275548e-08f}); // ln z + 2 gamma
-    const df a = df_mul(lz, j);
-    df b = df_mul_raw(z, v);
-    b = df{2.f * b.h, 2.f * b.l};
-    *A = df_add(a, b);
-    *J = j;
-}
 // (A, J) and their z-derivatives (target gradient): A' = J/z + (ln z + 2 gamma) J' + 2 V'
 struct HVal {
     df A, J, dA, dJ;
@@ -119,14 +77,6 @@ __device__ __noinline__ void h0_slow_grad(double x, HVal *o)
     o->dA = df_of(-4.0 * M_PI * c * g1.re);
     o->dJ = df_of(4.0 * c * g1.im);
 }
-// the same from the FP64 functions, x = k r of the FP64 coordinates
-__device__ __noinline__ void h0_slow(double x, df *A, df *J)
-{
-    const zd g = h0_free64(x);
-    *A = df_of(-4.0 * M_PI * g.re);
-    *J = df_of(4.0 * g.im);
-}
-
 // ---------------------------------------------------------------------------
 // Tables
 // ---------------------------------------------------------------------------

@@ -1,0 +1,594 @@
+// lmfmm_oz.cu -- the FP64 form's M2L on the tensor cores (tcgen05, kind::f16) by
+// error-free slicing (Ozaki, Ogita, Oishi and Rump, Numer. Algorithms 59, 2012;
+// Mukunoki et al., ISC 2020): tables and multipoles are scaled to fixed point and cut
+// into 5 signed digits of 10 bits, held exactly in FP16.  A product of two digits has
+// at most 18 bits, so a sum over the 2(2p+1) <= 128 input orders is an integer that
+// the FP32 accumulator holds exactly; the digit pairs i + j <= 4 are kept, those of one
+// weight 2^{-10 (i + j)} in one accumulator, and the 5 integers of an output are
+// combined in double-float (50 bits against the 48 of the double-float contraction it
+// replaces).  Levels of at least OZ_MINBOX boxes of uniform trees; the others run on
+// the CUDA cores (k_m2l_dx).
+//
+// A tile is 64 columns: 64 / nvs target boxes of one row and parity class, nvs vectors
+// each.  An interior box's V list depends only on its row and its column's parity, so
+// the tiles of a (row, parity) share one entry list (table slot, column offset dc, source
+// row).  A source outside the strip is a zero box: each row of split multipoles is padded.
+// One entry adds D_{i+j}[128 x 64] += A_i[128 x K] B_j[64 x K]^T over 15 digit pairs, with
+// A the real-block table ([Re -Im; Im Re], 2(2p+1) rows) and K = 2(2p+1) padded to 16.
+//
+// Operands lie in global memory as [digit][8-wide K chunk][row][8 FP16]: 8 rows of a
+// chunk are a core matrix of the canonical K-major no-swizzle layout (stride 128 B between
+// 8-row groups), and any run of boxes is one bulk copy per digit and chunk, whatever its
+// offset.  Stages of up to 48 K (91 KB), two in flight.  Roles as in lmfmm_tc_tiles.cu:
+// a producer warp (a lane per copy), an MMA warp, 8 epilogue warps that read the 5
+// accumulators (320 columns of tensor memory) once per entry.
+// Bound: 45 MMAs of 128 x 64 x 16 a stage, limited by the shared-memory reads of their
+// operands (6 KB a MMA at 128 B per clock).
+#include <algorithm>
+#include <map>
+#include <tuple>
+
+#include <cuda_fp16.h>
+
+#include "df.cuh"
+#include "internal.h"
+#include "lists.cuh"
+#include "near64.cuh"
+#include "tc_common.cuh"
+
+#define OZ_S 5        // digits
+#define OZ_BITS 10
+#define OZ_N 64       // columns of a tile
+#define OZ_KC 6       // 8-wide K chunks of a full stage
+#define OZ_NST 2
+#define OZ_A_BYTES (OZ_S * OZ_KC * 128 * 16)
+#define OZ_B_BYTES (OZ_S * OZ_KC * OZ_N * 16)
+#define OZ_STAGE (OZ_A_BYTES + OZ_B_BYTES)
+#define OZ_EPI 8
+#define OZ_THREADS ((OZ_EPI + 2) * 32)
+#define OZ_SMEM (OZ_NST * OZ_STAGE + 128)
+#define OZ_MINBOX 2048
+#define OZ_PADL 2
+
+struct OzEnt {
+    int32_t slot, dc, rs, pad;
+};
+struct OzLevel {
+    int64_t tile0;          // first tile of the level in the launch
+    int32_t ncl, tpr;       // boxes of a (row, parity) class, tiles of one
+    int64_t ncol;
+    const int32_t *e0;      // [2 nrow + 1] entries of each class
+    const OzEnt *ents;
+    const unsigned char *A; // split tables
+    unsigned char *B;       // split multipoles: planes of a (row, parity)
+    const uint32_t *tmax;   // [2] largest table component and row sum of the level (float bits)
+    uint32_t *mmax;         // [LM_MAXV] largest multipole component per vector
+    const float4 *M;
+    float4 *L;
+    int64_t nrow;
+};
+
+__device__ __forceinline__ int oz_exp(uint32_t bits) { return bits ? (int)((bits >> 23) & 0xff) - 127 : -126; }
+// the level's table exponent: components below 2^(e-1), row sums at most 2^(e+4), so that the leading
+// digits' sum over K stays below 2^24 (|digit| <= 512 on either side)
+__device__ __forceinline__ int oz_ea(const uint32_t *t) { return max(oz_exp(t[0]) + 2, oz_exp(t[1]) - 3); }
+__device__ __forceinline__ float oz_pow2(int e) { return __int_as_float((max(-126, min(127, e)) + 127) << 23); }
+__host__ __device__ __forceinline__ int oz_rows(int np) { return (2 * np + 7) / 8 * 8; }
+__host__ __device__ __forceinline__ int oz_chunks(int np) { return (2 * np + 15) / 16 * 2; }
+__host__ __device__ __forceinline__ int64_t oz_prow(int ncl, int tb, int nvs) { return (int64_t)(OZ_PADL + ncl + tb + 2) * nvs; }
+
+// ---------------------------------------------------------------------------
+// operands
+// ---------------------------------------------------------------------------
+__global__ void __launch_bounds__(256) k_oz_tmax(const zd *tab, int np, uint32_t *tmax)
+{
+    const zd *T = tab + (int64_t)blockIdx.x * np * np;
+    float mx = 0.f, l1 = 0.f;
+    for (int p = threadIdx.x; p < np; p += blockDim.x) {
+        double s = 0.0;
+        for (int q = 0; q < np; ++q) {
+            const zd a = T[p * np + q];
+            mx = fmaxf(mx, (float)fmax(fabs(a.re), fabs(a.im)));
+            s += fabs(a.re) + fabs(a.im);
+        }
+        l1 = fmaxf(l1, (float)s);
+    }
+    if (mx > 0.f) atomicMax(tmax, __float_as_uint(mx));
+    if (l1 > 0.f) atomicMax(tmax + 1, __float_as_uint(l1));
+}
+// one thread per (class, 8-wide K chunk, row): 8 components into 5 digit planes
+__global__ void __launch_bounds__(256) k_oz_tsplit(const zd *tab, int64_t ncls, int np, const uint32_t *tmax,
+                                                   unsigned char *A)
+{
+    const int RA = oz_rows(np), KC = oz_chunks(np);
+    const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (idx >= ncls * KC * RA) return;
+    const int row = (int)(idx % RA), c = (int)(idx / RA % KC);
+    const int64_t cls = idx / ((int64_t)RA * KC);
+    const zd *T = tab + cls * np * np;
+    const double sc = ldexp(1.0, -oz_ea(tmax));
+    uint16_t d[OZ_S][8];
+    for (int i = 0; i < 8; ++i) {
+        const int k = 8 * c + i;
+        double x = 0.0;
+        if (row < 2 * np && k < 2 * np) {
+            const int p = row < np ? row : row - np, q = k < np ? k : k - np;
+            const zd a = T[p * np + q];
+            x = ((row < np) == (k < np)) ? a.re : (row < np ? -a.im : a.im);
+        }
+        x *= sc;
+        for (int s = 0; s < OZ_S; ++s) {
+            x *= 1024.0;
+            const double r = rint(x);
+            d[s][i] = __half_as_ushort(__float2half_rn((float)r));
+            x -= r;
+        }
+    }
+    // stage-major: [stage of OZ_KC chunks][digit][chunk][row]
+    const int st = c / OZ_KC, c0 = st * OZ_KC, kc = min(OZ_KC, KC - c0);
+    unsigned char *o = A + (cls * OZ_S * KC + (int64_t)OZ_S * c0) * RA * 16;
+    for (int s = 0; s < OZ_S; ++s)
+        *(uint4 *)(o + ((int64_t)(s * kc + c - c0) * RA + row) * 16) = *(const uint4 *)d[s];
+}
+
+// largest multipole component of each vector over a level's boxes
+__global__ void __launch_bounds__(256) k_oz_mmax(const OzLevel *lvs, int np, int nv)
+{
+    const OzLevel &lv = lvs[blockIdx.y];
+    const int64_t n = lv.ncol * lv.nrow * np;
+    const int per = blockDim.x / nv, v = threadIdx.x % nv; // threads per round of orders
+    float mx = 0.f;
+    if ((int)threadIdx.x < per * nv)
+        for (int64_t i = blockIdx.x * (int64_t)per + threadIdx.x / nv; i < n; i += (int64_t)gridDim.x * per) {
+            const float4 a = lv.M[i * nv + v];
+            mx = fmaxf(mx, fmaxf(fabsf(a.x), fabsf(a.z)));
+        }
+    __shared__ uint32_t s[LM_MAXV];
+    if (threadIdx.x < LM_MAXV) s[threadIdx.x] = 0;
+    __syncthreads();
+    if (mx > 0.f) atomicMax(&s[v], __float_as_uint(mx));
+    __syncthreads();
+    if ((int)threadIdx.x < nv && s[threadIdx.x]) atomicMax(&lv.mmax[threadIdx.x], s[threadIdx.x]);
+}
+// one thread per (plane, row of it, 8-wide K chunk): 8 orders of a (box, vector) into 5 digit
+// planes; the padding boxes and vectors beyond nv are written as zeros
+__global__ void __launch_bounds__(256) k_oz_split(const OzLevel *lvs, int np, int nv, int nvs)
+{
+    const OzLevel &lv = lvs[blockIdx.y];
+    const int KC = oz_chunks(np);
+    const int64_t rows = oz_prow(lv.ncl, OZ_N / nvs, nvs), tot = 2 * lv.nrow * rows * KC;
+    for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < tot; idx += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t r = idx % rows, pc = idx / rows;
+        const int c = (int)(pc % KC);
+        const int64_t plane = pc / KC, row = plane >> 1;
+        const int par = (int)(plane & 1), v = (int)(r % nvs);
+        const int64_t i = r / nvs - OZ_PADL;
+        uint16_t d[OZ_S][8];
+        const bool on = i >= 0 && i < lv.ncl && v < nv;
+        const int64_t box = row * lv.ncol + 2 * i + par;
+        const float sc = on ? oz_pow2(-(oz_exp(lv.mmax[v]) + 2)) : 0.f;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const int k = 8 * c + j;
+            float h = 0.f, l = 0.f;
+            if (on && k < 2 * np) {
+                const float4 a = lv.M[(box * np + (k < np ? k : k - np)) * nv + v];
+                h = (k < np ? a.x : a.z) * sc;
+                l = (k < np ? a.y : a.w) * sc;
+            }
+#pragma unroll
+            for (int s = 0; s < OZ_S; ++s) { // digits of h + l, exact
+                h *= 1024.f;
+                l *= 1024.f;
+                const float g = rintf(h);
+                d[s][j] = __half_as_ushort(__float2half_rn(g));
+                const df t = two_sum(__fsub_rn(h, g), l);
+                h = t.h;
+                l = t.l;
+            }
+        }
+        unsigned char *o = lv.B + (plane * OZ_S * KC + c) * rows * 16 + r * 16;
+#pragma unroll
+        for (int s = 0; s < OZ_S; ++s) *(uint4 *)(o + (int64_t)s * KC * rows * 16) = *(const uint4 *)d[s];
+    }
+}
+
+// ---------------------------------------------------------------------------
+// M2L
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ uint64_t oz_desc(uint32_t saddr, uint32_t lbo)
+{
+    uint64_t d = 0;
+    d |= (uint64_t)((saddr & 0x3FFFF) >> 4);
+    d |= (uint64_t)(lbo >> 4) << 16;  // K-direction core-matrix stride
+    d |= (uint64_t)(128 >> 4) << 32;  // 8-row-group stride
+    d |= (uint64_t)1 << 46;
+    return d;
+}
+__device__ __forceinline__ void oz_mma(uint32_t dtmem, uint64_t ad, uint64_t bd, uint32_t idesc, uint32_t acc)
+{
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+                 "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(dtmem),
+                 "l"(ad), "l"(bd), "r"(idesc), "r"(acc));
+}
+// 16 columns of each of the 5 accumulators, one wait
+__device__ __forceinline__ void oz_ld16x5(uint32_t t0, float d[OZ_S][16])
+{
+    uint32_t r[OZ_S][16];
+#pragma unroll
+    for (int k = 0; k < OZ_S; ++k)
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, "
+                     "%12, %13, %14, %15}, [%16];"
+                     : "=r"(r[k][0]), "=r"(r[k][1]), "=r"(r[k][2]), "=r"(r[k][3]), "=r"(r[k][4]), "=r"(r[k][5]),
+                       "=r"(r[k][6]), "=r"(r[k][7]), "=r"(r[k][8]), "=r"(r[k][9]), "=r"(r[k][10]), "=r"(r[k][11]),
+                       "=r"(r[k][12]), "=r"(r[k][13]), "=r"(r[k][14]), "=r"(r[k][15])
+                     : "r"(t0 + (uint32_t)(OZ_N * k)));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int k = 0; k < OZ_S; ++k)
+#pragma unroll
+        for (int i = 0; i < 16; ++i) d[k][i] = __uint_as_float(r[k][i]);
+}
+// tile -> level, class, first box of the class
+__device__ __forceinline__ const OzLevel &oz_tile(const OzLevel *lvs, int nlev, int64_t tile, int *cls, int *i0, int tb)
+{
+    int l = nlev - 1;
+    while (tile < lvs[l].tile0) --l;
+    const int64_t r = tile - lvs[l].tile0;
+    *cls = (int)(r / lvs[l].tpr);
+    *i0 = (int)(r % lvs[l].tpr) * tb;
+    return lvs[l];
+}
+__device__ __forceinline__ void oz_fail(volatile int *abort_s, int *err)
+{
+    *abort_s = 1;
+    atomicOr(err, 1);
+}
+
+__global__ void __launch_bounds__(OZ_THREADS, 1) k_m2l_oz(const OzLevel *lvs, int nlev, int64_t ntiles, int np, int nv, int nvs,
+                                                          int *err)
+{
+    extern __shared__ __align__(1024) unsigned char smem[];
+    uint64_t *bars = (uint64_t *)(smem + OZ_NST * OZ_STAGE);
+    uint32_t *tslot = (uint32_t *)(bars + 2 * OZ_NST + 2);
+    volatile int *abort_s = (volatile int *)(tslot + 1);
+    const uint32_t sbase = smem_u32(smem), bfull = smem_u32(bars), bempty = bfull + 8 * OZ_NST, btfull = bfull + 16 * OZ_NST,
+                   btempty = btfull + 8;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int KC = oz_chunks(np), RA = oz_rows(np), nst = (KC + OZ_KC - 1) / OZ_KC, tb = OZ_N / nvs;
+
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < OZ_NST; ++i) {
+            mbar_init(bfull + 8 * i, 1);
+            mbar_init(bempty + 8 * i, 1);
+        }
+        mbar_init(btfull, 1);
+        mbar_init(btempty, OZ_EPI);
+        *abort_s = *(volatile int *)err; // an earlier CTA gave up: do no work
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)), "r"(512));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem = *tslot;
+
+    if (warp == OZ_EPI) {
+        // ---- producer: lane 0 waits for a free stage; each lane then issues one table and one
+        // multipole copy (5 digits x up to 6 chunks) ----
+        uint32_t it = 0;
+        int last[OZ_NST];
+#pragma unroll
+        for (int s = 0; s < OZ_NST; ++s) last[s] = -1;
+        bool stop = false;
+        for (int64_t tile = blockIdx.x; tile < ntiles && !stop; tile += gridDim.x) {
+            int cls, i0;
+            const OzLevel &lv = oz_tile(lvs, nlev, tile, &cls, &i0, tb);
+            const int e0 = lv.e0[cls], e1 = lv.e0[cls + 1], c0 = 2 * i0 + (cls & 1);
+            const int64_t rows = oz_prow(lv.ncl, tb, nvs);
+            for (int base = e0; base < e1 && !stop; base += 32) {
+                const int cnt = min(32, e1 - base);
+                const OzEnt mine = lane < cnt ? lv.ents[base + lane] : OzEnt{0, 0, 0, 0};
+                for (int i = 0; i < cnt && !stop; ++i) {
+                    const int slot = __shfl_sync(0xffffffffu, mine.slot, i), dc = __shfl_sync(0xffffffffu, mine.dc, i),
+                              rs = __shfl_sync(0xffffffffu, mine.rs, i);
+                    const int cs = c0 - dc, par = cs & 1;
+                    const int64_t sbox = ((cs - par) >> 1) + OZ_PADL; // first source in its padded plane
+                    const unsigned char *a = lv.A + (int64_t)slot * OZ_S * KC * RA * 16;
+                    const unsigned char *b = lv.B + ((int64_t)rs * 2 + par) * OZ_S * KC * rows * 16 + sbox * nvs * 16;
+                    for (int st = 0; st < nst; ++st, ++it) {
+                        const int s = (int)(it % OZ_NST), k0 = st * OZ_KC, kc = min(OZ_KC, KC - k0);
+                        int ok = 1;
+                        if (lane == 0) {
+                            ok = mbar_wait_lim(bempty + 8 * s, ((it / OZ_NST) & 1) ^ 1, TC_WAIT_LIMIT, abort_s, err);
+                            if (ok) mbar_expect_tx(bfull + 8 * s, OZ_S * kc * (RA + OZ_N) * 16);
+                            else oz_fail(abort_s, err);
+                        }
+                        ok = __shfl_sync(0xffffffffu, ok, 0);
+                        if (!ok) {
+                            stop = true;
+                            break;
+                        }
+                        const uint32_t sa = sbase + s * OZ_STAGE, sb = sa + OZ_A_BYTES, fb = bfull + 8 * s;
+                        if (lane < OZ_S * kc) {
+                            const int dg = lane / kc, c = lane - dg * kc;
+                            bulk_g2s(sa + (dg * OZ_KC + c) * 128 * 16, a + ((int64_t)OZ_S * k0 + lane) * RA * 16, RA * 16, fb);
+                            bulk_g2s(sb + (dg * OZ_KC + c) * OZ_N * 16, b + ((int64_t)dg * KC + k0 + c) * rows * 16, OZ_N * 16, fb);
+                        }
+                        last[s] = (int)it;
+                        __syncwarp();
+                    }
+                }
+            }
+        }
+        // copies in flight land before the CTA's shared memory is released
+        if (lane == 0)
+            for (int s = 0; s < OZ_NST; ++s)
+                if (last[s] >= 0) mbar_wait_lim(bfull + 8 * s, (last[s] / OZ_NST) & 1, TC_WAIT_LIMIT, nullptr, nullptr);
+        __syncwarp();
+    } else if (warp == OZ_EPI + 1) {
+        // ---- MMA issuer ----
+        if (lane == 0) {
+            const uint32_t idesc = (1u << 4) | ((uint32_t)(OZ_N >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+            uint32_t it = 0, item = 0;
+            int done = -1;
+            bool stop = false;
+            for (int64_t tile = blockIdx.x; tile < ntiles && !stop && !*abort_s; tile += gridDim.x) {
+                int cls, i0;
+                const OzLevel &lv = oz_tile(lvs, nlev, tile, &cls, &i0, tb);
+                const int ne = lv.e0[cls + 1] - lv.e0[cls];
+                for (int e = 0; e < ne && !stop; ++e, ++item) {
+                    if (!mbar_wait_lim(btempty, (item & 1) ^ 1, TC_WAIT_LIMIT, abort_s, err)) {
+                        oz_fail(abort_s, err);
+                        stop = true;
+                        break;
+                    }
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    int issued = 0;
+                    for (int st = 0; st < nst; ++st, ++it) {
+                        const int s = (int)(it % OZ_NST), ks = min(OZ_KC, KC - st * OZ_KC) / 2;
+                        if (!mbar_wait_lim(bfull + 8 * s, (it / OZ_NST) & 1, TC_WAIT_LIMIT, abort_s, err)) {
+                            oz_fail(abort_s, err);
+                            stop = true;
+                            break;
+                        }
+                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                        const uint32_t sa = sbase + s * OZ_STAGE, sb = sa + OZ_A_BYTES;
+                        for (int kk = 0; kk < ks; ++kk)
+#pragma unroll
+                            for (int i = 0; i < OZ_S; ++i)
+#pragma unroll
+                                for (int j = 0; i + j < OZ_S; ++j)
+                                    oz_mma(tmem + OZ_N * (i + j), oz_desc(sa + (i * OZ_KC + 2 * kk) * 128 * 16, 128 * 16),
+                                           oz_desc(sb + (j * OZ_KC + 2 * kk) * OZ_N * 16, OZ_N * 16), idesc,
+                                           (st > 0 || kk > 0 || i > 0) ? 1u : 0u);
+                        tc_commit(bempty + 8 * s);
+                        ++issued;
+                    }
+                    if (issued > 0) { // (after a failed wait too: the drain below then covers every MMA issued)
+                        tc_commit(btfull);
+                        done = (int)item;
+                    }
+                }
+            }
+            // MMAs in flight complete before tensor memory is freed
+            if (done >= 0) mbar_wait_lim(btfull, done & 1, TC_WAIT_LIMIT, nullptr, nullptr);
+        }
+        __syncwarp();
+    } else {
+        // ---- epilogue: warp (quadrant Q, half H): accumulator rows 32 Q .. + 31, columns 32 H .. + 31 ----
+        const int Q = warp & 3, H = warp >> 2, row = 32 * Q + lane;
+        const bool live = 32 * Q < 2 * np;
+        const uint32_t base = tmem + ((uint32_t)(32 * Q) << 16) + 32u * H;
+        uint32_t item = 0;
+        bool bad = false;
+        for (int64_t tile = blockIdx.x; tile < ntiles && !bad; tile += gridDim.x) {
+            int cls, i0;
+            const OzLevel &lv = oz_tile(lvs, nlev, tile, &cls, &i0, tb);
+            const int ne = lv.e0[cls + 1] - lv.e0[cls];
+            df acc[32];
+#pragma unroll
+            for (int c = 0; c < 32; ++c) acc[c] = df{0.f, 0.f};
+            for (int e = 0; e < ne; ++e, ++item) {
+                if (!mbar_wait_lim(btfull, item & 1, TC_WAIT_LIMIT, abort_s, err)) {
+                    oz_fail(abort_s, err);
+                    bad = true;
+                    break;
+                }
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                if (live) {
+#pragma unroll
+                    for (int hf = 0; hf < 2; ++hf) {
+                        float d[OZ_S][16];
+                        oz_ld16x5(base + 16u * hf, d);
+                        if (hf == 1) {
+                            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                            __syncwarp();
+                            if (lane == 0) mbar_arrive(btempty);
+                        }
+#pragma unroll
+                        for (int c = 0; c < 16; ++c) { // integers of weight 2^{-10 k}
+                            const df s = two_sum(d[0][c], d[1][c] * 0x1p-10f);
+                            const df u = two_sum(d[2][c] * 0x1p-20f, fmaf(d[4][c], 0x1p-40f, d[3][c] * 0x1p-30f));
+                            acc[16 * hf + c] = df_add(acc[16 * hf + c], df_add(s, u));
+                        }
+                    }
+                } else {
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(btempty);
+                }
+            }
+            if (bad) break;
+            if (row < 2 * np) {
+                const int ea = oz_ea(lv.tmax), p = row < np ? row : row - np, off = row < np ? 0 : 1;
+                const int64_t r0 = (int64_t)(cls >> 1) * lv.ncol + (cls & 1);
+#pragma unroll
+                for (int c = 0; c < 32; ++c) {
+                    const int col = 32 * H + c, j = col / nvs, v = col - j * nvs;
+                    if (i0 + j < lv.ncl && v < nv) {
+                        const int ex = ea + oz_exp(lv.mmax[v]) + 2 - 2 * OZ_BITS, x1 = ex / 2;
+                        const float f = oz_pow2(x1), g = oz_pow2(ex - x1);
+                        float2 *o = (float2 *)&lv.L[((r0 + 2 * (int64_t)(i0 + j)) * np + p) * nv + v];
+                        o[off] = make_float2(acc[c].h * f * g, acc[c].l * f * g);
+                    }
+                }
+            }
+        }
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
+}
+
+// ---------------------------------------------------------------------------
+// host side
+// ---------------------------------------------------------------------------
+#define TRY_O(x)                     \
+    do {                             \
+        lm_status s_ = (x);          \
+        if (s_ != LM_OK) return s_;  \
+    } while (0)
+static int nv_slots(int nv) { return nv <= 1 ? 1 : nv <= 2 ? 2 : nv <= 4 ? 4 : nv <= 8 ? 8 : 16; }
+
+// whether level l of a uniform FP64 tree takes the tensor cores: its boxes fill the SMs with tiles, its
+// order fits the operand
+bool lm_oz_level(const lm_tree_s *t, int l)
+{
+    return !t->adaptive && t->m2l_df && l >= 1 && 2 * t->np <= 128 && t->lev[l].nbox >= OZ_MINBOX;
+}
+
+static std::vector<OzLevel> oz_levels(const lm_tree_s *t, int nvs)
+{
+    std::vector<OzLevel> v;
+    const int tb = OZ_N / nvs;
+    int64_t tiles = 0;
+    for (const OzData::Lv &z : t->oz.lv) {
+        const Level &lv = t->lev[z.l];
+        OzLevel o{};
+        o.tile0 = tiles;
+        o.ncl = (int32_t)(lv.ncol / 2);
+        o.tpr = (o.ncl + tb - 1) / tb;
+        o.ncol = lv.ncol;
+        o.nrow = lv.nrow;
+        o.e0 = z.e0;
+        o.ents = (const OzEnt *)z.ents;
+        o.A = z.A;
+        o.B = z.B;
+        o.tmax = z.tmax;
+        o.mmax = t->oz.mmax + (size_t)LM_MAXV * v.size();
+        o.M = (const float4 *)lv.M;
+        o.L = (float4 *)lv.Lc;
+        v.push_back(o);
+        tiles += 2 * lv.nrow * o.tpr;
+    }
+    return v;
+}
+
+lm_status lm_setup_oz(lm_tree_s *t, cudaStream_t st)
+{
+    OzData &Z = t->oz;
+    const int np = t->np, RA = oz_rows(np), KC = oz_chunks(np);
+    for (int l = t->L; l >= 1; --l) { // deepest (most tiles) first
+        if (!lm_oz_level(t, l)) continue;
+        const Level &lv = t->lev[l];
+        OzData::Lv z{};
+        z.l = l;
+        std::map<std::tuple<int, int, int>, int> slot;
+        for (size_t i = 0; i < lv.cls_term.size(); ++i) slot[{lv.cls_term[i], lv.cls_dc[i], lv.cls_dr[i]}] = (int)i;
+        std::vector<OzEnt> ents;
+        std::vector<int32_t> e0;
+        for (int64_t rt = 0; rt < lv.nrow; ++rt)
+            for (int par = 0; par < 2; ++par) {
+                e0.push_back((int32_t)ents.size());
+                const int64_t ct = 8 + par; // an interior column
+                for (int term = 0; term < 5; ++term) {
+                    const int64_t a = src_row(term, rt - 3, lv.nrow), b = src_row(term, rt + 3, lv.nrow);
+                    const int64_t rlo = std::max<int64_t>(0, std::min(a, b)), rhi = std::min(lv.nrow - 1, std::max(a, b));
+                    for (int64_t rs = rlo; rs <= rhi; ++rs) {
+                        const int64_t ri = img_row(term, rs, lv.nrow);
+                        for (int64_t cs = ct - 3; cs <= ct + 3; ++cs) {
+                            if (!v_rule(l, ct, rt, cs, ri)) continue;
+                            auto f = slot.find({term, (int)(ct - cs), (int)(rt - ri)});
+                            if (f == slot.end()) {
+                                lm_set_error("build_tree: internal error, an interaction has no translation class");
+                                return LM_ECUDA;
+                            }
+                            ents.push_back(OzEnt{f->second, (int32_t)(ct - cs), (int32_t)rs, 0});
+                        }
+                    }
+                }
+            }
+        e0.push_back((int32_t)ents.size());
+        const size_t ncls = std::max<size_t>(1, lv.cls_term.size());
+        OzEnt *de;
+        TRY_O(lm_dalloc(t, &de, ents.size()));
+        z.ents = de;
+        TRY_O(lm_dalloc(t, &z.e0, e0.size()));
+        TRY_O(lm_dalloc(t, &z.A, ncls * OZ_S * KC * RA * 16));
+        TRY_O(lm_dalloc(t, &z.tmax, 2));
+        size_t bb = 0; // every vector form shares the buffer
+        for (int s = 1; s <= LM_MAXV; s *= 2)
+            bb = std::max(bb, (size_t)(2 * lv.nrow * OZ_S * KC) * oz_prow((int)(lv.ncol / 2), OZ_N / s, s) * 16);
+        TRY_O(lm_dalloc(t, &z.B, bb));
+        Z.lv.push_back(z); // owned from here on
+        LM_CUDA(cudaMemcpyAsync(de, ents.data(), ents.size() * sizeof(OzEnt), cudaMemcpyHostToDevice, st));
+        LM_CUDA(cudaMemcpyAsync(z.e0, e0.data(), e0.size() * sizeof(int32_t), cudaMemcpyHostToDevice, st));
+        LM_CUDA(cudaMemsetAsync(z.tmax, 0, 2 * sizeof(uint32_t), st));
+        k_oz_tmax<<<(unsigned)ncls, 256, 0, st>>>(lv.tab, np, z.tmax);
+        const int64_t nt = (int64_t)ncls * KC * RA;
+        k_oz_tsplit<<<(unsigned)((nt + 255) / 256), 256, 0, st>>>(lv.tab, (int64_t)ncls, np, z.tmax, z.A);
+        LM_CUDA(cudaGetLastError());
+        LM_CUDA(cudaStreamSynchronize(st)); // host temporaries
+    }
+    if (Z.lv.empty()) return LM_OK;
+    TRY_O(lm_dalloc(t, &Z.mmax, Z.lv.size() * LM_MAXV));
+    int f = 0;
+    for (int s = 1; s <= 16; s *= 2, ++f) {
+        const std::vector<OzLevel> lv = oz_levels(t, s);
+        OzLevel *d;
+        TRY_O(lm_dalloc(t, &d, lv.size()));
+        Z.desc[f] = d;
+        const OzLevel &e = lv.back();
+        Z.ntile[f] = e.tile0 + 2 * e.nrow * e.tpr;
+        LM_CUDA(cudaMemcpyAsync(d, lv.data(), lv.size() * sizeof(OzLevel), cudaMemcpyHostToDevice, st));
+        LM_CUDA(cudaStreamSynchronize(st));
+    }
+    int dev = 0;
+    LM_CUDA(cudaGetDevice(&dev));
+    LM_CUDA(cudaDeviceGetAttribute(&Z.nsm, cudaDevAttrMultiProcessorCount, dev));
+    LM_CUDA(cudaFuncSetAttribute(k_m2l_oz, cudaFuncAttributeMaxDynamicSharedMemorySize, OZ_SMEM));
+    return LM_OK;
+}
+
+// the M2L of the tensor-core levels (sets their L); returns the kernels launched
+lm_status lm_launch_m2l_oz(lm_tree_s *t, int nv, cudaStream_t st, int *launches)
+{
+    OzData &Z = t->oz;
+    *launches = 0;
+    if (Z.lv.empty()) return LM_OK;
+    const int nvs = nv_slots(nv), f = nvs == 1 ? 0 : nvs == 2 ? 1 : nvs == 4 ? 2 : nvs == 8 ? 3 : 4, nl = (int)Z.lv.size();
+    const OzLevel *d = (const OzLevel *)Z.desc[f];
+    LM_CUDA(cudaMemsetAsync(Z.mmax, 0, Z.lv.size() * LM_MAXV * sizeof(uint32_t), st));
+    k_oz_mmax<<<dim3(2 * (unsigned)Z.nsm, nl), 256, 0, st>>>(d, t->np, nv);
+    k_oz_split<<<dim3(8 * (unsigned)Z.nsm, nl), 256, 0, st>>>(d, t->np, nv, nvs);
+    k_m2l_oz<<<(unsigned)std::min<int64_t>(Z.nsm, Z.ntile[f]), OZ_THREADS, OZ_SMEM, st>>>(d, nl, Z.ntile[f], t->np, nv, nvs,
+                                                                                           t->dflag + 1);
+    *launches = 3;
+    LM_CUDA(cudaGetLastError());
+    return LM_OK;
+}
+
+void lm_free_oz(lm_tree_s *t)
+{
+    for (OzData::Lv &z : t->oz.lv)
+        for (void *p : {(void *)z.ents, (void *)z.e0, (void *)z.A, (void *)z.B, (void *)z.tmax})
+            if (p) cudaFree(p);
+    for (void *p : t->oz.desc)
+        if (p) cudaFree(p);
+    if (t->oz.mmax) cudaFree(t->oz.mmax);
+    t->oz = OzData();
+}

@@ -8,6 +8,7 @@
 #include <tuple>
 
 #include "internal.h"
+#include "lists.cuh"
 #include "tables.cuh"
 
 // ---------------------------------------------------------------------------
@@ -140,29 +141,6 @@ __global__ void k_gather_pts(const double *x, const double *y, const int64_t *pe
 // nrow rows: free r; tt -1-r (mirror in y = 0); bb 2nrow-1-r (mirror in
 // y = -d); tb r-2nrow (shift +2d); bt r+2nrow (shift -2d).
 // ---------------------------------------------------------------------------
-// inverse: source row whose image row is ri
-__host__ __device__ inline int64_t src_row(int term, int64_t ri, int64_t nrow)
-{
-    switch (term) {
-    case 0: return ri;
-    case 1: return -1 - ri;
-    case 2: return 2 * nrow - 1 - ri;
-    case 3: return ri + 2 * nrow;
-    default: return ri - 2 * nrow;
-    }
-}
-__host__ __device__ inline int64_t floordiv2(int64_t a) { return a >= 0 ? a / 2 : -((-a + 1) / 2); }
-__host__ __device__ inline bool adj(int64_t c1, int64_t r1, int64_t c2, int64_t r2)
-{
-    return (c1 - c2 <= 1 && c2 - c1 <= 1) && (r1 - r2 <= 1 && r2 - r1 <= 1);
-}
-__host__ __device__ inline bool v_rule(int l, int64_t ct, int64_t rt, int64_t cs, int64_t ri)
-{
-    if (adj(ct, rt, cs, ri)) return false;
-    if (l == 0) return true;
-    return adj(ct / 2, floordiv2(rt), cs / 2, floordiv2(ri));
-}
-
 struct SlotMap {
     int DC;          // dc in [-DC, DC]
     int32_t *map;    // [5][2DC+1][7] slot or -1 (dr in [-3, 3])
@@ -774,6 +752,7 @@ void lm_free_tree_device(lm_tree_s *t)
 {
     lm_free_mixed(t);
     lm_free_adaptive(t);
+    lm_free_oz(t);
     void *ptrs[] = {t->xs, t->ys, t->perm, t->leaf_start, t->ustart, t->usrc, t->uterm, t->qs, t->us,
                     t->dflag, t->qexp, t->pwidx, t->pwC, t->nq.seg_lam, t->nq.seg_s2, t->nq.seg_w, t->nq.tail_lam, t->nq.tail_s2,
                     t->nq.tail_w, t->nq.tail_lam_g, t->nq.tail_s2_g, t->nq.tail_w_g, t->nq.tail_w2,

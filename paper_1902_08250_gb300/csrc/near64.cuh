@@ -2,6 +2,7 @@
 // their double-float near field (lmfmm_near_df.cu): box geometries, the density
 // exponent and the free-space kernel.
 #pragma once
+#include "df.cuh"
 #include "internal.h"
 
 // Box geometry of a launch: block i works on box id(i), whose centre and width
@@ -145,4 +146,59 @@ __device__ __forceinline__ zd h0_free64(double x)
     }
     const double y = 0.63661977236758134308 * ((log(0.5 * x) + 0.57721566490153286061) * j + sy);
     return zd{-0.25 * y, 0.25 * j};
+}
+
+// ---------------------------------------------------------------------------
+// The same in double-float.  A kernel value g = g_re + i g_im is kept as (A, J), g_re =
+// -A/(4 pi), g_im = J/4: A = (ln z + 2 gamma) J + 2 V, J = J0, z = (k r / 2)^2, so the constants
+// are applied once per target.
+// ---------------------------------------------------------------------------
+#define ND_TINY 8.0779357e-28f // 2^-90: closer pairs, and z > 1, take the FP64 functions
+// Series coefficients as double-floats (A&S 9.1.12, 9.1.13; H0Series of near64.cuh)
+struct H0DF {
+    float jh[H0S_TERMS], jl[H0S_TERMS], vh[H0S_TERMS], vl[H0S_TERMS];
+    constexpr H0DF() : jh(), jl(), vh(), vl()
+    {
+        const H0Series s = H0Series();
+        for (int m = 0; m < H0S_TERMS; ++m) {
+            jh[m] = df_hi(s.cj[m]);
+            jl[m] = df_lo(s.cj[m]);
+            vh[m] = df_hi(s.cy[m]);
+            vl[m] = df_lo(s.cy[m]);
+        }
+    }
+};
+static __constant__ H0DF c_h0df = H0DF();
+
+// (A, J) of a free pair at z = (k r / 2)^2.  The first D terms of both series in
+// double-float, the rest up to T in FP32: z^D / (D!)^2 < 2^-24 and z^T / (T!)^2 <
+// 2^-50 for z up to the instantiation's limit (1: D = 7, T = 12; 1/16: D = 4, T = 7).
+template <int D, int T>
+__device__ __forceinline__ void h0_df(const DfSmem &tab, df z, df *A, df *J)
+{
+    float fj = c_h0df.jh[T - 1], fv = c_h0df.vh[T - 1];
+#pragma unroll
+    for (int m = T - 2; m >= D; --m) {
+        fj = fmaf(fj, z.h, c_h0df.jh[m]);
+        fv = fmaf(fv, z.h, c_h0df.vh[m]);
+    }
+    df j = {fj, 0.f}, v = {fv, 0.f};
+#pragma unroll
+    for (int m = D - 1; m >= 0; --m) {
+        j = df_horner(df{c_h0df.jh[m], c_h0df.jl[m]}, z, j);
+        if (m >= 1) v = df_horner(df{c_h0df.vh[m], c_h0df.vl[m]}, z, v);
+    }
+    const df lz = df_add(df_log(tab, z), df{1.1544313f, -1.3275548e-08f}); // ln z + 2 gamma
+    const df a = df_mul(lz, j);
+    df b = df_mul_raw(z, v);
+    b = df{2.f * b.h, 2.f * b.l};
+    *A = df_add(a, b);
+    *J = j;
+}
+// the same from the FP64 functions, x = k r of the FP64 coordinates
+static __device__ __noinline__ void h0_slow(double x, df *A, df *J)
+{
+    const zd g = h0_free64(x);
+    *A = df_of(-4.0 * M_PI * g.re);
+    *J = df_of(4.0 * g.im);
 }
