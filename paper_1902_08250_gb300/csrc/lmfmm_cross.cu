@@ -15,10 +15,10 @@
 // table depends on the target and source rows separately, so a class is
 // (term, dc, rt, rs).  g_2^b never reaches the near field (its image is d or
 // more below every target).
-// Precision: LM_FP64 runs every step in FP64.  LM_MIXED builds the tables and the
-// near-field quadrature in FP64 and keeps FP32 copies of the tables; the
-// expansions and every multiply-add are FP32, the near kernel values FP64 rounded
-// to FP32.
+// Precision: LM_FP64 builds tables and quadratures in FP64 and runs every step of an
+// apply in double-float on the FP32 pipes (lmfmm_exp_df.cu's expansions and
+// k_cross_near_df), or in IEEE FP64 with opt.m2l_fp64.  LM_MIXED keeps FP32 copies
+// of the tables; its expansions and translations are FP32, its near pairs as above.
 #include <algorithm>
 #include <map>
 #include <tuple>
@@ -26,7 +26,9 @@
 
 #include <cmath>
 
+#include "df.cuh"
 #include "internal.h"
+#include "near64.cuh"
 #include "tables.cuh"
 
 // kernels shared with the middle-layer operator
@@ -47,6 +49,8 @@ __global__ void k_m2l64(int64_t nbox, int P, int nvec, const int64_t *vstart, co
                         const int32_t *vslot, const zd *tab, const zd *M, zd *Lc);
 __global__ void k_permute_in(const zd *q, const int64_t *perm, int64_t n, int nvec, int conjugate, zd *qs);
 __global__ void k_permute_out(const zd *us, const int64_t *perm, int64_t n, int nvec, int conjugate, zd *u);
+__global__ void k_qexp(const zd *qs, int64_t n, int nvec, int *qexp);
+__global__ void k_q_df(const zd *qs, int64_t n, int nvec, const int *qexp, float4 *q);
 #define CROSS_P2M_CHUNK 16 // points staged per round by k_p2m64
 
 struct CrossLevel {
@@ -62,6 +66,7 @@ struct CrossLevel {
     zd *tab; // [ncls][np][np]
     // mixed form: FP32 copies of the tables, FP32 expansions
     zf *tab32, *m2m32, *l2l32, *M32, *L32;
+    float4 *tabdft, *m2mdf, *l2ldf; // double-float form: transposed tables (M and Lc then hold double-floats)
 };
 
 struct lm_cross_s {
@@ -79,6 +84,15 @@ struct lm_cross_s {
     int nseg, nray, ntail;
     zd *seg_lam, *seg_s1, *seg_s2, *seg_w, *tail_lam, *tail_s1, *tail_s2, *tail_w;
     zd *qs, *us; // [LM_MAXV][ns], [LM_MAXV][nt]
+    // double-float near pairs (unless opt.m2l_fp64) and expansions (xdf)
+    bool ndf, xdf;
+    float4 *qdf;                                       // [ns][nvec] densities scaled by 2^-qexp
+    int *qexp;
+    float4 *seg_node, *seg_wdf, *tail_node, *tail_wdf; // quadrature of the near pairs (k_cross_tab)
+    float4 *rel_s, *rel_t;                             // [n] offsets from the leaf centres times k1/2, k2/2
+    BesselDF bes_s, bes_t;
+    M2LLevelDF *mlev;
+    int64_t nblk;
     int *dflag;
     std::vector<void *> allocs;
 };
@@ -243,11 +257,146 @@ __device__ zd cross_near(const CrossNear &q, double k2, double X, double y, doub
     return acc;
 }
 
+// ---------------------------------------------------------------------------
+// Near pairs in double-float: a warp per target, the lanes over the quadrature nodes of a
+// pair (2 nseg folded segment nodes, then ntail nodes of its ray), each lane multiplying its
+// part of g by the densities; the lanes are summed once per target.  A pair takes about 240
+// node pairs of two complex exponentials: few pairs reach the near field, and a thread per
+// target left the kernel to a handful of serial threads (20k sources, 24k targets: k_cross_leaf
+// 12.4 ms, of which the near pairs nearly all).
+// Node tables: lambda, s2 and s1 as (exponent, phase) coefficients in df_cexp's units; weights
+// of the two exponentials, complex (segment) or as P and iM of P Re(E) + i M Im(E) (tail).
+// ---------------------------------------------------------------------------
+__global__ void k_cross_tab(int n, const zd *lam, const zd *s1, const zd *s2, const zd *w, int tail, float4 *node, float4 *wt)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const double u = 64.0 / 0.693147180559945309417, v = 256.0 / 6.283185307179586476925;
+    const zd l = lam[i], a = s2[i], b = s1[i];
+    node[3 * i] = df_pack(df_of(-l.im * u), df_of(l.re * v)); // i lambda
+    node[3 * i + 1] = df_pack(df_of(a.re * u), df_of(a.im * v));
+    node[3 * i + 2] = df_pack(df_of(b.re * u), df_of(b.im * v));
+    if (!tail) {
+        wt[2 * i] = df_split(w[i]);
+        wt[2 * i + 1] = df_split(-w[n + i]);
+    } else {
+        const zd Ma = w[n + i], Mb = w[3 * n + i];
+        wt[4 * i] = df_split(w[i]);
+        wt[4 * i + 1] = df_split(zd{-Ma.im, Ma.re});
+        wt[4 * i + 2] = df_split(-w[2 * n + i]);
+        wt[4 * i + 3] = df_split(zd{Mb.im, -Mb.re});
+    }
+}
+struct CrossNearDF {
+    int nseg, nray, ntail;
+    const float4 *seg, *segw, *tail, *tailw;
+};
+__device__ __forceinline__ df dot3(df a, df x, df b, df y, df c, df z)
+{
+    df s = df_mul_raw(a, x);
+    df_mac(s, b, y);
+    df_mac(s, c, z);
+    return quick_two_sum(s.h, s.l);
+}
+template <int NV>
+__global__ void __launch_bounds__(128) k_cross_near_df(double k2, const double *xt, const double *yt, const int64_t *lt,
+                                                       const int64_t *ustart, const int32_t *usrc, const double *xs,
+                                                       const double *ysm, const int64_t *lsrc, CrossNearDF nq,
+                                                       const float4 *qd, const int *qexp, int64_t nt, int nv, zd *us)
+{
+    __shared__ DfSmem tab;
+    const int64_t b = blockIdx.x, lo = lt[b], hi = lt[b + 1];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    if (lo + (int64_t)blockIdx.y * nw >= hi) return;
+    tab.load();
+    __syncthreads();
+    const df none = {0.f, 0.f};
+    for (int64_t i = lo + (int64_t)blockIdx.y * nw + warp; i < hi; i += (int64_t)gridDim.y * nw) {
+        const double xi = xt[i], yi = yt[i];
+        const df yd = df_of(yi);
+        float4 acc[NV];
+#pragma unroll
+        for (int v = 0; v < NV; ++v) acc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int64_t e = ustart[b]; e < ustart[b + 1]; ++e) {
+            const int32_t s = usrc[e];
+            for (int64_t j0 = lsrc[s]; j0 < lsrc[s + 1]; j0 += 32) {
+                const int cnt = (int)min((int64_t)32, lsrc[s + 1] - j0);
+                // lane j: source j's offset, height and closed-form part (i/4) H0(k2 R)
+                df X = none, Y = none, A = none, J = none;
+                if (lane < cnt) {
+                    const double dx = fabs(xi - xs[j0 + lane]), y0 = -ysm[j0 + lane];
+                    X = df_of(dx);
+                    Y = df_of(y0);
+                    const df kap = df_of(0.5 * k2), dy = df_of(y0 - yi);
+                    const df z = df_add(df_sq(df_mul(X, kap)), df_sq(df_mul(dy, kap)));
+                    if (z.h > 1.0f || z.h < ND_TINY) h0_slow(k2 * hypot(dx, y0 - yi), &A, &J);
+                    else h0_df<7, 12>(tab, z, &A, &J);
+                    A = df_mul(A, df{-0.07957747f, -3.2103191e-09f}); // -1/(4 pi)
+                    J = df{0.25f * J.h, 0.25f * J.l};
+                }
+                for (int j = 0; j < cnt; ++j) {
+                    const df Xj = {__shfl_sync(0xffffffffu, X.h, j), __shfl_sync(0xffffffffu, X.l, j)};
+                    const df y0 = {__shfl_sync(0xffffffffu, Y.h, j), __shfl_sync(0xffffffffu, Y.l, j)};
+                    const df ny0 = df_neg(y0), dy = df_sub(yd, y0);
+                    float4 g = lane == j ? df_pack(A, J) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    for (int k = lane; k < 2 * nq.nseg; k += 32) {
+                        const float4 *nd = nq.seg + 3 * (k >> 1), *w = nq.segw + 2 * (k >> 1);
+                        const df x = (k & 1) ? df_neg(Xj) : Xj;
+                        const float4 ea = df_cexp(tab, dot3(df_re(nd[0]), x, df_re(nd[1]), yd, df_re(nd[2]), ny0),
+                                                  dot3(df_im(nd[0]), x, df_im(nd[1]), yd, df_im(nd[2]), ny0));
+                        const float4 eb = df_cexp(tab, dot3(df_re(nd[0]), x, df_re(nd[1]), dy, none, none),
+                                                  dot3(df_im(nd[0]), x, df_im(nd[1]), dy, none, none));
+                        dfc_mac(g, w[0], ea);
+                        dfc_mac(g, w[1], eb);
+                    }
+                    const int ray = nq.nray > 1 ? (int)rintf(atan2f(Xj.h, -dy.h) * (float)(nq.nray - 1) * 0.63661977f) : 0;
+                    for (int k = lane; k < nq.ntail; k += 32) {
+                        const float4 *nd = nq.tail + 3 * ((int64_t)ray * nq.ntail + k), *w = nq.tailw + 4 * ((int64_t)ray * nq.ntail + k);
+                        const float4 ea = df_cexp(tab, dot3(df_re(nd[0]), Xj, df_re(nd[1]), yd, df_re(nd[2]), ny0),
+                                                  dot3(df_im(nd[0]), Xj, df_im(nd[1]), yd, df_im(nd[2]), ny0));
+                        const float4 eb = df_cexp(tab, dot3(df_re(nd[0]), Xj, df_re(nd[1]), dy, none, none),
+                                                  dot3(df_im(nd[0]), Xj, df_im(nd[1]), dy, none, none));
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            const float4 E = h ? eb : ea, P = w[2 * h], M = w[2 * h + 1];
+                            df_mac(g.x, g.y, P.x, P.y, E.x, E.y);
+                            df_mac(g.z, g.w, P.z, P.w, E.x, E.y);
+                            df_mac(g.x, g.y, M.x, M.y, E.z, E.w);
+                            df_mac(g.z, g.w, M.z, M.w, E.z, E.w);
+                        }
+                    }
+                    g = df_norm(g);
+#pragma unroll
+                    for (int v = 0; v < NV; ++v)
+                        if (v < nv) dfc_mac(acc[v], g, qd[(j0 + j) * nv + v]);
+                }
+            }
+        }
+        const int ex = qexp_of(qexp);
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+            const float4 a = df_norm(acc[v]);
+            const df re = df_warp_sum(df_re(a)), im = df_warp_sum(df_im(a));
+            if (lane == v && v < nv) {
+                zd &o = us[(int64_t)v * nt + i];
+                o = o + zd{ldexp(df_double(re), ex), ldexp(df_double(im), ex)};
+            }
+        }
+    }
+}
+__global__ void k_cross_rel(LeafGeom g, double kap, const double *xs, const double *ys, const int64_t *ls, float4 *rel)
+{
+    double cx, cy;
+    leaf_centre(g, blockIdx.x, &cx, &cy);
+    for (int64_t i = ls[blockIdx.x] + threadIdx.x; i < ls[blockIdx.x + 1]; i += blockDim.x)
+        rel[i] = df_pack(df_of((xs[i] - cx) * kap), df_of((ys[i] - cy) * kap));
+}
+
 // L2T (k2) and the near g_2^t pairs of every target of a leaf
 __global__ void k_cross_leaf(LeafGeom g, int P, double k2, const double *xt, const double *yt, const int64_t *lt,
                              const int64_t *ustart, const int32_t *usrc, const double *xs, const double *ysm,
                              const int64_t *lsrc, CrossNear nq, const zd *Lc, const zd *qs, int64_t ns,
-                             int64_t nt, int nvec, zd *us)
+                             int64_t nt, int nvec, int near, zd *us)
 {
     const int np = 2 * P + 1;
     const int64_t b = blockIdx.x;
@@ -275,7 +424,7 @@ __global__ void k_cross_leaf(LeafGeom g, int P, double k2, const double *xt, con
                 }
             }
         }
-        for (int64_t e = ustart[b]; e < ustart[b + 1]; ++e) {
+        for (int64_t e = ustart[b]; near && e < ustart[b + 1]; ++e) {
             const int32_t s = usrc[e];
             for (int64_t j = lsrc[s]; j < lsrc[s + 1]; ++j) {
                 const zd gij = cross_near(nq, k2, fabs(xi - xs[j]), yi, -ysm[j]);
@@ -426,7 +575,7 @@ __global__ void k_cross_m2l32(int64_t nbox, int P, int nvec, const int64_t *vsta
 __global__ void k_cross_leaf32(LeafGeom g, int P, double k2, const double *xt, const double *yt, const int64_t *lt,
                                const int64_t *ustart, const int32_t *usrc, const double *xs, const double *ysm,
                                const int64_t *lsrc, CrossNear nq, const zf *Lc, const zd *qs, int64_t ns,
-                               int64_t nt, int nvec, zd *us)
+                               int64_t nt, int nvec, int near, zd *us)
 {
     const int np = 2 * P + 1;
     const int64_t b = blockIdx.x;
@@ -454,7 +603,7 @@ __global__ void k_cross_leaf32(LeafGeom g, int P, double k2, const double *xt, c
                 }
             }
         }
-        for (int64_t e = ustart[b]; e < ustart[b + 1]; ++e) {
+        for (int64_t e = ustart[b]; near && e < ustart[b + 1]; ++e) {
             const int32_t s = usrc[e];
             zf part[LM_MAXV]; // one source leaf summed on its own
             for (int v = 0; v < nvec; ++v) part[v] = zf{0.f, 0.f};
@@ -741,6 +890,62 @@ static lm_status cross_setup(lm_cross_s *c, const double *xs, const double *ys, 
         lm_set_error("build_cross: an M2L table could not be built at this order");
         return LM_ENOTSUP;
     }
+    // double-float form
+    const double wl = c->lev[L].w;
+    c->ndf = c->med.opt.precision == LM_MIXED || !c->med.opt.m2l_fp64;
+    c->xdf = c->med.opt.precision == LM_FP64 && !c->med.opt.m2l_fp64 && lm_exp_df_fits(k1, wl) && lm_exp_df_fits(k2, wl);
+    if (c->ndf) {
+        const int nt = c->nray * c->ntail;
+        CTRY(calloc_dev(c, &c->qdf, (size_t)LM_MAXV * c->ns));
+        CTRY(calloc_dev(c, &c->qexp, 1));
+        CTRY(calloc_dev(c, &c->seg_node, 3 * c->nseg));
+        CTRY(calloc_dev(c, &c->seg_wdf, 2 * c->nseg));
+        CTRY(calloc_dev(c, &c->tail_node, 3 * nt));
+        CTRY(calloc_dev(c, &c->tail_wdf, 4 * nt));
+        k_cross_tab<<<gridc(c->nseg, 64), 64, 0, st>>>(c->nseg, c->seg_lam, c->seg_s1, c->seg_s2, c->seg_w, 0, c->seg_node,
+                                                       c->seg_wdf);
+        k_cross_tab<<<gridc(nt, 64), 64, 0, st>>>(nt, c->tail_lam, c->tail_s1, c->tail_s2, c->tail_w, 1, c->tail_node,
+                                                  c->tail_wdf);
+    }
+    if (c->xdf) {
+        std::vector<float> hs, ht;
+        float2 *bs, *bt;
+        lm_bessel_df(P, k1, wl, hs, &c->bes_s.N, &c->bes_s.nt);
+        lm_bessel_df(P, k2, wl, ht, &c->bes_t.N, &c->bes_t.nt);
+        CTRY(calloc_dev(c, &bs, hs.size() / 2));
+        CTRY(calloc_dev(c, &bt, ht.size() / 2));
+        c->bes_s.c = bs;
+        c->bes_t.c = bt;
+        LM_CUDA(cudaMemcpyAsync(bs, hs.data(), hs.size() * sizeof(float), cudaMemcpyHostToDevice, st));
+        LM_CUDA(cudaMemcpyAsync(bt, ht.data(), ht.size() * sizeof(float), cudaMemcpyHostToDevice, st));
+        CTRY(calloc_dev(c, &c->rel_s, c->ns));
+        CTRY(calloc_dev(c, &c->rel_t, c->nt));
+        const LeafGeom g{c->lev[L].ncol, c->x0, wl};
+        k_cross_rel<<<(unsigned)c->nleaf, 64, 0, st>>>(g, 0.5 * k1, c->xs_s, c->ys_s, c->ls_s, c->rel_s);
+        k_cross_rel<<<(unsigned)c->nleaf, 64, 0, st>>>(g, 0.5 * k2, c->xs_t, c->ys_t, c->ls_t, c->rel_t);
+        std::vector<M2LLevelDF> ml;
+        c->nblk = 0;
+        for (int l = 0; l <= L; ++l) {
+            CrossLevel &lv = c->lev[l];
+            const int64_t nc = std::max(1, lv.ncls);
+            CTRY(calloc_dev(c, &lv.tabdft, (size_t)nc * np * np));
+            lm_tab_df_t(lv.tab, nc, np, lv.tabdft, st);
+            if (lv.m2m) {
+                CTRY(calloc_dev(c, &lv.m2mdf, (size_t)4 * np * np));
+                lm_tab_df_t(lv.m2m, 4, np, lv.m2mdf, st);
+            }
+            if (lv.l2l) {
+                CTRY(calloc_dev(c, &lv.l2ldf, (size_t)4 * np * np));
+                lm_tab_df_t(lv.l2l, 4, np, lv.l2ldf, st);
+            }
+            ml.push_back({c->nblk, lv.vstart, lv.vsrc, lv.vslot, lv.tabdft, (const float4 *)lv.M, (float4 *)lv.Lc});
+            c->nblk += lv.nbox;
+        }
+        CTRY(calloc_dev(c, &c->mlev, ml.size()));
+        LM_CUDA(cudaMemcpyAsync(c->mlev, ml.data(), ml.size() * sizeof(M2LLevelDF), cudaMemcpyHostToDevice, st));
+        LM_CUDA(cudaStreamSynchronize(st)); // host temporaries
+    }
+    LM_CUDA(cudaGetLastError());
     if (c->med.opt.precision == LM_MIXED) {
         for (int l = 0; l <= L; ++l) {
             CrossLevel &lv = c->lev[l];
@@ -818,6 +1023,23 @@ extern "C" lm_status lm_cross_info(lm_cross c, int64_t *ns, int64_t *nt, int *R,
     return LM_OK;
 }
 
+// near pairs of the leaves of the top row (no other has any), added to us
+static void cross_near_df(lm_cross_s *c, int nv, cudaStream_t st)
+{
+    if (!c->ndf || c->nu == 0) return;
+    const CrossLevel &lv = c->lev[c->L];
+    const CrossNearDF nq{c->nseg, c->nray, c->ntail, c->seg_node, c->seg_wdf, c->tail_node, c->tail_wdf};
+    const dim3 g((unsigned)lv.ncol, (unsigned)std::max<int64_t>(1, std::min<int64_t>(16, 1216 / lv.ncol)));
+    auto run = [&](auto kern) {
+        kern<<<g, 128, 0, st>>>(c->med.k2, c->xs_t, c->ys_t, c->ls_t, c->ustart, c->usrc, c->xs_s, c->ys_s, c->ls_s, nq, c->qdf,
+                                c->qexp, c->nt, nv, c->us);
+    };
+    if (nv == 1) run(k_cross_near_df<1>);
+    else if (nv == 2) run(k_cross_near_df<2>);
+    else if (nv <= 4) run(k_cross_near_df<4>);
+    else run(k_cross_near_df<16>);
+}
+
 extern "C" lm_status lm_cross_apply(lm_cross c, const void *q, int nvec, void *u, void *stream)
 {
     if (!c || !q || !u || nvec < 1) {
@@ -838,6 +1060,28 @@ extern "C" lm_status lm_cross_apply(lm_cross c, const void *q, int nvec, void *u
     for (int v0 = 0; v0 < nvec; v0 += LM_MAXV) {
         const int nv = std::min(LM_MAXV, nvec - v0);
         k_permute_in<<<gridc(c->ns, 256), 256, 0, st>>>(qd + (int64_t)v0 * c->ns, c->perm_s, c->ns, nv, 0, c->qs);
+        if (c->ndf || c->xdf) {
+            LM_CUDA(cudaMemsetAsync(c->qexp, 0x80, sizeof(int), st)); // below any exponent
+            k_qexp<<<std::min(1024, gridc(c->ns * nv, 256)), 256, 0, st>>>(c->qs, c->ns, nv, c->qexp);
+            k_q_df<<<gridc(c->ns * nv, 256), 256, 0, st>>>(c->qs, c->ns, nv, c->qexp, c->qdf);
+        }
+        if (c->xdf) {
+            auto M = [&](int l) { return (float4 *)c->lev[l].M; };
+            auto Lx = [&](int l) { return (float4 *)c->lev[l].Lc; };
+            const CrossLevel &lf = c->lev[L];
+            const LeafGeom g{lf.ncol, c->x0, lf.w};
+            lm_df_s2m(c->bes_s, g, lf.nbox, P, c->med.k1, c->rel_s, c->ls_s, c->qdf, nv, M(L), st);
+            for (int l = L - 1; l >= 0; --l)
+                lm_df_m2m(c->lev[l].ncol, c->lev[l].nbox, P, nv, c->lev[l].m2mdf, M(l + 1), M(l), st);
+            lm_df_m2l(c->mlev, L + 1, c->nblk, P, nv, st);
+            for (int l = 1; l <= L; ++l)
+                lm_df_l2l(c->lev[l - 1].ncol, c->lev[l - 1].nbox, P, nv, c->lev[l].l2ldf, Lx(l - 1), Lx(l), st);
+            lm_df_l2t(c->bes_t, g, lf.nbox, P, c->med.k2, c->rel_t, c->ls_t, Lx(L), nv, c->qexp, c->nt, c->us, st);
+            cross_near_df(c, nv, st);
+            k_permute_out<<<gridc(c->nt, 256), 256, 0, st>>>(c->us, c->perm_t, c->nt, nv, 0, ud + (int64_t)v0 * c->nt);
+            LM_CUDA(cudaGetLastError());
+            continue;
+        }
         if (c->med.opt.precision == LM_MIXED) {
             {
                 const CrossLevel &lv = c->lev[L];
@@ -864,7 +1108,8 @@ extern "C" lm_status lm_cross_apply(lm_cross c, const void *q, int nvec, void *u
             const CrossLevel &lv = c->lev[L];
             k_cross_leaf32<<<(unsigned)lv.nbox, 64, 0, st>>>(LeafGeom{lv.ncol, c->x0, lv.w}, P, c->med.k2, c->xs_t,
                                                              c->ys_t, c->ls_t, c->ustart, c->usrc, c->xs_s, c->ys_s,
-                                                             c->ls_s, nq, lv.L32, c->qs, c->ns, c->nt, nv, c->us);
+                                                             c->ls_s, nq, lv.L32, c->qs, c->ns, c->nt, nv, !c->ndf, c->us);
+            cross_near_df(c, nv, st);
             k_permute_out<<<gridc(c->nt, 256), 256, 0, st>>>(c->us, c->perm_t, c->nt, nv, 0, ud + (int64_t)v0 * c->nt);
             LM_CUDA(cudaGetLastError());
             continue;
@@ -895,7 +1140,8 @@ extern "C" lm_status lm_cross_apply(lm_cross c, const void *q, int nvec, void *u
             const CrossLevel &lv = c->lev[L];
             k_cross_leaf<<<(unsigned)lv.nbox, 64, 0, st>>>(LeafGeom{lv.ncol, c->x0, lv.w}, P, c->med.k2, c->xs_t,
                                                            c->ys_t, c->ls_t, c->ustart, c->usrc, c->xs_s, c->ys_s,
-                                                           c->ls_s, nq, lv.Lc, c->qs, c->ns, c->nt, nv, c->us);
+                                                           c->ls_s, nq, lv.Lc, c->qs, c->ns, c->nt, nv, !c->ndf, c->us);
+            cross_near_df(c, nv, st);
         }
         k_permute_out<<<gridc(c->nt, 256), 256, 0, st>>>(c->us, c->perm_t, c->nt, nv, 0, ud + (int64_t)v0 * c->nt);
         LM_CUDA(cudaGetLastError());
