@@ -158,6 +158,7 @@ struct AdaptTree {
     float4 *tabdft = nullptr;                          // double-float copy (as Level)
     // mixed form: FP32 copies of the tables and expansions, and per level the boxes with V entries
     zf *tab32 = nullptr, *M32 = nullptr, *L32 = nullptr;
+    zf *tab32t = nullptr;                              // tab32 transposed ([q][p])
     std::vector<int32_t *> m2l_tgt;
     std::vector<int64_t> m2l_ntgt;
 };
@@ -266,6 +267,7 @@ struct lm_tree_s {
     bool near_pw64; // FP64 reflected near field: segment factorised per leaf (k_near_pw64)
     int32_t *pwidx; // [boxes of the leaf level / of the tree] slot of an interface leaf, or -1
     zd *pwC;        // [slots][2 terms][2 nseg][LM_MAXV] per-leaf segment coefficients (k_pw_src64)
+    bool few32;     // mixed form: applies of up to 4 vectors take lmfmm_few32.cu's kernels
     bool adaptive;  // boxes refined where the points are (AdaptTree), FP64 only
     AdaptTree at;
     int *dflag;  // device error flag
@@ -325,6 +327,7 @@ lm_status lm_run_apply(lm_tree_s *t, const zd *q, int nvec, zd *u, bool adjoint,
 size_t lm_near_pw64_smem(int nseg);
 lm_status lm_near_pw64_attr(size_t bytes);
 lm_status lm_setup_pwsrc(lm_tree_s *t, cudaStream_t st); // interface-leaf slots and coefficient buffer
+lm_status lm_setup_pwidx(lm_tree_s *t, int64_t *npw, cudaStream_t st);
 lm_status lm_setup_df(lm_tree_s *t, cudaStream_t st); // the FP64 form's double-float data
 lm_status lm_setup_near_df(lm_tree_s *t, cudaStream_t st); // double-float near field (lmfmm_near_df.cu)
 void lm_launch_q_df(lm_tree_s *t, int nv, cudaStream_t st);
@@ -356,6 +359,12 @@ lm_status lm_autotune_mixed(lm_tree_s *t, cudaStream_t st, int *choice, float *m
 lm_status lm_run_apply_mixed(lm_tree_s *t, const void *q, int nvec, void *u, bool adjoint, bool c64, cudaStream_t st,
                              int part = 0);
 void lm_free_mixed(lm_tree_s *t);
+// applies of up to 4 vectors (lmfmm_few32.cu)
+struct NearQuadF;
+lm_status lm_setup_few32(lm_tree_s *t, cudaStream_t st);
+void lm_few32_s2m(lm_tree_s *t, int nv, cudaStream_t st);
+void lm_few32_m2l(lm_tree_s *t, int nv, cudaStream_t st);
+int lm_few32_leaf(lm_tree_s *t, const NearQuadF &nq, int nv, cudaStream_t st);
 // tensor-core M2L (lmfmm_tc.cu)
 lm_status lm_setup_tc(lm_tree_s *t, cudaStream_t st);
 lm_status lm_launch_m2l_tc(lm_tree_s *t, int l, cudaStream_t st, int nvs); // nvs: 4 or 16 vector slots

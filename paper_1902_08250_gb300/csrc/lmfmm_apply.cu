@@ -957,22 +957,19 @@ lm_status lm_setup_df(lm_tree_s *t, cudaStream_t st)
     return s;
 }
 
-// slots of the interface leaves (the blocks of k_pw_src64 / k_near_pw64) and their
-// per-apply plane-wave coefficients (FP64 form with the factorised segment)
-lm_status lm_setup_pwsrc(lm_tree_s *t, cudaStream_t st)
+// slots of the interface leaves (the blocks of the factorised segment's kernels): pwidx
+lm_status lm_setup_pwidx(lm_tree_s *t, int64_t *npw, cudaStream_t st)
 {
-    if (!t->near_pw64) return LM_OK;
     std::vector<int32_t> idx;
-    int64_t npw;
     if (t->adaptive) {
         idx.assign(t->at.nbox, -1);
-        npw = (int64_t)t->at.hpw.size();
-        for (int64_t i = 0; i < npw; ++i) idx[t->at.hpw[i]] = (int32_t)i;
+        *npw = (int64_t)t->at.hpw.size();
+        for (int64_t i = 0; i < *npw; ++i) idx[t->at.hpw[i]] = (int32_t)i;
     } else {
         const Level &lv = t->lev[t->L];
         idx.assign(lv.nbox, -1);
-        npw = lv.nrow == 1 ? lv.ncol : 2 * lv.ncol;
-        for (int64_t i = 0; i < npw; ++i) { // the block order of EdgeRowLeaves
+        *npw = lv.nrow == 1 ? lv.ncol : 2 * lv.ncol;
+        for (int64_t i = 0; i < *npw; ++i) { // the block order of EdgeRowLeaves
             const int64_t row = (lv.nrow == 1 || i < lv.ncol) ? 0 : lv.nrow - 1;
             idx[row * lv.ncol + i % lv.ncol] = (int32_t)i;
         }
@@ -981,5 +978,14 @@ lm_status lm_setup_pwsrc(lm_tree_s *t, cudaStream_t st)
     if (s != LM_OK) return s;
     LM_CUDA(cudaMemcpyAsync(t->pwidx, idx.data(), idx.size() * sizeof(int32_t), cudaMemcpyHostToDevice, st));
     LM_CUDA(cudaStreamSynchronize(st)); // idx is a host temporary
+    return LM_OK;
+}
+// and the per-apply plane-wave coefficients of the FP64 form
+lm_status lm_setup_pwsrc(lm_tree_s *t, cudaStream_t st)
+{
+    if (!t->near_pw64) return LM_OK;
+    int64_t npw = 0;
+    lm_status s = lm_setup_pwidx(t, &npw, st);
+    if (s != LM_OK) return s;
     return lm_dalloc(t, &t->pwC, (size_t)std::max<int64_t>(1, npw) * 2 * 2 * t->nq.nseg * LM_MAXV);
 }

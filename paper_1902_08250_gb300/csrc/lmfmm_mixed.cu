@@ -17,36 +17,6 @@ static int gridm(int64_t n, int b) { return (int)((n + b - 1) / b); }
 
 LM_HD zf f2(zd a) { return zf{(float)a.re, (float)a.im}; }
 
-// Box geometry of the FP32 kernels.  Grid32: leaf i of the uniform leaf lattice
-// (ncol columns of width w); List32: box ids[i] of the adaptive tree, with
-// centres and widths from its arrays.  offset(t, s) = centre_t - centre_s.
-struct Grid32 {
-    int64_t ncol;
-    float w;
-    __device__ int64_t id(int64_t i) const { return i; }
-    __device__ float width(int64_t) const { return w; }
-    __device__ void offset(int64_t bt, int64_t bs, float &ox, float &oy) const
-    {
-        const int rt = (int)(bt / ncol), ct = (int)(bt % ncol), rs = (int)(bs / ncol), cs = (int)(bs % ncol);
-        ox = (float)(ct - cs) * w;
-        oy = -(float)(rt - rs) * w;
-    }
-};
-struct EdgeGrid32 : Grid32 { // the leaves of the top row, then (nrow > 1) of the bottom row
-    int64_t nrow;
-    __device__ int64_t id(int64_t i) const { return ((nrow == 1 || i < ncol) ? 0 : nrow - 1) * ncol + i % ncol; }
-};
-struct List32 {
-    const int32_t *ids;
-    const double *bx, *by, *bw;
-    __device__ int64_t id(int64_t i) const { return ids[i]; }
-    __device__ float width(int64_t b) const { return (float)bw[b]; }
-    __device__ void offset(int64_t bt, int64_t bs, float &ox, float &oy) const
-    {
-        ox = (float)(bx[bt] - bx[bs]);
-        oy = (float)(by[bt] - by[bs]);
-    }
-};
 // parents and their four children: the lattice one level down, or the adaptive tree's links
 struct GridKids32 {
     int64_t ncol;
@@ -266,7 +236,7 @@ static lm_status setup_mixed_points(lm_tree_s *t, cudaStream_t st)
     }
     LM_CUDA(lm_raise_smem((const void *)k_near_pw32<EdgeGrid32>, LM_SMEM_NEAR_PW, (int)shm));
     LM_CUDA(lm_raise_smem((const void *)k_near_pw32<List32>, LM_SMEM_NEAR_PW_A, (int)shm));
-    return LM_OK;
+    return lm_setup_few32(t, st);
 }
 
 // leaf-local coordinates of the adaptive tree's leaves (box centres from its arrays)
@@ -341,7 +311,7 @@ void lm_free_mixed(lm_tree_s *t)
     lm_free_leaf_tt(t);
     {
         AdaptTree &A = t->at;
-        void *ap[] = {A.tab32, A.M32, A.L32};
+        void *ap[] = {A.tab32, A.tab32t, A.M32, A.L32};
         for (void *p : ap)
             if (p) cudaFree(p);
         for (int32_t *p : A.m2l_tgt)
@@ -1396,6 +1366,15 @@ static void launch_l2l_list(const AdaptTree &A, const Level &lv, int l, cudaStre
         k_l2l32<NP, LM_MAXV, false, ListPar32><<<(unsigned)nb, 128, 0, st>>>(par, lv.l2l32, A.L32, A.L32,
                                                                              nullptr);
 }
+// up to 4 vectors: adds to the M2L's local expansions
+template <int P>
+static void launch_l2l_list_acc(const AdaptTree &A, const Level &lv, int l, cudaStream_t st)
+{
+    const int64_t b0 = A.lev_start[l], nb = A.lev_start[l + 1] - b0;
+    if (nb > 0)
+        k_l2l32<2 * P + 1, 4, true, ListPar32><<<(unsigned)nb, 128, 0, st>>>(ListPar32{b0, A.parent, A.pos}, lv.l2l32, A.L32,
+                                                                             A.L32, nullptr);
+}
 template <int P>
 static void launch_rest_list(const AdaptTree &A, int l, cudaStream_t st, int nvs)
 {
@@ -1445,7 +1424,9 @@ static lm_status run_mixed_adaptive(lm_tree_s *t, const void *q, int nvec, void 
                                                              adjoint, t->qs32, nullptr);
         lm_phase_end(t, PH_PERMUTE, st, 1);
         lm_phase_begin(t, PH_S2M, st);
-        if (A.nleaf > 0) {
+        const bool few = nv <= 4 && t->few32;
+        if (few) lm_few32_s2m(t, nv, st);
+        else if (A.nleaf > 0) {
             const size_t shm = (P2M32_CHUNK * np + P2M32_CHUNK * LM_MAXV) * sizeof(zf);
             k_p2m32<List32><<<(unsigned)A.nleaf, 128, shm, st>>>(leaves, P, k, t->xl32, t->yl32, t->leaf_start,
                                                                  t->qs32, nvs, A.M32);
@@ -1454,7 +1435,15 @@ static lm_status run_mixed_adaptive(lm_tree_s *t, const void *q, int nvec, void 
         if (L > 0) lm_phase_begin(t, PH_M2M, st);
         for (int l = L - 1; l >= 0; --l) MX_DISPATCH(P, launch_m2m_list, A, t->lev[l], l, st, nvs);
         if (L > 0) lm_phase_end(t, PH_M2M, st, L);
-        for (int l = 0; l <= L; ++l) {
+        if (few) { // M2L of every level at once, then L2L adds
+            lm_phase_begin(t, PH_M2L, st);
+            lm_few32_m2l(t, nv, st);
+            lm_phase_end(t, PH_M2L, st, 1);
+            if (L > 0) lm_phase_begin(t, PH_L2L, st);
+            for (int l = 1; l <= L; ++l) MX_DISPATCH(P, launch_l2l_list_acc, A, t->lev[l], l, st);
+            if (L > 0) lm_phase_end(t, PH_L2L, st, L);
+        }
+        for (int l = 0; l <= L && !few; ++l) {
             lm_phase_begin(t, PH_L2L, st);
             if (l == 0) {
                 const int64_t nb = A.lev_start[1] - A.lev_start[0];
@@ -1468,12 +1457,13 @@ static lm_status run_mixed_adaptive(lm_tree_s *t, const void *q, int nvec, void 
             lm_phase_end(t, PH_M2L, st, A.m2l_ntgt[l] > 0);
         }
         lm_phase_begin(t, PH_LEAF, st);
-        if (A.nleaf > 0) MX_DISPATCH(P, launch_leaf_list, t, nq, st, nv);
-        if (A.npw > 0)
+        const int few_k = few ? lm_few32_leaf(t, nq, nv, st) : 0;
+        if (!few && A.nleaf > 0) MX_DISPATCH(P, launch_leaf_list, t, nq, st, nv);
+        if (!few && A.npw > 0)
             k_near_pw32<List32><<<(unsigned)A.npw, 256, near_pw_smem(t), st>>>(
                 pwl, (float)t->med.d, t->xl32, t->y32, t->leaf_start, t->ustart, t->usrc, t->uterm, nq, t->qs32,
                 t->us32);
-        lm_phase_end(t, PH_LEAF, st, 1 + (A.npw > 0));
+        lm_phase_end(t, PH_LEAF, st, few ? few_k : 1 + (A.npw > 0));
         lm_phase_begin(t, PH_PERMUTE, st);
         if (c64)
             k_permute_out32<zf><<<gridm(n, 256), 256, 0, st>>>(t->us32, t->iperm, n, nv, adjoint,
@@ -1532,7 +1522,9 @@ lm_status lm_run_apply_mixed(lm_tree_s *t, const void *q, int nvec, void *u, boo
         lm_phase_begin(t, PH_S2M, st);
         {
             Level &lv = t->lev[L];
-            if (s2m16_ok(t, nvs)) {
+            if (nv <= 4 && t->few32) {
+                lm_few32_s2m(t, nv, st);
+            } else if (s2m16_ok(t, nvs)) {
                 MX_DISPATCH(P, launch_s2m16, lv, k, t, st);
             } else {
                 size_t shm = (P2M32_CHUNK * np + P2M32_CHUNK * LM_MAXV) * sizeof(zf);
@@ -1591,8 +1583,11 @@ lm_status lm_run_apply_mixed(lm_tree_s *t, const void *q, int nvec, void *u, boo
             lm_phase_end(t, PH_M2L, st, launches);
         }
         lm_phase_begin(t, PH_LEAF, st);
-        MX_DISPATCH(P, launch_leaf, t, nq, st, nv);
-        {
+        int leafk = 2;
+        if (nv <= 4 && t->few32) {
+            leafk = lm_few32_leaf(t, nq, nv, st);
+        } else {
+            MX_DISPATCH(P, launch_leaf, t, nq, st, nv);
             const Level &lv = t->lev[L];
             const unsigned nb = (unsigned)(lv.nrow == 1 ? lv.ncol : 2 * lv.ncol);
             EdgeGrid32 eg;
@@ -1603,7 +1598,7 @@ lm_status lm_run_apply_mixed(lm_tree_s *t, const void *q, int nvec, void *u, boo
                                                           t->y32, t->leaf_start, t->ustart, t->usrc, t->uterm, nq,
                                                           t->qs32, t->us32);
         }
-        lm_phase_end(t, PH_LEAF, st, 2);
+        lm_phase_end(t, PH_LEAF, st, leafk);
         lm_phase_begin(t, PH_PERMUTE, st);
         if (c64)
             k_permute_out32<zf><<<gridm(n, 256), 256, 0, st>>>(t->us32, t->iperm, n, nv, adjoint,

@@ -4,6 +4,37 @@
 #pragma once
 #include "internal.h"
 
+// Box geometry of the FP32 kernels.  Grid32: leaf i of the uniform leaf lattice
+// (ncol columns of width w); List32: box ids[i] of the adaptive tree, with
+// centres and widths from its arrays.  offset(t, s) = centre_t - centre_s.
+struct Grid32 {
+    int64_t ncol;
+    float w;
+    __device__ int64_t id(int64_t i) const { return i; }
+    __device__ float width(int64_t) const { return w; }
+    __device__ void offset(int64_t bt, int64_t bs, float &ox, float &oy) const
+    {
+        const int rt = (int)(bt / ncol), ct = (int)(bt % ncol), rs = (int)(bs / ncol), cs = (int)(bs % ncol);
+        ox = (float)(ct - cs) * w;
+        oy = -(float)(rt - rs) * w;
+    }
+};
+struct EdgeGrid32 : Grid32 { // the leaves of the top row, then (nrow > 1) of the bottom row
+    int64_t nrow;
+    __device__ int64_t id(int64_t i) const { return ((nrow == 1 || i < ncol) ? 0 : nrow - 1) * ncol + i % ncol; }
+};
+struct List32 {
+    const int32_t *ids;
+    const double *bx, *by, *bw;
+    __device__ int64_t id(int64_t i) const { return ids[i]; }
+    __device__ float width(int64_t b) const { return (float)bw[b]; }
+    __device__ void offset(int64_t bt, int64_t bs, float &ox, float &oy) const
+    {
+        ox = (float)(bx[bt] - bx[bs]);
+        oy = (float)(by[bt] - by[bs]);
+    }
+};
+
 // asynchronous global -> shared copies (cp.async), completed per commit group
 __device__ __forceinline__ void cp_async4(void *sdst, const void *gsrc)
 {
@@ -139,3 +170,4 @@ static __device__ __noinline__ zf near_tail32(const NearQuadF &q, int m, float X
     return zf{re, im};
 }
 
+int lm_h0_terms(double xmax); // lmfmm_mixed.cu
