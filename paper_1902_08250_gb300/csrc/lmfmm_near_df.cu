@@ -13,8 +13,9 @@
 // the argument of the ascending series; densities by 2^-qexp (as the multipoles).
 // A kernel value g = g_re + i g_im is kept as (A, J), g_re = -A/(4 pi), g_im = J/4:
 // for the free pair A = (ln z + 2 gamma) J + 2 V, J = J0, so the constants are
-// applied once per target.  Pairs outside the series' range (z > 1, or closer than
-// 2^-45 in these units) take the FP64 functions.
+// applied once per target.  A pair closer than 2^-10 leaf widths takes its offset from the
+// FP64 coordinates (the leaf-relative ones are good to 2^-49 of the leaf); pairs outside the
+// series' range (z > 1, or closer than 2^-45 in these units) take the FP64 functions.
 #include <algorithm>
 
 #include "df.cuh"
@@ -304,6 +305,7 @@ __global__ void __launch_bounds__(ND_THREADS, GRAD ? 3 : 4)
     tab.load();
     double cx, cy, bw;
     geo.centre(b, &cx, &cy, &bw);
+    const float zclose = (float)(kap * kap * bw * bw) * 0x1p-20f;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t u0 = ustart[b], u1 = ustart[b + 1];
     constexpr int ROWS = TG / (ND_THREADS / 32), HALF = SRC / 32;
@@ -385,14 +387,19 @@ __global__ void __launch_bounds__(ND_THREADS, GRAD ? 3 : 4)
                     if (s >= ns) continue;
                     const float4 tp = tr[row], p = sp[s];
                     const int term = st[s];
-                    const df dx = df_sub(df_re(tp), df_re(p));
+                    df dx = df_sub(df_re(tp), df_re(p));
                     GradVal G; // [1..]: d/dx, d/dy (GRAD)
 #pragma unroll
                     for (int c = 0; c < 3; ++c) G.A[c] = G.J[c] = df{0.f, 0.f};
                     if (term == 0) {
                         if (sj[s] != t0 + row) {
-                            const df dy = df_sub(df_im(tp), df_im(p));
-                            const df z = df_add(df_sq(dx), df_sq(dy));
+                            df dy = df_sub(df_im(tp), df_im(p));
+                            df z = df_add(df_sq(dx), df_sq(dy));
+                            if (z.h < zclose) {
+                                dx = df_of((xs[t0 + row] - xs[sj[s]]) * kap);
+                                dy = df_of((ys[t0 + row] - ys[sj[s]]) * kap);
+                                z = df_add(df_sq(dx), df_sq(dy));
+                            }
                             const bool slow = z.h > 1.0f || z.h < ND_TINY;
                             if (GRAD) {
                                 HVal H;
@@ -410,10 +417,11 @@ __global__ void __launch_bounds__(ND_THREADS, GRAD ? 3 : 4)
                         }
                     } else {
                         const int m = term - 1;
-                        const df X = dx.h < 0.f ? df_neg(dx) : dx;
                         const float4 hh = th[row];
                         df h = df_add(m == 0 ? df_re(hh) : df_im(hh), df_im(p));
                         if (m == 0) h = df_neg(h); // tt: -(y + y0); bb: (y + d) + (y0 + d)
+                        if (dx.h * dx.h + h.h * h.h < zclose) dx = df_of((xs[t0 + row] - xs[sj[s]]) * kap);
+                        const df X = dx.h < 0.f ? df_neg(dx) : dx;
                         const int64_t wo = (int64_t)m * (GRAD ? 6 : 2) * nq.nray * nq.ntail;
                         if (GRAD) seg_df_grad(tab, nq, m, X, h, &G);
                         auto tail = [&](const float4 *w, float hr) {
