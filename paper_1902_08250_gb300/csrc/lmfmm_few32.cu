@@ -93,29 +93,35 @@ __global__ void __launch_bounds__(64) k_s2m_f32(G geo, int P, float k, BesselDF 
 }
 
 // ---------------------------------------------------------------------------
-// L2T and the direct interactions.  One block: up to tb <= 16 targets of a leaf at a time, 4 rows
-// per warp.  The leaf's near sources are flattened and staged 64 at a time in the target leaf's
-// frame; each lane takes two of them against the warp's rows, kernel value and multiply-adds in
-// registers, and the lanes' sums are folded once per target by exchanging halves.  Reflected pairs
-// add their tails (the segment part comes from k_near_pw_f32).
-// DEG as in k_leaf32.
+// L2T and the direct interactions.  One block: up to tb targets of a leaf at a time, ROWS rows per
+// warp.  The leaf's near sources are flattened and staged 64 at a time in the target leaf's frame; each
+// lane takes two of them against the warp's rows, kernel value and multiply-adds in registers, and the
+// lanes' sums are folded once per target by exchanging halves.  Reflected pairs add their tails (the
+// segment part comes from k_near_pw_f32).  DEG as in k_leaf32.
+// Bound by FP32 issue and, between the rounds, by the staging and the barriers: more rows a warp
+// spread those over more pairs.  Uniform 100k points, 1 vector: 193 us with 4 rows, 153 us with 8;
+// 12 trees of 4 vectors: 3.46 ms with 4 rows, 3.29 ms with 6 (8 spill).  Clustered adaptive 100k, whose
+// leaves hold fewer points than 32: 186 us with 4 rows, 256 us with 8.
 // ---------------------------------------------------------------------------
-#define F32_TGT 16
+// rows of a warp on large uniform trees (4 vectors' sums take more registers), F32_ROWS elsewhere
+__host__ __device__ constexpr int f32_rows(int nv) { return nv == 4 ? 6 : 8; }
+#define F32_ROWS 4
 #define F32_SRC 64
 #define F32_ENT 64
-template <int NV, int DEG, class G>
+template <int NV, int DEG, int ROWS, class G>
 __global__ void __launch_bounds__(128) k_leaf_f32(G geo, int P, float k, float d, BesselDF B, const float *xl, const float *yl,
                                                   const float *y32, const int64_t *ls, const int64_t *ustart,
                                                   const int32_t *usrc, const int32_t *uterm, NearQuadF nq, const zf *Lc,
                                                   const zf *qs, zf *us, int nv, int tb, int free_on)
 {
+    constexpr int TGT = 4 * ROWS;
     __shared__ int fj0[F32_ENT], fpre[F32_ENT + 1], fterm[F32_ENT];
     __shared__ float2 foff[F32_ENT];
     __shared__ float2 sp[F32_SRC];
     __shared__ int sj[F32_SRC], st[F32_SRC];
     __shared__ zf sq[F32_SRC][NV];
-    __shared__ float4 tr[F32_TGT]; // x, y relative to the leaf centre, absolute y
-    __shared__ zf bz[F32_TGT][25], PQ[25][NV][2], uL[F32_TGT][NV];
+    __shared__ float4 tr[TGT]; // x, y relative to the leaf centre, absolute y
+    __shared__ zf bz[TGT][25], PQ[25][NV][2], uL[TGT][NV];
     const int np = 2 * P + 1;
     const int64_t b = geo.id(blockIdx.x);
     const int lo = (int)ls[b], hi = (int)ls[b + 1];
@@ -149,16 +155,16 @@ __global__ void __launch_bounds__(128) k_leaf_f32(G geo, int P, float k, float d
             }
             uL[j][v] = a;
         }
-        float tx[4], ty[4];
+        float tx[ROWS], ty[ROWS];
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {
+        for (int r = 0; r < ROWS; ++r) {
             const float4 t = tr[min(warp + 4 * r, nt - 1)];
             tx[r] = t.x;
             ty[r] = t.y;
         }
-        zf acc[4][NV];
+        zf acc[ROWS][NV];
 #pragma unroll
-        for (int r = 0; r < 4; ++r)
+        for (int r = 0; r < ROWS; ++r)
 #pragma unroll
             for (int v = 0; v < NV; ++v) acc[r][v] = zf{0.f, 0.f};
         for (int c0 = e0; c0 < e1; c0 += F32_ENT) {
@@ -215,7 +221,7 @@ __global__ void __launch_bounds__(128) k_leaf_f32(G geo, int P, float k, float d
                     for (int v = 0; v < NV; ++v) q[v] = sq[s][v];
                     if (term == 0) {
 #pragma unroll
-                        for (int r = 0; r < 4; ++r) {
+                        for (int r = 0; r < ROWS; ++r) {
                             if (warp + 4 * r >= nt) break;
                             const float dx = tx[r] - p.x, dy = ty[r] - p.y;
                             const bool self = j == t0 + warp + 4 * r;
@@ -232,7 +238,7 @@ __global__ void __launch_bounds__(128) k_leaf_f32(G geo, int P, float k, float d
                         }
                     } else {
 #pragma unroll
-                        for (int r = 0; r < 4; ++r) {
+                        for (int r = 0; r < ROWS; ++r) {
                             if (warp + 4 * r >= nt) break;
                             const float ya = tr[warp + 4 * r].z;
                             const float hh = term == 1 ? -(ya + p.y) : ya + p.y + 2.0f * d;
@@ -245,35 +251,41 @@ __global__ void __launch_bounds__(128) k_leaf_f32(G geo, int P, float k, float d
                 __syncthreads(); // the sources are overwritten by the next round
             }
         }
-        // 8 NV sums over the lanes: at each step a lane keeps one half of them
-        float val[8 * NV];
+        // 2 NV sums of each row over the lanes, RP rows at a time: at each step a lane keeps one half of
+        // them
+        constexpr int RP = NV * ROWS <= 16 ? ROWS : 2, CNT = 2 * NV * RP; // 8, 16 or 32 sums
 #pragma unroll
-        for (int r = 0; r < 4; ++r)
+        for (int r0 = 0; r0 < ROWS; r0 += RP) {
+            if (warp + 4 * r0 >= nt) break;
+            float val[CNT];
 #pragma unroll
-            for (int v = 0; v < NV; ++v) {
-                val[2 * (r * NV + v)] = acc[r][v].re;
-                val[2 * (r * NV + v) + 1] = acc[r][v].im;
+            for (int r = 0; r < RP; ++r)
+#pragma unroll
+                for (int v = 0; v < NV; ++v) {
+                    val[2 * (r * NV + v)] = acc[r0 + r][v].re;
+                    val[2 * (r * NV + v) + 1] = acc[r0 + r][v].im;
+                }
+            int cnt = CNT;
+#pragma unroll
+            for (int o = 16; o >= 1; o >>= 1) {
+                if (cnt > 1) {
+                    cnt >>= 1;
+#pragma unroll
+                    for (int i = 0; i < CNT / 2; ++i)
+                        if (i < cnt) {
+                            const float x = val[i], y = val[i + cnt];
+                            const bool up = (lane & o) != 0;
+                            val[i] = (up ? y : x) + __shfl_xor_sync(0xffffffffu, up ? x : y, o);
+                        }
+                } else
+                    val[0] += __shfl_xor_sync(0xffffffffu, val[0], o);
             }
-        int cnt = 8 * NV;
-#pragma unroll
-        for (int o = 16; o >= 1; o >>= 1) {
-            if (cnt > 1) {
-                cnt >>= 1;
-#pragma unroll
-                for (int i = 0; i < 4 * NV; ++i)
-                    if (i < cnt) {
-                        const float x = val[i], y = val[i + cnt];
-                        const bool up = (lane & o) != 0;
-                        val[i] = (up ? y : x) + __shfl_xor_sync(0xffffffffu, up ? x : y, o);
-                    }
-            } else
-                val[0] += __shfl_xor_sync(0xffffffffu, val[0], o);
-        }
-        constexpr int REP = 32 / (8 * NV); // lanes holding the same sum
-        const int id = lane / REP, row = warp + 4 * (id / (2 * NV)), vv = (id / 2) % NV;
-        if (lane % REP == 0 && row < nt && vv < nv) {
-            const zf l = uL[row][vv];
-            ((float *)&us[(int64_t)(t0 + row) * LM_MAXV + vv])[id & 1] = val[0] + ((id & 1) ? l.im : l.re);
+            constexpr int REP = 32 / CNT; // lanes holding the same sum
+            const int id = lane / REP, row = warp + 4 * (r0 + id / (2 * NV)), vv = (id / 2) % NV;
+            if (lane % REP == 0 && row < nt && vv < nv) {
+                const zf l = uL[row][vv];
+                ((float *)&us[(int64_t)(t0 + row) * LM_MAXV + vv])[id & 1] = val[0] + ((id & 1) ? l.im : l.re);
+            }
         }
     }
 }
@@ -510,9 +522,12 @@ int lm_few32_leaf(lm_tree_s *t, const NearQuadF &nq, int nv, cudaStream_t st)
     const float k = (float)t->med.k2, d = (float)t->med.d;
     const int free_on = t->med.opt.kernel == LM_KERNEL_G;
     const int64_t nleaf = t->adaptive ? t->at.nleaf : t->lev[t->L].nbox;
-    // targets a pass: 16, fewer while that leaves fewer than 4 blocks per SM (small trees)
+    // targets a pass: 32 (24 for 4 vectors) on a uniform tree that fills 4 blocks per SM with them,
+    // else 16, fewer while that leaves fewer than 4 blocks per SM (small trees)
     const int64_t per = std::max<int64_t>(1, (t->n + nleaf - 1) / nleaf);
-    int tb = F32_TGT;
+    const int big = 4 * f32_rows(nv <= 2 ? nv : 4);
+    const bool wide = !t->adaptive && nleaf * ((per + big - 1) / big) >= 608;
+    int tb = wide ? big : 4 * F32_ROWS;
     while (tb > 4 && nleaf * ((per + tb - 1) / tb) < 608) tb >>= 1;
     const unsigned gy = (unsigned)std::min<int64_t>(64, (per + tb - 1) / tb);
     const size_t shm = (size_t)2 * t->nq.nseg * (nv <= 2 ? nv : 4) * sizeof(zf);
@@ -528,7 +543,7 @@ int lm_few32_leaf(lm_tree_s *t, const NearQuadF &nq, int nv, cudaStream_t st)
     if (t->adaptive) {
         const AdaptTree &A = t->at;
         const List32 g{A.leaves, A.cx, A.cy, A.w}, e{A.pwleaves, A.cx, A.cy, A.w};
-        NV_FEW(nv, (leaf(k_leaf_f32<NV, 0, List32>, g, A.L32)));
+        NV_FEW(nv, (leaf(k_leaf_f32<NV, 0, F32_ROWS, List32>, g, A.L32)));
         if (A.npw == 0) return 1;
         NV_FEW(nv, (pw(k_pw_src_f32<NV, List32>, k_near_pw_f32<NV, List32>, e, A.npw)));
         return 3;
@@ -541,8 +556,9 @@ int lm_few32_leaf(lm_tree_s *t, const NearQuadF &nq, int nv, cudaStream_t st)
     e.nrow = lv.nrow;
     // largest k r of a direct pair: two leaves apart diagonally
     const double xmax = t->med.k2 * lv.w * 2.0 * 1.4142135623730951 * 1.0001;
-    if (xmax <= 2.0 && lm_h0_terms(xmax) <= 6) NV_FEW(nv, (leaf(k_leaf_f32<NV, 6, Grid32>, g, lv.L32)))
-    else NV_FEW(nv, (leaf(k_leaf_f32<NV, 0, Grid32>, g, lv.L32)))
+    const bool deg6 = xmax <= 2.0 && lm_h0_terms(xmax) <= 6;
+    NV_FEW(nv, (deg6 ? (wide ? leaf(k_leaf_f32<NV, 6, f32_rows(NV), Grid32>, g, lv.L32) : leaf(k_leaf_f32<NV, 6, F32_ROWS, Grid32>, g, lv.L32))
+                     : (wide ? leaf(k_leaf_f32<NV, 0, f32_rows(NV), Grid32>, g, lv.L32) : leaf(k_leaf_f32<NV, 0, F32_ROWS, Grid32>, g, lv.L32))));
     NV_FEW(nv, (pw(k_pw_src_f32<NV, EdgeGrid32>, k_near_pw_f32<NV, EdgeGrid32>, e, lv.nrow == 1 ? lv.ncol : 2 * lv.ncol)));
     return 3;
 }
