@@ -300,40 +300,59 @@ __global__ void __launch_bounds__(512) k_l2l_dx(Geo geo, int P, int nv, const fl
 }
 
 // M2L over the V lists of every level in one launch: one block per target box; sets L.
-// The entries form GS interleaved subsets, each summed on its own, then added in order: a vector's
-// sums do not depend on how many vectors are applied or on how many threads share a box.  PAR: a group
-// of threads per subset (up to 2 vectors, whose threads would be too few), else a thread takes them all.
-template <int NV, bool PAR>
-__global__ void __launch_bounds__(512) k_m2l_dx(const M2LLevelDF *lev, int nlev, int P, int nv, int GS)
+// The entries form GS interleaved subsets (3, or 12 for small trees), each summed on its own; the
+// sums of equal index mod 3 are added in order, then the three: a vector's result does not depend on
+// how many vectors are applied or on how many threads share a box.  G groups of threads (GS, 3 or 1)
+// take the subsets.  Bound by FP32 issue on large trees (24 multiply-adds a complex product) and by the
+// reads of table and multipoles in the two or three blocks an SM gets on small ones.
+template <int NV, int MINB>
+__global__ void __launch_bounds__(512, MINB) k_m2l_dx(const M2LLevelDF *lev, int nlev, int P, int nv, int GS, int G)
 {
     constexpr int VPT = NV < 4 ? NV : 4;
-    extern __shared__ float4 red[]; // PAR: [GS - 1][np][VPT]
+    extern __shared__ float4 red[]; // [G - 1][items][VPT]
     const int np = 2 * P + 1, vg = (nv + VPT - 1) / VPT, item = np * vg;
     int l = nlev - 1;
     while ((int64_t)blockIdx.x < lev[l].box0) --l;
     const M2LLevelDF &v = lev[l];
     const int64_t b = blockIdx.x - v.box0, e0 = v.vstart[b], e1 = v.vstart[b + 1];
-    const int p = threadIdx.x % np, r = threadIdx.x / np, g = PAR ? r : 0, v0 = PAR ? 0 : r * VPT, nvv = min(VPT, nv - v0);
-    if (!PAR && (int)threadIdx.x >= item) return;
+    const int it = threadIdx.x % item, g = threadIdx.x / item, p = it % np, v0 = it / np * VPT, nvv = min(VPT, nv - v0);
+    const int k3 = min(3, GS); // the last level of the sum
     float4 tot[VPT];
-    for (int s = g; s < (PAR ? min(g + 1, GS) : GS); ++s) {
-        float4 acc[VPT];
 #pragma unroll
-        for (int i = 0; i < VPT; ++i) acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int64_t e = e0 + s; e < e1; e += GS)
-            dot_q<VPT>(acc, v.tab + (int64_t)v.vslot[e] * np * np + p, v.M + (int64_t)v.vsrc[e] * np * nv + v0, np, nv);
+    for (int i = 0; i < VPT; ++i) tot[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (g < G) {
+        // G = GS: subset g; G = 3: subsets g, g + 3, ..; G = 1: all of them, class by class
+        for (int c = G == 1 ? 0 : g; c < (G == 1 ? k3 : g + 1); ++c) {
+            float4 part[VPT];
+            for (int s = c; s < (G == GS && G > 1 ? c + 1 : GS); s += 3) {
+                float4 acc[VPT];
 #pragma unroll
-        for (int i = 0; i < VPT; ++i) tot[i] = s == g ? df_norm(acc[i]) : dfc_add(tot[i], df_norm(acc[i]));
+                for (int i = 0; i < VPT; ++i) acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+                for (int64_t e = e0 + s; e < e1; e += GS)
+                    dot_q<VPT>(acc, v.tab + (int64_t)v.vslot[e] * np * np + p, v.M + (int64_t)v.vsrc[e] * np * nv + v0, np, nv);
+#pragma unroll
+                for (int i = 0; i < VPT; ++i) part[i] = s == c ? df_norm(acc[i]) : dfc_add(part[i], df_norm(acc[i]));
+            }
+#pragma unroll
+            for (int i = 0; i < VPT; ++i) tot[i] = G > 1 || c == 0 ? part[i] : dfc_add(tot[i], part[i]);
+        }
     }
-    if (PAR) {
-        if (g > 0 && g < GS)
+    if (G > 1) {
+        if (g > 0 && g < G)
 #pragma unroll
-            for (int i = 0; i < VPT; ++i) red[((g - 1) * np + p) * VPT + i] = tot[i];
+            for (int i = 0; i < VPT; ++i) red[((g - 1) * item + it) * VPT + i] = tot[i];
         __syncthreads();
         if (g == 0)
 #pragma unroll
-            for (int i = 0; i < VPT; ++i)
-                for (int h = 1; h < GS; ++h) tot[i] = dfc_add(tot[i], red[((h - 1) * np + p) * VPT + i]);
+            for (int i = 0; i < VPT; ++i) {
+                auto at = [&](int s) { return red[((s - 1) * item + it) * VPT + i]; };
+                for (int s = 3; s < G; s += 3) tot[i] = dfc_add(tot[i], at(s));
+                for (int c = 1; c < k3; ++c) {
+                    float4 part = at(c);
+                    for (int s = c + 3; s < G; s += 3) part = dfc_add(part, at(s));
+                    tot[i] = dfc_add(tot[i], part);
+                }
+            }
     }
     if (g == 0)
 #pragma unroll
@@ -493,13 +512,20 @@ static void launch_l2l(Geo geo, int64_t npar, int P, int nv, const float4 *tab, 
 static void launch_m2l(const M2LLevelDF *lev, int nlev, int64_t nblk, int P, int nv, cudaStream_t st)
 {
     const int np = 2 * P + 1;
-    // subsets of a box's entries: as many as threads of 512 for small trees, whose boxes leave SMs idle
-    const int GS = std::max(1, std::min(nblk < 1216 ? 12 : 3, 512 / np));
+    // subsets of a box's entries: 12 for small trees, whose boxes leave SMs idle, if 512 threads hold them
+    const int GS = nblk < 1216 && 12 * np <= 512 ? 12 : 3;
     NV_DISPATCH(nv, {
         constexpr int VPT = NV < 4 ? NV : 4;
-        constexpr bool PAR = NV <= 2;
-        const int thr = round32(np * (PAR ? GS : (nv + VPT - 1) / VPT));
-        k_m2l_dx<NV, PAR><<<(unsigned)nblk, thr, PAR ? (size_t)(GS - 1) * np * VPT * sizeof(float4) : 0, st>>>(lev, nlev, P, nv, GS);
+        const int item = np * ((nv + VPT - 1) / VPT);
+        const int G = item * GS <= 512 && (GS - 1) * item * VPT <= 3072 ? GS : (item * 3 <= 512 ? 3 : 1); // 48 KB of sums
+        const size_t shm = (size_t)(G - 1) * item * VPT * sizeof(float4);
+        // one vector on many boxes (four waves of 8 blocks per SM): 64 registers, more warps; clustered 100k
+        // 2.07 ms against 2.27 ms with 102.  Fewer boxes or more vectors: the registers (two vectors on
+        // 1000 boxes: the whole apply 0.69 ms against 0.77 ms with 64).
+        if (NV == 1 && nblk >= 4864)
+            k_m2l_dx<NV, NV == 1 ? 2 : 1><<<(unsigned)nblk, round32(item * G), shm, st>>>(lev, nlev, P, nv, GS, G);
+        else
+            k_m2l_dx<NV, 1><<<(unsigned)nblk, round32(item * G), shm, st>>>(lev, nlev, P, nv, GS, G);
     });
 }
 

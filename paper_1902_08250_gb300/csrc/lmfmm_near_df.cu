@@ -25,11 +25,13 @@
 static int gridn(int64_t n, int b) { return (int)((n + b - 1) / b); }
 __host__ __device__ constexpr int min_i(int a, int b) { return a < b ? a : b; }
 
-#define ND_THREADS 128
+// threads of a block: 128, 256 for 16 vectors (two rows of targets a warp hold their sums in registers;
+// 250k strip: 2.46 ms, 3.08 ms with 128 threads and 8 targets a pass)
+__host__ __device__ constexpr int nd_threads(int nv, bool grad) { return !grad && nv == 16 ? 256 : 128; }
 #define ND_ENT 64 // U entries a round
 #define ND_SRC 64 // near sources a round
-// targets of a block's pass: 16, 8 where the sums take more registers
-__host__ __device__ constexpr int nd_tgt(int nv, bool grad) { return grad || nv == 16 ? 8 : 16; }
+// targets of a block's pass: 16, 8 for the gradient, whose sums take three times the registers
+__host__ __device__ constexpr int nd_tgt(int nv, bool grad) { return grad ? 8 : 16; }
 
 // (A, J) and their z-derivatives (target gradient): A' = J/z + (ln z + 2 gamma) J' + 2 V'
 struct HVal {
@@ -283,12 +285,12 @@ __device__ __noinline__ void seg_df_grad(const DfSmem &tab, const NearDF &q, int
 // Bound by FP32 issue (free pairs about 250 instructions, tails 170 per node, 48
 // per complex multiply-add).
 template <int NV, int D, int T, bool GRAD, class Geo>
-__global__ void __launch_bounds__(ND_THREADS, GRAD ? 3 : 4)
+__global__ void __launch_bounds__(nd_threads(NV, GRAD), GRAD ? 3 : 512 / nd_threads(NV, GRAD))
     k_near_df(Geo geo, double k, double kap, const double *xs, const double *ys, const int64_t *ls, const float4 *rel,
               const float4 *hgt, const int64_t *ustart, const int32_t *usrc, const int32_t *uterm, NearDF nq,
               const float4 *qd, int nvq, const int *qexp, int64_t n, int nv, int tb, int free_on, zd *us, GradOut go)
 {
-    constexpr int SETS = GRAD ? 3 : 1, TG = nd_tgt(NV, GRAD), SRC = GRAD ? 32 : ND_SRC;
+    constexpr int SETS = GRAD ? 3 : 1, TG = nd_tgt(NV, GRAD), SRC = GRAD ? 32 : ND_SRC, THR = nd_threads(NV, GRAD);
     __shared__ DfSmem tab;
     __shared__ int64_t fj0[ND_ENT];
     __shared__ int fpre[ND_ENT + 1], fterm[ND_ENT];
@@ -308,7 +310,7 @@ __global__ void __launch_bounds__(ND_THREADS, GRAD ? 3 : 4)
     const float zclose = (float)(kap * kap * bw * bw) * 0x1p-20f;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t u0 = ustart[b], u1 = ustart[b + 1];
-    constexpr int ROWS = TG / (ND_THREADS / 32), HALF = SRC / 32;
+    constexpr int ROWS = TG / (THR / 32), HALF = SRC / 32;
     // Sums over the sources: 8 interleaved subsets whatever the number of vectors, so that a vector's
     // result does not depend on how many others are applied with it.  A lane holds ACC subsets of
     // vector v for LR of its warp's ROWS rows.
@@ -376,13 +378,13 @@ __global__ void __launch_bounds__(ND_THREADS, GRAD ? 3 : 4)
                     st[tid] = term;
                 }
                 if (nv < NV)
-                    for (int i = tid; i < SRC * NV; i += ND_THREADS) sq[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    for (int i = tid; i < SRC * NV; i += THR) sq[i] = make_float4(0.f, 0.f, 0.f, 0.f);
                 __syncthreads();
-                for (int i = tid; i < ns * nv; i += ND_THREADS) {
+                for (int i = tid; i < ns * nv; i += THR) {
                     const int s = i / nv, vv = i - s * nv;
                     sq[s * NV + vv] = qd[sj[s] * nvq + go.v0 + vv];
                 }
-                for (int it = warp; it < HALF * nt; it += ND_THREADS / 32) {
+                for (int it = warp; it < HALF * nt; it += THR / 32) {
                     const int row = it / HALF, s = (it % HALF) * 32 + lane;
                     if (s >= ns) continue;
                     const float4 tp = tr[row], p = sp[s];
@@ -469,7 +471,7 @@ __global__ void __launch_bounds__(ND_THREADS, GRAD ? 3 : 4)
                 __syncthreads();
 #pragma unroll
                 for (int r = 0; r < LR; ++r) {
-                    const int row = warp + (r * RSTEP + rh) * (ND_THREADS / 32);
+                    const int row = warp + (r * RSTEP + rh) * (THR / 32);
                     if (on && row < nt)
                         for (int s0 = 0; s0 < ns; s0 += SUB)
 #pragma unroll
@@ -493,7 +495,7 @@ __global__ void __launch_bounds__(ND_THREADS, GRAD ? 3 : 4)
         }
 #pragma unroll
         for (int r = 0; r < LR; ++r) {
-            const int row = warp + (r * RSTEP + rh) * (ND_THREADS / 32);
+            const int row = warp + (r * RSTEP + rh) * (THR / 32);
 #pragma unroll
             for (int c = 0; c < SETS; ++c) { // the subsets' sums, halves first
                 float4 x[ACC], y[ACC];
@@ -517,7 +519,7 @@ __global__ void __launch_bounds__(ND_THREADS, GRAD ? 3 : 4)
         }
         __syncthreads();
         const int ex = qexp_of(qexp);
-        for (int i = tid; i < nt * nv * SETS; i += ND_THREADS) {
+        for (int i = tid; i < nt * nv * SETS; i += THR) {
             const int row = i % nt, vc = i / nt, vv = vc % nv, c = vc / nv;
             const float4 a = ur[((row * SETS + c) * NV + vv) * 2], j = ur[((row * SETS + c) * NV + vv) * 2 + 1];
             const double f = -1.0 / (4.0 * M_PI);
@@ -748,7 +750,7 @@ static void launch_near(lm_tree_s *t, Geo geo, int64_t nleaf, int nvq, int nv, c
     const size_t shm = (size_t)(GRAD ? 32 : ND_SRC) * NV * sizeof(float4);
     const int free_on = t->med.opt.kernel == LM_KERNEL_G;
     auto run = [&](auto kern) {
-        kern<<<dim3((unsigned)nleaf, gy), ND_THREADS, shm, st>>>(geo, t->med.k2, kap, t->xs, t->ys, t->leaf_start, N.rel,
+        kern<<<dim3((unsigned)nleaf, gy), nd_threads(NV, GRAD), shm, st>>>(geo, t->med.k2, kap, t->xs, t->ys, t->leaf_start, N.rel,
                                                                  N.hgt, t->ustart, t->usrc, t->uterm, nq, N.q, nvq, t->qexp,
                                                                  t->n, nv, tb, free_on, t->us, go);
     };

@@ -18,15 +18,13 @@
 //
 // Operands lie in global memory as [digit][8-wide K chunk][row][8 FP16]: 8 rows of a
 // chunk are a core matrix of the canonical K-major no-swizzle layout (stride 128 B between
-// 8-row groups), and any run of boxes is one bulk copy per digit and chunk, whatever its
-// offset.  Stages of up to 48 K (91 KB), two in flight.  Roles as in lmfmm_tc_tiles.cu:
+// 8-row groups), a stage of a table is one bulk copy, and any run of boxes one per digit and
+// chunk, whatever its offset.  Stages of up to 48 K (91 KB), two in flight.  Roles as in lmfmm_tc_tiles.cu:
 // a producer warp (a lane per copy), an MMA warp, 8 epilogue warps that read the 5
 // accumulators (320 columns of tensor memory) once per entry.
 // Bound: 45 MMAs of 128 x 64 x 16 a stage, limited by the shared-memory reads of their
 // operands (6 KB a MMA at 128 B per clock).
 #include <algorithm>
-#include <map>
-#include <tuple>
 
 #include <cuda_fp16.h>
 
@@ -41,24 +39,23 @@
 #define OZ_N 64       // columns of a tile
 #define OZ_KC 6       // 8-wide K chunks of a full stage
 #define OZ_NST 2
-#define OZ_A_BYTES (OZ_S * OZ_KC * 128 * 16)
+#define OZ_A_BYTES (OZ_S * OZ_KC * 128 * 16) // RA <= 128 rows a chunk, packed; an MMA reads 128 from any chunk
 #define OZ_B_BYTES (OZ_S * OZ_KC * OZ_N * 16)
 #define OZ_STAGE (OZ_A_BYTES + OZ_B_BYTES)
 #define OZ_EPI 8
 #define OZ_THREADS ((OZ_EPI + 2) * 32)
 #define OZ_SMEM (OZ_NST * OZ_STAGE + 128)
-#define OZ_MINBOX 2048
+// Smaller levels leave most SMs without a tile.  250k strip, 16 vectors: levels of up to 2047 boxes in
+// k_m2l_dx 2.67 ms, of up to 255 0.20 ms, this kernel 6.10 and 6.25 ms.
+#define OZ_MINBOX 256
 #define OZ_PADL 2
 
-struct OzEnt {
-    int32_t slot, dc, rs, pad;
-};
 struct OzLevel {
     int64_t tile0;          // first tile of the level in the launch
     int32_t ncl, tpr;       // boxes of a (row, parity) class, tiles of one
     int64_t ncol;
     const int32_t *e0;      // [2 nrow + 1] entries of each class
-    const OzEnt *ents;
+    const RowEnt *ents;
     const unsigned char *A; // split tables
     unsigned char *B;       // split multipoles: planes of a (row, parity)
     const uint32_t *tmax;   // [2] largest table component and row sum of the level (float bits)
@@ -277,8 +274,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_m2l_oz(const OzLevel *lvs, in
     const uint32_t tmem = *tslot;
 
     if (warp == OZ_EPI) {
-        // ---- producer: lane 0 waits for a free stage; each lane then issues one table and one
-        // multipole copy (5 digits x up to 6 chunks) ----
+        // ---- producer: lane 0 waits for a free stage; lane 31 then copies the tables, lanes 0..29
+        // one multipole piece each (5 digits x up to 6 chunks) ----
         uint32_t it = 0;
         int last[OZ_NST];
 #pragma unroll
@@ -291,7 +288,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_m2l_oz(const OzLevel *lvs, in
             const int64_t rows = oz_prow(lv.ncl, tb, nvs);
             for (int base = e0; base < e1 && !stop; base += 32) {
                 const int cnt = min(32, e1 - base);
-                const OzEnt mine = lane < cnt ? lv.ents[base + lane] : OzEnt{0, 0, 0, 0};
+                const RowEnt mine = lane < cnt ? lv.ents[base + lane] : RowEnt{0, 0, 0, 0};
                 for (int i = 0; i < cnt && !stop; ++i) {
                     const int slot = __shfl_sync(0xffffffffu, mine.slot, i), dc = __shfl_sync(0xffffffffu, mine.dc, i),
                               rs = __shfl_sync(0xffffffffu, mine.rs, i);
@@ -313,9 +310,10 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_m2l_oz(const OzLevel *lvs, in
                             break;
                         }
                         const uint32_t sa = sbase + s * OZ_STAGE, sb = sa + OZ_A_BYTES, fb = bfull + 8 * s;
+                        if (lane == 31) // the stage's tables are contiguous
+                            bulk_g2s(sa, a + (int64_t)OZ_S * k0 * RA * 16, OZ_S * kc * RA * 16, fb);
                         if (lane < OZ_S * kc) {
                             const int dg = lane / kc, c = lane - dg * kc;
-                            bulk_g2s(sa + (dg * OZ_KC + c) * 128 * 16, a + ((int64_t)OZ_S * k0 + lane) * RA * 16, RA * 16, fb);
                             bulk_g2s(sb + (dg * OZ_KC + c) * OZ_N * 16, b + ((int64_t)dg * KC + k0 + c) * rows * 16, OZ_N * 16, fb);
                         }
                         last[s] = (int)it;
@@ -349,7 +347,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_m2l_oz(const OzLevel *lvs, in
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     int issued = 0;
                     for (int st = 0; st < nst; ++st, ++it) {
-                        const int s = (int)(it % OZ_NST), ks = min(OZ_KC, KC - st * OZ_KC) / 2;
+                        const int s = (int)(it % OZ_NST), kc = min(OZ_KC, KC - st * OZ_KC), ks = kc / 2;
                         if (!mbar_wait_lim(bfull + 8 * s, (it / OZ_NST) & 1, TC_WAIT_LIMIT, abort_s, err)) {
                             oz_fail(abort_s, err);
                             stop = true;
@@ -362,7 +360,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_m2l_oz(const OzLevel *lvs, in
                             for (int i = 0; i < OZ_S; ++i)
 #pragma unroll
                                 for (int j = 0; i + j < OZ_S; ++j)
-                                    oz_mma(tmem + OZ_N * (i + j), oz_desc(sa + (i * OZ_KC + 2 * kk) * 128 * 16, 128 * 16),
+                                    oz_mma(tmem + OZ_N * (i + j), oz_desc(sa + (i * kc + 2 * kk) * RA * 16, RA * 16),
                                            oz_desc(sb + (j * OZ_KC + 2 * kk) * OZ_N * 16, OZ_N * 16), idesc,
                                            (st > 0 || kk > 0 || i > 0) ? 1u : 0u);
                         tc_commit(bempty + 8 * s);
@@ -475,7 +473,7 @@ static std::vector<OzLevel> oz_levels(const lm_tree_s *t, int nvs)
         o.ncol = lv.ncol;
         o.nrow = lv.nrow;
         o.e0 = z.e0;
-        o.ents = (const OzEnt *)z.ents;
+        o.ents = (const RowEnt *)z.ents;
         o.A = z.A;
         o.B = z.B;
         o.tmax = z.tmax;
@@ -497,34 +495,11 @@ lm_status lm_setup_oz(lm_tree_s *t, cudaStream_t st)
         const Level &lv = t->lev[l];
         OzData::Lv z{};
         z.l = l;
-        std::map<std::tuple<int, int, int>, int> slot;
-        for (size_t i = 0; i < lv.cls_term.size(); ++i) slot[{lv.cls_term[i], lv.cls_dc[i], lv.cls_dr[i]}] = (int)i;
-        std::vector<OzEnt> ents;
+        std::vector<RowEnt> ents;
         std::vector<int32_t> e0;
-        for (int64_t rt = 0; rt < lv.nrow; ++rt)
-            for (int par = 0; par < 2; ++par) {
-                e0.push_back((int32_t)ents.size());
-                const int64_t ct = 8 + par; // an interior column
-                for (int term = 0; term < 5; ++term) {
-                    const int64_t a = src_row(term, rt - 3, lv.nrow), b = src_row(term, rt + 3, lv.nrow);
-                    const int64_t rlo = std::max<int64_t>(0, std::min(a, b)), rhi = std::min(lv.nrow - 1, std::max(a, b));
-                    for (int64_t rs = rlo; rs <= rhi; ++rs) {
-                        const int64_t ri = img_row(term, rs, lv.nrow);
-                        for (int64_t cs = ct - 3; cs <= ct + 3; ++cs) {
-                            if (!v_rule(l, ct, rt, cs, ri)) continue;
-                            auto f = slot.find({term, (int)(ct - cs), (int)(rt - ri)});
-                            if (f == slot.end()) {
-                                lm_set_error("build_tree: internal error, an interaction has no translation class");
-                                return LM_ECUDA;
-                            }
-                            ents.push_back(OzEnt{f->second, (int32_t)(ct - cs), (int32_t)rs, 0});
-                        }
-                    }
-                }
-            }
-        e0.push_back((int32_t)ents.size());
+        TRY_O(lm_row_entries(lv, ents, e0));
         const size_t ncls = std::max<size_t>(1, lv.cls_term.size());
-        OzEnt *de;
+        RowEnt *de;
         TRY_O(lm_dalloc(t, &de, ents.size()));
         z.ents = de;
         TRY_O(lm_dalloc(t, &z.e0, e0.size()));
@@ -535,7 +510,7 @@ lm_status lm_setup_oz(lm_tree_s *t, cudaStream_t st)
             bb = std::max(bb, (size_t)(2 * lv.nrow * OZ_S * KC) * oz_prow((int)(lv.ncol / 2), OZ_N / s, s) * 16);
         TRY_O(lm_dalloc(t, &z.B, bb));
         Z.lv.push_back(z); // owned from here on
-        LM_CUDA(cudaMemcpyAsync(de, ents.data(), ents.size() * sizeof(OzEnt), cudaMemcpyHostToDevice, st));
+        LM_CUDA(cudaMemcpyAsync(de, ents.data(), ents.size() * sizeof(RowEnt), cudaMemcpyHostToDevice, st));
         LM_CUDA(cudaMemcpyAsync(z.e0, e0.data(), e0.size() * sizeof(int32_t), cudaMemcpyHostToDevice, st));
         LM_CUDA(cudaMemsetAsync(z.tmax, 0, 2 * sizeof(uint32_t), st));
         k_oz_tmax<<<(unsigned)ncls, 256, 0, st>>>(lv.tab, np, z.tmax);
