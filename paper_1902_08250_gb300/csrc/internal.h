@@ -2,6 +2,7 @@
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
+#include <algorithm>
 #include <string>
 #include <vector>
 
@@ -94,6 +95,22 @@ struct NearQuad {
     // subtracts (imp_beta); beta = k2 alpha per wall, 0 without one
     zd *seg_c, *tail_c_g;
     double beta[2];
+};
+
+// Device memory of one tree, cut from slabs that are given back together: a cudaMalloc that maps new
+// memory takes 70 to 120 us and a cudaFree 10 to 50 us, and a tree has about 150 arrays (build and apply of
+// 100k points: 7.5 ms, 2.8 ms with slabs).  A slab is as large as the slabs before it, 4 to 64 MB; a block of
+// more than half of that has a slab of its own, and where a slab cannot be had the block alone is tried.
+struct LmArena {
+    std::vector<void *> slabs;
+    char *cur = nullptr;
+    size_t left = 0, total = 0;
+    cudaError_t get(void **p, size_t bytes);
+    void release();
+    LmArena() = default;
+    LmArena(const LmArena &) = delete;
+    LmArena &operator=(const LmArena &) = delete;
+    ~LmArena() { release(); }
 };
 
 struct Level {
@@ -226,7 +243,7 @@ struct lm_tree_s {
     int64_t *perm;       // [n] tree position -> input index
     int64_t *leaf_start; // [nleaf + 1]
     // U list (leaf level, target-major CSR)
-    int64_t nu;
+    int64_t nu, umax; // entries; largest number of one leaf (uniform tree)
     int64_t *ustart;  // [nleaf + 1]
     int32_t *usrc;    // [nu]
     int32_t *uterm;   // [nu]
@@ -275,6 +292,7 @@ struct lm_tree_s {
     NearTabDF ndf;
     ExpDF xdf;
     OzData oz;
+    LmArena mem, tmp; // the tree's arrays; temporaries of its build
     int *qexp;   // device: binary exponent of the largest |density| component of the apply
     int64_t bytes;
     // phase profiling
@@ -303,13 +321,13 @@ struct M2LClass { // one M2L table: [2P+1][2P+1] at out, scaled by S_t(p) S_s(q)
     const double *scale_t, *scale_s;  // device: S(n), n = 0..P (free space)
     zd *out;
 };
-lm_status lm_build_m2l_tables(const MediumD &md, int P, const std::vector<M2LClass> &cls, int *dflag, cudaStream_t st);
+lm_status lm_build_m2l_tables(const MediumD &md, int P, const std::vector<M2LClass> &cls, int *dflag, LmArena &tmp, cudaStream_t st);
 struct ShiftJob { // M2M and L2L tables between a level of box width wc and its parent level; m2m or l2l may be null
     double k, wc;
     const double *sc_child, *sc_par;
     zd *m2m, *l2l; // [4 child positions][2P+1][2P+1]
 };
-lm_status lm_build_shift_tables(int P, const std::vector<ShiftJob> &jobs, cudaStream_t st);
+lm_status lm_build_shift_tables(int P, const std::vector<ShiftJob> &jobs, LmArena &tmp, cudaStream_t st);
 // setup (lmfmm_setup.cu)
 lm_status lm_setup_tree(lm_tree_s *t, const double *x, const double *y, cudaStream_t st);
 lm_status lm_setup_tables(lm_tree_s *t, cudaStream_t st);
@@ -318,7 +336,6 @@ lm_status lm_setup_near(lm_tree_s *t, cudaStream_t st);                      // 
 // adaptive tree (lmfmm_adaptive.cu)
 lm_status lm_setup_adaptive(lm_tree_s *t, const double *x, const double *y, cudaStream_t st);
 lm_status lm_adaptive_lists_to_host(lm_tree_s *t, int which, std::vector<int64_t> &rows, cudaStream_t st);
-void lm_free_adaptive(lm_tree_s *t);
 lm_status lm_list_to_host(lm_tree_s *t, int which, int level, std::vector<int64_t> &rows,
                           cudaStream_t st);
 void lm_free_tree_device(lm_tree_s *t);
@@ -349,7 +366,6 @@ void lm_df_m2l(const M2LLevelDF *lev, int nlev, int64_t nblk, int P, int nv, cud
 bool lm_oz_level(const lm_tree_s *t, int l); // tensor-core M2L of the FP64 form (lmfmm_oz.cu)
 lm_status lm_setup_oz(lm_tree_s *t, cudaStream_t st);
 lm_status lm_launch_m2l_oz(lm_tree_s *t, int nv, cudaStream_t st, int *launches);
-void lm_free_oz(lm_tree_s *t);
 lm_status lm_run_df(lm_tree_s *t, const zd *q, int nvec, zd *u, bool adjoint, zd *ux, zd *uy, cudaStream_t st);
 lm_status lm_run_apply_grad(lm_tree_s *t, const zd *q, int nvec, zd *u, zd *ux, zd *uy, cudaStream_t st);
 // mixed precision (lmfmm_mixed.cu)
@@ -358,7 +374,6 @@ lm_status lm_setup_mixed_adaptive(lm_tree_s *t, cudaStream_t st);
 lm_status lm_autotune_mixed(lm_tree_s *t, cudaStream_t st, int *choice, float *ms);
 lm_status lm_run_apply_mixed(lm_tree_s *t, const void *q, int nvec, void *u, bool adjoint, bool c64, cudaStream_t st,
                              int part = 0);
-void lm_free_mixed(lm_tree_s *t);
 // applies of up to 4 vectors (lmfmm_few32.cu)
 struct NearQuadF;
 lm_status lm_setup_few32(lm_tree_s *t, cudaStream_t st);
@@ -377,7 +392,6 @@ lm_status lm_launch_msplit_tt(lm_tree_s *t, cudaStream_t st, int nvs);
 struct NearQuadF;
 lm_status lm_setup_leaf_tt(lm_tree_s *t, cudaStream_t st);
 lm_status lm_launch_leaf_tt(lm_tree_s *t, const NearQuadF &nq, cudaStream_t st);
-void lm_free_leaf_tt(lm_tree_s *t);
 struct lm_tt_batch_s;
 lm_status lm_tt_batch_build(lm_tree_s *const *trees, int count, int nvs, lm_tt_batch_s **out);
 lm_status lm_tt_batch_launch(const lm_tt_batch_s *b, cudaStream_t st);
@@ -386,16 +400,21 @@ void lm_tt_batch_free(lm_tt_batch_s *b);
 // 2 from L2L on (after a tile M2L of the tree has run).  Parts 1 and 2 need the tile
 // form and at most 16 vectors.
 bool lm_mixed_tiles(const lm_tree_s *t, int nvec);
-void lm_free_tt(lm_tree_s *t);
 template <typename T>
-lm_status lm_dalloc(lm_tree_s *t, T **p, size_t count)
+lm_status lm_dalloc(LmArena &a, T **p, size_t count)
 {
     if (count == 0) count = 1;
-    cudaError_t e = cudaMalloc((void **)p, count * sizeof(T));
+    cudaError_t e = a.get((void **)p, count * sizeof(T));
     if (e != cudaSuccess) {
         lm_set_error("cudaMalloc of %zu bytes failed: %s", count * sizeof(T), cudaGetErrorString(e));
         return LM_ENOMEM;
     }
-    t->bytes += count * sizeof(T);
     return LM_OK;
+}
+template <typename T>
+lm_status lm_dalloc(lm_tree_s *t, T **p, size_t count)
+{
+    const lm_status s = lm_dalloc(t->mem, p, count);
+    if (s == LM_OK) t->bytes += std::max<size_t>(1, count) * sizeof(T);
+    return s;
 }

@@ -31,8 +31,9 @@ __host__ __device__ inline bool v_rule(int l, int64_t ct, int64_t rt, int64_t cs
 }
 
 // An interior box's V list depends only on its row and its column's parity (levels >= 1): the entry
-// lists of every (row, parity) class of level l, [2 row + parity], e0 their offsets.  A source column
-// c - dc outside the level is an entry that the target does not have.
+// lists of every (row, parity) class of a level, [2 row + parity], e0 their offsets.  A source column
+// c - dc outside the level is an entry that the target does not have.  Level 0 is one row of boxes whose
+// lists hold every class: one list.
 struct RowEnt {
     int32_t slot, dc, rs, pad; // table slot, target column - source column, source row
 };
@@ -42,6 +43,11 @@ inline lm_status lm_row_entries(const Level &lv, std::vector<RowEnt> &ents, std:
     for (size_t i = 0; i < lv.cls_term.size(); ++i) slot[{lv.cls_term[i], lv.cls_dc[i], lv.cls_dr[i]}] = (int)i;
     ents.clear();
     e0.clear();
+    if (lv.l == 0) {
+        e0 = {0, (int32_t)lv.cls_term.size()};
+        for (size_t i = 0; i < lv.cls_term.size(); ++i) ents.push_back(RowEnt{(int32_t)i, lv.cls_dc[i], 0, 0});
+        return LM_OK;
+    }
     for (int64_t rt = 0; rt < lv.nrow; ++rt)
         for (int par = 0; par < 2; ++par) {
             e0.push_back((int32_t)ents.size());

@@ -457,13 +457,14 @@ lm_status lm_setup_adaptive(lm_tree_s *t, const double *x, const double *y, cuda
         for (int j = 0; j < ncls; ++j)
             tcls.push_back({cterm[j], cdx[j], cdy[j], md.k2 * ldexp(d, -clt[j]), md.k2 * ldexp(d, -cls[j]),
                             t->lev[clt[j]].scale, t->lev[cls[j]].scale, A.tab + (size_t)j * np * np});
-        TRY_A(lm_build_m2l_tables(md, P, tcls, t->dflag, st));
+        TRY_A(lm_build_m2l_tables(md, P, tcls, t->dflag, t->tmp, st));
     }
-    // expansions and tree-order scratch
-    TRY_A(lm_dalloc(t, &A.M, (size_t)nbox * np * LM_MAXV));
-    TRY_A(lm_dalloc(t, &A.Lc, (size_t)nbox * np * LM_MAXV));
-    TRY_A(lm_dalloc(t, &t->qs, (size_t)LM_MAXV * n));
-    TRY_A(lm_dalloc(t, &t->us, (size_t)LM_MAXV * n));
+    if (t->precision == LM_FP64) { // expansions and tree-order scratch
+        TRY_A(lm_dalloc(t, &A.M, (size_t)nbox * np * LM_MAXV));
+        TRY_A(lm_dalloc(t, &A.Lc, (size_t)nbox * np * LM_MAXV));
+        TRY_A(lm_dalloc(t, &t->qs, (size_t)LM_MAXV * n));
+        TRY_A(lm_dalloc(t, &t->us, (size_t)LM_MAXV * n));
+    }
     int hflag = 0;
     LM_CUDA(cudaMemcpyAsync(&hflag, t->dflag, sizeof(int), cudaMemcpyDeviceToHost, st));
     LM_CUDA(cudaStreamSynchronize(st));
@@ -498,17 +499,6 @@ lm_status lm_adaptive_lists_to_host(lm_tree_s *t, int which, std::vector<int64_t
             rows[3 * e + 2] = hsrc[e];
         }
     return LM_OK;
-}
-
-void lm_free_adaptive(lm_tree_s *t)
-{
-    AdaptTree &A = t->at;
-    void *ptrs[] = {A.cx,     A.cy,     A.w,      A.parent, A.pos,   A.child, A.leaves, A.nonleaf,
-                    A.pwleaves, A.vstart, A.vsrc, A.vslot,  A.vterm, A.tab,   A.M,      A.Lc,
-                    A.tabdft};
-    for (void *p : ptrs)
-        if (p) cudaFree(p);
-    A = AdaptTree();
 }
 
 extern "C" lm_status lm_adaptive_plan(const double *x, const double *y, int64_t n, double d, int leaf_target,

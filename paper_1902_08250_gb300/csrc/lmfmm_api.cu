@@ -192,6 +192,7 @@ extern "C" lm_status lm_build_tree(lm_medium m, const double *x, const double *y
         lm_destroy_tree(t);
         return s;
     }
+    t->tmp.release(); // the set-up has synchronised
     *out = t;
     return LM_OK;
 }

@@ -976,8 +976,8 @@ lm_status lm_setup_pwidx(lm_tree_s *t, int64_t *npw, cudaStream_t st)
     }
     lm_status s = lm_dalloc(t, &t->pwidx, idx.size());
     if (s != LM_OK) return s;
+    // (a copy from pageable memory has read it when the call returns)
     LM_CUDA(cudaMemcpyAsync(t->pwidx, idx.data(), idx.size() * sizeof(int32_t), cudaMemcpyHostToDevice, st));
-    LM_CUDA(cudaStreamSynchronize(st)); // idx is a host temporary
     return LM_OK;
 }
 // and the per-apply plane-wave coefficients of the FP64 form

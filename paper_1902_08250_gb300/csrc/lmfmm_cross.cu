@@ -764,7 +764,11 @@ static lm_status cross_setup(lm_cross_s *c, const double *xs, const double *ys, 
         jobs.push_back({k1, ch.w, ch.sc_s, par.sc_s, par.m2m, nullptr});
         jobs.push_back({k2, ch.w, ch.sc_t, par.sc_t, nullptr, ch.l2l});
     }
-    CTRY(lm_build_shift_tables(P, jobs, st));
+    {
+        LmArena tmp;
+        CTRY(lm_build_shift_tables(P, jobs, tmp, st));
+        LM_CUDA(cudaStreamSynchronize(st));
+    }
 
     // V lists and classes (host): target-major, then term, then source box
     const size_t shm = (2 * 16 * np + 16) * sizeof(zd); // m2l_table_body's staging

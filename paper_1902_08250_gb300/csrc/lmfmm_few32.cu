@@ -487,7 +487,6 @@ lm_status lm_setup_few32(lm_tree_s *t, cudaStream_t st)
         TRY_F(lm_dalloc(t, &t->at.tab32t, (size_t)cnt));
         k_tab32_t<<<gridf(cnt, 256), 256, 0, st>>>(t->at.tab32, cnt, np, t->at.tab32t);
     }
-    LM_CUDA(cudaStreamSynchronize(st)); // host temporaries
     LM_CUDA(cudaGetLastError());
     t->few32 = true;
     return LM_OK;

@@ -846,33 +846,22 @@ lm_status lm_setup_leaf_tt(lm_tree_s *t, cudaStream_t st)
     }
     // the L2T basis series holds for k2 w <= 2 (t = (k2 r / 2)^2 <= 1/2 inside a leaf)
     if (!inst || t->L < 1 || t->n >= ((int64_t)1 << 29) || t->med.k2 * t->lev[t->L].w > 2.0) return LM_OK;
-    std::vector<int64_t> us(t->nleaf + 1);
-    LM_CUDA(cudaMemcpyAsync(us.data(), t->ustart, us.size() * sizeof(int64_t), cudaMemcpyDeviceToHost, st));
-    LM_CUDA(cudaStreamSynchronize(st));
-    for (int64_t b = 0; b < t->nleaf; ++b)
-        if (us[b + 1] - us[b] > LF_MAXE) return LM_OK;
+    if (t->umax > LF_MAXE) return LM_OK;
     int dev = 0, nsm = 0;
     LM_CUDA(cudaGetDevice(&dev));
     LM_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
     t->lf_grid = (int)std::max<int64_t>(1, std::min<int64_t>(nsm, t->nleaf));
     const lm_status s = lf_set_attr(t->p);
     if (s != LM_OK) return s;
-    if (!t->lf_pts) {
-        LM_CUDA(cudaMalloc((void **)&t->lf_pts, (size_t)std::max<int64_t>(1, t->n) * sizeof(float4)));
-        t->bytes += (int64_t)std::max<int64_t>(1, t->n) * sizeof(float4);
-    }
-    if (!t->lf_ent) {
-        LM_CUDA(cudaMalloc((void **)&t->lf_ent, (size_t)t->nleaf * LF_MAXE * sizeof(int4)));
-        t->bytes += t->nleaf * LF_MAXE * (int64_t)sizeof(int4);
-    }
-    if (!t->lf_scl) {
-        LM_CUDA(cudaMalloc((void **)&t->lf_scl, 2 * sizeof(uint32_t)));
-        t->bytes += 2 * sizeof(uint32_t);
-    }
-    if (!t->lf_tot) {
-        LM_CUDA(cudaMalloc((void **)&t->lf_tot, (size_t)t->nleaf * sizeof(int32_t)));
-        t->bytes += t->nleaf * (int64_t)sizeof(int32_t);
-    }
+    float4 *pts;
+    int4 *ent;
+    lm_status r = lm_dalloc(t, &pts, (size_t)t->n);
+    if (r == LM_OK) r = lm_dalloc(t, &ent, (size_t)t->nleaf * LF_MAXE);
+    if (r == LM_OK) r = lm_dalloc(t, &t->lf_scl, 2);
+    if (r == LM_OK) r = lm_dalloc(t, &t->lf_tot, (size_t)t->nleaf);
+    if (r != LM_OK) return r;
+    t->lf_pts = pts;
+    t->lf_ent = ent;
     k_lf_pts<<<(unsigned)((t->n + 255) / 256), 256, 0, st>>>(t->xl32, t->yl32, t->y32, t->n, (float4 *)t->lf_pts);
     k_lf_tot<<<(unsigned)((t->nleaf + 255) / 256), 256, 0, st>>>(t->leaf_start, t->ustart, t->usrc, t->nleaf,
                                                                   t->lf_tot);
@@ -905,19 +894,6 @@ static lm_status lf_launch(lm_tree_s *t, const NearQuadF &nq, cudaStream_t st)
             t->us32, t->dflag + 1, first);
     LM_CUDA(cudaGetLastError());
     return LM_OK;
-}
-
-void lm_free_leaf_tt(lm_tree_s *t)
-{
-    cudaFree(t->lf_pts);
-    cudaFree(t->lf_tot);
-    cudaFree(t->lf_scl);
-    cudaFree(t->lf_ent);
-    t->lf_ent = nullptr;
-    t->lf_pts = nullptr;
-    t->lf_tot = nullptr;
-    t->lf_scl = nullptr;
-    t->lf_ready = false;
 }
 
 lm_status lm_launch_leaf_tt(lm_tree_s *t, const NearQuadF &nq, cudaStream_t st)

@@ -72,47 +72,17 @@ __global__ void k_local_coords(int64_t ncol, double x0, double w, const int64_t 
 
 // entries of the V list that the free-space stencil kernel does not cover
 __global__ void k_rest(int l, int64_t nbox, const int64_t *vstart, const int32_t *vsrc,
-                       const int32_t *vslot, const int32_t *vterm, int64_t *rstart, int32_t *rsrc,
-                       int32_t *rslot, int pass)
+                       const int32_t *vslot, const int32_t *vterm, const int64_t *rstart, int32_t *rsrc,
+                       int32_t *rslot)
 {
     int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (b >= nbox) return;
-    int64_t pos = pass ? rstart[b] : 0, cnt = 0;
+    int64_t pos = rstart[b];
     for (int64_t e = vstart[b]; e < vstart[b + 1]; ++e) {
         if (l > 0 && vterm[e] == 0) continue;
-        if (pass) {
-            rsrc[pos] = vsrc[e];
-            rslot[pos] = vslot[e];
-            ++pos;
-        }
-        ++cnt;
-    }
-    if (!pass) rstart[b] = cnt;
-}
-__global__ void k_scan64b(int64_t *c, int64_t m)
-{
-    __shared__ int64_t part[1024];
-    int64_t chunk = (m + blockDim.x - 1) / blockDim.x;
-    int64_t lo = threadIdx.x * chunk, hi = min(m, lo + chunk);
-    int64_t s = 0;
-    for (int64_t i = lo; i < hi; ++i) s += c[i];
-    part[threadIdx.x] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int64_t acc = 0;
-        for (int i = 0; i < (int)blockDim.x; ++i) {
-            int64_t v = part[i];
-            part[i] = acc;
-            acc += v;
-        }
-        c[m] = acc;
-    }
-    __syncthreads();
-    int64_t acc = part[threadIdx.x];
-    for (int64_t i = lo; i < hi; ++i) {
-        int64_t v = c[i];
-        c[i] = acc;
-        acc += v;
+        rsrc[pos] = vsrc[e];
+        rslot[pos] = vslot[e];
+        ++pos;
     }
 }
 
@@ -159,12 +129,6 @@ lm_status lm_setup_mixed(lm_tree_s *t, cudaStream_t st)
                 sten[(lv.cls_dc[i] + 3) * 7 + lv.cls_dr[i] + 3] = i;
         TRYM(lm_dalloc(t, &lv.stencil, 49));
         LM_CUDA(cudaMemcpyAsync(lv.stencil, sten.data(), 49 * sizeof(int32_t), cudaMemcpyHostToDevice, st));
-        TRYM(lm_dalloc(t, &lv.rstart, lv.nbox + 1));
-        k_rest<<<gridm(lv.nbox, 128), 128, 0, st>>>(l, lv.nbox, lv.vstart, lv.vsrc, lv.vslot, lv.vterm,
-                                                     lv.rstart, nullptr, nullptr, 0);
-        k_scan64b<<<1, 1024, 0, st>>>(lv.rstart, lv.nbox);
-        LM_CUDA(cudaMemcpyAsync(&lv.nrest, lv.rstart + lv.nbox, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
-        LM_CUDA(cudaStreamSynchronize(st));
         // the stencil kernel assumes every free-space offset of an interior box has a table
         if (l > 0)
             for (int dc = -3; dc <= 3; ++dc)
@@ -177,20 +141,7 @@ lm_status lm_setup_mixed(lm_tree_s *t, cudaStream_t st)
         TRYM(lm_dalloc(t, &lv.rsrc, lv.nrest));
         TRYM(lm_dalloc(t, &lv.rslot, lv.nrest));
         k_rest<<<gridm(lv.nbox, 128), 128, 0, st>>>(l, lv.nbox, lv.vstart, lv.vsrc, lv.vslot, lv.vterm,
-                                                     lv.rstart, lv.rsrc, lv.rslot, 1);
-        {
-            // targets that have entries on this list
-            std::vector<int64_t> hs(lv.nbox + 1);
-            LM_CUDA(cudaMemcpyAsync(hs.data(), lv.rstart, (lv.nbox + 1) * sizeof(int64_t), cudaMemcpyDeviceToHost, st));
-            LM_CUDA(cudaStreamSynchronize(st));
-            std::vector<int32_t> tg;
-            for (int64_t b2 = 0; b2 < lv.nbox; ++b2)
-                if (hs[b2 + 1] > hs[b2]) tg.push_back((int32_t)b2);
-            lv.nrtgt = (int64_t)tg.size();
-            TRYM(lm_dalloc(t, &lv.rtgt, tg.size()));
-            if (!tg.empty())
-                LM_CUDA(cudaMemcpyAsync(lv.rtgt, tg.data(), tg.size() * sizeof(int32_t), cudaMemcpyHostToDevice, st));
-        }
+                                                     lv.rstart, lv.rsrc, lv.rslot);
     }
     const int64_t n = t->n;
     TRYM(lm_dalloc(t, &t->xl32, n));
@@ -303,30 +254,6 @@ lm_status lm_setup_mixed_adaptive(lm_tree_s *t, cudaStream_t st)
     LM_CUDA(cudaGetLastError());
     LM_CUDA(cudaStreamSynchronize(st));
     return LM_OK;
-}
-
-void lm_free_mixed(lm_tree_s *t)
-{
-    lm_free_tt(t);
-    lm_free_leaf_tt(t);
-    {
-        AdaptTree &A = t->at;
-        void *ap[] = {A.tab32, A.tab32t, A.M32, A.L32};
-        for (void *p : ap)
-            if (p) cudaFree(p);
-        for (int32_t *p : A.m2l_tgt)
-            if (p) cudaFree(p);
-    }
-    void *ptrs[] = {t->xl32, t->yl32, t->y32, t->qs32, t->us32, t->iperm, t->nq_seg_lam, t->nq_seg_s2, t->nq_seg_w,
-                    t->nq_tail_lam, t->nq_tail_s2, t->nq_tail_w};
-    for (void *p : ptrs)
-        if (p) cudaFree(p);
-    for (Level &lv : t->lev) {
-        void *lp[] = {lv.tab32, lv.m2m32, lv.l2l32, lv.M32, lv.L32, lv.stencil, lv.rstart, lv.rsrc, lv.rslot,
-                      lv.rtgt};
-        for (void *p : lp)
-            if (p) cudaFree(p);
-    }
 }
 
 // ---------------------------------------------------------------------------

@@ -557,13 +557,3 @@ lm_status lm_launch_m2l_oz(lm_tree_s *t, int nv, cudaStream_t st, int *launches)
     return LM_OK;
 }
 
-void lm_free_oz(lm_tree_s *t)
-{
-    for (OzData::Lv &z : t->oz.lv)
-        for (void *p : {(void *)z.ents, (void *)z.e0, (void *)z.A, (void *)z.B, (void *)z.tmax})
-            if (p) cudaFree(p);
-    for (void *p : t->oz.desc)
-        if (p) cudaFree(p);
-    if (t->oz.mmax) cudaFree(t->oz.mmax);
-    t->oz = OzData();
-}

@@ -150,15 +150,16 @@ __host__ __device__ inline int slot_index(int DC, int term, int dc, int dr)
     return (term * (2 * DC + 1) + (dc + DC)) * 7 + (dr + 3);
 }
 
-// pass 0: count; pass 1: fill. One thread per target box.
+// pass 0: count (rstart, optional: the entries that the free-space stencil kernels do not cover);
+// pass 1: fill. One thread per target box.
 __global__ void k_vlist(int l, int64_t ncol, int64_t nrow, int DC, const int32_t *slotmap,
                         int64_t *vstart, int32_t *vsrc, int32_t *vslot, int32_t *vterm, int pass,
-                        int *flag)
+                        int *flag, int64_t *rstart)
 {
     int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (t >= ncol * nrow) return;
     int64_t rt = t / ncol, ct = t % ncol;
-    int64_t pos = pass ? vstart[t] : 0, cnt = 0;
+    int64_t pos = pass ? vstart[t] : 0, cnt = 0, rest = 0;
     for (int term = 0; term < 5; ++term) {
         // source rows in ascending order
         int64_t rlo = 0, rhi = nrow - 1;
@@ -185,10 +186,12 @@ __global__ void k_vlist(int l, int64_t ncol, int64_t nrow, int DC, const int32_t
                     ++pos;
                 }
                 ++cnt;
+                rest += l == 0 || term > 0;
             }
         }
     }
-    if (!pass) vstart[t] = cnt; // counts, scanned on the host side afterwards
+    if (!pass) vstart[t] = cnt; // counts, scanned by k_scan_lists
+    if (!pass && rstart) rstart[t] = rest;
 }
 
 // U list at the leaf level: image adjacent to target (free term includes itself)
@@ -218,31 +221,59 @@ __global__ void k_ulist(int64_t ncol, int64_t nrow, int64_t *ustart, int32_t *us
     if (!pass) ustart[t] = cnt;
 }
 
-// in-place exclusive scan of counts c[0..m) (stored as int64) -> start[0..m]
-__global__ void k_scan64(int64_t *c, int64_t m)
+// One block per list: counts c[0..m) -> starts c[0..m], in place; tot: their sum, the largest count and
+// the number of nonzero counts, whose boxes go to tgt in ascending order (optional)
+struct ScanJob {
+    int64_t *c;
+    int64_t m;
+    int64_t *tot; // [3]
+    int32_t *tgt; // [m]
+};
+__global__ void __launch_bounds__(1024) k_scan_lists(const ScanJob *jobs)
 {
-    __shared__ int64_t part[1024];
-    int64_t chunk = (m + blockDim.x - 1) / blockDim.x;
-    int64_t lo = threadIdx.x * chunk, hi = min(m, lo + chunk);
-    int64_t s = 0;
-    for (int64_t i = lo; i < hi; ++i) s += c[i];
-    part[threadIdx.x] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int64_t acc = 0;
-        for (int i = 0; i < (int)blockDim.x; ++i) {
-            int64_t v = part[i];
-            part[i] = acc;
-            acc += v;
+    __shared__ int64_t ws[32], wn[32], wm[32];
+    const ScanJob J = jobs[blockIdx.x];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t chunk = (J.m + 1023) / 1024, lo = threadIdx.x * chunk, hi = min(J.m, lo + chunk);
+    int64_t s = 0, nz = 0, mx = 0;
+    for (int64_t i = lo; i < hi; ++i) {
+        const int64_t v = J.c[i];
+        s += v;
+        nz += v > 0;
+        mx = max(mx, v);
+    }
+    int64_t is = s, in = nz;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int64_t a = __shfl_up_sync(0xffffffffu, is, o), b = __shfl_up_sync(0xffffffffu, in, o);
+        if (lane >= o) {
+            is += a;
+            in += b;
         }
-        c[m] = acc;
+        mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    }
+    if (lane == 31) {
+        ws[warp] = is;
+        wn[warp] = in;
+        wm[warp] = mx;
     }
     __syncthreads();
-    int64_t acc = part[threadIdx.x];
+    int64_t as = is - s, an = in - nz; // exclusive
+    for (int w = 0; w < warp; ++w) {
+        as += ws[w];
+        an += wn[w];
+    }
+    if (threadIdx.x == 1023) {
+        J.c[J.m] = as + s;
+        J.tot[0] = as + s;
+        for (int w = 0; w < 32; ++w) mx = max(mx, wm[w]);
+        J.tot[1] = mx;
+        J.tot[2] = an + nz;
+    }
     for (int64_t i = lo; i < hi; ++i) {
-        int64_t v = c[i];
-        c[i] = acc;
-        acc += v;
+        const int64_t v = J.c[i];
+        J.c[i] = as;
+        as += v;
+        if (v > 0 && J.tgt) J.tgt[an++] = (int32_t)i;
     }
 }
 
@@ -345,18 +376,42 @@ __global__ void k_near_tail(MediumD m, double c, int nray, int order, zd *lam_o,
 // ---------------------------------------------------------------------------
 // host orchestration
 // ---------------------------------------------------------------------------
-template <typename T>
-static lm_status dalloc(lm_tree_s *t, T **p, size_t count)
+cudaError_t LmArena::get(void **p, size_t bytes)
 {
-    if (count == 0) count = 1;
-    cudaError_t e = cudaMalloc((void **)p, count * sizeof(T));
-    if (e != cudaSuccess) {
-        lm_set_error("cudaMalloc of %zu bytes failed: %s", count * sizeof(T), cudaGetErrorString(e));
-        return LM_ENOMEM;
+    bytes = (bytes + 511) / 512 * 512; // what cudaMalloc aligns to
+    if (bytes > left) {
+        const size_t unit = std::min<size_t>(64u << 20, std::max<size_t>(4u << 20, total));
+        size_t want = bytes > unit / 2 ? bytes : unit;
+        slabs.reserve(slabs.size() + 1);
+        void *m = nullptr;
+        cudaError_t e = cudaMalloc(&m, want);
+        if (e == cudaErrorMemoryAllocation && want > bytes) {
+            cudaGetLastError();
+            e = cudaMalloc(&m, want = bytes);
+        }
+        if (e != cudaSuccess) return e;
+        slabs.push_back(m);
+        total += want;
+        if (want == bytes) { // the open slab stays open
+            *p = m;
+            return cudaSuccess;
+        }
+        cur = (char *)m;
+        left = want;
     }
-    t->bytes += count * sizeof(T);
-    return LM_OK;
+    *p = cur;
+    cur += bytes;
+    left -= bytes;
+    return cudaSuccess;
 }
+void LmArena::release()
+{
+    for (void *m : slabs) cudaFree(m);
+    slabs.clear();
+    cur = nullptr;
+    left = total = 0;
+}
+
 #define TRY(x)                       \
     do {                             \
         lm_status s_ = (x);          \
@@ -369,22 +424,19 @@ lm_status lm_setup_tree(lm_tree_s *t, const double *x, const double *y, cudaStre
 {
     const int64_t n = t->n;
     const double d = t->med.d;
-    TRY(dalloc(t, &t->dflag, 4));
+    TRY(lm_dalloc(t, &t->dflag, 4));
     LM_CUDA(cudaMemsetAsync(t->dflag, 0, 4 * sizeof(int), st));
     int nb = (int)std::min<int64_t>(1024, (n + 255) / 256);
     double *bmin, *bmax;
-    TRY(dalloc(t, &bmin, nb));
-    TRY(dalloc(t, &bmax, nb));
+    TRY(lm_dalloc(t->tmp, &bmin, 2 * nb));
+    bmax = bmin + nb;
     k_minmax<<<nb, 256, 0, st>>>(x, y, n, d, bmin, bmax, t->dflag);
-    std::vector<double> hmin(nb), hmax(nb);
+    std::vector<double> hmin(2 * nb);
+    const double *hmax = hmin.data() + nb;
     int hflag = 0;
-    LM_CUDA(cudaMemcpyAsync(hmin.data(), bmin, nb * sizeof(double), cudaMemcpyDeviceToHost, st));
-    LM_CUDA(cudaMemcpyAsync(hmax.data(), bmax, nb * sizeof(double), cudaMemcpyDeviceToHost, st));
+    LM_CUDA(cudaMemcpyAsync(hmin.data(), bmin, 2 * nb * sizeof(double), cudaMemcpyDeviceToHost, st));
     LM_CUDA(cudaMemcpyAsync(&hflag, t->dflag, sizeof(int), cudaMemcpyDeviceToHost, st));
     LM_CUDA(cudaStreamSynchronize(st));
-    cudaFree(bmin);
-    cudaFree(bmax);
-    t->bytes -= 2 * nb * sizeof(double);
     if (hflag & 1) {
         lm_set_error("build_tree: a point is non-finite or not strictly inside -d < y < 0");
         return LM_EINVAL;
@@ -415,27 +467,23 @@ lm_status lm_setup_tree(lm_tree_s *t, const double *x, const double *y, cudaStre
         int L = 0;
         while ((double)n > (double)t->med.opt.leaf_target * t->R * pow(4.0, L)) ++L;
         int32_t *key = nullptr, *cnt = nullptr;
-        TRY(dalloc(t, &key, n));
+        TRY(lm_dalloc(t->tmp, &key, n));
         for (;; ++L) {
             const int64_t ncol = (int64_t)t->R << L, nrow = (int64_t)1 << L, nl = ncol * nrow;
             if (L >= 14 || nl > std::max<int64_t>(2 * n, t->R)) {
                 --L;
                 break;
             }
-            TRY(dalloc(t, &cnt, nl));
+            TRY(lm_dalloc(t->tmp, &cnt, nl));
             LM_CUDA(cudaMemsetAsync(cnt, 0, nl * sizeof(int32_t), st));
             k_keys<<<grid_for(n, 256), 256, 0, st>>>(x, y, n, t->x0, ldexp(d, -L), ncol, nrow, key, cnt);
             std::vector<int32_t> hc(nl);
             LM_CUDA(cudaMemcpyAsync(hc.data(), cnt, nl * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
             LM_CUDA(cudaStreamSynchronize(st));
-            cudaFree(cnt);
-            t->bytes -= nl * sizeof(int32_t);
             double s2 = 0.0;
             for (int32_t c : hc) s2 += (double)c * c;
             if (s2 / n <= 1.5 * t->med.opt.leaf_target) break;
         }
-        cudaFree(key);
-        t->bytes -= n * sizeof(int32_t);
         t->L = std::max(L, 0);
     }
     const int L = t->L;
@@ -447,34 +495,23 @@ lm_status lm_setup_tree(lm_tree_s *t, const double *x, const double *y, cudaStre
     }
     int32_t *key, *cnt, *cursor;
     int64_t *tmp;
-    TRY(dalloc(t, &key, n));
-    TRY(dalloc(t, &cnt, t->nleaf));
-    TRY(dalloc(t, &cursor, t->nleaf));
-    TRY(dalloc(t, &t->leaf_start, t->nleaf + 1));
-    TRY(dalloc(t, &t->perm, n));
-    LM_CUDA(cudaMemsetAsync(cnt, 0, t->nleaf * sizeof(int32_t), st));
-    LM_CUDA(cudaMemsetAsync(cursor, 0, t->nleaf * sizeof(int32_t), st));
+    TRY(lm_dalloc(t->tmp, &key, n));
+    TRY(lm_dalloc(t->tmp, &cnt, 2 * t->nleaf));
+    cursor = cnt + t->nleaf;
+    TRY(lm_dalloc(t, &t->leaf_start, t->nleaf + 1));
+    TRY(lm_dalloc(t, &t->perm, n));
+    LM_CUDA(cudaMemsetAsync(cnt, 0, 2 * t->nleaf * sizeof(int32_t), st));
     double w = ldexp(d, -L);
     k_keys<<<grid_for(n, 256), 256, 0, st>>>(x, y, n, t->x0, w, ncol, nrow, key, cnt);
     k_scan<<<1, 1024, 0, st>>>(cnt, t->nleaf, t->leaf_start);
     tmp = t->perm;
     k_scatter<<<grid_for(n, 256), 256, 0, st>>>(key, n, t->leaf_start, cursor, tmp);
     k_leafsort<<<(unsigned)t->nleaf, 256, 0, st>>>(t->leaf_start, t->perm, t->dflag);
-    TRY(dalloc(t, &t->xs, n));
-    TRY(dalloc(t, &t->ys, n));
+    TRY(lm_dalloc(t, &t->xs, n));
+    TRY(lm_dalloc(t, &t->ys, n));
     k_gather_pts<<<grid_for(n, 256), 256, 0, st>>>(x, y, t->perm, n, t->xs, t->ys);
     LM_CUDA(cudaGetLastError());
-    LM_CUDA(cudaMemcpyAsync(&hflag, t->dflag, sizeof(int), cudaMemcpyDeviceToHost, st));
-    LM_CUDA(cudaStreamSynchronize(st));
-    cudaFree(key);
-    cudaFree(cnt);
-    cudaFree(cursor);
-    t->bytes -= (n + 2 * t->nleaf) * sizeof(int32_t);
-    if (hflag & 2) {
-        lm_set_error("build_tree: a leaf holds more than %d points; use a deeper tree", LM_MAXLEAF);
-        return LM_ENOTSUP;
-    }
-    return LM_OK;
+    return LM_OK; // an overfull leaf (k_leafsort's flag) is reported by lm_setup_tables
 }
 
 // classes (term, dc, dr) reachable under the list rules at level l
@@ -509,12 +546,15 @@ static void enumerate_classes(int l, int R, std::vector<std::tuple<int, int, int
 }
 
 // Levels 0..L of the strip forest: scale vectors, the M2M / L2L tables and,
-// with boxes set, the per-level expansion arrays of the uniform tree.
+// with boxes set, the FP64 form's per-level expansion arrays of the uniform tree.
 lm_status lm_setup_levels(lm_tree_s *t, int L, bool boxes, cudaStream_t st)
 {
     const int P = t->p, np = 2 * P + 1;
     const double k = t->med.k2, d = t->med.d;
     t->lev.resize(L + 1);
+    double *scale;
+    TRY(lm_dalloc(t, &scale, (size_t)(L + 1) * (P + 1)));
+    std::vector<double> sc((size_t)(L + 1) * (P + 1));
     for (int l = 0; l <= L; ++l) {
         Level &lv = t->lev[l];
         lv.l = l;
@@ -522,33 +562,32 @@ lm_status lm_setup_levels(lm_tree_s *t, int L, bool boxes, cudaStream_t st)
         lv.nrow = (int64_t)1 << l;
         lv.nbox = lv.ncol * lv.nrow;
         lv.w = ldexp(d, -l);
-        std::vector<double> sc(P + 1);
         double f = 0.5 * k * lv.w, v = 1.0;
         for (int n = 0; n <= P; ++n) {
-            sc[n] = v;
+            sc[(size_t)l * (P + 1) + n] = v;
             v *= f / (n + 1);
         }
-        TRY(dalloc(t, &lv.scale, P + 1));
-        LM_CUDA(cudaMemcpyAsync(lv.scale, sc.data(), (P + 1) * sizeof(double), cudaMemcpyHostToDevice, st));
-        if (boxes) {
-            TRY(dalloc(t, &lv.M, lv.nbox * np * LM_MAXV));
-            TRY(dalloc(t, &lv.Lc, lv.nbox * np * LM_MAXV));
+        lv.scale = scale + (size_t)l * (P + 1);
+        if (boxes && t->precision == LM_FP64) {
+            TRY(lm_dalloc(t, &lv.M, lv.nbox * np * LM_MAXV));
+            TRY(lm_dalloc(t, &lv.Lc, lv.nbox * np * LM_MAXV));
         }
     }
+    LM_CUDA(cudaMemcpyAsync(scale, sc.data(), sc.size() * sizeof(double), cudaMemcpyHostToDevice, st));
     // shift tables
     for (int l = 0; l <= L; ++l) {
         Level &lv = t->lev[l];
         lv.m2m = nullptr;
         lv.l2l = nullptr;
-        if (l < L) TRY(dalloc(t, &lv.m2m, 4 * np * np));
-        if (l > 0) TRY(dalloc(t, &lv.l2l, 4 * np * np));
+        if (l < L) TRY(lm_dalloc(t, &lv.m2m, 4 * np * np));
+        if (l > 0) TRY(lm_dalloc(t, &lv.l2l, 4 * np * np));
     }
     std::vector<ShiftJob> jobs;
     for (int l = 0; l < L; ++l) { // child level l+1 -> parent level l
         const Level &par = t->lev[l], &ch = t->lev[l + 1];
         jobs.push_back({k, ch.w, ch.scale, par.scale, par.m2m, ch.l2l});
     }
-    return lm_build_shift_tables(P, jobs, st);
+    return lm_build_shift_tables(P, jobs, t->tmp, st);
 }
 
 // Near-field quadrature tables of the reflected direct terms (shared by both tree kinds)
@@ -577,30 +616,30 @@ lm_status lm_setup_near(lm_tree_s *t, cudaStream_t st)
     q.nseg = (nflat + 2) * order;
     q.nray = t->med.opt.tail_rays;
     q.ntail = t->med.opt.tail_order;
-    TRY(dalloc(t, &q.seg_lam, q.nseg));
-    TRY(dalloc(t, &q.seg_s2, q.nseg));
-    TRY(dalloc(t, &q.seg_w, 2 * q.nseg));
+    TRY(lm_dalloc(t, &q.seg_lam, q.nseg));
+    TRY(lm_dalloc(t, &q.seg_s2, q.nseg));
+    TRY(lm_dalloc(t, &q.seg_w, 2 * q.nseg));
     int nt = q.nray * q.ntail;
-    TRY(dalloc(t, &q.tail_lam, nt));
-    TRY(dalloc(t, &q.tail_s2, nt));
-    TRY(dalloc(t, &q.tail_w, 4 * nt));
+    TRY(lm_dalloc(t, &q.tail_lam, nt));
+    TRY(lm_dalloc(t, &q.tail_s2, nt));
+    TRY(lm_dalloc(t, &q.tail_w, 4 * nt));
     const bool impc = t->precision == LM_FP64 && (imp_beta(md, 0) != 0.0 || imp_beta(md, 1) != 0.0);
     q.beta[0] = imp_beta(md, 0);
     q.beta[1] = imp_beta(md, 1);
-    if (impc) TRY(dalloc(t, &q.seg_c, 2 * q.nseg));
+    if (impc) TRY(lm_dalloc(t, &q.seg_c, 2 * q.nseg));
     k_near_seg<<<grid_for(q.nseg, 64), 64, 0, st>>>(md, q.c, a, delta, nflat, order, q.seg_lam, q.seg_s2,
                                                      q.seg_w, q.nseg, impc ? q.seg_c : nullptr);
-    if (q.split) TRY(dalloc(t, &q.tail_w2, 4 * nt));
+    if (q.split) TRY(lm_dalloc(t, &q.tail_w2, 4 * nt));
     k_near_tail<<<grid_for(nt, 64), 64, 0, st>>>(md, q.c, q.nray, q.ntail, q.tail_lam, q.tail_s2, q.tail_w,
                                                   q.split ? q.tail_w2 : nullptr);
     if (t->precision == LM_FP64) {
         q.ntail_g = std::max(64, q.ntail);
         const int ng = q.nray * q.ntail_g;
-        TRY(dalloc(t, &q.tail_lam_g, ng));
-        TRY(dalloc(t, &q.tail_s2_g, ng));
-        TRY(dalloc(t, &q.tail_w_g, 4 * ng));
-        if (q.split) TRY(dalloc(t, &q.tail_w2_g, 4 * ng));
-        if (impc) TRY(dalloc(t, &q.tail_c_g, 4 * ng));
+        TRY(lm_dalloc(t, &q.tail_lam_g, ng));
+        TRY(lm_dalloc(t, &q.tail_s2_g, ng));
+        TRY(lm_dalloc(t, &q.tail_w_g, 4 * ng));
+        if (q.split) TRY(lm_dalloc(t, &q.tail_w2_g, 4 * ng));
+        if (impc) TRY(lm_dalloc(t, &q.tail_c_g, 4 * ng));
         k_near_tail<<<grid_for(ng, 64), 64, 0, st>>>(md, q.c, q.nray, q.ntail_g, q.tail_lam_g, q.tail_s2_g,
                                                       q.tail_w_g, q.split ? q.tail_w2_g : nullptr,
                                                       impc ? q.tail_c_g : nullptr);
@@ -629,38 +668,84 @@ lm_status lm_setup_tables(lm_tree_s *t, cudaStream_t st)
                {t->med.opt.top_bc, t->med.opt.bottom_bc},
                {t->med.opt.top_alpha, t->med.opt.bottom_alpha}};
     TRY(lm_setup_levels(t, L, true, st));
-    // lists and M2L classes
-    std::vector<M2LClass> tcls;
+    // M2L classes and lists.  The lists are counted and scanned for all levels before the one
+    // synchronisation that their sizes need.
+    const bool mixed = t->precision == LM_MIXED;
+    std::vector<int32_t> smap;
+    std::vector<size_t> smap0;
+    std::vector<int> dcs;
     for (int l = 0; l <= L; ++l) {
         Level &lv = t->lev[l];
         std::vector<std::tuple<int, int, int>> cls;
         enumerate_classes(l, t->R, cls);
         int DC = l == 0 ? (int)std::max<int64_t>(3, lv.ncol - 1) : 3;
-        std::vector<int32_t> smap((size_t)5 * (2 * DC + 1) * 7, -1);
+        smap0.push_back(smap.size());
+        dcs.push_back(DC);
+        smap.resize(smap.size() + (size_t)5 * (2 * DC + 1) * 7, -1);
         for (size_t i = 0; i < cls.size(); ++i) {
             int term = std::get<0>(cls[i]), dc = std::get<1>(cls[i]), dr = std::get<2>(cls[i]);
             lv.cls_term.push_back(term);
             lv.cls_dc.push_back(dc);
             lv.cls_dr.push_back(dr);
-            smap[slot_index(DC, term, dc, dr)] = (int32_t)i;
+            smap[smap0[l] + slot_index(DC, term, dc, dr)] = (int32_t)i;
         }
-        int32_t *dmap;
-        TRY(dalloc(t, &dmap, smap.size()));
-        LM_CUDA(cudaMemcpyAsync(dmap, smap.data(), smap.size() * sizeof(int32_t), cudaMemcpyHostToDevice, st));
-        TRY(dalloc(t, &lv.vstart, lv.nbox + 1));
-        k_vlist<<<grid_for(lv.nbox, 128), 128, 0, st>>>(l, lv.ncol, lv.nrow, DC, dmap, lv.vstart,
-                                                        nullptr, nullptr, nullptr, 0, t->dflag);
-        k_scan64<<<1, 1024, 0, st>>>(lv.vstart, lv.nbox);
-        LM_CUDA(cudaMemcpyAsync(&lv.nv, lv.vstart + lv.nbox, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
-        LM_CUDA(cudaStreamSynchronize(st));
-        TRY(dalloc(t, &lv.vsrc, lv.nv));
-        TRY(dalloc(t, &lv.vslot, lv.nv));
-        TRY(dalloc(t, &lv.vterm, lv.nv));
-        k_vlist<<<grid_for(lv.nbox, 128), 128, 0, st>>>(l, lv.ncol, lv.nrow, DC, dmap, lv.vstart,
-                                                        lv.vsrc, lv.vslot, lv.vterm, 1, t->dflag);
+    }
+    int32_t *dmap;
+    ScanJob *djobs;
+    int64_t *dtot;
+    TRY(lm_dalloc(t->tmp, &dmap, smap.size()));
+    LM_CUDA(cudaMemcpyAsync(dmap, smap.data(), smap.size() * sizeof(int32_t), cudaMemcpyHostToDevice, st));
+    const int nj = (mixed ? 2 : 1) * (L + 1) + 1; // V, rest (mixed) of every level; U
+    TRY(lm_dalloc(t->tmp, &djobs, nj));
+    TRY(lm_dalloc(t->tmp, &dtot, 3 * nj));
+    std::vector<ScanJob> sj;
+    auto vlist = [&](Level &lv, int pass) {
+        k_vlist<<<grid_for(lv.nbox, 128), 128, 0, st>>>(lv.l, lv.ncol, lv.nrow, dcs[lv.l], dmap + smap0[lv.l], lv.vstart,
+                                                        lv.vsrc, lv.vslot, lv.vterm, pass, t->dflag, lv.rstart);
+    };
+    for (Level &lv : t->lev) {
+        TRY(lm_dalloc(t, &lv.vstart, lv.nbox + 1));
+        sj.push_back({lv.vstart, lv.nbox, dtot + 3 * sj.size(), nullptr});
+        if (mixed) {
+            TRY(lm_dalloc(t, &lv.rstart, lv.nbox + 1));
+            TRY(lm_dalloc(t, &lv.rtgt, lv.nbox));
+            sj.push_back({lv.rstart, lv.nbox, dtot + 3 * sj.size(), lv.rtgt});
+        }
+        vlist(lv, 0);
+    }
+    const int64_t ncol = (int64_t)t->R << L, nrow = (int64_t)1 << L;
+    TRY(lm_dalloc(t, &t->ustart, t->nleaf + 1));
+    sj.push_back({t->ustart, t->nleaf, dtot + 3 * sj.size(), nullptr});
+    k_ulist<<<grid_for(t->nleaf, 128), 128, 0, st>>>(ncol, nrow, t->ustart, nullptr, nullptr, 0);
+    LM_CUDA(cudaMemcpyAsync(djobs, sj.data(), nj * sizeof(ScanJob), cudaMemcpyHostToDevice, st));
+    k_scan_lists<<<nj, 1024, 0, st>>>(djobs);
+    LM_CUDA(cudaGetLastError());
+    std::vector<int64_t> tot(3 * nj);
+    int hflag = 0;
+    LM_CUDA(cudaMemcpyAsync(tot.data(), dtot, tot.size() * sizeof(int64_t), cudaMemcpyDeviceToHost, st));
+    LM_CUDA(cudaMemcpyAsync(&hflag, t->dflag, sizeof(int), cudaMemcpyDeviceToHost, st));
+    LM_CUDA(cudaStreamSynchronize(st));
+    if (hflag & 2) {
+        lm_set_error("build_tree: a leaf holds more than %d points; use a deeper tree", LM_MAXLEAF);
+        return LM_ENOTSUP;
+    }
+    const int64_t *ht = tot.data();
+    std::vector<M2LClass> tcls;
+    for (Level &lv : t->lev) {
+        lv.nv = ht[0];
+        ht += 3;
+        if (mixed) {
+            lv.nrest = ht[0];
+            lv.nrtgt = ht[2];
+            ht += 3;
+        }
+        TRY(lm_dalloc(t, &lv.vsrc, lv.nv));
+        TRY(lm_dalloc(t, &lv.vslot, lv.nv));
+        TRY(lm_dalloc(t, &lv.vterm, lv.nv));
+        vlist(lv, 1);
         // tables
-        int ncls = (int)cls.size();
-        TRY(dalloc(t, &lv.tab, (size_t)std::max(1, ncls) * np * np));
+        int ncls = (int)lv.cls_term.size();
+        TRY(lm_dalloc(t, &lv.tab, (size_t)std::max(1, ncls) * np * np));
         if (md.deriv) // the free part does not depend on d: its tables stay zero
             LM_CUDA(cudaMemsetAsync(lv.tab, 0, (size_t)std::max(1, ncls) * np * np * sizeof(zd), st));
         for (int i = 0; i < ncls; ++i) { // free space: target centre - source centre = (dc w, -dr w)
@@ -668,30 +753,22 @@ lm_status lm_setup_tables(lm_tree_s *t, cudaStream_t st)
             tcls.push_back({lv.cls_term[i], lv.cls_dc[i] * lv.w, dy, k * lv.w, k * lv.w, lv.scale, lv.scale,
                             lv.tab + (size_t)i * np * np});
         }
-        LM_CUDA(cudaGetLastError());
-        LM_CUDA(cudaStreamSynchronize(st));
-        cudaFree(dmap);
-        t->bytes -= smap.size() * sizeof(int32_t);
     }
-    TRY(lm_build_m2l_tables(md, P, tcls, t->dflag, st));
-    // U list
-    {
-        const int64_t ncol = (int64_t)t->R << L, nrow = (int64_t)1 << L;
-        TRY(dalloc(t, &t->ustart, t->nleaf + 1));
-        k_ulist<<<grid_for(t->nleaf, 128), 128, 0, st>>>(ncol, nrow, t->ustart, nullptr, nullptr, 0);
-        k_scan64<<<1, 1024, 0, st>>>(t->ustart, t->nleaf);
-        LM_CUDA(cudaMemcpyAsync(&t->nu, t->ustart + t->nleaf, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
-        LM_CUDA(cudaStreamSynchronize(st));
-        TRY(dalloc(t, &t->usrc, t->nu));
-        TRY(dalloc(t, &t->uterm, t->nu));
-        k_ulist<<<grid_for(t->nleaf, 128), 128, 0, st>>>(ncol, nrow, t->ustart, t->usrc, t->uterm, 1);
-    }
+    TRY(lm_build_m2l_tables(md, P, tcls, t->dflag, t->tmp, st));
+    t->nu = ht[0];
+    t->umax = ht[1];
+    TRY(lm_dalloc(t, &t->usrc, t->nu));
+    TRY(lm_dalloc(t, &t->uterm, t->nu));
+    k_ulist<<<grid_for(t->nleaf, 128), 128, 0, st>>>(ncol, nrow, t->ustart, t->usrc, t->uterm, 1);
     TRY(lm_setup_near(t, st));
-    // tree-order scratch for densities and potentials
-    TRY(dalloc(t, &t->qs, (size_t)LM_MAXV * t->n));
-    TRY(dalloc(t, &t->us, (size_t)LM_MAXV * t->n));
-    int hflag = 0;
     LM_CUDA(cudaGetLastError());
+    if (mixed) {
+        TRY(lm_setup_mixed(t, st));
+    } else {
+        // tree-order scratch for densities and potentials
+        TRY(lm_dalloc(t, &t->qs, (size_t)LM_MAXV * t->n));
+        TRY(lm_dalloc(t, &t->us, (size_t)LM_MAXV * t->n));
+    }
     LM_CUDA(cudaMemcpyAsync(&hflag, t->dflag, sizeof(int), cudaMemcpyDeviceToHost, st));
     LM_CUDA(cudaStreamSynchronize(st));
     if (hflag & 4) {
@@ -702,8 +779,7 @@ lm_status lm_setup_tables(lm_tree_s *t, cudaStream_t st)
         lm_set_error("build_tree: a layered M2L table overflowed; lower p");
         return LM_ENOTSUP;
     }
-    if (t->precision == LM_MIXED) return lm_setup_mixed(t, st);
-    return lm_setup_df(t, st);
+    return mixed ? LM_OK : lm_setup_df(t, st);
 }
 
 lm_status lm_list_to_host(lm_tree_s *t, int which, int level, std::vector<int64_t> &rows,
@@ -750,22 +826,7 @@ lm_status lm_list_to_host(lm_tree_s *t, int which, int level, std::vector<int64_
 
 void lm_free_tree_device(lm_tree_s *t)
 {
-    lm_free_mixed(t);
-    lm_free_adaptive(t);
-    lm_free_oz(t);
-    void *ptrs[] = {t->xs, t->ys, t->perm, t->leaf_start, t->ustart, t->usrc, t->uterm, t->qs, t->us,
-                    t->dflag, t->qexp, t->pwidx, t->pwC, t->nq.seg_lam, t->nq.seg_s2, t->nq.seg_w, t->nq.tail_lam, t->nq.tail_s2,
-                    t->nq.tail_w, t->nq.tail_lam_g, t->nq.tail_s2_g, t->nq.tail_w_g, t->nq.tail_w2,
-                    t->nq.tail_w2_g, t->nq.seg_c, t->nq.tail_c_g, t->ndf.node, t->ndf.w, t->ndf.w2, t->ndf.seg,
-                    t->ndf.segw, t->ndf.rel, t->ndf.hgt, t->ndf.q, t->ndf.node_g, t->ndf.w_g, t->ndf.w2_g, t->ndf.segw_g,
-                    t->xdf.bes, t->xdf.lev};
-    for (void *p : ptrs)
-        if (p) cudaFree(p);
-    for (Level &lv : t->lev) {
-        void *lp[] = {lv.vstart, lv.vsrc, lv.vslot, lv.vterm, lv.tab, lv.scale, lv.m2m, lv.l2l, lv.M, lv.Lc,
-                      lv.tabdft, lv.m2mdf, lv.l2ldf};
-        for (void *p : lp)
-            if (p) cudaFree(p);
-    }
+    t->tmp.release();
+    t->mem.release();
     cudaGetLastError(); // teardown leaves no error behind for the caller's next call
 }

@@ -57,9 +57,9 @@ __device__ inline int ti_seg_rounds(const TabContour &C) { return (C.nseg() + TI
 // node's weight and the powers Z^-n; the mirror's powers are (-1)^n Z^-n
 // (segment, lambda -> -lambda) or (-1)^n conj(Z^-n) (ray, lambda -> -conj lambda).
 // Bound by the FP64 pipe (2 DFMA per clock and SM): about 1600 DFMAs to evaluate
-// a pair of nodes, 12P + 8 (4P + 1) per pair for powers and sums.  Measured with
-// k_image_expand, 100k mixed tree of five levels (p = 14): 78.0 ms for the
-// (2P + 1)^2 integrals of a class one block each, before.
+// a pair of nodes, 12P + 8 (4P + 1) per pair for powers and sums.  100k mixed tree
+// of five levels (p = 14): 0.66 ms, k_image_expand 0.02 ms; 78.0 ms with a block per
+// class for its (2P + 1)^2 integrals.
 __global__ void __launch_bounds__(TI_THREADS) k_image_int(MediumD m, int P, const ImgInt *ints, const ImgItem *items,
                                                           zd *part)
 {
@@ -234,23 +234,19 @@ template <typename T> size_t put(std::vector<unsigned char> &buf, const std::vec
 
 } // namespace
 
-lm_status lm_build_shift_tables(int P, const std::vector<ShiftJob> &jobs, cudaStream_t st)
+lm_status lm_build_shift_tables(int P, const std::vector<ShiftJob> &jobs, LmArena &tmp, cudaStream_t st)
 {
     if (jobs.empty()) return LM_OK;
     ShiftJob *d;
-    LM_CUDA(cudaMalloc((void **)&d, jobs.size() * sizeof(ShiftJob)));
-    cudaError_t e = cudaMemcpyAsync(d, jobs.data(), jobs.size() * sizeof(ShiftJob), cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) {
-        k_shift_tab<<<(unsigned)(4 * jobs.size()), 256, 0, st>>>(P, d);
-        e = cudaGetLastError();
-    }
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st); // the job list is a temporary
-    cudaFree(d);
-    LM_CUDA(e);
+    const lm_status r = lm_dalloc(tmp, &d, jobs.size());
+    if (r != LM_OK) return r;
+    LM_CUDA(cudaMemcpyAsync(d, jobs.data(), jobs.size() * sizeof(ShiftJob), cudaMemcpyHostToDevice, st));
+    k_shift_tab<<<(unsigned)(4 * jobs.size()), 256, 0, st>>>(P, d);
+    LM_CUDA(cudaGetLastError());
     return LM_OK;
 }
 
-lm_status lm_build_m2l_tables(const MediumD &md, int P, const std::vector<M2LClass> &cls, int *dflag, cudaStream_t st)
+lm_status lm_build_m2l_tables(const MediumD &md, int P, const std::vector<M2LClass> &cls, int *dflag, LmArena &tmp, cudaStream_t st)
 {
     const int nn = 4 * P + 1;
     const double km = fmax(md.k1, fmax(md.k2, md.k3)), kmin = fmin(md.k1, fmin(md.k2, md.k3));
@@ -286,22 +282,18 @@ lm_status lm_build_m2l_tables(const MediumD &md, int P, const std::vector<M2LCla
     if (buf.empty()) return LM_OK;
     const size_t op = (buf.size() + 15) / 16 * 16;
     unsigned char *d;
-    LM_CUDA(cudaMalloc((void **)&d, op + items.size() * nn * sizeof(zd)));
-    cudaError_t e = cudaMemcpyAsync(d, buf.data(), buf.size(), cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess && !fc.empty()) k_free_tab<<<(unsigned)fc.size(), 256, 0, st>>>(md.k2, P, (const FreeCls *)(d + of));
-    if (e == cudaSuccess && !ic.empty()) {
+    const lm_status r = lm_dalloc(tmp, &d, op + items.size() * nn * sizeof(zd));
+    if (r != LM_OK) return r;
+    LM_CUDA(cudaMemcpyAsync(d, buf.data(), buf.size(), cudaMemcpyHostToDevice, st));
+    if (!fc.empty()) k_free_tab<<<(unsigned)fc.size(), 256, 0, st>>>(md.k2, P, (const FreeCls *)(d + of));
+    if (!ic.empty()) {
         const size_t shm = ((size_t)TI_CHUNK * nn + 2 * TI_CHUNK) * sizeof(zd);
-        e = lm_raise_smem((const void *)k_image_int, LM_SMEM_IMAGE_M2L, (int)shm);
-        if (e == cudaSuccess) {
-            k_image_int<<<(unsigned)items.size(), TI_THREADS, shm, st>>>(md, P, (const ImgInt *)(d + oi),
-                                                                       (const ImgItem *)(d + ot), (zd *)(d + op));
-            k_image_expand<<<(unsigned)ic.size(), 256, 0, st>>>(P, (const ImgInt *)(d + oi), (const ImgCls *)(d + oc),
-                                                                (const zd *)(d + op), dflag);
-        }
+        LM_CUDA(lm_raise_smem((const void *)k_image_int, LM_SMEM_IMAGE_M2L, (int)shm));
+        k_image_int<<<(unsigned)items.size(), TI_THREADS, shm, st>>>(md, P, (const ImgInt *)(d + oi),
+                                                                   (const ImgItem *)(d + ot), (zd *)(d + op));
+        k_image_expand<<<(unsigned)ic.size(), 256, 0, st>>>(P, (const ImgInt *)(d + oi), (const ImgCls *)(d + oc),
+                                                            (const zd *)(d + op), dflag);
     }
-    if (e == cudaSuccess) e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st); // the class lists and partial sums are temporaries
-    cudaFree(d);
-    LM_CUDA(e);
+    LM_CUDA(cudaGetLastError());
     return LM_OK;
 }

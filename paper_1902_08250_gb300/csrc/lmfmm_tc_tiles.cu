@@ -53,12 +53,12 @@
 // the launch's error flag, the others stop at their next wait, copies and
 // MMAs in flight are waited for (bounded) and tensor memory is freed.
 #include <algorithm>
-#include <map>
 #include <tuple>
 #include <type_traits>
 #include <vector>
 
 #include "internal.h"
+#include "lists.cuh"
 #include "tc_common.cuh"
 
 #include <cuda_fp16.h>
@@ -649,11 +649,11 @@ static lm_status tt_set_attr(int p)
     return LM_ENOTSUP;
 }
 
-// Tiles of tb class-consecutive boxes over every level, from the host copies of the
-// V lists: per tile the union of its boxes' entries, each with the mask of boxes that have it
-static void tt_build_tiles(const std::vector<std::vector<int64_t>> &vs, const std::vector<std::vector<int32_t>> &vsrc,
-                           const std::vector<std::vector<int32_t>> &vslot, const lm_tree_s *t, int tb,
-                           std::vector<TtTile> &tiles, std::vector<TtEnt> &ents)
+// Tiles of tb class-consecutive boxes over every level: per tile the union of its boxes' entries, by
+// (slot, column offset, source row), each with the mask of boxes that have it.  re, e0: the classes'
+// entry lists (lm_row_entries) in that order.
+static void tt_build_tiles(const std::vector<std::vector<RowEnt>> &re, const std::vector<std::vector<int32_t>> &e0,
+                           const lm_tree_s *t, int tb, std::vector<TtTile> &tiles, std::vector<TtEnt> &ents)
 {
     for (int l = 0; l <= t->L; ++l) {
         const Level &lv = t->lev[l];
@@ -665,18 +665,20 @@ static void tt_build_tiles(const std::vector<std::vector<int64_t>> &vs, const st
                 for (int64_t i0 = 0; i0 < ncl; i0 += tb) {
                     TtTile T{l, (int32_t)r, (int32_t)(i0 * cstride + pc), cstride,
                              (int32_t)std::min<int64_t>(tb, ncl - i0), (int32_t)ents.size(), 0, 0};
-                    std::map<std::tuple<int32_t, int32_t, int32_t>, uint32_t> m;
-                    for (int j = 0; j < T.nbox; ++j) {
-                        const int64_t c = T.c0 + (int64_t)j * cstride, b = r * ncol + c;
-                        for (int64_t e = vs[l][b]; e < vs[l][b + 1]; ++e) {
-                            const int64_t src = vsrc[l][e];
-                            const int32_t dc = (int32_t)(c - src % ncol), rs = (int32_t)(src / ncol);
-                            m[std::make_tuple(vslot[l][e], dc, rs)] |= 1u << j;
+                    const int64_t c0 = T.c0, c1 = c0 + (int64_t)(T.nbox - 1) * cstride;
+                    const int64_t cls = r * npar + pc;
+                    for (int32_t e = e0[l][cls]; e < e0[l][cls + 1]; ++e) {
+                        const RowEnt &E = re[l][e];
+                        uint32_t m = 0xffffffffu >> (32 - T.nbox);
+                        if (c0 - E.dc < 0 || c1 - E.dc >= ncol) {
+                            m = 0;
+                            for (int j = 0; j < T.nbox; ++j) {
+                                const int64_t cs = c0 + (int64_t)j * cstride - E.dc;
+                                if (cs >= 0 && cs < ncol) m |= 1u << j;
+                            }
                         }
+                        if (m) ents.push_back(TtEnt{E.slot, E.dc, E.rs, m});
                     }
-                    for (const auto &kv : m)
-                        ents.push_back(TtEnt{std::get<0>(kv.first), std::get<1>(kv.first), std::get<2>(kv.first),
-                                             kv.second});
                     T.e1 = (int32_t)ents.size();
                     tiles.push_back(T);
                 }
@@ -696,7 +698,7 @@ static lm_status tt_upload(lm_tree_s *t, const std::vector<T> &h, void **out, cu
 // Set-up of the tile form: split tables, the split-multipole buffer (sized for the
 // 16-vector form, with one zero box at the end for masked sources), the level
 // descriptors of both vector forms and their tile / entry lists, built on the host
-// from the V lists of every level.  Leaves tt_ready false (the per-level kernels
+// from the list rules.  Leaves tt_ready false (the per-level kernels
 // then run) where the form does not apply.
 lm_status lm_setup_tt(lm_tree_s *t, cudaStream_t st)
 {
@@ -734,26 +736,20 @@ lm_status lm_setup_tt(lm_tree_s *t, cudaStream_t st)
         k_tsplit<<<(unsigned)((nt + 255) / 256), 256, 0, st>>>(t->lev[l].tab, ncls, np, t->tt_tmax + l,
                                                                t->tt_tab + t->tt_tbase[l] * TT_TAB_FLOATS);
     }
-    // host copies of the V lists
-    std::vector<std::vector<int64_t>> vs(L + 1);
-    std::vector<std::vector<int32_t>> vsrc(L + 1), vslot(L + 1);
+    std::vector<std::vector<RowEnt>> re(L + 1);
+    std::vector<std::vector<int32_t>> e0(L + 1);
     for (int l = 0; l <= L; ++l) {
-        const Level &lv = t->lev[l];
-        vs[l].resize(lv.nbox + 1);
-        vsrc[l].resize(std::max<int64_t>(1, lv.nv));
-        vslot[l].resize(std::max<int64_t>(1, lv.nv));
-        LM_CUDA(cudaMemcpyAsync(vs[l].data(), lv.vstart, (lv.nbox + 1) * sizeof(int64_t), cudaMemcpyDeviceToHost, st));
-        if (lv.nv > 0) {
-            LM_CUDA(cudaMemcpyAsync(vsrc[l].data(), lv.vsrc, lv.nv * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-            LM_CUDA(cudaMemcpyAsync(vslot[l].data(), lv.vslot, lv.nv * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-        }
+        TT_TRY(lm_row_entries(t->lev[l], re[l], e0[l]));
+        for (size_t c = 0; c + 1 < e0[l].size(); ++c)
+            std::sort(re[l].begin() + e0[l][c], re[l].begin() + e0[l][c + 1], [](const RowEnt &a, const RowEnt &b) {
+                return std::tie(a.slot, a.dc, a.rs) < std::tie(b.slot, b.dc, b.rs);
+            });
     }
-    LM_CUDA(cudaStreamSynchronize(st));
     int64_t maxtiles = 0;
     for (int f = 0; f < 2; ++f) {
         std::vector<TtTile> tiles;
         std::vector<TtEnt> ents;
-        tt_build_tiles(vs, vsrc, vslot, t, f == 0 ? TtShape<16>::TB : TtShape<4>::TB, tiles, ents);
+        tt_build_tiles(re, e0, t, f == 0 ? TtShape<16>::TB : TtShape<4>::TB, tiles, ents);
         if (ents.size() > (size_t)INT32_MAX || tiles.size() > (size_t)INT32_MAX) return LM_OK;
         t->tt_ntile[f] = (int64_t)tiles.size();
         t->tt_nent[f] = (int64_t)ents.size();
@@ -762,7 +758,6 @@ lm_status lm_setup_tt(lm_tree_s *t, cudaStream_t st)
         TT_TRY(tt_upload(t, tt_levels(t, f == 0 ? 16 : 4), &t->tt_lv[f], st));
         maxtiles = std::max(maxtiles, t->tt_ntile[f]);
     }
-    LM_CUDA(cudaStreamSynchronize(st));
     t->tt_grid = std::max(1, (int)std::min<int64_t>(nsm, maxtiles));
     TT_TRY(tt_set_attr(t->p));
     t->tt_ready = true;
@@ -900,18 +895,3 @@ void lm_tt_batch_free(lm_tt_batch_s *b)
     delete b;
 }
 
-void lm_free_tt(lm_tree_s *t)
-{
-    for (int f = 0; f < 2; ++f) {
-        void *ptrs[] = {t->tt_tiles[f], t->tt_ents[f], t->tt_lv[f]};
-        for (void *p : ptrs)
-            if (p) cudaFree(p);
-        t->tt_tiles[f] = t->tt_ents[f] = t->tt_lv[f] = nullptr;
-    }
-    if (t->tt_tab) cudaFree(t->tt_tab);
-    if (t->tt_msplit) cudaFree(t->tt_msplit);
-    if (t->tt_tmax) cudaFree(t->tt_tmax);
-    if (t->tt_mmax) cudaFree(t->tt_mmax);
-    t->tt_tab = t->tt_msplit = nullptr;
-    t->tt_tmax = t->tt_mmax = nullptr;
-}

@@ -55,8 +55,6 @@ NEAR = {
     "leaf_of_65": (A, 65, 0.9, (-0.9, -0.1), 8, dict(p=20, depth=0)),           # one past a round of sources
     "low_order": (A, 500, 2.0, (-0.9, -0.1), 4, dict(p=1, depth=2)),
     "high_order": (A, 500, 2.0, (-0.9, -0.1), 16, dict(p=48, depth=1)),
-    "wide_tiles": (A, 30000, 3.0, (-0.95, -0.05), dict(p=14, depth=4)),
-    "wide_tiles_full_series": (A, 30000, 9.0, (-0.95, -0.05), dict(p=14, depth=3)),
     "interface": (A, 1500, 2.0, (-0.02, -1e-7), 11, dict(p=20, depth=3)),
     "adaptive": (A, 1500, 2.0, (-0.02, -1e-7), 3, dict(p=20, adaptive=True, leaf_target=16)),
     "impedance": (A, 900, 2.0, (-0.99, -0.01), 3, dict(p=22, depth=2, top_bc="impedance", top_alpha=0.7,
@@ -125,6 +123,8 @@ FEW = {
     "far_series": (B, 300, 1.9, (-0.95, -0.05), dict(p=24, depth=0)),
     "leaf_of_17": (A, 17, 0.9, (-0.9, -0.1), dict(p=14, depth=0)),
     "short_series": (A, 4000, 3.0, (-0.95, -0.05), dict(p=14, depth=4)),
+    "wide_tiles": (A, 30000, 3.0, (-0.95, -0.05), dict(p=14, depth=4)),
+    "wide_tiles_full_series": (A, 30000, 9.0, (-0.95, -0.05), dict(p=14, depth=3)),
     "interface": (A, 1500, 2.0, (-0.02, -1e-6), dict(p=14, depth=3)),
     "adaptive": (A, 1500, 2.0, (-0.02, -1e-6), dict(p=14, adaptive=True, leaf_target=16)),
     "adaptive_high": (A, 1500, 2.0, (-0.5, -1e-6), dict(p=24, adaptive=True, leaf_target=16)),
