@@ -21,7 +21,9 @@
 // 8-row groups), a stage of a table is one bulk copy, and any run of boxes one per digit and
 // chunk, whatever its offset.  Stages of up to 48 K (91 KB), two in flight.  Roles as in lmfmm_tc_tiles.cu:
 // a producer warp (a lane per copy), an MMA warp, 8 epilogue warps that read the 5
-// accumulators (320 columns of tensor memory) once per entry.
+// accumulators (320 columns of tensor memory) once per 4 entries: there is room for one
+// set of accumulators, so that reading them (about 50 FP32 instructions an element) and
+// the MMAs take turns.  250k strip, 16 vectors: 4.86 ms, 6.25 ms with a reading per entry.
 // Bound: 45 MMAs of 128 x 64 x 16 a stage, limited by the shared-memory reads of their
 // operands (6 KB a MMA at 128 B per clock).
 #include <algorithm>
@@ -49,6 +51,7 @@
 // k_m2l_dx 2.67 ms, of up to 255 0.20 ms, this kernel 6.10 and 6.25 ms.
 #define OZ_MINBOX 256
 #define OZ_PADL 2
+#define OZ_GRP 4 // entries summed in the accumulators before they are read
 
 struct OzLevel {
     int64_t tile0;          // first tile of the level in the launch
@@ -66,9 +69,9 @@ struct OzLevel {
 };
 
 __device__ __forceinline__ int oz_exp(uint32_t bits) { return bits ? (int)((bits >> 23) & 0xff) - 127 : -126; }
-// the level's table exponent: components below 2^(e-1), row sums at most 2^(e+4), so that the leading
-// digits' sum over K stays below 2^24 (|digit| <= 512 on either side)
-__device__ __forceinline__ int oz_ea(const uint32_t *t) { return max(oz_exp(t[0]) + 2, oz_exp(t[1]) - 3); }
+// the level's table exponent: components below 2^(e-1), row sums at most 2^(e+2), so that the leading
+// digits' sum over K and OZ_GRP = 4 entries stays below 2^24 (|digit| <= 512 on either side)
+__device__ __forceinline__ int oz_ea(const uint32_t *t) { return max(oz_exp(t[0]) + 2, oz_exp(t[1]) - 1); }
 __device__ __forceinline__ float oz_pow2(int e) { return __int_as_float((max(-126, min(127, e)) + 127) << 23); }
 __host__ __device__ __forceinline__ int oz_rows(int np) { return (2 * np + 7) / 8 * 8; }
 __host__ __device__ __forceinline__ int oz_chunks(int np) { return (2 * np + 15) / 16 * 2; }
@@ -338,7 +341,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_m2l_oz(const OzLevel *lvs, in
                 int cls, i0;
                 const OzLevel &lv = oz_tile(lvs, nlev, tile, &cls, &i0, tb);
                 const int ne = lv.e0[cls + 1] - lv.e0[cls];
-                for (int e = 0; e < ne && !stop; ++e, ++item) {
+                for (int e = 0; e < ne && !stop; e += OZ_GRP, ++item) {
                     if (!mbar_wait_lim(btempty, (item & 1) ^ 1, TC_WAIT_LIMIT, abort_s, err)) {
                         oz_fail(abort_s, err);
                         stop = true;
@@ -346,7 +349,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_m2l_oz(const OzLevel *lvs, in
                     }
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     int issued = 0;
-                    for (int st = 0; st < nst; ++st, ++it) {
+                    const int nstg = nst * min(OZ_GRP, ne - e);
+                    for (int q = 0, st = 0; q < nstg; ++q, ++it, st = st + 1 == nst ? 0 : st + 1) {
                         const int s = (int)(it % OZ_NST), kc = min(OZ_KC, KC - st * OZ_KC), ks = kc / 2;
                         if (!mbar_wait_lim(bfull + 8 * s, (it / OZ_NST) & 1, TC_WAIT_LIMIT, abort_s, err)) {
                             oz_fail(abort_s, err);
@@ -362,7 +366,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_m2l_oz(const OzLevel *lvs, in
                                 for (int j = 0; i + j < OZ_S; ++j)
                                     oz_mma(tmem + OZ_N * (i + j), oz_desc(sa + (i * kc + 2 * kk) * RA * 16, RA * 16),
                                            oz_desc(sb + (j * OZ_KC + 2 * kk) * OZ_N * 16, OZ_N * 16), idesc,
-                                           (st > 0 || kk > 0 || i > 0) ? 1u : 0u);
+                                           (q > 0 || kk > 0 || i > 0) ? 1u : 0u);
                         tc_commit(bempty + 8 * s);
                         ++issued;
                     }
@@ -390,7 +394,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_m2l_oz(const OzLevel *lvs, in
             df acc[32];
 #pragma unroll
             for (int c = 0; c < 32; ++c) acc[c] = df{0.f, 0.f};
-            for (int e = 0; e < ne; ++e, ++item) {
+            for (int e = 0; e < ne; e += OZ_GRP, ++item) {
                 if (!mbar_wait_lim(btfull, item & 1, TC_WAIT_LIMIT, abort_s, err)) {
                     oz_fail(abort_s, err);
                     bad = true;
