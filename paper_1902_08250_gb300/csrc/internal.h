@@ -217,17 +217,23 @@ struct ExpDF {
 // Tensor-core M2L of the FP64 form (lmfmm_oz.cu): its levels, and per vector form (1, 2, 4, 8, 16
 // slots) the device descriptors
 struct OzData {
-    struct Lv {
-        int l;
+    struct Op { // tables and entry lists of a contraction
         void *ents;
         int32_t *e0;
-        unsigned char *A, *B;
+        unsigned char *A;
         uint32_t *tmax;
     };
-    std::vector<Lv> lv;
+    struct Lv { // a level whose M2L (M2M to and L2L from the level above) runs on the tensor cores
+        int l;
+        Op op[3];
+        unsigned char *B; // digits of its multipoles, then of its local expansions
+    };
+    std::vector<Lv> lv; // L, L - 1, ..
+    size_t nshift = 0;  // of which the first take M2M and L2L too
     uint32_t *mmax = nullptr;
+    unsigned char *Btop = nullptr; // digits of the local expansions of the level above the last
     void *desc[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
-    int64_t ntile[5] = {0, 0, 0, 0, 0};
+    int64_t ntile[5] = {0, 0, 0, 0, 0}; // of the M2L
     int nsm = 0;
 };
 
@@ -366,6 +372,9 @@ void lm_df_m2l(const M2LLevelDF *lev, int nlev, int64_t nblk, int P, int nv, cud
 bool lm_oz_level(const lm_tree_s *t, int l); // tensor-core M2L of the FP64 form (lmfmm_oz.cu)
 lm_status lm_setup_oz(lm_tree_s *t, cudaStream_t st);
 lm_status lm_launch_m2l_oz(lm_tree_s *t, int nv, cudaStream_t st, int *launches);
+lm_status lm_launch_m2m_oz(lm_tree_s *t, int nv, cudaStream_t st, int *lmin, int *launches);
+bool lm_oz_shift(const lm_tree_s *t, int l);
+lm_status lm_launch_l2l_oz(lm_tree_s *t, int l, int nv, cudaStream_t st, int *launches);
 lm_status lm_run_df(lm_tree_s *t, const zd *q, int nvec, zd *u, bool adjoint, zd *ux, zd *uy, cudaStream_t st);
 lm_status lm_run_apply_grad(lm_tree_s *t, const zd *q, int nvec, zd *u, zd *ux, zd *uy, cudaStream_t st);
 // mixed precision (lmfmm_mixed.cu)

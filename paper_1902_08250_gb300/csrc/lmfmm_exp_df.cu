@@ -587,8 +587,9 @@ lm_status lm_run_df(lm_tree_s *t, const zd *q, int nvec, zd *u, bool adjoint, zd
         else launch_s2m(B, gleaves, nleaf, P, k2, t->ndf.rel, t->leaf_start, t->ndf.q, nv, Mof(L), st);
         lm_phase_end(t, PH_S2M, st, 1);
         if (L > 0) lm_phase_begin(t, PH_M2M, st);
-        int nl = 0;
-        for (int l = L - 1; l >= 0; --l) {
+        int nl = 0, lm2m = L;
+        if (!ad) TRY_X(lm_launch_m2m_oz(t, nv, st, &lm2m, &nl));
+        for (int l = lm2m - 1; l >= 0; --l) {
             const int64_t npar = ad ? A.nl_start[l + 1] - A.nl_start[l] : t->lev[l].nbox;
             if (npar == 0) continue;
             if (ad) launch_m2m(ListParents{A.nonleaf + A.nl_start[l], A.child}, npar, P, nv, t->lev[l].m2mdf, Mof(0), Mof(0), st);
@@ -607,6 +608,12 @@ lm_status lm_run_df(lm_tree_s *t, const zd *q, int nvec, zd *u, bool adjoint, zd
         for (int l = 1; l <= L; ++l) {
             const int64_t npar = ad ? A.nl_start[l] - A.nl_start[l - 1] : t->lev[l - 1].nbox;
             if (npar == 0) continue;
+            if (lm_oz_shift(t, l)) {
+                int k = 0;
+                TRY_X(lm_launch_l2l_oz(t, l, nv, st, &k));
+                nl += k;
+                continue;
+            }
             if (ad) launch_l2l(ListParents{A.nonleaf + A.nl_start[l - 1], A.child}, npar, P, nv, t->lev[l].l2ldf, Lof(0), Lof(0), st);
             else launch_l2l(GridParents{t->lev[l - 1].ncol}, npar, P, nv, t->lev[l].l2ldf, Lof(l - 1), Lof(l), st);
             ++nl;

@@ -6,8 +6,8 @@
 // the FP32 accumulator holds exactly; the digit pairs i + j <= 4 are kept, those of one
 // weight 2^{-10 (i + j)} in one accumulator, and the 5 integers of an output are
 // combined in double-float (50 bits against the 48 of the double-float contraction it
-// replaces).  Levels of at least OZ_MINBOX boxes of uniform trees; the others run on
-// the CUDA cores (k_m2l_dx).
+// replaces).  Levels of at least OZ_MINBOX boxes of uniform trees, their M2M and L2L
+// from OZ_MINSHIFT; the others run on the CUDA cores (lmfmm_exp_df.cu).
 //
 // A tile is 64 columns: 64 / nvs target boxes of one row and parity class, nvs vectors
 // each.  An interior box's V list depends only on its row and its column's parity, so
@@ -46,26 +46,38 @@
 #define OZ_STAGE (OZ_A_BYTES + OZ_B_BYTES)
 #define OZ_EPI 8
 #define OZ_THREADS ((OZ_EPI + 2) * 32)
-#define OZ_SMEM (OZ_NST * OZ_STAGE + 128)
+#define OZ_XROW 33 // floats of a row of an epilogue warp's exchange
+#define OZ_XCH (OZ_EPI * 32 * OZ_XROW * 4)
+#define OZ_SMEM (OZ_NST * OZ_STAGE + OZ_XCH + 128)
 // Smaller levels leave most SMs without a tile.  250k strip, 16 vectors: levels of up to 2047 boxes in
 // k_m2l_dx 2.67 ms, of up to 255 0.20 ms, this kernel 6.10 and 6.25 ms.
 #define OZ_MINBOX 256
+// M2M and L2L read and write a level for one or four entries a tile and split the sources in a launch
+// of their own.  250k strip, 16 vectors (levels of 20480 and 5120 boxes): 4.5 ms on the CUDA cores,
+// 1.7 ms with these two levels here; walled adjoint of 20k points (no level as large): 658 us, 680 us
+// with its levels of 256 boxes here.
+#define OZ_MINSHIFT 4096
 #define OZ_PADL 2
 #define OZ_GRP 4 // entries summed in the accumulators before they are read
 
+// One level of a contraction: M2L (sources and targets a level's boxes), M2M (sources the children,
+// targets a level) or L2L (sources the parents).  Sources lie in planes of consecutive boxes: (row, column
+// parity) for M2L and M2M, so that the children (i, j) of consecutive parents are one run; rows for L2L.
 struct OzLevel {
     int64_t tile0;          // first tile of the level in the launch
-    int32_t ncl, tpr;       // boxes of a (row, parity) class, tiles of one
-    int64_t ncol;
-    const int32_t *e0;      // [2 nrow + 1] entries of each class
-    const RowEnt *ents;
+    int32_t ncl, tpr;       // boxes of a target class = of a source plane, tiles of a class
+    int32_t tstep, sstep;   // 2: target classes / source planes are (row, parity), 1: rows
+    int32_t add, planes;    // L += (L2L); source planes
+    int64_t ncol;           // target columns
+    const int32_t *e0;      // [classes + 1] entries of each class
+    const RowEnt *ents;     // (pad: rs is the source plane itself, its run starts at the tile's first box)
     const unsigned char *A; // split tables
-    unsigned char *B;       // split multipoles: planes of a (row, parity)
+    unsigned char *B;       // split sources
     const uint32_t *tmax;   // [2] largest table component and row sum of the level (float bits)
-    uint32_t *mmax;         // [LM_MAXV] largest multipole component per vector
-    const float4 *M;
-    float4 *L;
-    int64_t nrow;
+    uint32_t *mmax;         // [LM_MAXV] largest source component per vector
+    uint32_t *omax;         // the same of the result, or null
+    const float4 *M;        // sources
+    float4 *L;              // targets
 };
 
 __device__ __forceinline__ int oz_exp(uint32_t bits) { return bits ? (int)((bits >> 23) & 0xff) - 127 : -126; }
@@ -131,11 +143,11 @@ __global__ void __launch_bounds__(256) k_oz_tsplit(const zd *tab, int64_t ncls, 
         *(uint4 *)(o + ((int64_t)(s * kc + c - c0) * RA + row) * 16) = *(const uint4 *)d[s];
 }
 
-// largest multipole component of each vector over a level's boxes
+// largest component of each vector over a level's sources
 __global__ void __launch_bounds__(256) k_oz_mmax(const OzLevel *lvs, int np, int nv)
 {
     const OzLevel &lv = lvs[blockIdx.y];
-    const int64_t n = lv.ncol * lv.nrow * np;
+    const int64_t n = (int64_t)lv.planes * lv.ncl * np;
     const int per = blockDim.x / nv, v = threadIdx.x % nv; // threads per round of orders
     float mx = 0.f;
     if ((int)threadIdx.x < per * nv)
@@ -156,16 +168,16 @@ __global__ void __launch_bounds__(256) k_oz_split(const OzLevel *lvs, int np, in
 {
     const OzLevel &lv = lvs[blockIdx.y];
     const int KC = oz_chunks(np);
-    const int64_t rows = oz_prow(lv.ncl, OZ_N / nvs, nvs), tot = 2 * lv.nrow * rows * KC;
+    const int64_t rows = oz_prow(lv.ncl, OZ_N / nvs, nvs), tot = lv.planes * rows * KC;
     for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < tot; idx += (int64_t)gridDim.x * blockDim.x) {
         const int64_t r = idx % rows, pc = idx / rows;
         const int c = (int)(pc % KC);
-        const int64_t plane = pc / KC, row = plane >> 1;
-        const int par = (int)(plane & 1), v = (int)(r % nvs);
+        const int64_t plane = pc / KC;
+        const int v = (int)(r % nvs);
         const int64_t i = r / nvs - OZ_PADL;
         uint16_t d[OZ_S][8];
         const bool on = i >= 0 && i < lv.ncl && v < nv;
-        const int64_t box = row * lv.ncol + 2 * i + par;
+        const int64_t box = lv.sstep == 2 ? (plane >> 1) * 2 * lv.ncl + 2 * i + (plane & 1) : plane * lv.ncl + i;
         const float sc = on ? oz_pow2(-(oz_exp(lv.mmax[v]) + 2)) : 0.f;
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
@@ -249,7 +261,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_m2l_oz(const OzLevel *lvs, in
                                                           int *err)
 {
     extern __shared__ __align__(1024) unsigned char smem[];
-    uint64_t *bars = (uint64_t *)(smem + OZ_NST * OZ_STAGE);
+    uint64_t *bars = (uint64_t *)(smem + OZ_NST * OZ_STAGE + OZ_XCH);
     uint32_t *tslot = (uint32_t *)(bars + 2 * OZ_NST + 2);
     volatile int *abort_s = (volatile int *)(tslot + 1);
     const uint32_t sbase = smem_u32(smem), bfull = smem_u32(bars), bempty = bfull + 8 * OZ_NST, btfull = bfull + 16 * OZ_NST,
@@ -294,11 +306,12 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_m2l_oz(const OzLevel *lvs, in
                 const RowEnt mine = lane < cnt ? lv.ents[base + lane] : RowEnt{0, 0, 0, 0};
                 for (int i = 0; i < cnt && !stop; ++i) {
                     const int slot = __shfl_sync(0xffffffffu, mine.slot, i), dc = __shfl_sync(0xffffffffu, mine.dc, i),
-                              rs = __shfl_sync(0xffffffffu, mine.rs, i);
+                              rs = __shfl_sync(0xffffffffu, mine.rs, i), direct = __shfl_sync(0xffffffffu, mine.pad, i);
                     const int cs = c0 - dc, par = cs & 1;
-                    const int64_t sbox = ((cs - par) >> 1) + OZ_PADL; // first source in its padded plane
+                    const int64_t plane = direct ? rs : (int64_t)rs * 2 + par;
+                    const int64_t sbox = (direct ? i0 : (cs - par) >> 1) + OZ_PADL; // first source in its padded plane
                     const unsigned char *a = lv.A + (int64_t)slot * OZ_S * KC * RA * 16;
-                    const unsigned char *b = lv.B + ((int64_t)rs * 2 + par) * OZ_S * KC * rows * 16 + sbox * nvs * 16;
+                    const unsigned char *b = lv.B + plane * OZ_S * KC * rows * 16 + sbox * nvs * 16;
                     for (int st = 0; st < nst; ++st, ++it) {
                         const int s = (int)(it % OZ_NST), k0 = st * OZ_KC, kc = min(OZ_KC, KC - k0);
                         int ok = 1;
@@ -424,19 +437,80 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_m2l_oz(const OzLevel *lvs, in
                 }
             }
             if (bad) break;
-            if (row < 2 * np) {
-                const int ea = oz_ea(lv.tmax), p = row < np ? row : row - np, off = row < np ? 0 : 1;
-                const int64_t r0 = (int64_t)(cls >> 1) * lv.ncol + (cls & 1);
+            const int64_t r0 = lv.tstep == 2 ? (int64_t)(cls >> 1) * lv.ncol + (cls & 1) : cls * lv.ncol;
+            const int ea = oz_ea(lv.tmax);
+            float omx = 0.f; // largest result of column 32 H + lane
+            // where result (row, column) goes, and its scale 2^x
+            auto out = [&](int rw, int col, int *x) -> float2 * {
+                const int j = col / nvs, v = col - j * nvs, p = rw < np ? rw : rw - np;
+                if (rw >= 2 * np || i0 + j >= lv.ncl || v >= nv) return nullptr;
+                *x = ea + oz_exp(lv.mmax[v]) + 2 - 2 * OZ_BITS;
+                return (float2 *)&lv.L[((r0 + lv.tstep * (int64_t)(i0 + j)) * np + p) * nv + v] + (rw < np ? 0 : 1);
+            };
+            if (nvs >= 8) {
+                // a lane takes a column: neighbouring vectors are neighbours in memory
+                float *xc = (float *)(smem + OZ_NST * OZ_STAGE) + warp * 32 * OZ_XROW;
+                float h[32];
+                __syncwarp();
 #pragma unroll
-                for (int c = 0; c < 32; ++c) {
-                    const int col = 32 * H + c, j = col / nvs, v = col - j * nvs;
-                    if (i0 + j < lv.ncl && v < nv) {
-                        const int ex = ea + oz_exp(lv.mmax[v]) + 2 - 2 * OZ_BITS, x1 = ex / 2;
-                        const float f = oz_pow2(x1), g = oz_pow2(ex - x1);
-                        float2 *o = (float2 *)&lv.L[((r0 + 2 * (int64_t)(i0 + j)) * np + p) * nv + v];
-                        o[off] = make_float2(acc[c].h * f * g, acc[c].l * f * g);
+                for (int c = 0; c < 32; ++c) xc[lane * OZ_XROW + c] = acc[c].h;
+                __syncwarp();
+#pragma unroll
+                for (int r = 0; r < 32; ++r) h[r] = xc[r * OZ_XROW + lane];
+                __syncwarp();
+#pragma unroll
+                for (int c = 0; c < 32; ++c) xc[lane * OZ_XROW + c] = acc[c].l;
+                __syncwarp();
+#pragma unroll
+                for (int r8 = 0; r8 < 32; r8 += 8) {
+                    float2 *o[8], b[8];
+                    int x = 0;
+#pragma unroll
+                    for (int r = 0; r < 8; ++r) {
+                        o[r] = out(32 * Q + r8 + r, 32 * H + lane, &x);
+                        b[r] = lv.add && o[r] ? *o[r] : make_float2(0.f, 0.f);
+                    }
+                    const float f = oz_pow2(x / 2), g = oz_pow2(x - x / 2);
+#pragma unroll
+                    for (int r = 0; r < 8; ++r)
+                        if (o[r]) {
+                            df y = {h[r8 + r] * f * g, xc[(r8 + r) * OZ_XROW + lane] * f * g};
+                            if (lv.add) y = df_add(df{b[r].x, b[r].y}, y);
+                            *o[r] = make_float2(y.h, y.l);
+                            omx = fmaxf(omx, fabsf(y.h));
+                        }
+                }
+            } else {
+                // a lane takes a row: with few vectors, neighbouring orders are near in memory
+#pragma unroll
+                for (int c8 = 0; c8 < 32; c8 += 8) {
+                    float2 *o[8], b[8];
+                    int x[8];
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) {
+                        o[c] = out(row, 32 * H + c8 + c, &x[c]);
+                        b[c] = lv.add && o[c] ? *o[c] : make_float2(0.f, 0.f);
+                    }
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) {
+                        float m = 0.f;
+                        if (o[c]) {
+                            const float f = oz_pow2(x[c] / 2), g = oz_pow2(x[c] - x[c] / 2);
+                            df y = {acc[c8 + c].h * f * g, acc[c8 + c].l * f * g};
+                            if (lv.add) y = df_add(df{b[c].x, b[c].y}, y);
+                            *o[c] = make_float2(y.h, y.l);
+                            m = fabsf(y.h);
+                        }
+                        if (lv.omax) {
+                            const float w = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(m)));
+                            if (lane == c8 + c) omx = w;
+                        }
                     }
                 }
+            }
+            if (lv.omax) {
+                uint32_t *o = lv.omax + (32 * H + lane) % nvs;
+                if (__float_as_uint(omx) > *(volatile uint32_t *)o) atomicMax(o, __float_as_uint(omx));
             }
         }
     }
@@ -454,7 +528,6 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_m2l_oz(const OzLevel *lvs, in
         lm_status s_ = (x);          \
         if (s_ != LM_OK) return s_;  \
     } while (0)
-static int nv_slots(int nv) { return nv <= 1 ? 1 : nv <= 2 ? 2 : nv <= 4 ? 4 : nv <= 8 ? 8 : 16; }
 
 // whether level l of a uniform FP64 tree takes the tensor cores: its boxes fill the SMs with tiles, its
 // order fits the operand
@@ -463,78 +536,123 @@ bool lm_oz_level(const lm_tree_s *t, int l)
     return !t->adaptive && t->m2l_df && l >= 1 && 2 * t->np <= 128 && t->lev[l].nbox >= OZ_MINBOX;
 }
 
-static std::vector<OzLevel> oz_levels(const lm_tree_s *t, int nvs)
+// M2L descriptors of the tensor-core levels, their M2M to the level above, their L2L from it
+enum { OZ_M2L = 0, OZ_M2M = 1, OZ_L2L = 2 };
+static std::vector<OzLevel> oz_levels(const lm_tree_s *t, int op, int nvs)
 {
     std::vector<OzLevel> v;
+    const OzData &Z = t->oz;
     const int tb = OZ_N / nvs;
+    const size_t nl = Z.lv.size();
     int64_t tiles = 0;
-    for (const OzData::Lv &z : t->oz.lv) {
-        const Level &lv = t->lev[z.l];
+    for (size_t i = 0; i < nl; ++i) {
+        const OzData::Lv &z = Z.lv[i];
+        const Level &lv = t->lev[z.l], &up = t->lev[z.l - 1];
+        const OzData::Op &x = z.op[op];
         OzLevel o{};
-        o.tile0 = tiles;
+        o.tile0 = op == OZ_M2L ? tiles : 0;
         o.ncl = (int32_t)(lv.ncol / 2);
         o.tpr = (o.ncl + tb - 1) / tb;
-        o.ncol = lv.ncol;
-        o.nrow = lv.nrow;
-        o.e0 = z.e0;
-        o.ents = (const RowEnt *)z.ents;
-        o.A = z.A;
-        o.B = z.B;
-        o.tmax = z.tmax;
-        o.mmax = t->oz.mmax + (size_t)LM_MAXV * v.size();
-        o.M = (const float4 *)lv.M;
-        o.L = (float4 *)lv.Lc;
+        o.tstep = op == OZ_M2M ? 1 : 2;
+        o.sstep = op == OZ_L2L ? 1 : 2;
+        o.add = op == OZ_L2L;
+        o.planes = (int32_t)(op == OZ_L2L ? up.nrow : 2 * lv.nrow);
+        o.ncol = op == OZ_M2M ? up.ncol : lv.ncol;
+        o.e0 = x.e0;
+        o.ents = (const RowEnt *)x.ents;
+        o.A = x.A;
+        o.tmax = x.tmax;
+        // level i's multipoles and their digits; the parents' local expansions take those of level i + 1
+        o.B = op == OZ_L2L ? (i + 1 < nl ? Z.lv[i + 1].B : Z.Btop) : z.B;
+        o.mmax = Z.mmax + (size_t)LM_MAXV * (op == OZ_L2L ? nl + i + 1 : i);
+        o.omax = op == OZ_M2M && i + 1 < nl ? Z.mmax + (size_t)LM_MAXV * (i + 1) : op == OZ_L2L ? Z.mmax + (size_t)LM_MAXV * (nl + i) : nullptr;
+        o.M = (const float4 *)(op == OZ_L2L ? up.Lc : lv.M);
+        o.L = (float4 *)(op == OZ_M2M ? up.M : lv.Lc);
         v.push_back(o);
         tiles += 2 * lv.nrow * o.tpr;
     }
     return v;
 }
 
+// split tables [ncls][np][np] of one contraction and its entry lists
+static lm_status oz_setup_op(lm_tree_s *t, const zd *tab, size_t ncls, const std::vector<RowEnt> &ents,
+                             const std::vector<int32_t> &e0, OzData::Op &x, cudaStream_t st)
+{
+    const int np = t->np, RA = oz_rows(np), KC = oz_chunks(np);
+    RowEnt *de;
+    TRY_O(lm_dalloc(t, &de, ents.size()));
+    x.ents = de;
+    TRY_O(lm_dalloc(t, &x.e0, e0.size()));
+    TRY_O(lm_dalloc(t, &x.A, ncls * OZ_S * KC * RA * 16));
+    TRY_O(lm_dalloc(t, &x.tmax, 2));
+    LM_CUDA(cudaMemcpyAsync(de, ents.data(), ents.size() * sizeof(RowEnt), cudaMemcpyHostToDevice, st));
+    LM_CUDA(cudaMemcpyAsync(x.e0, e0.data(), e0.size() * sizeof(int32_t), cudaMemcpyHostToDevice, st));
+    LM_CUDA(cudaMemsetAsync(x.tmax, 0, 2 * sizeof(uint32_t), st));
+    k_oz_tmax<<<(unsigned)ncls, 256, 0, st>>>(tab, np, x.tmax);
+    const int64_t nt = (int64_t)ncls * KC * RA;
+    k_oz_tsplit<<<(unsigned)((nt + 255) / 256), 256, 0, st>>>(tab, (int64_t)ncls, np, x.tmax, x.A);
+    LM_CUDA(cudaGetLastError());
+    return LM_OK;
+}
+
 lm_status lm_setup_oz(lm_tree_s *t, cudaStream_t st)
 {
     OzData &Z = t->oz;
-    const int np = t->np, RA = oz_rows(np), KC = oz_chunks(np);
+    const int KC = oz_chunks(t->np);
+    auto buf = [&](int64_t planes, int64_t ncl, unsigned char **B) { // every vector form shares the buffer
+        size_t bb = 0;
+        for (int s = 1; s <= LM_MAXV; s *= 2)
+            bb = std::max(bb, (size_t)(planes * OZ_S * KC) * oz_prow((int)ncl, OZ_N / s, s) * 16);
+        return lm_dalloc(t, B, bb);
+    };
     for (int l = t->L; l >= 1; --l) { // deepest (most tiles) first
         if (!lm_oz_level(t, l)) continue;
-        const Level &lv = t->lev[l];
+        const Level &lv = t->lev[l], &up = t->lev[l - 1];
         OzData::Lv z{};
         z.l = l;
         std::vector<RowEnt> ents;
         std::vector<int32_t> e0;
         TRY_O(lm_row_entries(lv, ents, e0));
-        const size_t ncls = std::max<size_t>(1, lv.cls_term.size());
-        RowEnt *de;
-        TRY_O(lm_dalloc(t, &de, ents.size()));
-        z.ents = de;
-        TRY_O(lm_dalloc(t, &z.e0, e0.size()));
-        TRY_O(lm_dalloc(t, &z.A, ncls * OZ_S * KC * RA * 16));
-        TRY_O(lm_dalloc(t, &z.tmax, 2));
-        size_t bb = 0; // every vector form shares the buffer
-        for (int s = 1; s <= LM_MAXV; s *= 2)
-            bb = std::max(bb, (size_t)(2 * lv.nrow * OZ_S * KC) * oz_prow((int)(lv.ncol / 2), OZ_N / s, s) * 16);
-        TRY_O(lm_dalloc(t, &z.B, bb));
-        Z.lv.push_back(z); // owned from here on
-        LM_CUDA(cudaMemcpyAsync(de, ents.data(), ents.size() * sizeof(RowEnt), cudaMemcpyHostToDevice, st));
-        LM_CUDA(cudaMemcpyAsync(z.e0, e0.data(), e0.size() * sizeof(int32_t), cudaMemcpyHostToDevice, st));
-        LM_CUDA(cudaMemsetAsync(z.tmax, 0, 2 * sizeof(uint32_t), st));
-        k_oz_tmax<<<(unsigned)ncls, 256, 0, st>>>(lv.tab, np, z.tmax);
-        const int64_t nt = (int64_t)ncls * KC * RA;
-        k_oz_tsplit<<<(unsigned)((nt + 255) / 256), 256, 0, st>>>(lv.tab, (int64_t)ncls, np, z.tmax, z.A);
-        LM_CUDA(cudaGetLastError());
-        LM_CUDA(cudaStreamSynchronize(st)); // host temporaries
+        TRY_O(oz_setup_op(t, lv.tab, std::max<size_t>(1, lv.cls_term.size()), ents, e0, z.op[OZ_M2L], st));
+        if (lv.nbox < OZ_MINSHIFT) {
+            TRY_O(buf(2 * lv.nrow, lv.ncol / 2, &z.B));
+            Z.lv.push_back(z);
+            continue;
+        }
+        // M2M: the children of a parent row, by position; L2L: one parent of a child
+        ents.clear();
+        e0.assign(1, 0);
+        for (int64_t r = 0; r < up.nrow; ++r) {
+            for (int pos = 0; pos < 4; ++pos) ents.push_back(RowEnt{pos, 0, (int32_t)(2 * (2 * r + (pos >> 1)) + (pos & 1)), 1});
+            e0.push_back((int32_t)ents.size());
+        }
+        TRY_O(oz_setup_op(t, up.m2m, 4, ents, e0, z.op[OZ_M2M], st));
+        ents.clear();
+        e0.assign(1, 0);
+        for (int64_t c = 0; c < 2 * lv.nrow; ++c) {
+            ents.push_back(RowEnt{(int32_t)((c >> 1 & 1) * 2 + (c & 1)), 0, (int32_t)(c >> 2), 1});
+            e0.push_back((int32_t)ents.size());
+        }
+        TRY_O(oz_setup_op(t, lv.l2l, 4, ents, e0, z.op[OZ_L2L], st));
+        TRY_O(buf(2 * lv.nrow, lv.ncol / 2, &z.B));
+        Z.lv.push_back(z);
+        Z.nshift = Z.lv.size();
     }
     if (Z.lv.empty()) return LM_OK;
-    TRY_O(lm_dalloc(t, &Z.mmax, Z.lv.size() * LM_MAXV));
+    const size_t nl = Z.lv.size();
+    const Level &top = t->lev[Z.lv.back().l - 1];
+    if (Z.nshift == nl) TRY_O(buf(top.nrow, top.ncol, &Z.Btop));
+    TRY_O(lm_dalloc(t, &Z.mmax, (2 * nl + 1) * LM_MAXV)); // multipoles of a level; local expansions, to the level above
     int f = 0;
     for (int s = 1; s <= 16; s *= 2, ++f) {
-        const std::vector<OzLevel> lv = oz_levels(t, s);
         OzLevel *d;
-        TRY_O(lm_dalloc(t, &d, lv.size()));
+        TRY_O(lm_dalloc(t, &d, 3 * nl));
         Z.desc[f] = d;
-        const OzLevel &e = lv.back();
-        Z.ntile[f] = e.tile0 + 2 * e.nrow * e.tpr;
-        LM_CUDA(cudaMemcpyAsync(d, lv.data(), lv.size() * sizeof(OzLevel), cudaMemcpyHostToDevice, st));
-        LM_CUDA(cudaStreamSynchronize(st));
+        for (int op = 0; op < 3; ++op) {
+            const std::vector<OzLevel> lv = oz_levels(t, op, s);
+            LM_CUDA(cudaMemcpyAsync(d + op * nl, lv.data(), nl * sizeof(OzLevel), cudaMemcpyHostToDevice, st));
+            if (op == OZ_M2L) Z.ntile[f] = lv.back().tile0 + 2 * t->lev[Z.lv.back().l].nrow * lv.back().tpr;
+        }
     }
     int dev = 0;
     LM_CUDA(cudaGetDevice(&dev));
@@ -543,21 +661,62 @@ lm_status lm_setup_oz(lm_tree_s *t, cudaStream_t st)
     return LM_OK;
 }
 
-// the M2L of the tensor-core levels (sets their L); returns the kernels launched
-lm_status lm_launch_m2l_oz(lm_tree_s *t, int nv, cudaStream_t st, int *launches)
+static int oz_form(int nv) { return nv <= 1 ? 0 : nv <= 2 ? 1 : nv <= 4 ? 2 : nv <= 8 ? 3 : 4; }
+// one contraction of tensor-core level i (M2M, L2L), its sources' digits first
+static int oz_step(lm_tree_s *t, int op, size_t i, bool mmax, int nv, cudaStream_t st)
 {
-    OzData &Z = t->oz;
+    const OzData &Z = t->oz;
+    const int f = oz_form(nv), nvs = 1 << f, tb = OZ_N / nvs;
+    const OzLevel *d = (const OzLevel *)Z.desc[f] + op * Z.lv.size() + i;
+    const Level &lv = t->lev[Z.lv[i].l];
+    const int64_t ncl = lv.ncol / 2, planes = op == OZ_L2L ? lv.nrow / 2 : 2 * lv.nrow;
+    const int64_t work = planes * oz_prow((int)ncl, tb, nvs) * oz_chunks(t->np);
+    if (mmax) k_oz_mmax<<<2 * (unsigned)Z.nsm, 256, 0, st>>>(d, t->np, nv);
+    k_oz_split<<<(unsigned)std::min<int64_t>(8 * Z.nsm, (work + 255) / 256), 256, 0, st>>>(d, t->np, nv, nvs);
+    const int64_t tiles = (op == OZ_M2M ? lv.nrow / 2 : 2 * lv.nrow) * ((ncl + tb - 1) / tb);
+    k_m2l_oz<<<(unsigned)std::min<int64_t>(Z.nsm, tiles), OZ_THREADS, OZ_SMEM, st>>>(d, 1, tiles, t->np, nv, nvs, t->dflag + 1);
+    return 2 + mmax;
+}
+
+// M2M from the levels of at least OZ_MINSHIFT boxes, whose multipoles' digits the M2L takes too; *lmin: the
+// level that it has reached
+lm_status lm_launch_m2m_oz(lm_tree_s *t, int nv, cudaStream_t st, int *lmin, int *launches)
+{
+    const OzData &Z = t->oz;
     *launches = 0;
+    *lmin = t->L;
     if (Z.lv.empty()) return LM_OK;
-    const int nvs = nv_slots(nv), f = nvs == 1 ? 0 : nvs == 2 ? 1 : nvs == 4 ? 2 : nvs == 8 ? 3 : 4, nl = (int)Z.lv.size();
-    const OzLevel *d = (const OzLevel *)Z.desc[f];
-    LM_CUDA(cudaMemsetAsync(Z.mmax, 0, Z.lv.size() * LM_MAXV * sizeof(uint32_t), st));
-    k_oz_mmax<<<dim3(2 * (unsigned)Z.nsm, nl), 256, 0, st>>>(d, t->np, nv);
-    k_oz_split<<<dim3(8 * (unsigned)Z.nsm, nl), 256, 0, st>>>(d, t->np, nv, nvs);
-    k_m2l_oz<<<(unsigned)std::min<int64_t>(Z.nsm, Z.ntile[f]), OZ_THREADS, OZ_SMEM, st>>>(d, nl, Z.ntile[f], t->np, nv, nvs,
-                                                                                           t->dflag + 1);
-    *launches = 3;
+    LM_CUDA(cudaMemsetAsync(Z.mmax, 0, (2 * Z.lv.size() + 1) * LM_MAXV * sizeof(uint32_t), st));
+    for (size_t i = 0; i < Z.nshift; ++i) *launches += oz_step(t, OZ_M2M, i, i == 0, nv, st);
+    *lmin = t->L - (int)Z.nshift;
+    LM_CUDA(cudaGetLastError());
+    return LM_OK;
+}
+bool lm_oz_shift(const lm_tree_s *t, int l) { return t->L - l < (int)t->oz.nshift; }
+// L2L to such a level l (adds to its L)
+lm_status lm_launch_l2l_oz(lm_tree_s *t, int l, int nv, cudaStream_t st, int *launches)
+{
+    const size_t i = (size_t)(t->L - l);
+    *launches = oz_step(t, OZ_L2L, i, i + 1 == t->oz.nshift, nv, st);
     LM_CUDA(cudaGetLastError());
     return LM_OK;
 }
 
+// the M2L of the tensor-core levels (sets their L; after their M2M); returns the kernels launched
+lm_status lm_launch_m2l_oz(lm_tree_s *t, int nv, cudaStream_t st, int *launches)
+{
+    const OzData &Z = t->oz;
+    *launches = 0;
+    if (Z.lv.empty()) return LM_OK;
+    const int f = oz_form(nv), nl = (int)Z.lv.size(), n0 = (int)Z.nshift;
+    const OzLevel *d = (const OzLevel *)Z.desc[f];
+    if (n0 < nl) { // the digits of the levels without M2M here
+        k_oz_mmax<<<dim3(2 * (unsigned)Z.nsm, nl - n0), 256, 0, st>>>(d + n0, t->np, nv);
+        k_oz_split<<<dim3(8 * (unsigned)Z.nsm, nl - n0), 256, 0, st>>>(d + n0, t->np, nv, 1 << f);
+    }
+    k_m2l_oz<<<(unsigned)std::min<int64_t>(Z.nsm, Z.ntile[f]), OZ_THREADS, OZ_SMEM, st>>>(
+        d, nl, Z.ntile[f], t->np, nv, 1 << f, t->dflag + 1);
+    *launches = n0 < nl ? 3 : 1;
+    LM_CUDA(cudaGetLastError());
+    return LM_OK;
+}

@@ -117,6 +117,15 @@ def test_digit_m2l_vector_forms_and_scales(lm, nvec):
     assert np.array_equal(ua[-1], _apply(lm, a, q[-1]))  # alone or among others: the same bits
 
 
+@pytest.mark.parametrize("p", [7, 20, 24, 32])
+@pytest.mark.parametrize("nvec", [1, 3, 8, 16])
+def test_digit_shifts(lm, p, nvec):
+    """M2M and L2L by digits on two levels (20480 and 5120 boxes, ragged tiles, most leaves empty)."""
+    x, y, q = workloads.uniform_strip(9001, 0.0, 4.9, -0.99, -0.01, nvec=nvec, seed=p)
+    a, b = (_tree(lm, A, x, y, p=p, depth=6, m2l_fp64=f) for f in (False, True))
+    assert _rel(_apply(lm, a, q), _apply(lm, b, q)) <= 1e-12
+
+
 FEW = {
     "one_point": (A, 1, 1.0, (-0.6, -0.4), dict(p=14)),
     "one_root": (A, 200, 0.9, (-0.95, -0.05), dict(p=16, depth=0)),
