@@ -9,23 +9,29 @@
 // replaces).  Levels of at least OZ_MINBOX boxes of uniform trees, their M2M and L2L
 // from OZ_MINSHIFT; the others run on the CUDA cores (lmfmm_exp_df.cu).
 //
-// A tile is 64 columns: 64 / nvs target boxes of one row and parity class, nvs vectors
+// A tile is 128 columns: 128 / nvs target boxes of one row and parity class, nvs vectors
 // each.  An interior box's V list depends only on its row and its column's parity, so
 // the tiles of a (row, parity) share one entry list (table slot, column offset dc, source
 // row).  A source outside the strip is a zero box: each row of split multipoles is padded.
-// One entry adds D_{i+j}[128 x 64] += A_i[128 x K] B_j[64 x K]^T over 15 digit pairs, with
-// A the real-block table ([Re -Im; Im Re], 2(2p+1) rows) and K = 2(2p+1) padded to 16.
+// One entry adds D_{i+j}[128 x R] += S_i[128 x K] T_j[R x K]^T over 15 digit pairs, with S
+// the sources, T the real-block table ([Re -Im; Im Re], rows 2 p + re / im) and
+// K = 2(2p+1) padded to 16.  R <= 96: five accumulators of R columns share the 512 columns
+// of tensor memory; orders with more rows take two sweeps.  (Tables as the 128-row operand
+// against 64 columns, 38 of whose rows are padding at p = 22, read 6 KB of shared memory an
+// MMA for half the columns: 250k strip, 16 vectors, M2L, M2M and L2L 5.85 ms, 3.07 ms
+// this way round.)
 //
 // Operands lie in global memory as [digit][8-wide K chunk][row][8 FP16]: 8 rows of a
 // chunk are a core matrix of the canonical K-major no-swizzle layout (stride 128 B between
 // 8-row groups), a stage of a table is one bulk copy, and any run of boxes one per digit and
-// chunk, whatever its offset.  Stages of up to 48 K (91 KB), two in flight.  Roles as in lmfmm_tc_tiles.cu:
+// chunk, whatever its offset.  Stages of up to 48 K (107 KB), two in flight.  Roles as in lmfmm_tc_tiles.cu:
 // a producer warp (a lane per copy), an MMA warp, 8 epilogue warps that read the 5
-// accumulators (320 columns of tensor memory) once per 4 entries: there is room for one
-// set of accumulators, so that reading them (about 50 FP32 instructions an element) and
-// the MMAs take turns.  250k strip, 16 vectors: 4.86 ms, 6.25 ms with a reading per entry.
-// Bound: 45 MMAs of 128 x 64 x 16 a stage, limited by the shared-memory reads of their
-// operands (6 KB a MMA at 128 B per clock).
+// accumulators once per 4 entries: there is room for one set of accumulators, so that
+// reading them (about 50 FP32 instructions an element) and the MMAs take turns (with a
+// reading per entry 6.25 ms where 4.86 ms).  A lane of an epilogue warp holds a column,
+// so that it writes whole components, neighbouring vectors beside each other.
+// Bound by the copies from L2 (215 KB an entry and 128 columns at p = 22) and the
+// shared-memory reads of the MMAs' operands (7 KB each at 128 B per clock).
 #include <algorithm>
 
 #include <cuda_fp16.h>
@@ -38,19 +44,19 @@
 
 #define OZ_S 5        // digits
 #define OZ_BITS 10
-#define OZ_N 64       // columns of a tile
+#define OZ_N 128      // columns of a tile
+#define OZ_RN 96      // most table rows of a sweep: 5 accumulators of OZ_RN columns in 512 of tensor memory
 #define OZ_KC 6       // 8-wide K chunks of a full stage
 #define OZ_NST 2
-#define OZ_A_BYTES (OZ_S * OZ_KC * 128 * 16) // RA <= 128 rows a chunk, packed; an MMA reads 128 from any chunk
-#define OZ_B_BYTES (OZ_S * OZ_KC * OZ_N * 16)
+#define OZ_A_BYTES (OZ_S * OZ_KC * OZ_N * 16)  // sources
+#define OZ_B_BYTES (OZ_S * OZ_KC * OZ_RN * 16) // tables
 #define OZ_STAGE (OZ_A_BYTES + OZ_B_BYTES)
 #define OZ_EPI 8
 #define OZ_THREADS ((OZ_EPI + 2) * 32)
-#define OZ_XROW 33 // floats of a row of an epilogue warp's exchange
-#define OZ_XCH (OZ_EPI * 32 * OZ_XROW * 4)
-#define OZ_SMEM (OZ_NST * OZ_STAGE + OZ_XCH + 128)
+#define OZ_SMEM (OZ_NST * OZ_STAGE + 128)
+
 // Smaller levels leave most SMs without a tile.  250k strip, 16 vectors: levels of up to 2047 boxes in
-// k_m2l_dx 2.67 ms, of up to 255 0.20 ms, this kernel 6.10 and 6.25 ms.
+// k_m2l_dx 2.67 ms, of up to 255 0.20 ms and 0.15 ms more here.
 #define OZ_MINBOX 256
 // M2M and L2L read and write a level for one or four entries a tile and split the sources in a launch
 // of their own.  250k strip, 16 vectors (levels of 20480 and 5120 boxes): 4.5 ms on the CUDA cores,
@@ -85,7 +91,9 @@ __device__ __forceinline__ int oz_exp(uint32_t bits) { return bits ? (int)((bits
 // digits' sum over K and OZ_GRP = 4 entries stays below 2^24 (|digit| <= 512 on either side)
 __device__ __forceinline__ int oz_ea(const uint32_t *t) { return max(oz_exp(t[0]) + 2, oz_exp(t[1]) - 1); }
 __device__ __forceinline__ float oz_pow2(int e) { return __int_as_float((max(-126, min(127, e)) + 127) << 23); }
-__host__ __device__ __forceinline__ int oz_rows(int np) { return (2 * np + 7) / 8 * 8; }
+// table rows (2 p + re / im) in sweeps of oz_rows(np), a multiple of 16, at most OZ_RN
+__host__ __device__ __forceinline__ int oz_sweeps(int np) { return 2 * np <= OZ_RN ? 1 : 2; }
+__host__ __device__ __forceinline__ int oz_rows(int np) { return (2 * np / oz_sweeps(np) + 15) / 16 * 16; }
 __host__ __device__ __forceinline__ int oz_chunks(int np) { return (2 * np + 15) / 16 * 2; }
 __host__ __device__ __forceinline__ int64_t oz_prow(int ncl, int tb, int nvs) { return (int64_t)(OZ_PADL + ncl + tb + 2) * nvs; }
 
@@ -112,11 +120,12 @@ __global__ void __launch_bounds__(256) k_oz_tmax(const zd *tab, int np, uint32_t
 __global__ void __launch_bounds__(256) k_oz_tsplit(const zd *tab, int64_t ncls, int np, const uint32_t *tmax,
                                                    unsigned char *A)
 {
-    const int RA = oz_rows(np), KC = oz_chunks(np);
+    const int RN = oz_rows(np), ns = oz_sweeps(np), KC = oz_chunks(np);
     const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (idx >= ncls * KC * RA) return;
-    const int row = (int)(idx % RA), c = (int)(idx / RA % KC);
-    const int64_t cls = idx / ((int64_t)RA * KC);
+    if (idx >= ncls * ns * KC * RN) return;
+    const int lrow = (int)(idx % RN), c = (int)(idx / RN % KC);
+    const int64_t cs = idx / ((int64_t)RN * KC), cls = cs / ns;
+    const int row = (int)(cs % ns) * RN + lrow, p = row >> 1, im = row & 1;
     const zd *T = tab + cls * np * np;
     const double sc = ldexp(1.0, -oz_ea(tmax));
     uint16_t d[OZ_S][8];
@@ -124,9 +133,8 @@ __global__ void __launch_bounds__(256) k_oz_tsplit(const zd *tab, int64_t ncls, 
         const int k = 8 * c + i;
         double x = 0.0;
         if (row < 2 * np && k < 2 * np) {
-            const int p = row < np ? row : row - np, q = k < np ? k : k - np;
-            const zd a = T[p * np + q];
-            x = ((row < np) == (k < np)) ? a.re : (row < np ? -a.im : a.im);
+            const zd a = T[p * np + (k < np ? k : k - np)];
+            x = (im != 0) == (k >= np) ? a.re : (im ? a.im : -a.im);
         }
         x *= sc;
         for (int s = 0; s < OZ_S; ++s) {
@@ -138,9 +146,9 @@ __global__ void __launch_bounds__(256) k_oz_tsplit(const zd *tab, int64_t ncls, 
     }
     // stage-major: [stage of OZ_KC chunks][digit][chunk][row]
     const int st = c / OZ_KC, c0 = st * OZ_KC, kc = min(OZ_KC, KC - c0);
-    unsigned char *o = A + (cls * OZ_S * KC + (int64_t)OZ_S * c0) * RA * 16;
+    unsigned char *o = A + (cs * OZ_S * KC + (int64_t)OZ_S * c0) * RN * 16;
     for (int s = 0; s < OZ_S; ++s)
-        *(uint4 *)(o + ((int64_t)(s * kc + c - c0) * RA + row) * 16) = *(const uint4 *)d[s];
+        *(uint4 *)(o + ((int64_t)(s * kc + c - c0) * RN + lrow) * 16) = *(const uint4 *)d[s];
 }
 
 // largest component of each vector over a level's sources
@@ -223,32 +231,33 @@ __device__ __forceinline__ void oz_mma(uint32_t dtmem, uint64_t ad, uint64_t bd,
                  "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(dtmem),
                  "l"(ad), "l"(bd), "r"(idesc), "r"(acc));
 }
-// 16 columns of each of the 5 accumulators, one wait
-__device__ __forceinline__ void oz_ld16x5(uint32_t t0, float d[OZ_S][16])
+// 8 columns of each of the 5 accumulators (nc columns apart), one wait
+__device__ __forceinline__ void oz_ld8x5(uint32_t t0, uint32_t nc, float d[OZ_S][8])
 {
-    uint32_t r[OZ_S][16];
+    uint32_t r[OZ_S][8];
 #pragma unroll
     for (int k = 0; k < OZ_S; ++k)
-        asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, "
-                     "%12, %13, %14, %15}, [%16];"
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                      : "=r"(r[k][0]), "=r"(r[k][1]), "=r"(r[k][2]), "=r"(r[k][3]), "=r"(r[k][4]), "=r"(r[k][5]),
-                       "=r"(r[k][6]), "=r"(r[k][7]), "=r"(r[k][8]), "=r"(r[k][9]), "=r"(r[k][10]), "=r"(r[k][11]),
-                       "=r"(r[k][12]), "=r"(r[k][13]), "=r"(r[k][14]), "=r"(r[k][15])
-                     : "r"(t0 + (uint32_t)(OZ_N * k)));
+                       "=r"(r[k][6]), "=r"(r[k][7])
+                     : "r"(t0 + nc * k));
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
     for (int k = 0; k < OZ_S; ++k)
 #pragma unroll
-        for (int i = 0; i < 16; ++i) d[k][i] = __uint_as_float(r[k][i]);
+        for (int i = 0; i < 8; ++i) d[k][i] = __uint_as_float(r[k][i]);
 }
-// tile -> level, class, first box of the class
-__device__ __forceinline__ const OzLevel &oz_tile(const OzLevel *lvs, int nlev, int64_t tile, int *cls, int *i0, int tb)
+// tile -> level, class, first box of the class, sweep
+__device__ __forceinline__ const OzLevel &oz_tile(const OzLevel *lvs, int nlev, int64_t tile, int ns, int *cls, int *i0, int *sw,
+                                                  int tb)
 {
     int l = nlev - 1;
     while (tile < lvs[l].tile0) --l;
     const int64_t r = tile - lvs[l].tile0;
+    const int x = (int)(r % lvs[l].tpr);
     *cls = (int)(r / lvs[l].tpr);
-    *i0 = (int)(r % lvs[l].tpr) * tb;
+    *i0 = x / ns * tb;
+    *sw = x % ns;
     return lvs[l];
 }
 __device__ __forceinline__ void oz_fail(volatile int *abort_s, int *err)
@@ -261,13 +270,13 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_m2l_oz(const OzLevel *lvs, in
                                                           int *err)
 {
     extern __shared__ __align__(1024) unsigned char smem[];
-    uint64_t *bars = (uint64_t *)(smem + OZ_NST * OZ_STAGE + OZ_XCH);
+    uint64_t *bars = (uint64_t *)(smem + OZ_NST * OZ_STAGE);
     uint32_t *tslot = (uint32_t *)(bars + 2 * OZ_NST + 2);
     volatile int *abort_s = (volatile int *)(tslot + 1);
     const uint32_t sbase = smem_u32(smem), bfull = smem_u32(bars), bempty = bfull + 8 * OZ_NST, btfull = bfull + 16 * OZ_NST,
                    btempty = btfull + 8;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int KC = oz_chunks(np), RA = oz_rows(np), nst = (KC + OZ_KC - 1) / OZ_KC, tb = OZ_N / nvs;
+    const int KC = oz_chunks(np), RN = oz_rows(np), ns = oz_sweeps(np), nst = (KC + OZ_KC - 1) / OZ_KC, tb = OZ_N / nvs;
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < OZ_NST; ++i) {
@@ -297,8 +306,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_m2l_oz(const OzLevel *lvs, in
         for (int s = 0; s < OZ_NST; ++s) last[s] = -1;
         bool stop = false;
         for (int64_t tile = blockIdx.x; tile < ntiles && !stop; tile += gridDim.x) {
-            int cls, i0;
-            const OzLevel &lv = oz_tile(lvs, nlev, tile, &cls, &i0, tb);
+            int cls, i0, sw;
+            const OzLevel &lv = oz_tile(lvs, nlev, tile, ns, &cls, &i0, &sw, tb);
             const int e0 = lv.e0[cls], e1 = lv.e0[cls + 1], c0 = 2 * i0 + (cls & 1);
             const int64_t rows = oz_prow(lv.ncl, tb, nvs);
             for (int base = e0; base < e1 && !stop; base += 32) {
@@ -310,14 +319,14 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_m2l_oz(const OzLevel *lvs, in
                     const int cs = c0 - dc, par = cs & 1;
                     const int64_t plane = direct ? rs : (int64_t)rs * 2 + par;
                     const int64_t sbox = (direct ? i0 : (cs - par) >> 1) + OZ_PADL; // first source in its padded plane
-                    const unsigned char *a = lv.A + (int64_t)slot * OZ_S * KC * RA * 16;
+                    const unsigned char *a = lv.A + ((int64_t)slot * ns + sw) * OZ_S * KC * RN * 16;
                     const unsigned char *b = lv.B + plane * OZ_S * KC * rows * 16 + sbox * nvs * 16;
                     for (int st = 0; st < nst; ++st, ++it) {
                         const int s = (int)(it % OZ_NST), k0 = st * OZ_KC, kc = min(OZ_KC, KC - k0);
                         int ok = 1;
                         if (lane == 0) {
                             ok = mbar_wait_lim(bempty + 8 * s, ((it / OZ_NST) & 1) ^ 1, TC_WAIT_LIMIT, abort_s, err);
-                            if (ok) mbar_expect_tx(bfull + 8 * s, OZ_S * kc * (RA + OZ_N) * 16);
+                            if (ok) mbar_expect_tx(bfull + 8 * s, OZ_S * kc * (RN + OZ_N) * 16);
                             else oz_fail(abort_s, err);
                         }
                         ok = __shfl_sync(0xffffffffu, ok, 0);
@@ -327,10 +336,10 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_m2l_oz(const OzLevel *lvs, in
                         }
                         const uint32_t sa = sbase + s * OZ_STAGE, sb = sa + OZ_A_BYTES, fb = bfull + 8 * s;
                         if (lane == 31) // the stage's tables are contiguous
-                            bulk_g2s(sa, a + (int64_t)OZ_S * k0 * RA * 16, OZ_S * kc * RA * 16, fb);
+                            bulk_g2s(sb, a + (int64_t)OZ_S * k0 * RN * 16, OZ_S * kc * RN * 16, fb);
                         if (lane < OZ_S * kc) {
                             const int dg = lane / kc, c = lane - dg * kc;
-                            bulk_g2s(sb + (dg * OZ_KC + c) * OZ_N * 16, b + ((int64_t)dg * KC + k0 + c) * rows * 16, OZ_N * 16, fb);
+                            bulk_g2s(sa + (dg * OZ_KC + c) * OZ_N * 16, b + ((int64_t)dg * KC + k0 + c) * rows * 16, OZ_N * 16, fb);
                         }
                         last[s] = (int)it;
                         __syncwarp();
@@ -346,13 +355,13 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_m2l_oz(const OzLevel *lvs, in
     } else if (warp == OZ_EPI + 1) {
         // ---- MMA issuer ----
         if (lane == 0) {
-            const uint32_t idesc = (1u << 4) | ((uint32_t)(OZ_N >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+            const uint32_t idesc = (1u << 4) | ((uint32_t)(RN >> 3) << 17) | ((uint32_t)(OZ_N >> 4) << 24);
             uint32_t it = 0, item = 0;
             int done = -1;
             bool stop = false;
             for (int64_t tile = blockIdx.x; tile < ntiles && !stop && !*abort_s; tile += gridDim.x) {
-                int cls, i0;
-                const OzLevel &lv = oz_tile(lvs, nlev, tile, &cls, &i0, tb);
+                int cls, i0, sw;
+                const OzLevel &lv = oz_tile(lvs, nlev, tile, ns, &cls, &i0, &sw, tb);
                 const int ne = lv.e0[cls + 1] - lv.e0[cls];
                 for (int e = 0; e < ne && !stop; e += OZ_GRP, ++item) {
                     if (!mbar_wait_lim(btempty, (item & 1) ^ 1, TC_WAIT_LIMIT, abort_s, err)) {
@@ -377,8 +386,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_m2l_oz(const OzLevel *lvs, in
                             for (int i = 0; i < OZ_S; ++i)
 #pragma unroll
                                 for (int j = 0; i + j < OZ_S; ++j)
-                                    oz_mma(tmem + OZ_N * (i + j), oz_desc(sa + (i * kc + 2 * kk) * RA * 16, RA * 16),
-                                           oz_desc(sb + (j * OZ_KC + 2 * kk) * OZ_N * 16, OZ_N * 16), idesc,
+                                    oz_mma(tmem + RN * (i + j), oz_desc(sa + (i * OZ_KC + 2 * kk) * OZ_N * 16, OZ_N * 16),
+                                           oz_desc(sb + (j * kc + 2 * kk) * RN * 16, RN * 16), idesc,
                                            (q > 0 || kk > 0 || i > 0) ? 1u : 0u);
                         tc_commit(bempty + 8 * s);
                         ++issued;
@@ -394,19 +403,18 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_m2l_oz(const OzLevel *lvs, in
         }
         __syncwarp();
     } else {
-        // ---- epilogue: warp (quadrant Q, half H): accumulator rows 32 Q .. + 31, columns 32 H .. + 31 ----
-        const int Q = warp & 3, H = warp >> 2, row = 32 * Q + lane;
-        const bool live = 32 * Q < 2 * np;
-        const uint32_t base = tmem + ((uint32_t)(32 * Q) << 16) + 32u * H;
+        // ---- epilogue: warp (quadrant Q, half H): tile columns 32 Q .. + 31, one a lane, half the sweep's rows ----
+        const int Q = warp & 3, H = warp >> 2, col = 32 * Q + lane, nr = RN / 2, j = col / nvs, v = col - j * nvs;
+        const uint32_t base = tmem + ((uint32_t)(32 * Q) << 16) + (uint32_t)(nr * H);
         uint32_t item = 0;
         bool bad = false;
         for (int64_t tile = blockIdx.x; tile < ntiles && !bad; tile += gridDim.x) {
-            int cls, i0;
-            const OzLevel &lv = oz_tile(lvs, nlev, tile, &cls, &i0, tb);
+            int cls, i0, sw;
+            const OzLevel &lv = oz_tile(lvs, nlev, tile, ns, &cls, &i0, &sw, tb);
             const int ne = lv.e0[cls + 1] - lv.e0[cls];
-            df acc[32];
+            df acc[OZ_RN / 2];
 #pragma unroll
-            for (int c = 0; c < 32; ++c) acc[c] = df{0.f, 0.f};
+            for (int r = 0; r < OZ_RN / 2; ++r) acc[r] = df{0.f, 0.f};
             for (int e = 0; e < ne; e += OZ_GRP, ++item) {
                 if (!mbar_wait_lim(btfull, item & 1, TC_WAIT_LIMIT, abort_s, err)) {
                     oz_fail(abort_s, err);
@@ -414,103 +422,55 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_m2l_oz(const OzLevel *lvs, in
                     break;
                 }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                if (live) {
 #pragma unroll
-                    for (int hf = 0; hf < 2; ++hf) {
-                        float d[OZ_S][16];
-                        oz_ld16x5(base + 16u * hf, d);
-                        if (hf == 1) {
-                            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                            __syncwarp();
-                            if (lane == 0) mbar_arrive(btempty);
-                        }
-#pragma unroll
-                        for (int c = 0; c < 16; ++c) { // integers of weight 2^{-10 k}
-                            const df s = two_sum(d[0][c], d[1][c] * 0x1p-10f);
-                            const df u = two_sum(d[2][c] * 0x1p-20f, fmaf(d[4][c], 0x1p-40f, d[3][c] * 0x1p-30f));
-                            acc[16 * hf + c] = df_add(acc[16 * hf + c], df_add(s, u));
-                        }
+                for (int r8 = 0; r8 < OZ_RN / 2; r8 += 8) {
+                    if (r8 >= nr) break;
+                    float d[OZ_S][8];
+                    oz_ld8x5(base + r8, RN, d);
+                    if (r8 + 8 == nr) {
+                        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(btempty);
                     }
-                } else {
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(btempty);
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) { // integers of weight 2^{-10 k}
+                        const df s = two_sum(d[0][c], d[1][c] * 0x1p-10f);
+                        const df u = two_sum(d[2][c] * 0x1p-20f, fmaf(d[4][c], 0x1p-40f, d[3][c] * 0x1p-30f));
+                        acc[r8 + c] = df_add(acc[r8 + c], df_add(s, u));
+                    }
                 }
             }
             if (bad) break;
-            const int64_t r0 = lv.tstep == 2 ? (int64_t)(cls >> 1) * lv.ncol + (cls & 1) : cls * lv.ncol;
-            const int ea = oz_ea(lv.tmax);
-            float omx = 0.f; // largest result of column 32 H + lane
-            // where result (row, column) goes, and its scale 2^x
-            auto out = [&](int rw, int col, int *x) -> float2 * {
-                const int j = col / nvs, v = col - j * nvs, p = rw < np ? rw : rw - np;
-                if (rw >= 2 * np || i0 + j >= lv.ncl || v >= nv) return nullptr;
-                *x = ea + oz_exp(lv.mmax[v]) + 2 - 2 * OZ_BITS;
-                return (float2 *)&lv.L[((r0 + lv.tstep * (int64_t)(i0 + j)) * np + p) * nv + v] + (rw < np ? 0 : 1);
-            };
-            if (nvs >= 8) {
-                // a lane takes a column: neighbouring vectors are neighbours in memory
-                float *xc = (float *)(smem + OZ_NST * OZ_STAGE) + warp * 32 * OZ_XROW;
-                float h[32];
-                __syncwarp();
+            if (i0 + j < lv.ncl && v < nv) {
+                const int64_t r0 = lv.tstep == 2 ? (int64_t)(cls >> 1) * lv.ncol + (cls & 1) : cls * lv.ncol;
+                const int x = oz_ea(lv.tmax) + oz_exp(lv.mmax[v]) + 2 - 2 * OZ_BITS, p0 = (sw * RN + H * nr) / 2;
+                const float f = oz_pow2(x / 2), g = oz_pow2(x - x / 2);
+                float4 *o = lv.L + ((r0 + lv.tstep * (int64_t)(i0 + j)) * np + p0) * nv + v;
+                float omx = 0.f;
 #pragma unroll
-                for (int c = 0; c < 32; ++c) xc[lane * OZ_XROW + c] = acc[c].h;
-                __syncwarp();
+                for (int r8 = 0; r8 < OZ_RN / 2; r8 += 8) {
+                    if (r8 >= nr) break;
+                    float4 b[4];
 #pragma unroll
-                for (int r = 0; r < 32; ++r) h[r] = xc[r * OZ_XROW + lane];
-                __syncwarp();
+                    for (int c = 0; c < 4; ++c)
+                        b[c] = lv.add && p0 + r8 / 2 + c < np ? o[(int64_t)(r8 / 2 + c) * nv] : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-                for (int c = 0; c < 32; ++c) xc[lane * OZ_XROW + c] = acc[c].l;
-                __syncwarp();
-#pragma unroll
-                for (int r8 = 0; r8 < 32; r8 += 8) {
-                    float2 *o[8], b[8];
-                    int x = 0;
-#pragma unroll
-                    for (int r = 0; r < 8; ++r) {
-                        o[r] = out(32 * Q + r8 + r, 32 * H + lane, &x);
-                        b[r] = lv.add && o[r] ? *o[r] : make_float2(0.f, 0.f);
-                    }
-                    const float f = oz_pow2(x / 2), g = oz_pow2(x - x / 2);
-#pragma unroll
-                    for (int r = 0; r < 8; ++r)
-                        if (o[r]) {
-                            df y = {h[r8 + r] * f * g, xc[(r8 + r) * OZ_XROW + lane] * f * g};
-                            if (lv.add) y = df_add(df{b[r].x, b[r].y}, y);
-                            *o[r] = make_float2(y.h, y.l);
-                            omx = fmaxf(omx, fabsf(y.h));
+                    for (int c = 0; c < 4; ++c)
+                        if (p0 + r8 / 2 + c < np) {
+                            const df a = acc[r8 + 2 * c], i = acc[r8 + 2 * c + 1];
+                            df yr = {a.h * f * g, a.l * f * g}, yi = {i.h * f * g, i.l * f * g};
+                            if (lv.add) {
+                                yr = df_add(df{b[c].x, b[c].y}, yr);
+                                yi = df_add(df{b[c].z, b[c].w}, yi);
+                            }
+                            o[(int64_t)(r8 / 2 + c) * nv] = make_float4(yr.h, yr.l, yi.h, yi.l);
+                            omx = fmaxf(omx, fmaxf(fabsf(yr.h), fabsf(yi.h)));
                         }
                 }
-            } else {
-                // a lane takes a row: with few vectors, neighbouring orders are near in memory
-#pragma unroll
-                for (int c8 = 0; c8 < 32; c8 += 8) {
-                    float2 *o[8], b[8];
-                    int x[8];
-#pragma unroll
-                    for (int c = 0; c < 8; ++c) {
-                        o[c] = out(row, 32 * H + c8 + c, &x[c]);
-                        b[c] = lv.add && o[c] ? *o[c] : make_float2(0.f, 0.f);
-                    }
-#pragma unroll
-                    for (int c = 0; c < 8; ++c) {
-                        float m = 0.f;
-                        if (o[c]) {
-                            const float f = oz_pow2(x[c] / 2), g = oz_pow2(x[c] - x[c] / 2);
-                            df y = {acc[c8 + c].h * f * g, acc[c8 + c].l * f * g};
-                            if (lv.add) y = df_add(df{b[c].x, b[c].y}, y);
-                            *o[c] = make_float2(y.h, y.l);
-                            m = fabsf(y.h);
-                        }
-                        if (lv.omax) {
-                            const float w = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(m)));
-                            if (lane == c8 + c) omx = w;
-                        }
-                    }
+                if (lv.omax) {
+                    const uint32_t m = __float_as_uint(omx);
+                    if (m > *(volatile uint32_t *)&lv.omax[v]) atomicMax(&lv.omax[v], m);
                 }
-            }
-            if (lv.omax) {
-                uint32_t *o = lv.omax + (32 * H + lane) % nvs;
-                if (__float_as_uint(omx) > *(volatile uint32_t *)o) atomicMax(o, __float_as_uint(omx));
             }
         }
     }
@@ -552,7 +512,7 @@ static std::vector<OzLevel> oz_levels(const lm_tree_s *t, int op, int nvs)
         OzLevel o{};
         o.tile0 = op == OZ_M2L ? tiles : 0;
         o.ncl = (int32_t)(lv.ncol / 2);
-        o.tpr = (o.ncl + tb - 1) / tb;
+        o.tpr = (o.ncl + tb - 1) / tb * oz_sweeps(t->np);
         o.tstep = op == OZ_M2M ? 1 : 2;
         o.sstep = op == OZ_L2L ? 1 : 2;
         o.add = op == OZ_L2L;
@@ -578,18 +538,18 @@ static std::vector<OzLevel> oz_levels(const lm_tree_s *t, int op, int nvs)
 static lm_status oz_setup_op(lm_tree_s *t, const zd *tab, size_t ncls, const std::vector<RowEnt> &ents,
                              const std::vector<int32_t> &e0, OzData::Op &x, cudaStream_t st)
 {
-    const int np = t->np, RA = oz_rows(np), KC = oz_chunks(np);
+    const int np = t->np, rows = oz_rows(np) * oz_sweeps(np), KC = oz_chunks(np);
     RowEnt *de;
     TRY_O(lm_dalloc(t, &de, ents.size()));
     x.ents = de;
     TRY_O(lm_dalloc(t, &x.e0, e0.size()));
-    TRY_O(lm_dalloc(t, &x.A, ncls * OZ_S * KC * RA * 16));
+    TRY_O(lm_dalloc(t, &x.A, ncls * OZ_S * KC * rows * 16));
     TRY_O(lm_dalloc(t, &x.tmax, 2));
     LM_CUDA(cudaMemcpyAsync(de, ents.data(), ents.size() * sizeof(RowEnt), cudaMemcpyHostToDevice, st));
     LM_CUDA(cudaMemcpyAsync(x.e0, e0.data(), e0.size() * sizeof(int32_t), cudaMemcpyHostToDevice, st));
     LM_CUDA(cudaMemsetAsync(x.tmax, 0, 2 * sizeof(uint32_t), st));
     k_oz_tmax<<<(unsigned)ncls, 256, 0, st>>>(tab, np, x.tmax);
-    const int64_t nt = (int64_t)ncls * KC * RA;
+    const int64_t nt = (int64_t)ncls * KC * rows;
     k_oz_tsplit<<<(unsigned)((nt + 255) / 256), 256, 0, st>>>(tab, (int64_t)ncls, np, x.tmax, x.A);
     LM_CUDA(cudaGetLastError());
     return LM_OK;
@@ -673,7 +633,7 @@ static int oz_step(lm_tree_s *t, int op, size_t i, bool mmax, int nv, cudaStream
     const int64_t work = planes * oz_prow((int)ncl, tb, nvs) * oz_chunks(t->np);
     if (mmax) k_oz_mmax<<<2 * (unsigned)Z.nsm, 256, 0, st>>>(d, t->np, nv);
     k_oz_split<<<(unsigned)std::min<int64_t>(8 * Z.nsm, (work + 255) / 256), 256, 0, st>>>(d, t->np, nv, nvs);
-    const int64_t tiles = (op == OZ_M2M ? lv.nrow / 2 : 2 * lv.nrow) * ((ncl + tb - 1) / tb);
+    const int64_t tiles = (op == OZ_M2M ? lv.nrow / 2 : 2 * lv.nrow) * ((ncl + tb - 1) / tb) * oz_sweeps(t->np);
     k_m2l_oz<<<(unsigned)std::min<int64_t>(Z.nsm, tiles), OZ_THREADS, OZ_SMEM, st>>>(d, 1, tiles, t->np, nv, nvs, t->dflag + 1);
     return 2 + mmax;
 }
