@@ -282,7 +282,9 @@ struct lm_tree_s {
     bool lf_ready;
     void *lf_pts;               // [n] float4 (x, y relative to the leaf centre, absolute y, 0)
     int32_t *lf_tot;            // [nleaf] U-list source points per leaf
-    void *lf_ent;               // [nleaf][32] int4 (first point, points, U term, source leaf) per U entry
+    void *lf_ent;               // [nleaf][32] int4 (first point, points, first slot, 0) per U entry
+    int64_t lf_nchunk, *lf_cbase; // chunks of 64 U-list sources of all leaves with points; first of each leaf
+    void *lf_src;               // [lf_nchunk][64] float4 records of the sources (k_lf_src)
     uint32_t *lf_scl;           // [2] largest |component| of the apply's densities and leaf-level local
                                 // expansions (float bits), for the FP16 scales
     int lf_grid;                // persistent CTAs (one per SM)

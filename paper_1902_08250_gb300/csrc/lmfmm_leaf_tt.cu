@@ -23,19 +23,18 @@
 // are the expensive part) and no thread multiplies over the vectors.
 //
 // Roles (16 warps, one CTA per SM, persistent over the leaves):
-//   warp 0     producer: tables the leaf's flattened U-list sources once per
-//              leaf; per chunk its lanes write each source's record (offset of
-//              the source leaf, point, U term), and the lane at the start of
-//              each run of consecutive points bulk-copies the run's densities
-//              (rows of 128 B) and coordinates (rows of 16 B), or lane 0 the
-//              leaf's local expansion;
+//   warp 0     producer: per chunk, bulk copies of the sources' records (one run,
+//              laid out with the tree), of each U entry's part of the densities
+//              (rows of 128 B, a lane per entry), with a pass's first chunk of its
+//              target rows; or of the leaf's local expansion;
 //   warps 1, 3 converters: split a stage's densities into the B operand
 //              (canonical K-major layout, hi/lo parts, real-block signs), 8
-//              vectors each; warp 1 also turns the records into coordinates;
+//              vectors each;
 //   warp 2     MMA issuer, owner of the tensor memory;
-//   warps 4-11 kernel values: warp 4 + g evaluates G for target slots
-//              32 (g & 1) .. + 31 and the chunk's sources 16 (g >> 1) .. + 15 and
-//              stores their hi and lo rows of A;
+//   warps 4-11 kernel values: items of 8 targets x 16 sources in turn, a lane per
+//              target and 4 sources, stored as hi and lo rows of A (a lane per
+//              target would leave a quarter of the lanes of leaves of 49 points
+//              idle, this leaves 7 %);
 //   warps 12-15 epilogue: warp 12 + Q reads tensor-memory lanes 32 Q .. + 31 of
 //              each chunk's accumulator; at the end of a pass the lo-part rows
 //              meet their hi-part rows in shared memory and the potentials are
@@ -61,27 +60,17 @@
 #define LF_NA 2                           // A buffers
 #define LF_ND 4                           // accumulators (64 tensor-memory columns each)
 #define LF_GW 8                           // kernel-value warps
-#define LF_JS 16                          // sources (order slots) per kernel-value thread and chunk
-#define LF_RB 4                           // of which one round of evaluations takes LF_RB
+#define LF_RB 4                           // sources (order slots) of a kernel-value thread's round
 #define LF_EPI0 (4 + LF_GW)               // first epilogue warp (a multiple of 4)
 #define LF_THREADS ((LF_EPI0 + 4) * 32)
 #define LF_MAXE 32                        // U entries of a leaf (one per producer lane)
 #define LF_A_BYTES (128 * LF_K * 2)       // 32 KB: FP16
 #define LF_B_BYTES (64 * LF_K * 2)        // 16 KB
 #define LF_GSCALE 1024.0f                 // kernel values enter A multiplied by 2^10
-#define LF_Q_BYTES (LF_CH * LM_MAXV * 8)  // 8 KB: rows of 16 complex densities
-#define LF_RAW_BYTES (LF_Q_BYTES + LF_CH * 16) // + coordinate rows (x, y local; y absolute; 0)
-#define LF_XS 33                          // floats per target row of the exchange buffer
-
-// one stage's sources as the kernel-value warps read them, one 16-byte record each:
-// (x, y relative to the target leaf's centre, absolute y, code = point << 2 | U term;
-// an empty slot has point -1).  The producer writes the offsets centre_t - centre_s
-// into x, y and the converter turns them into coordinates.
-struct LfMeta {
-    float4 src[LF_CH];
-    int32_t n, pad[3]; // sources in the chunk (orders in the L2T chunk)
-};
-#define LF_MAXT 1024 // flattened U-list sources of a leaf tabled by the producer
+#define LF_RAW_BYTES (LF_CH * LM_MAXV * 8) // 8 KB: rows of 16 complex densities
+#define LF_META_BYTES (LF_CH * 16)         // 1 KB: records of the chunk's sources
+#define LF_NT 4                            // target-row buffers (a pass's is free 3 passes later)
+#define LF_XS 33                           // floats per target row of the exchange buffer
 
 template <int P>
 struct LfSmem {
@@ -89,10 +78,9 @@ struct LfSmem {
     static constexpr int B_OFF = A_OFF + LF_NA * LF_A_BYTES;
     static constexpr int RAW_OFF = B_OFF + LF_NS * LF_B_BYTES;
     static constexpr int META_OFF = RAW_OFF + LF_NS * LF_RAW_BYTES;
-    static constexpr int XCH_OFF = META_OFF + LF_NS * (int)sizeof(LfMeta);
-    static constexpr int ETAB_OFF = XCH_OFF + 2 * LF_TGT * LF_XS * 4;
-    static constexpr int TAB_OFF = ETAB_OFF + 6 * (LF_MAXE + 1) * 4;
-    static constexpr int BAR_OFF = (TAB_OFF + LF_MAXT * 5 + 7) / 8 * 8;
+    static constexpr int TGT_OFF = META_OFF + LF_NS * LF_META_BYTES;
+    static constexpr int XCH_OFF = TGT_OFF + LF_NT * LF_TGT * 16;
+    static constexpr int BAR_OFF = (XCH_OFF + 2 * LF_TGT * LF_XS * 4 + 7) / 8 * 8;
     static constexpr int NBAR = 3 * LF_NS + 2 * LF_NA + 2 * LF_ND;
     static constexpr int BYTES = BAR_OFF + NBAR * 8 + 16;
 };
@@ -203,32 +191,30 @@ __device__ __forceinline__ zf lf_h0s(float t)
     return zf{fmaf(wc, im, sh), im};
 }
 
-// L2T basis of the order slots E .. E + NS - 1 (slot P + n <-> order n) for a target at
-// (x, y) relative to its leaf centre, zeta = (x + i y) / w, t = (k r / 2)^2:
-//   n >= 0: s_n(t) zeta^n,   n < 0: (-1)^|n| s_|n|(t) conj(zeta)^|n|,
+// L2T basis of the orders n = 0 .. P for a target at (x, y) relative to its leaf centre,
+// zeta = (x + i y) / w, t = (k r / 2)^2:  v_n = s_n(t) zeta^n (order -n: (-1)^n conj(v_n)),
 // s_m(t) = sum_j (-t)^j m! / (j! (j + m)!) = J_m(k r) / ((k r / 2)^m / m!), the scaled
-// Bessel function of the local expansion (Eq. (local)), from its ascending series
-// (A&S 9.1.10) by Horner's rule to j = 8 (first dropped term < 2e-14 for t <= 1/2).
-template <int P, int E, int NS>
-__device__ __forceinline__ void lf_basis(float xs, float ys, float t, zf *gv)
+// Bessel function of the local expansion (Eq. (local)).  s_P and s_{P-1} from the ascending
+// series (A&S 9.1.10) by Horner's rule to j = 8 (first dropped term < 2e-14 for t <= 1/2), the
+// others by s_{m-1} = s_m - t / (m (m + 1)) s_{m+1} (A&S 9.1.27), which only adds small terms.
+template <int P>
+__device__ __forceinline__ void lf_basis(float xs, float ys, float t, zf *v)
 {
-    constexpr int NP = 2 * P + 1;
-    zf pw[P + 1];
-    pw[0] = zf{1.f, 0.f};
+    float sv[P + 1];
 #pragma unroll
-    for (int m = 1; m <= P; ++m) pw[m] = pw[m - 1] * zf{xs, ys};
+    for (int a = P; a >= P - 1; --a) {
+        float f = 1.0f;
 #pragma unroll
-    for (int ii = 0; ii < NS; ++ii) {
-        const int j = E + ii, n = j - P, a = n < 0 ? -n : n;
-        if (j >= NP) {
-            gv[ii] = zf{0.f, 0.f};
-            continue;
-        }
-        float sv = 1.0f;
+        for (int q = 8; q >= 1; --q) f = fmaf(-t * (1.0f / (float)(q * (q + a))), f, 1.0f);
+        sv[a] = f;
+    }
 #pragma unroll
-        for (int q = 8; q >= 1; --q) sv = fmaf(-t * (1.0f / (float)(q * (q + a))), sv, 1.0f);
-        const zf z = n >= 0 ? pw[a] : conj(pw[a]);
-        gv[ii] = (((n < 0 && (a & 1)) ? -sv : sv) * LF_GSCALE) * z;
+    for (int m = P - 1; m >= 1; --m) sv[m - 1] = fmaf(-t * (1.0f / (float)(m * (m + 1))), sv[m + 1], sv[m]);
+    zf pw = {LF_GSCALE, 0.f};
+#pragma unroll
+    for (int m = 0; m <= P; ++m) {
+        v[m] = sv[m] * pw;
+        pw = pw * zf{xs, ys};
     }
 }
 
@@ -245,30 +231,52 @@ __device__ __forceinline__ bool lf_bar_or(int id, int nthreads, bool p)
     return r != 0;
 }
 
-// per leaf: its U-list source points (the length of its flattened source list)
-__global__ void k_lf_tot(const int64_t *ls, const int64_t *ustart, const int32_t *usrc, int64_t nleaf,
-                         int32_t *tot)
+// Per leaf with points: the length of its flattened U list, its entries (first point, points, first
+// slot of the flattened list, 0; zeros past the entries) and the list's records in chunks of 64: x, y
+// relative to the target leaf's centre in units of 2/k, absolute y, U term (zeros past the list)
+__global__ void __launch_bounds__(128) k_lf_src(const int64_t *ls, const int64_t *ustart, const int32_t *usrc,
+                                                const int32_t *uterm, int64_t ncol, float w, float kh, const float *xl,
+                                                const float *yl, const float *y32, const int64_t *cbase, float4 *src,
+                                                int4 *ent, int32_t *tot)
 {
-    const int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (b >= nleaf) return;
-    int64_t T = 0;
-    for (int64_t e = ustart[b]; e < ustart[b + 1]; ++e) T += ls[usrc[e] + 1] - ls[usrc[e]];
-    tot[b] = (int32_t)T;
-}
-// per (leaf, entry slot < LF_MAXE): (first point, points, U term, source leaf) of the entry;
-// zeros past the leaf's entries (and the free-term entries of a dG/dd tree would be dropped)
-__global__ void k_lf_ent(const int64_t *ls, const int64_t *ustart, const int32_t *usrc, const int32_t *uterm,
-                         int64_t nleaf, int4 *ent)
-{
-    const int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (x >= nleaf * LF_MAXE) return;
-    const int64_t b = x / LF_MAXE, e = x % LF_MAXE, e0 = ustart[b];
-    int4 r = make_int4(0, 0, 0, 0);
-    if (e0 + e < ustart[b + 1]) {
-        const int s = usrc[e0 + e];
-        r = make_int4((int)ls[s], (int)(ls[s + 1] - ls[s]), uterm[e0 + e], s);
+    const int64_t b = blockIdx.x, e0 = ustart[b];
+    const int ne = (int)(ustart[b + 1] - e0);
+    __shared__ int4 rec[LF_MAXE];
+    __shared__ int T;
+    if (threadIdx.x < LF_MAXE) {
+        int4 r = make_int4(0, 0, 0, 0);
+        const int s = (int)threadIdx.x < ne ? usrc[e0 + threadIdx.x] : -1;
+        if (s >= 0) {
+            r.x = (int)ls[s];
+            r.y = (int)(ls[s + 1] - ls[s]);
+        }
+        int incl = r.y;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, incl, o);
+            if ((int)threadIdx.x >= o) incl += y;
+        }
+        r.z = incl - r.y;
+        rec[threadIdx.x] = r;
+        ent[b * LF_MAXE + threadIdx.x] = r;
+        if (threadIdx.x == LF_MAXE - 1) {
+            T = incl;
+            tot[b] = incl;
+        }
     }
-    ent[x] = r;
+    __syncthreads();
+    if (ls[b + 1] <= ls[b]) return;
+    float4 *o = src + cbase[b] * LF_CH;
+    const int64_t rt = b / ncol, ct = b % ncol;
+    for (int e = threadIdx.x >> 5; e < ne; e += 4) {
+        const int64_t s = usrc[e0 + e], rs = s / ncol, cs = s % ncol;
+        const float ox = __fmul_rn((float)(ct - cs), w), oy = -__fmul_rn((float)(rt - rs), w); // centre_t - centre_s
+        const float tm = __int_as_float(uterm[e0 + e]);
+        const int4 r = rec[e];
+        for (int i = threadIdx.x & 31; i < r.y; i += 32)
+            o[r.z + i] = make_float4(__fmul_rn(kh, xl[r.x + i] - ox), __fmul_rn(kh, yl[r.x + i] - oy), y32[r.x + i], tm);
+    }
+    for (int i = T + threadIdx.x; i < (T + LF_CH - 1) / LF_CH * LF_CH; i += 128) o[i] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
 // a leaf's target range and U-list length, loaded one leaf ahead by every role
@@ -291,28 +299,21 @@ __global__ void k_lf_pts(const float *xl, const float *yl, const float *y32, int
 // first_limit >= 0: poll limit of the MMA issuer's first wait (the timeout path's test)
 template <int P, int DEG>
 __global__ void __launch_bounds__(LF_THREADS, 1)
-    k_leaf_tt(int64_t nleaf, int64_t ncol, float w, float k, float d, const float *xl, const float *yl,
-              const float *y32, const float4 *pts, const int64_t *ls, const int4 *ent, const int32_t *tot,
-              const uint32_t *scl, NearQuadF nq, const zf *Lc,
+    k_leaf_tt(int64_t nleaf, float w, float k, float d, const float4 *pts, const int64_t *ls, const int4 *ent,
+              const int32_t *tot, const int64_t *cbase, const float4 *src, const uint32_t *scl, NearQuadF nq, const zf *Lc,
               const zf *qs, zf *us, int *err, int first_limit)
 {
     constexpr int NP = 2 * P + 1;
     static_assert(2 * NP <= 64, "the local expansion's orders must fit one chunk");
     using S = LfSmem<P>;
     extern __shared__ __align__(1024) unsigned char smem[];
-    LfMeta *meta = (LfMeta *)(smem + S::META_OFF);
     float *xch = (float *)(smem + S::XCH_OFF);
-    int32_t *eterm = (int32_t *)(smem + S::ETAB_OFF);
-    int32_t *epref = eterm + (LF_MAXE + 1), *ebase = epref + (LF_MAXE + 1);
-    float *eox = (float *)(ebase + (LF_MAXE + 1)), *eoy = eox + (LF_MAXE + 1);
-    int32_t *tpi = (int32_t *)(smem + S::TAB_OFF);            // [LF_MAXT] point of flattened source g
-    uint8_t *te = (uint8_t *)(tpi + LF_MAXT);                 // [LF_MAXT] its entry
     uint64_t *bars = (uint64_t *)(smem + S::BAR_OFF);
     uint32_t *tslot = (uint32_t *)(bars + S::NBAR);
     volatile int *abort_s = (volatile int *)(tslot + 1);
     const uint32_t sbase = smem_u32(smem);
     const uint32_t b0 = smem_u32(bars);
-    // barriers: rfull (copies landed), bfull (B converted, meta ready), sempty (stage free),
+    // barriers: rfull (copies landed), bfull (B converted), sempty (stage free),
     // afull (A stored), aempty (A read), dfull (accumulator written), dempty (accumulator read)
     auto rfull = [&](int s) { return b0 + 8u * s; };
     auto bfull = [&](int s) { return b0 + 8u * (LF_NS + s); };
@@ -368,126 +369,57 @@ __global__ void __launch_bounds__(LF_THREADS, 1)
 
     if (warp == 0) {
         // ---------------- producer ----------------
-        uint32_t cc = 0;
+        uint32_t cc = 0, pp = 0;
         int last[LF_NS]; // last chunk copied into each stage (lane 0)
 #pragma unroll
         for (int s = 0; s < LF_NS; ++s) last[s] = -1;
         bool stop = *abort_s != 0;
         LfLeaf nx = lf_leaf(ls, tot, blockIdx.x, nleaf);
         int4 nrec = blockIdx.x < nleaf ? ent[blockIdx.x * LF_MAXE + lane] : make_int4(0, 0, 0, 0);
+        int64_t ncb = blockIdx.x < nleaf ? cbase[blockIdx.x] : 0;
         for (int64_t b = blockIdx.x; b < nleaf && !stop; b += gridDim.x) {
             const LfLeaf cu = nx;
-            const int4 rec = nrec;
+            const int4 rec = nrec; // this lane's U entry
+            const float4 *ms = src + ncb * LF_CH;
             nx = lf_leaf(ls, tot, b + gridDim.x, nleaf); // in flight while this leaf is served
-            if (b + gridDim.x < nleaf) nrec = ent[(b + gridDim.x) * LF_MAXE + lane];
-            const int lo = cu.lo, hi = cu.hi;
+            if (b + gridDim.x < nleaf) {
+                nrec = ent[(b + gridDim.x) * LF_MAXE + lane];
+                ncb = cbase[b + gridDim.x];
+            }
+            const int lo = cu.lo, hi = cu.hi, T = cu.T;
             if (hi <= lo) continue;
-            // this lane's U entry (zeros past the leaf's entries)
-            const int base = rec.x, cnt = rec.y, term = rec.z, src = rec.w;
-            int incl = cnt;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int y = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += y;
-            }
-            const int T = __shfl_sync(0xffffffffu, incl, 31);
-            {
-                const int64_t rt = b / ncol, ct = b % ncol, rs = src / ncol, cs = src % ncol;
-                eox[lane] = (float)(ct - cs) * w; // centre_t - centre_s
-                eoy[lane] = -(float)(rt - rs) * w;
-            }
-            eterm[lane] = term;
-            ebase[lane] = base;
-            epref[lane + 1] = incl;
-            if (lane == 0) epref[0] = 0;
-            __syncwarp();
-            const bool tabled = T <= LF_MAXT;
-            if (tabled) {
-                // the entries with points, one after the other (their data by shuffle)
-                for (uint32_t live = __ballot_sync(0xffffffffu, cnt > 0); live; live &= live - 1) {
-                    const int e = __ffs(live) - 1;
-                    const int p0 = __shfl_sync(0xffffffffu, incl - cnt, e), ce = __shfl_sync(0xffffffffu, cnt, e);
-                    const int be = __shfl_sync(0xffffffffu, base, e);
-                    for (int k2 = lane; k2 < ce; k2 += 32) {
-                        tpi[p0 + k2] = be + k2;
-                        te[p0 + k2] = (uint8_t)e;
-                    }
-                }
-                __syncwarp();
-            }
             const int nreg = (T + LF_CH - 1) / LF_CH, nch = nreg + 1;
-            for (int i0 = lo; i0 < hi && !stop; i0 += LF_TGT) {
+            for (int i0 = lo; i0 < hi && !stop; i0 += LF_TGT, ++pp) {
                 for (int c = 0; c < nch; ++c, ++cc) {
                     const int s = (int)(cc % LF_NS);
+                    const uint32_t raw = sbase + S::RAW_OFF + s * LF_RAW_BYTES;
+                    const int g0 = c * LF_CH, n = c < nreg ? min(LF_CH, T - g0) : NP;
+                    const int ntb = c == 0 ? min(LF_TGT, hi - i0) * 16 : 0; // the pass's target rows
                     int ok = 1;
-                    if (lane == 0)
+                    if (lane == 0) {
                         ok = lf_wait(sempty(s), ((cc / LF_NS) & 1) ^ 1, LF_WAIT_LIMIT, abort_s, err);
+                        if (ok) {
+                            mbar_expect_tx(rfull(s), (uint32_t)(n * LM_MAXV * 8 + (c < nreg ? LF_META_BYTES : 0) + ntb));
+                            last[s] = (int)cc;
+                        }
+                    }
                     ok = __shfl_sync(0xffffffffu, ok, 0);
                     if (!ok) {
                         if (lane == 0) lf_fail(abort_s, err);
                         stop = true;
                         break;
                     }
-                    LfMeta &m = meta[s];
-                    const uint32_t raw = sbase + S::RAW_OFF + s * LF_RAW_BYTES;
                     if (c < nreg) {
-                        const int g0 = c * LF_CH, n = min(LF_CH, T - g0);
-                        // slots lane and 32 + lane: point, meta record, start of a run of consecutive points
-                        int pi[2], last0 = -2;
-                        uint32_t starts[2];
-#pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-                            const int slot = 32 * h + lane;
-                            const bool valid = slot < n;
-                            int e = 0;
-                            pi[h] = -1;
-                            if (valid) {
-                                const int g = g0 + slot;
-                                if (tabled) {
-                                    pi[h] = tpi[g];
-                                    e = te[g];
-                                } else {
-                                    while (epref[e + 1] <= g) ++e;
-                                    pi[h] = ebase[e] + (g - epref[e]);
-                                }
-                            }
-                            m.src[slot] = valid ? make_float4(eox[e], eoy[e], 0.f, __int_as_float((pi[h] << 2) | eterm[e]))
-                                                : make_float4(0.f, 0.f, 0.f, __int_as_float(-4));
-                            int prev = __shfl_up_sync(0xffffffffu, pi[h], 1);
-                            if (lane == 0) prev = last0; // slot 31 before slot 32; none before slot 0
-                            starts[h] = __ballot_sync(0xffffffffu, valid && pi[h] != prev + 1);
-                            last0 = __shfl_sync(0xffffffffu, pi[0], 31);
-                        }
-                        if (lane == 0) m.n = n;
-                        __syncwarp();
-                        if (lane == 0) mbar_expect_tx(rfull(s), (uint32_t)n * (LM_MAXV * 8 + 16));
-                        __syncwarp();
-                        // runs of consecutive points: the lane at a run's first slot copies its densities and
-                        // coordinates (the copies of a chunk are issued in parallel)
-                        const uint64_t st64 = (uint64_t)starts[0] | ((uint64_t)starts[1] << 32);
-#pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-                            const int r = 32 * h + lane;
-                            if ((st64 >> r) & 1) {
-                                const uint64_t after = r < 63 ? st64 >> (r + 1) : 0;
-                                const int r1 = after ? r + __ffsll((long long)after) : n;
-                                const uint32_t len = (uint32_t)(r1 - r);
-                                bulk_g2s(raw + (uint32_t)r * LM_MAXV * 8, qs + (int64_t)pi[h] * LM_MAXV, len * LM_MAXV * 8,
-                                         rfull(s));
-                                bulk_g2s(raw + LF_Q_BYTES + (uint32_t)r * 16, pts + pi[h], len * 16, rfull(s));
-                            }
-                        }
-                    } else {
-                        // the L2T chunk: the leaf's local expansion, orders as sources
-                        if (lane == 0) {
-                            m.n = NP;
-                            mbar_expect_tx(rfull(s), NP * LM_MAXV * 8);
-                            bulk_g2s(raw, Lc + b * NP * LM_MAXV, NP * LM_MAXV * 8, rfull(s));
-                        }
-                    }
-                    if (lane == 0) last[s] = (int)cc;
-                    stop = __shfl_sync(0xffffffffu, (int)(*abort_s != 0), 0) != 0;
-                    if (stop) break;
+                        // each lane copies its entry's part of the chunk
+                        const int a0 = max(rec.z, g0), a1 = min(rec.z + rec.y, g0 + n);
+                        if (a1 > a0)
+                            bulk_g2s(raw + (uint32_t)(a0 - g0) * LM_MAXV * 8, qs + (int64_t)(rec.x + a0 - rec.z) * LM_MAXV,
+                                     (uint32_t)(a1 - a0) * LM_MAXV * 8, rfull(s));
+                        if (lane == 31) bulk_g2s(sbase + S::META_OFF + s * LF_META_BYTES, ms + g0, LF_META_BYTES, rfull(s));
+                        if (lane == 30 && ntb)
+                            bulk_g2s(sbase + S::TGT_OFF + (pp % LF_NT) * LF_TGT * 16, pts + i0, (uint32_t)ntb, rfull(s));
+                    } else if (lane == 0) // the L2T chunk: the leaf's local expansion, orders as sources
+                        bulk_g2s(raw, Lc + b * NP * LM_MAXV, NP * LM_MAXV * 8, rfull(s));
                 }
             }
         }
@@ -498,7 +430,7 @@ __global__ void __launch_bounds__(LF_THREADS, 1)
                     lf_wait(rfull(s), (last[s] / LF_NS) & 1, LF_WAIT_LIMIT, nullptr, nullptr);
         __syncwarp();
     } else if (warp == 1 || warp == 3) {
-        // ---------------- converters: warp 1 vectors 0..7 (and the coordinates), warp 3 vectors 8..15 ----------------
+        // ---------------- converters: warp 1 vectors 0..7, warp 3 vectors 8..15 ----------------
         uint32_t cc = 0;
         bool stop = *abort_s != 0;
         const int cw = warp == 1 ? 0 : 1, v = 8 * cw + (lane & 7), kbp = lane >> 3;
@@ -517,39 +449,33 @@ __global__ void __launch_bounds__(LF_THREADS, 1)
                         stop = true;
                         break;
                     }
-                    LfMeta &m = meta[s];
-                    const int n = m.n;
+                    const int n = c < nreg ? min(LF_CH, cu.T - c * LF_CH) : NP;
                     const zf *raw = (const zf *)(smem + S::RAW_OFF + s * LF_RAW_BYTES);
-                    if (cw == 0 && c < nreg) { // coordinates relative to the target leaf: X = x_s - (centre_t - centre_s)
-#pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-                            const int slot = 32 * h + lane;
-                            const float4 pt = slot < n ? ((const float4 *)(raw + LF_CH * LM_MAXV))[slot]
-                                                       : make_float4(0.f, 0.f, 0.f, 0.f);
-                            const float4 o = m.src[slot];
-                            m.src[slot] = make_float4(kh * (pt.x - o.x), kh * (pt.y - o.y), pt.z, o.w);
-                        }
-                    }
                     unsigned char *B = smem + S::B_OFF + s * LF_B_BYTES;
                     const float sc = scq[c < nreg ? 0 : 1];
-                    // K block kb holds sources 4 kb .. 4 kb + 3 (real, imaginary part each)
+                    // K block kb holds sources 4 kb .. 4 kb + 3 (real, imaginary part each); this lane's 4 blocks
+                    // are read before any is stored
+                    zf q[4][4];
 #pragma unroll
-                    for (int kb = kbp; kb < LF_CH / 4; kb += 4) {
+                    for (int k4 = 0; k4 < 4; ++k4)
+#pragma unroll
+                        for (int jj = 0; jj < 4; ++jj) {
+                            const int j = 4 * (kbp + 4 * k4) + jj;
+                            q[k4][jj] = j < n ? raw[j * LM_MAXV + v] : zf{0.f, 0.f};
+                        }
+#pragma unroll
+                    for (int k4 = 0; k4 < 4; ++k4) {
                         uint32_t h[2][4], l[2][4]; // [output re / im][source]
 #pragma unroll
                         for (int jj = 0; jj < 4; ++jj) {
-                            const int j = 4 * kb + jj;
-                            const zf q = j < n ? raw[j * LM_MAXV + v] : zf{0.f, 0.f};
-                            const float qr = q.re * sc, qi = q.im * sc;
-                            uint32_t hr, lr, hi2, li2;
-                            lf_split2(qr, -qi, hr, lr);  // out re: (Re Q, -Im Q)
-                            lf_split2(qi, qr, hi2, li2); // out im: (Im Q, Re Q)
-                            h[0][jj] = hr;
-                            h[1][jj] = hi2;
-                            l[0][jj] = lr;
-                            l[1][jj] = li2;
+                            uint32_t hp, lp; // (Re Q, Im Q)
+                            lf_split2(q[k4][jj].re * sc, q[k4][jj].im * sc, hp, lp);
+                            h[0][jj] = hp ^ 0x80000000u;               // out re: (Re Q, -Im Q)
+                            h[1][jj] = __byte_perm(hp, hp, 0x1032);    // out im: (Im Q, Re Q)
+                            l[0][jj] = lp ^ 0x80000000u;
+                            l[1][jj] = __byte_perm(lp, lp, 0x1032);
                         }
-                        const int kk = 8 * kb;
+                        const int kk = 8 * (kbp + 4 * k4);
                         *(uint4 *)(B + lf_off(v, kk)) = make_uint4(h[0][0], h[0][1], h[0][2], h[0][3]);
                         *(uint4 *)(B + lf_off(16 + v, kk)) = make_uint4(h[1][0], h[1][1], h[1][2], h[1][3]);
                         *(uint4 *)(B + lf_off(32 + v, kk)) = make_uint4(l[0][0], l[0][1], l[0][2], l[0][3]);
@@ -614,114 +540,121 @@ __global__ void __launch_bounds__(LF_THREADS, 1)
         __syncwarp();
     } else if (warp >= 4 && warp < LF_EPI0) {
         // ---------------- kernel values ----------------
-        const int g = warp - 4, part = g >> 1, t = 32 * (g & 1) + lane;
-        const int j0 = LF_JS * part;
-        uint32_t cc = 0;
+        const int g = warp - 4, tq = lane & 7, sq = lane >> 3;
+        uint32_t cc = 0, pp = 0;
         bool bad = *abort_s != 0;
         LfLeaf nx = lf_leaf(ls, tot, blockIdx.x, nleaf);
-        int pre_i0 = -1; // the pass whose target row is prefetched, and the row
-        float4 pre_pt = make_float4(0.f, 0.f, 0.f, 0.f);
+        // hi and lo rows of target slot t, columns of the 4 sources (order slots) from j
+        auto store = [&](unsigned char *A, int t, int j, const zf *gv) {
+            uint32_t h[4], l[4];
+#pragma unroll
+            for (int jj = 0; jj < 4; ++jj) lf_split2(gv[jj].re, gv[jj].im, h[jj], l[jj]);
+            *(uint4 *)(A + lf_off(t, 2 * j)) = make_uint4(h[0], h[1], h[2], h[3]);
+            *(uint4 *)(A + lf_off(64 + t, 2 * j)) = make_uint4(l[0], l[1], l[2], l[3]);
+        };
         for (int64_t b = blockIdx.x; b < nleaf && !bad; b += gridDim.x) {
             const LfLeaf cu = nx;
             nx = lf_leaf(ls, tot, b + gridDim.x, nleaf);
             const int lo = cu.lo, hi = cu.hi;
             if (hi <= lo) continue;
             const int nreg = (cu.T + LF_CH - 1) / LF_CH, nch = nreg + 1;
-            for (int i0 = lo; i0 < hi && !bad; i0 += LF_TGT) {
-                const int i = i0 + t;
-                const bool act = i < hi;
-                const float4 pt = i0 == pre_i0 ? pre_pt : (act ? pts[i] : make_float4(0.f, 0.f, 0.f, 0.f));
-                {
-                    // the next pass's target row, in flight while this pass is served
-                    const int n0 = i0 + LF_TGT < hi ? i0 + LF_TGT : nx.lo, nh = i0 + LF_TGT < hi ? hi : nx.hi;
-                    pre_i0 = n0;
-                    pre_pt = n0 + t < nh ? pts[n0 + t] : make_float4(0.f, 0.f, 0.f, 0.f);
-                }
-                const float xi = pt.x, yi = pt.y, ya = pt.z;
-                const float xk = kh * xi, yk = kh * yi;
+            for (int i0 = lo; i0 < hi && !bad; i0 += LF_TGT, ++pp) {
+                const float4 *tg = (const float4 *)(smem + S::TGT_OFF) + (pp % LF_NT) * LF_TGT;
+                const int nt = min(LF_TGT, hi - i0), ng = (nt + 7) >> 3;
                 for (int c = 0; c < nch; ++c, ++cc) {
                     const int s = (int)(cc % LF_NS), a = (int)(cc % LF_NA);
-                    if (!lf_wait(bfull(s), (cc / LF_NS) & 1, LF_WAIT_LIMIT, abort_s, err) ||
+                    if (!lf_wait(rfull(s), (cc / LF_NS) & 1, LF_WAIT_LIMIT, abort_s, err) ||
                         !lf_wait(aempty(a), ((cc / LF_NA) & 1) ^ 1, LF_WAIT_LIMIT, abort_s, err)) {
                         lf_fail(abort_s, err);
                         bad = true;
                         break;
                     }
                     unsigned char *A = smem + S::A_OFF + a * LF_A_BYTES;
-                    if (act) {
-                        // this thread's LF_JS sources (or order slots) in rounds of LF_RB
+                    const int it0 = (g + 4 * (int)(cc & 1)) & (LF_GW - 1); // (uneven rounds even out over two chunks)
+                    if (c < nreg) {
+                        // Items of 8 targets x 16 sources, round robin over the warps: a lane takes a target
+                        // and 4 sources.  Columns past the chunk's sources (B is zero there) and rows past the
+                        // targets keep finite values of earlier chunks.
+                        const float4 *ms = (const float4 *)(smem + S::META_OFF + s * LF_META_BYTES);
+                        const int nit = ng * ((min(LF_CH, cu.T - c * LF_CH) + 15) >> 4);
+                        int grp = it0, blk = 0;
+                        float4 nr4[LF_RB], npt; // the next item's records and target, loaded ahead
+                        auto fetch = [&]() {
+                            while (grp >= ng) {
+                                grp -= ng;
+                                ++blk;
+                            }
+                            npt = tg[min(8 * grp + tq, nt - 1)];
+#pragma unroll
+                            for (int ii = 0; ii < LF_RB; ++ii) nr4[ii] = ms[16 * blk + LF_RB * sq + ii];
+                        };
+                        if (it0 < nit) fetch();
 #pragma unroll 1
-                        for (int hb = 0; hb < LF_JS / LF_RB; ++hb) {
-                            const int jb = j0 + LF_RB * hb;
+                        for (int it = it0; it < nit; it += LF_GW) {
+                            const int t = 8 * grp + tq, jb = 16 * blk + LF_RB * sq;
+                            const float4 pt = npt;
+                            float4 r4[LF_RB];
+#pragma unroll
+                            for (int ii = 0; ii < LF_RB; ++ii) r4[ii] = nr4[ii];
+                            grp += LF_GW;
+                            if (it + LF_GW < nit) fetch();
+                            const float xk = __fmul_rn(kh, pt.x), yk = __fmul_rn(kh, pt.y); // as in the records: t = 0 for the self pair
+                            // coordinates in units of 2/k, so that t = (k r / 2)^2 = dx^2 + dy^2; slots past
+                            // the chunk's sources hold zeros
                             zf gv[LF_RB];
-                            if (c < nreg) {
-                                // coordinates in units of 2/k, so that t = (k r / 2)^2 = dx^2 + dy^2; slots past
-                                // the chunk's sources hold zeros (finite values; B is zero there)
-                                const LfMeta &m = meta[s];
-                                float tv[LF_RB];
-                                bool special = false;
+                            float tv[LF_RB];
+                            bool special = false;
+#pragma unroll
+                            for (int ii = 0; ii < LF_RB; ++ii) {
+                                const float dx = xk - r4[ii].x, dy = yk - r4[ii].y;
+                                tv[ii] = fmaf(dx, dx, dy * dy);
+                                special |= (__float_as_int(r4[ii].w) != 0) | (!DEG && tv[ii] > 1.0f);
+                            }
+#pragma unroll
+                            for (int ii = 0; ii < LF_RB; ++ii) gv[ii] = lf_h0s<DEG ? DEG : 8>(tv[ii]);
+                            if (!special) {
+                                // t = 0: the self pair (and points that coincide) is left out
+#pragma unroll
+                                for (int ii = 0; ii < LF_RB; ++ii)
+                                    if (tv[ii] == 0.f) gv[ii] = zf{0.f, 0.f};
+                            } else {
 #pragma unroll
                                 for (int ii = 0; ii < LF_RB; ++ii) {
-                                    const float4 r4 = m.src[jb + ii];
-                                    const float dx = xk - r4.x, dy = yk - r4.y;
-                                    tv[ii] = fmaf(dx, dx, dy * dy);
-                                    special |= ((__float_as_int(r4.w) & 3) != 0) | (!DEG && tv[ii] > 1.0f);
-                                }
-#pragma unroll
-                                for (int ii = 0; ii < LF_RB; ++ii) gv[ii] = lf_h0s<DEG ? DEG : 8>(tv[ii]);
-                                if (!special) {
-                                    // t = 0: the self pair (and points that coincide) is left out
-#pragma unroll
-                                    for (int ii = 0; ii < LF_RB; ++ii)
-                                        if (tv[ii] == 0.f) gv[ii] = zf{0.f, 0.f};
-                                } else {
-#pragma unroll
-                                    for (int ii = 0; ii < LF_RB; ++ii) {
-                                        const float4 r4 = m.src[jb + ii]; // read again: the rare path
-                                        const int term = __float_as_int(r4.w) & 3;
-                                        if (term != 0) { // tail of a reflected direct term
-                                            const float X = fabsf(xk - r4.x) * (1.0f / kh);
-                                            const float h = term == 1 ? -(ya + r4.z) : ya + r4.z + 2.0f * d;
-                                            const zf tl = near_tail32(nq, term - 1, X, h);
-                                            gv[ii] = zf{tl.re * LF_GSCALE, tl.im * LF_GSCALE};
-                                        } else if (tv[ii] == 0.f) {
-                                            gv[ii] = zf{0.f, 0.f};
-                                        } else if (!DEG && tv[ii] > 1.0f) {
-                                            const zf fr = green_free32_far(tv[ii]);
-                                            gv[ii] = zf{fr.re * LF_GSCALE, fr.im * LF_GSCALE};
-                                        }
+                                    const int term = __float_as_int(r4[ii].w);
+                                    if (term != 0) { // tail of a reflected direct term
+                                        const float X = fabsf(xk - r4[ii].x) * (1.0f / kh);
+                                        const float h = term == 1 ? -(pt.z + r4[ii].z) : pt.z + r4[ii].z + 2.0f * d;
+                                        const zf tl = near_tail32(nq, term - 1, X, h);
+                                        gv[ii] = zf{tl.re * LF_GSCALE, tl.im * LF_GSCALE};
+                                    } else if (tv[ii] == 0.f) {
+                                        gv[ii] = zf{0.f, 0.f};
+                                    } else if (!DEG && tv[ii] > 1.0f) {
+                                        const zf fr = green_free32_far(tv[ii]);
+                                        gv[ii] = zf{fr.re * LF_GSCALE, fr.im * LF_GSCALE};
                                     }
                                 }
-                            } else {
-                                // the L2T chunk: order slots jb .. jb + LF_RB - 1 (a compile-time set per case)
-                                const float xs = xi / w, ys = yi / w, tt = fmaf(xk, xk, yk * yk);
-                                switch (jb / LF_RB) {
-                                case 0: lf_basis<P, 0, LF_RB>(xs, ys, tt, gv); break;
-                                case 1: lf_basis<P, LF_RB, LF_RB>(xs, ys, tt, gv); break;
-                                case 2: lf_basis<P, 2 * LF_RB, LF_RB>(xs, ys, tt, gv); break;
-                                case 3: lf_basis<P, 3 * LF_RB, LF_RB>(xs, ys, tt, gv); break;
-#if LF_RB == 4
-                                case 4: lf_basis<P, 16, 4>(xs, ys, tt, gv); break;
-                                case 5: lf_basis<P, 20, 4>(xs, ys, tt, gv); break;
-                                case 6: lf_basis<P, 24, 4>(xs, ys, tt, gv); break;
-                                case 7: lf_basis<P, 28, 4>(xs, ys, tt, gv); break;
-#endif
-                                default: // slots past 2 P + 1 <= 29 hold zeros
-#pragma unroll
-                                    for (int ii = 0; ii < LF_RB; ++ii) gv[ii] = zf{0.f, 0.f};
-                                    break;
-                                }
                             }
-                            // hi and lo rows of this target slot: one 16-byte store per 4 sources and part
+                            store(A, t, jb, gv);
+                        }
+                    } else {
+                        // the L2T chunk: a lane per target, all its orders; the other warps go on
+                        const int t = 32 * it0 + lane;
+                        if (t < nt) {
+                            const float4 pt = tg[t];
+                            const float xk = kh * pt.x, yk = kh * pt.y;
+                            zf v[P + 1];
+                            lf_basis<P>(pt.x / w, pt.y / w, fmaf(xk, xk, yk * yk), v);
 #pragma unroll
-                            for (int m4 = 0; m4 < LF_RB / 4; ++m4) {
-                                uint32_t h[4], l[4];
+                            for (int q = 0; q < (NP + 3) / 4; ++q) { // slot j: order j - P
+                                zf gv[4];
 #pragma unroll
-                                for (int jj = 0; jj < 4; ++jj)
-                                    lf_split2(gv[4 * m4 + jj].re, gv[4 * m4 + jj].im, h[jj], l[jj]);
-                                const int kk = 2 * (jb + 4 * m4);
-                                *(uint4 *)(A + lf_off(t, kk)) = make_uint4(h[0], h[1], h[2], h[3]);
-                                *(uint4 *)(A + lf_off(64 + t, kk)) = make_uint4(l[0], l[1], l[2], l[3]);
+                                for (int jj = 0; jj < 4; ++jj) {
+                                    const int j = 4 * q + jj, n = j - P;
+                                    if (j >= NP) gv[jj] = zf{0.f, 0.f};
+                                    else if (n >= 0) gv[jj] = v[n];
+                                    else gv[jj] = (n & 1) ? zf{-v[-n].re, v[-n].im} : conj(v[-n]);
+                                }
+                                store(A, t, 4 * q, gv);
                             }
                         }
                     }
@@ -853,20 +786,22 @@ lm_status lm_setup_leaf_tt(lm_tree_s *t, cudaStream_t st)
     t->lf_grid = (int)std::max<int64_t>(1, std::min<int64_t>(nsm, t->nleaf));
     const lm_status s = lf_set_attr(t->p);
     if (s != LM_OK) return s;
-    float4 *pts;
+    float4 *pts, *src;
     int4 *ent;
     lm_status r = lm_dalloc(t, &pts, (size_t)t->n);
+    if (r == LM_OK) r = lm_dalloc(t, &src, (size_t)t->lf_nchunk * LF_CH);
     if (r == LM_OK) r = lm_dalloc(t, &ent, (size_t)t->nleaf * LF_MAXE);
     if (r == LM_OK) r = lm_dalloc(t, &t->lf_scl, 2);
     if (r == LM_OK) r = lm_dalloc(t, &t->lf_tot, (size_t)t->nleaf);
     if (r != LM_OK) return r;
     t->lf_pts = pts;
     t->lf_ent = ent;
-    k_lf_pts<<<(unsigned)((t->n + 255) / 256), 256, 0, st>>>(t->xl32, t->yl32, t->y32, t->n, (float4 *)t->lf_pts);
-    k_lf_tot<<<(unsigned)((t->nleaf + 255) / 256), 256, 0, st>>>(t->leaf_start, t->ustart, t->usrc, t->nleaf,
-                                                                  t->lf_tot);
-    k_lf_ent<<<(unsigned)((t->nleaf * LF_MAXE + 255) / 256), 256, 0, st>>>(t->leaf_start, t->ustart, t->usrc,
-                                                                          t->uterm, t->nleaf, (int4 *)t->lf_ent);
+    t->lf_src = src;
+    const Level &lv = t->lev[t->L];
+    k_lf_pts<<<(unsigned)((t->n + 255) / 256), 256, 0, st>>>(t->xl32, t->yl32, t->y32, t->n, pts);
+    k_lf_src<<<(unsigned)t->nleaf, 128, 0, st>>>(t->leaf_start, t->ustart, t->usrc, t->uterm, lv.ncol, (float)lv.w,
+                                                 0.5f * (float)t->med.k2, t->xl32, t->yl32, t->y32, t->lf_cbase, src, ent,
+                                                 t->lf_tot);
     LM_CUDA(cudaGetLastError());
     t->lf_ready = true;
     return LM_OK;
@@ -882,15 +817,13 @@ static lm_status lf_launch(lm_tree_s *t, const NearQuadF &nq, cudaStream_t st)
     t->lf_poll_limit = -1; // a test limit applies to one launch
     if (xmax <= 2.0 && nterms <= 6)
         k_leaf_tt<P, 6><<<t->lf_grid, LF_THREADS, LfSmem<P>::BYTES, st>>>(
-            t->nleaf, lv.ncol, (float)lv.w, (float)t->med.k2, (float)t->med.d, t->xl32, t->yl32, t->y32,
-            (const float4 *)t->lf_pts, t->leaf_start, (const int4 *)t->lf_ent, t->lf_tot, t->lf_scl, nq, lv.L32,
-            t->qs32,
+            t->nleaf, (float)lv.w, (float)t->med.k2, (float)t->med.d, (const float4 *)t->lf_pts, t->leaf_start,
+            (const int4 *)t->lf_ent, t->lf_tot, t->lf_cbase, (const float4 *)t->lf_src, t->lf_scl, nq, lv.L32, t->qs32,
             t->us32, t->dflag + 1, first);
     else
         k_leaf_tt<P, 0><<<t->lf_grid, LF_THREADS, LfSmem<P>::BYTES, st>>>(
-            t->nleaf, lv.ncol, (float)lv.w, (float)t->med.k2, (float)t->med.d, t->xl32, t->yl32, t->y32,
-            (const float4 *)t->lf_pts, t->leaf_start, (const int4 *)t->lf_ent, t->lf_tot, t->lf_scl, nq, lv.L32,
-            t->qs32,
+            t->nleaf, (float)lv.w, (float)t->med.k2, (float)t->med.d, (const float4 *)t->lf_pts, t->leaf_start,
+            (const int4 *)t->lf_ent, t->lf_tot, t->lf_cbase, (const float4 *)t->lf_src, t->lf_scl, nq, lv.L32, t->qs32,
             t->us32, t->dflag + 1, first);
     LM_CUDA(cudaGetLastError());
     return LM_OK;

@@ -195,13 +195,14 @@ __global__ void k_vlist(int l, int64_t ncol, int64_t nrow, int DC, const int32_t
 }
 
 // U list at the leaf level: image adjacent to target (free term includes itself)
+// pass 0: count (chunks, optional: of 64 source points, for leaves with points); pass 1: fill
 __global__ void k_ulist(int64_t ncol, int64_t nrow, int64_t *ustart, int32_t *usrc, int32_t *uterm,
-                        int pass)
+                        int pass, const int64_t *ls, int64_t *chunks)
 {
     int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (t >= ncol * nrow) return;
     int64_t rt = t / ncol, ct = t % ncol;
-    int64_t pos = pass ? ustart[t] : 0, cnt = 0;
+    int64_t pos = pass ? ustart[t] : 0, cnt = 0, pts = 0;
     for (int term = 0; term < 5; ++term) {
         int64_t a = src_row(term, rt - 1, nrow), b = src_row(term, rt + 1, nrow);
         int64_t rlo = max((int64_t)0, min(a, b)), rhi = min(nrow - 1, max(a, b));
@@ -215,10 +216,12 @@ __global__ void k_ulist(int64_t ncol, int64_t nrow, int64_t *ustart, int32_t *us
                     ++pos;
                 }
                 ++cnt;
+                if (chunks) pts += ls[rs * ncol + cs + 1] - ls[rs * ncol + cs];
             }
         }
     }
     if (!pass) ustart[t] = cnt;
+    if (chunks) chunks[t] = ls[t + 1] > ls[t] ? (pts + 63) / 64 : 0;
 }
 
 // One block per list: counts c[0..m) -> starts c[0..m], in place; tot: their sum, the largest count and
@@ -695,7 +698,7 @@ lm_status lm_setup_tables(lm_tree_s *t, cudaStream_t st)
     int64_t *dtot;
     TRY(lm_dalloc(t->tmp, &dmap, smap.size()));
     LM_CUDA(cudaMemcpyAsync(dmap, smap.data(), smap.size() * sizeof(int32_t), cudaMemcpyHostToDevice, st));
-    const int nj = (mixed ? 2 : 1) * (L + 1) + 1; // V, rest (mixed) of every level; U
+    const int nj = mixed ? 2 * (L + 1) + 2 : L + 2; // V, rest (mixed) of every level; U, chunks (mixed)
     TRY(lm_dalloc(t->tmp, &djobs, nj));
     TRY(lm_dalloc(t->tmp, &dtot, 3 * nj));
     std::vector<ScanJob> sj;
@@ -716,7 +719,11 @@ lm_status lm_setup_tables(lm_tree_s *t, cudaStream_t st)
     const int64_t ncol = (int64_t)t->R << L, nrow = (int64_t)1 << L;
     TRY(lm_dalloc(t, &t->ustart, t->nleaf + 1));
     sj.push_back({t->ustart, t->nleaf, dtot + 3 * sj.size(), nullptr});
-    k_ulist<<<grid_for(t->nleaf, 128), 128, 0, st>>>(ncol, nrow, t->ustart, nullptr, nullptr, 0);
+    if (mixed) {
+        TRY(lm_dalloc(t, &t->lf_cbase, t->nleaf + 1));
+        sj.push_back({t->lf_cbase, t->nleaf, dtot + 3 * sj.size(), nullptr});
+    }
+    k_ulist<<<grid_for(t->nleaf, 128), 128, 0, st>>>(ncol, nrow, t->ustart, nullptr, nullptr, 0, t->leaf_start, t->lf_cbase);
     LM_CUDA(cudaMemcpyAsync(djobs, sj.data(), nj * sizeof(ScanJob), cudaMemcpyHostToDevice, st));
     k_scan_lists<<<nj, 1024, 0, st>>>(djobs);
     LM_CUDA(cudaGetLastError());
@@ -757,9 +764,10 @@ lm_status lm_setup_tables(lm_tree_s *t, cudaStream_t st)
     TRY(lm_build_m2l_tables(md, P, tcls, t->dflag, t->tmp, st));
     t->nu = ht[0];
     t->umax = ht[1];
+    if (mixed) t->lf_nchunk = ht[3];
     TRY(lm_dalloc(t, &t->usrc, t->nu));
     TRY(lm_dalloc(t, &t->uterm, t->nu));
-    k_ulist<<<grid_for(t->nleaf, 128), 128, 0, st>>>(ncol, nrow, t->ustart, t->usrc, t->uterm, 1);
+    k_ulist<<<grid_for(t->nleaf, 128), 128, 0, st>>>(ncol, nrow, t->ustart, t->usrc, t->uterm, 1, nullptr, nullptr);
     TRY(lm_setup_near(t, st));
     LM_CUDA(cudaGetLastError());
     if (mixed) {

@@ -152,6 +152,16 @@ def test_few_vector_mixed_kernels(lm, name, nvec):
     assert _rel(_apply(lm, t, q.astype(np.complex64)), ref) <= 1e-6
 
 
+@pytest.mark.parametrize("n", [1, 40, 270, 1100, 2100, 4000])
+@pytest.mark.parametrize("band", [(-0.95, -0.05), (-1.0 + 1e-6, -1e-6)])
+def test_tensor_core_leaf_tiles(lm, n, band):
+    """32 leaves of 0 to 150 points: target groups of 8, passes of 64, chunks of 64 sources, tails."""
+    x, y, q = workloads.uniform_strip(n, 0.0, 1.9, *band, nvec=16, seed=n)
+    t = _tree(lm, A, x, y, precision="mixed", p=14, depth=2)
+    ref = _apply(lm, _tree(lm, A, x, y, p=24, depth=2), q)
+    assert _rel(_apply(lm, t, q.astype(np.complex64)), ref) <= 1e-6
+
+
 @pytest.mark.parametrize("nvec", [1, 2, 3, 5, 16])
 @pytest.mark.parametrize("band", [(0.05, 0.95), (1e-6, 0.02)])
 def test_cross_double_float_matches_ieee(lm, nvec, band):
