@@ -220,10 +220,10 @@ __global__ void __launch_bounds__(128) k_l2t_df(Geo geo, int P, double k, Bessel
 // ---------------------------------------------------------------------------
 // (vectors beyond nv are summed with their neighbours' data, inside the 16-slot buffers, and not stored)
 template <int VPT>
-__device__ __forceinline__ void dot_q(float4 *acc, const float4 *T, const float4 *m, int np, int nv)
+__device__ __forceinline__ void dot_q(float4 *acc, const float4 *T, const float4 *m, int nq, int np, int nv)
 {
     int q = 0;
-    for (; q + 4 <= np; q += 4) { // four table entries in flight
+    for (; q + 4 <= nq; q += 4) { // four table entries in flight
         float4 t[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) t[j] = T[(q + j) * np];
@@ -233,69 +233,78 @@ __device__ __forceinline__ void dot_q(float4 *acc, const float4 *T, const float4
             for (int i = 0; i < VPT; ++i)
                 dfc_mac(acc[i], t[j], m[(q + j) * nv + i]);
     }
-    for (; q < np; ++q)
+    for (; q < nq; ++q)
 #pragma unroll
         for (int i = 0; i < VPT; ++i)
             dfc_mac(acc[i], T[q * np], m[q * nv + i]);
 }
 
-// M2M: one block per parent; up to 4 vectors: a thread per (child position, order),
-// the four positions summed through shared memory; more: a thread per (order, group of 4 vectors)
-template <int NV, class Geo>
-__global__ void __launch_bounds__(512) k_m2m_dx(Geo geo, int P, int nv, const float4 *tabs, const float4 *Mc, float4 *Mp)
+// M2M: one block per (parent, group of VPT vectors); a thread per (part of the sum over q, child
+// position, order).  Each position's parts are added in order, then the positions.  QS parts of the
+// sum (2 while 512 threads hold them) depend on the order alone: a vector's result does not depend on
+// the others.  Bound by FP32 issue on large levels, by the chain of multiply-adds on small ones: 250k
+// strip, 16 vectors, the four levels above 5120 boxes 456 us with a thread for the four positions of
+// (order, 4 vectors), 167 us; adjoint of 20k points, 2 vectors, 69 us with QS = 1, 52 us with 2.
+template <int VPT, class Geo>
+__global__ void __launch_bounds__(512) k_m2m_dx(Geo geo, int P, int nv, int QS, const float4 *tabs, const float4 *Mc, float4 *Mp)
 {
-    constexpr int VPT = NV < 4 ? NV : 4;
-    constexpr bool SPLIT = NV <= 4;
-    extern __shared__ float4 red[]; // SPLIT: [3][np][VPT]
-    const int np = 2 * P + 1, vg = (nv + VPT - 1) / VPT, nitem = np * vg * (SPLIT ? 4 : 1);
+    extern __shared__ float4 red[]; // [4 QS - 1][np][VPT]
+    const int np = 2 * P + 1, v0 = blockIdx.y * VPT, nvv = min(VPT, nv - v0);
     const int64_t b = geo.parent(blockIdx.x);
-    for (int it = threadIdx.x; it < (nitem + blockDim.x - 1) / blockDim.x * blockDim.x; it += blockDim.x) {
-        const bool on = it < nitem;
-        const int p = it % np, r = it / np, pos0 = SPLIT ? r : 0, v0 = SPLIT ? 0 : r * VPT, nvv = min(VPT, nv - v0);
-        float4 tot[VPT];
-        for (int pos = pos0; pos < (SPLIT ? pos0 + 1 : 4); ++pos) { // each position summed on its own
-            float4 acc[VPT];
+    const int p = threadIdx.x % np, r = threadIdx.x / np, pos = r & 3, qs = r >> 2;
+    const int q0 = qs * np / QS, q1 = (qs + 1) * np / QS;
+    float4 acc[VPT];
 #pragma unroll
-            for (int i = 0; i < VPT; ++i) acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (on)
-                dot_q<VPT>(acc, tabs + (int64_t)pos * np * np + p, Mc + geo.child(b, pos) * np * nv + v0, np, nv);
+    for (int i = 0; i < VPT; ++i) acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (qs < QS) {
+        dot_q<VPT>(acc, tabs + ((int64_t)pos * np + q0) * np + p, Mc + (geo.child(b, pos) * np + q0) * nv + v0, q1 - q0, np, nv);
 #pragma unroll
-            for (int i = 0; i < VPT; ++i) tot[i] = pos == pos0 ? df_norm(acc[i]) : dfc_add(tot[i], df_norm(acc[i]));
+        for (int i = 0; i < VPT; ++i) {
+            acc[i] = df_norm(acc[i]);
+            if (r > 0) red[((r - 1) * np + p) * VPT + i] = acc[i];
         }
-        if (SPLIT) { // a block has at least nitem threads (rounded up)
-            if (on && pos0 > 0)
+    }
+    __syncthreads();
+    if (r > 0) return;
 #pragma unroll
-                for (int i = 0; i < VPT; ++i) red[((pos0 - 1) * np + p) * VPT + i] = tot[i];
-            __syncthreads();
-            if (on && pos0 == 0)
-#pragma unroll
-                for (int i = 0; i < VPT; ++i)
-                    for (int pos = 1; pos < 4; ++pos) tot[i] = dfc_add(tot[i], red[((pos - 1) * np + p) * VPT + i]);
+    for (int i = 0; i < VPT; ++i) {
+        float4 tot = acc[i];
+        for (int c = 0; c < 4; ++c) {
+            float4 part = c == 0 ? acc[i] : red[((c - 1) * np + p) * VPT + i];
+            for (int h = 1; h < QS; ++h) part = dfc_add(part, red[((c + 4 * h - 1) * np + p) * VPT + i]);
+            tot = c == 0 ? part : dfc_add(tot, part);
         }
-        if (on && pos0 == 0)
-#pragma unroll
-            for (int i = 0; i < VPT; ++i)
-                if (i < nvv) Mp[(b * np + p) * nv + v0 + i] = tot[i];
+        if (i < nvv) Mp[(b * np + p) * nv + v0 + i] = tot;
     }
 }
 
-// L2L: one block per parent; a thread per (child, order, group of vectors); adds to the child's L
-template <int NV, class Geo>
-__global__ void __launch_bounds__(512) k_l2l_dx(Geo geo, int P, int nv, const float4 *tabs, const float4 *Lp, float4 *Lc)
+// L2L: one block per (parent, group of vectors), threads as in M2M; adds to the child's L
+template <int VPT, class Geo>
+__global__ void __launch_bounds__(512) k_l2l_dx(Geo geo, int P, int nv, int QS, const float4 *tabs, const float4 *Lp, float4 *Lc)
 {
-    constexpr int VPT = NV < 4 ? NV : 4;
-    const int np = 2 * P + 1, vg = (nv + VPT - 1) / VPT;
+    extern __shared__ float4 red[]; // [4 QS - 4][np][VPT]
+    const int np = 2 * P + 1, v0 = blockIdx.y * VPT, nvv = min(VPT, nv - v0);
     const int64_t b = geo.parent(blockIdx.x);
-    for (int it = threadIdx.x; it < 4 * np * vg; it += blockDim.x) {
-        const int p = it % np, r = it / np, pos = r & 3, v0 = (r >> 2) * VPT, nvv = min(VPT, nv - v0);
-        float4 acc[VPT];
+    const int p = threadIdx.x % np, r = threadIdx.x / np, pos = r & 3, qs = r >> 2;
+    const int q0 = qs * np / QS, q1 = (qs + 1) * np / QS;
+    float4 acc[VPT];
 #pragma unroll
-        for (int i = 0; i < VPT; ++i) acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-        dot_q<VPT>(acc, tabs + (int64_t)pos * np * np + p, Lp + b * np * nv + v0, np, nv);
-        float4 *o = Lc + (geo.child(b, pos) * np + p) * nv + v0;
+    for (int i = 0; i < VPT; ++i) acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (qs < QS) {
+        dot_q<VPT>(acc, tabs + ((int64_t)pos * np + q0) * np + p, Lp + (b * np + q0) * nv + v0, q1 - q0, np, nv);
 #pragma unroll
-        for (int i = 0; i < VPT; ++i)
-            if (i < nvv) o[i] = dfc_add(o[i], df_norm(acc[i]));
+        for (int i = 0; i < VPT; ++i) {
+            acc[i] = df_norm(acc[i]);
+            if (qs > 0) red[((r - 4) * np + p) * VPT + i] = acc[i];
+        }
+    }
+    if (QS > 1) __syncthreads();
+    if (qs > 0) return;
+    float4 *o = Lc + (geo.child(b, pos) * np + p) * nv + v0;
+#pragma unroll
+    for (int i = 0; i < VPT; ++i) {
+        for (int h = 1; h < QS; ++h) acc[i] = dfc_add(acc[i], red[((r + 4 * h - 4) * np + p) * VPT + i]);
+        if (i < nvv) o[i] = dfc_add(o[i], acc[i]);
     }
 }
 
@@ -329,7 +338,7 @@ __global__ void __launch_bounds__(512, MINB) k_m2l_dx(const M2LLevelDF *lev, int
 #pragma unroll
                 for (int i = 0; i < VPT; ++i) acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
                 for (int64_t e = e0 + s; e < e1; e += GS)
-                    dot_q<VPT>(acc, v.tab + (int64_t)v.vslot[e] * np * np + p, v.M + (int64_t)v.vsrc[e] * np * nv + v0, np, nv);
+                    dot_q<VPT>(acc, v.tab + (int64_t)v.vslot[e] * np * np + p, v.M + (int64_t)v.vsrc[e] * np * nv + v0, np, np, nv);
 #pragma unroll
                 for (int i = 0; i < VPT; ++i) part[i] = s == c ? df_norm(acc[i]) : dfc_add(part[i], df_norm(acc[i]));
             }
@@ -489,24 +498,30 @@ static int launch_l2t_all(const BesselDF &B, Geo geo, int64_t nleaf, int P, doub
                           L2TOut{us + (int64_t)w0 * n, nullptr, nullptr, nullptr}, st);
     return k_;
 }
+// parts of the sum over q of M2M and L2L
+static int shift_parts(int np) { return 8 * np <= 512 ? 2 : 1; }
+#define VPT_DISPATCH(nv, ...)                            \
+    switch (nv) {                                         \
+    case 1: { constexpr int VPT = 1; __VA_ARGS__; } break; \
+    case 2: { constexpr int VPT = 2; __VA_ARGS__; } break; \
+    default: { constexpr int VPT = 4; __VA_ARGS__; } break;\
+    }
 template <class Geo>
 static void launch_m2m(Geo geo, int64_t npar, int P, int nv, const float4 *tab, const float4 *Mc, float4 *Mp, cudaStream_t st)
 {
-    const int np = 2 * P + 1;
-    NV_DISPATCH(nv, {
-        constexpr int VPT = NV < 4 ? NV : 4;
-        const int thr = NV <= 4 ? round32(4 * np) : round32(np * ((nv + 3) / 4));
-        const size_t shm = NV <= 4 ? (size_t)3 * np * VPT * sizeof(float4) : 0;
-        k_m2m_dx<NV><<<(unsigned)npar, thr, shm, st>>>(geo, P, nv, tab, Mc, Mp);
+    const int np = 2 * P + 1, QS = shift_parts(np);
+    VPT_DISPATCH(nv, {
+        k_m2m_dx<VPT><<<dim3((unsigned)npar, (nv + VPT - 1) / VPT), round32(4 * QS * np), (size_t)(4 * QS - 1) * np * VPT * sizeof(float4),
+                        st>>>(geo, P, nv, QS, tab, Mc, Mp);
     });
 }
 template <class Geo>
 static void launch_l2l(Geo geo, int64_t npar, int P, int nv, const float4 *tab, const float4 *Lp, float4 *Lc, cudaStream_t st)
 {
-    const int np = 2 * P + 1;
-    NV_DISPATCH(nv, {
-        const int thr = std::min(512, round32(4 * np * ((nv + 3) / 4)));
-        k_l2l_dx<NV><<<(unsigned)npar, thr, 0, st>>>(geo, P, nv, tab, Lp, Lc);
+    const int np = 2 * P + 1, QS = shift_parts(np);
+    VPT_DISPATCH(nv, {
+        k_l2l_dx<VPT><<<dim3((unsigned)npar, (nv + VPT - 1) / VPT), round32(4 * QS * np), (size_t)(4 * QS - 4) * np * VPT * sizeof(float4),
+                        st>>>(geo, P, nv, QS, tab, Lp, Lc);
     });
 }
 static void launch_m2l(const M2LLevelDF *lev, int nlev, int64_t nblk, int P, int nv, cudaStream_t st)
