@@ -25,9 +25,9 @@
 static int gridn(int64_t n, int b) { return (int)((n + b - 1) / b); }
 __host__ __device__ constexpr int min_i(int a, int b) { return a < b ? a : b; }
 
-// threads of a block: 128, 256 for 16 vectors (two rows of targets a warp hold their sums in registers;
-// 250k strip: 2.46 ms, 3.08 ms with 128 threads and 8 targets a pass)
-__host__ __device__ constexpr int nd_threads(int nv, bool grad) { return !grad && nv == 16 ? 256 : 128; }
+// 16 vectors: 256 threads a block, the sums of a row spread over 4 warps (WIDE); else 128
+__host__ __device__ constexpr bool nd_wide(int nv, bool grad) { return !grad && nv == 16; }
+__host__ __device__ constexpr int nd_threads(int nv, bool grad) { return nd_wide(nv, grad) ? 256 : 128; }
 #define ND_ENT 64 // U entries a round
 #define ND_SRC 64 // near sources a round
 // targets of a block's pass: 16, 8 for the gradient, whose sums take three times the registers
@@ -311,12 +311,17 @@ __global__ void __launch_bounds__(nd_threads(NV, GRAD), GRAD ? 3 : 512 / nd_thre
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t u0 = ustart[b], u1 = ustart[b + 1];
     constexpr int ROWS = TG / (THR / 32), HALF = SRC / 32;
-    // Sums over the sources: 8 interleaved subsets whatever the number of vectors, so that a vector's
-    // result does not depend on how many others are applied with it.  A lane holds ACC subsets of
-    // vector v for LR of its warp's ROWS rows.
-    constexpr int SUB = 8, ACC = NV * SUB > 32 ? NV * SUB / 32 : 1, LS = SUB / ACC, RSTEP = min_i(ROWS, 32 / (NV * LS));
-    constexpr int LR = ROWS / RSTEP;
+    // Sums over the sources: 8 interleaved subsets whatever the number of vectors, added in the same
+    // order, so that a vector's result does not depend on how many others are applied with it.  A lane
+    // holds ACC subsets of vector v for LR of its warp's ROWS rows; WIDE (16 vectors): one subset of every
+    // second row, so that a leaf's rows are spread evenly over the warps whatever their number and a
+    // density is read once for up to 8 rows.
+    constexpr bool WIDE = nd_wide(NV, GRAD);
+    constexpr int SUB = 8, ACC = WIDE ? 1 : NV * SUB > 32 ? NV * SUB / 32 : 1, LS = WIDE ? 2 : SUB / ACC,
+                  RSTEP = WIDE ? 1 : min_i(ROWS, 32 / (NV * LS));
+    constexpr int LR = WIDE ? TG / 2 : ROWS / RSTEP;
     const int v = lane % NV, sub = (lane / NV) % LS, rh = lane / (NV * LS);
+    const int wg = warp & 3, wr = warp >> 2; // WIDE: subsets 2 wg + sub, rows wr + 2 r
     const bool on = rh < RSTEP; // one vector, 8 targets a pass: half the lanes have no row
     for (int64_t t0 = lo + (int64_t)blockIdx.y * tb; t0 < hi; t0 += (int64_t)gridDim.y * tb) {
         const int nt = (int)min((int64_t)tb, hi - t0);
@@ -469,6 +474,23 @@ __global__ void __launch_bounds__(nd_threads(NV, GRAD), GRAD ? 3 : 512 / nd_thre
                     for (int c = 0; c < SETS; ++c) g[c][row][s] = df_pack(G.A[c], G.J[c]);
                 }
                 __syncthreads();
+                if (WIDE) {
+                    for (int s0 = 2 * wg; s0 < ns; s0 += SUB) {
+                        const bool in = s0 + sub < ns;
+                        const int s = in ? s0 + sub : s0;
+                        const float4 q = in ? sq[s * NV + v] : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                        for (int r = 0; r < LR; ++r)
+                            if (wr + 2 * r < nt) {
+                                const float4 gg = g[0][wr + 2 * r][s];
+                                float4 &x = acA[0][r][0], &y = acJ[0][r][0];
+                                df_mac(x.x, x.y, gg.x, gg.y, q.x, q.y);
+                                df_mac(x.z, x.w, gg.x, gg.y, q.z, q.w);
+                                df_mac(y.x, y.y, gg.z, gg.w, q.x, q.y);
+                                df_mac(y.z, y.w, gg.z, gg.w, q.z, q.w);
+                            }
+                    }
+                } else
 #pragma unroll
                 for (int r = 0; r < LR; ++r) {
                     const int row = warp + (r * RSTEP + rh) * (THR / 32);
@@ -493,27 +515,43 @@ __global__ void __launch_bounds__(nd_threads(NV, GRAD), GRAD ? 3 : 512 / nd_thre
                 __syncthreads(); // sources and values are overwritten by the next round
             }
         }
+        // the subsets' sums: neighbours first
+        if (WIDE) {
+#pragma unroll
+            for (int r = 0; r < LR; ++r) {
+                const int row = wr + 2 * r;
+                if (row >= nt) break;
+                float4 a = df_norm(acA[0][r][0]), j = df_norm(acJ[0][r][0]);
+                a = dfc_add(a, shfl4(a, NV));
+                j = dfc_add(j, shfl4(j, NV));
+                if (sub == 0) {
+                    ur[(row * 4 + wg) * NV + v] = a;
+                    sq[(row * 4 + wg) * NV + v] = j;
+                }
+            }
+        } else
 #pragma unroll
         for (int r = 0; r < LR; ++r) {
             const int row = warp + (r * RSTEP + rh) * (THR / 32);
 #pragma unroll
-            for (int c = 0; c < SETS; ++c) { // the subsets' sums, halves first
+            for (int c = 0; c < SETS; ++c) {
                 float4 x[ACC], y[ACC];
 #pragma unroll
-                for (int i = 0; i < ACC; ++i) x[i] = df_norm(acA[c][r][i]), y[i] = df_norm(acJ[c][r][i]);
+                for (int i = 0; i < ACC; ++i) {
+                    x[i] = df_norm(acA[c][r][i]), y[i] = df_norm(acJ[c][r][i]);
 #pragma unroll
-                for (int h = ACC / 2; h > 0; h >>= 1)
-#pragma unroll
-                    for (int i = 0; i < h; ++i) x[i] = dfc_add(x[i], x[i + h]), y[i] = dfc_add(y[i], y[i + h]);
-                float4 a = x[0], j = y[0];
-#pragma unroll
-                for (int o = NV * LS / 2; o >= NV; o >>= 1) {
-                    a = dfc_add(a, shfl4(a, o));
-                    j = dfc_add(j, shfl4(j, o));
+                    for (int o = NV; o < NV * LS; o <<= 1) {
+                        x[i] = dfc_add(x[i], shfl4(x[i], o));
+                        y[i] = dfc_add(y[i], shfl4(y[i], o));
+                    }
                 }
+#pragma unroll
+                for (int h = 1; h < ACC; h <<= 1)
+#pragma unroll
+                    for (int i = 0; i < ACC; i += 2 * h) x[i] = dfc_add(x[i], x[i + h]), y[i] = dfc_add(y[i], y[i + h]);
                 if (on && row < nt && sub == 0) {
-                    ur[((row * SETS + c) * NV + v) * 2] = a;
-                    ur[((row * SETS + c) * NV + v) * 2 + 1] = j;
+                    ur[((row * SETS + c) * NV + v) * 2] = x[0];
+                    ur[((row * SETS + c) * NV + v) * 2 + 1] = y[0];
                 }
             }
         }
@@ -521,7 +559,15 @@ __global__ void __launch_bounds__(nd_threads(NV, GRAD), GRAD ? 3 : 512 / nd_thre
         const int ex = qexp_of(qexp);
         for (int i = tid; i < nt * nv * SETS; i += THR) {
             const int row = i % nt, vc = i / nt, vv = vc % nv, c = vc / nv;
-            const float4 a = ur[((row * SETS + c) * NV + vv) * 2], j = ur[((row * SETS + c) * NV + vv) * 2 + 1];
+            float4 a, j;
+            if (WIDE) {
+                const float4 *pa = ur + row * 4 * NV + vv, *pj = sq + row * 4 * NV + vv;
+                a = dfc_add(dfc_add(pa[0], pa[NV]), dfc_add(pa[2 * NV], pa[3 * NV]));
+                j = dfc_add(dfc_add(pj[0], pj[NV]), dfc_add(pj[2 * NV], pj[3 * NV]));
+            } else {
+                a = ur[((row * SETS + c) * NV + vv) * 2];
+                j = ur[((row * SETS + c) * NV + vv) * 2 + 1];
+            }
             const double f = -1.0 / (4.0 * M_PI);
             zd r = {f * df_double(df_re(a)) - 0.25 * df_double(df_im(j)), f * df_double(df_im(a)) + 0.25 * df_double(df_re(j))};
             r = zd{ldexp(r.re, ex), ldexp(r.im, ex)};

@@ -14,8 +14,8 @@
 // the tiles of a (row, parity) share one entry list (table slot, column offset dc, source
 // row).  A source outside the strip is a zero box: each row of split multipoles is padded.
 // One entry adds D_{i+j}[128 x R] += S_i[128 x K] T_j[R x K]^T over 15 digit pairs, with S
-// the sources, T the real-block table ([Re -Im; Im Re], rows 2 p + re / im) and
-// K = 2(2p+1) padded to 16.  R <= 96: five accumulators of R columns share the 512 columns
+// the sources, T the real-block table ([Re -Im; Im Re], rows and columns 2 n + re / im)
+// and K = 2(2p+1) padded to 16.  R <= 96: five accumulators of R columns share the 512 columns
 // of tensor memory; orders with more rows take two sweeps.  (Tables as the 128-row operand
 // against 64 columns, 38 of whose rows are padding at p = 22, read 6 KB of shared memory an
 // MMA for half the columns: 250k strip, 16 vectors, M2L, M2M and L2L 5.85 ms, 3.07 ms
@@ -133,8 +133,8 @@ __global__ void __launch_bounds__(256) k_oz_tsplit(const zd *tab, int64_t ncls, 
         const int k = 8 * c + i;
         double x = 0.0;
         if (row < 2 * np && k < 2 * np) {
-            const zd a = T[p * np + (k < np ? k : k - np)];
-            x = (im != 0) == (k >= np) ? a.re : (im ? a.im : -a.im);
+            const zd a = T[p * np + (k >> 1)];
+            x = im == (k & 1) ? a.re : (im ? a.im : -a.im);
         }
         x *= sc;
         for (int s = 0; s < OZ_S; ++s) {
@@ -192,9 +192,9 @@ __global__ void __launch_bounds__(256) k_oz_split(const OzLevel *lvs, int np, in
             const int k = 8 * c + j;
             float h = 0.f, l = 0.f;
             if (on && k < 2 * np) {
-                const float4 a = lv.M[(box * np + (k < np ? k : k - np)) * nv + v];
-                h = (k < np ? a.x : a.z) * sc;
-                l = (k < np ? a.y : a.w) * sc;
+                const float4 a = lv.M[(box * np + (k >> 1)) * nv + v];
+                h = (k & 1 ? a.z : a.x) * sc;
+                l = (k & 1 ? a.w : a.y) * sc;
             }
 #pragma unroll
             for (int s = 0; s < OZ_S; ++s) { // digits of h + l, exact
