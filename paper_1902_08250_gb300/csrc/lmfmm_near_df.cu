@@ -17,6 +17,7 @@
 // FP64 coordinates (the leaf-relative ones are good to 2^-49 of the leaf); pairs outside the
 // series' range (z > 1, or closer than 2^-45 in these units) take the FP64 functions.
 #include <algorithm>
+#include <type_traits>
 
 #include "df.cuh"
 #include "internal.h"
@@ -30,7 +31,8 @@ __host__ __device__ constexpr bool nd_wide(int nv, bool grad) { return !grad && 
 __host__ __device__ constexpr int nd_threads(int nv, bool grad) { return nd_wide(nv, grad) ? 256 : 128; }
 #define ND_ENT 64 // U entries a round
 #define ND_SRC 64 // near sources a round
-// targets of a block's pass: 16, 8 for the gradient, whose sums take three times the registers
+// targets of a block's pass: 16, 8 for the gradient, whose sums take three times the registers; up to 2
+// vectors twice as many on large uniform trees whose leaves hold more than that (launch_near)
 __host__ __device__ constexpr int nd_tgt(int nv, bool grad) { return grad ? 8 : 16; }
 
 // (A, J) and their z-derivatives (target gradient): A' = J/z + (ln z + 2 gamma) J' + 2 V'
@@ -284,13 +286,13 @@ __device__ __noinline__ void seg_df_grad(const DfSmem &tab, const NearDF &q, int
 // source into shared memory, then summed with a lane per (source subset, vector).
 // Bound by FP32 issue (free pairs about 250 instructions, tails 170 per node, 48
 // per complex multiply-add).
-template <int NV, int D, int T, bool GRAD, class Geo>
+template <int NV, int D, int T, bool GRAD, int TG, class Geo>
 __global__ void __launch_bounds__(nd_threads(NV, GRAD), GRAD ? 3 : 512 / nd_threads(NV, GRAD))
     k_near_df(Geo geo, double k, double kap, const double *xs, const double *ys, const int64_t *ls, const float4 *rel,
               const float4 *hgt, const int64_t *ustart, const int32_t *usrc, const int32_t *uterm, NearDF nq,
               const float4 *qd, int nvq, const int *qexp, int64_t n, int nv, int tb, int free_on, zd *us, GradOut go)
 {
-    constexpr int SETS = GRAD ? 3 : 1, TG = nd_tgt(NV, GRAD), SRC = GRAD ? 32 : ND_SRC, THR = nd_threads(NV, GRAD);
+    constexpr int SETS = GRAD ? 3 : 1, SRC = GRAD ? 32 : ND_SRC, THR = nd_threads(NV, GRAD);
     __shared__ DfSmem tab;
     __shared__ int64_t fj0[ND_ENT];
     __shared__ int fpre[ND_ENT + 1], fterm[ND_ENT];
@@ -788,9 +790,14 @@ static void launch_near(lm_tree_s *t, Geo geo, int64_t nleaf, int nvq, int nv, c
     const NearDF nq{q.nray, GRAD ? q.ntail_g : q.ntail, imp ? 1 : 0, q.a_zero ? 1 : 0, GRAD ? N.node_g : N.node,
                     GRAD ? N.w_g : N.w, GRAD ? N.w2_g : N.w2, df{(float)(2.0 * t->med.d * kap), 0.f},
                     (float)(q.hray * kap), {q.rinf[0], q.rinf[1]}, q.nseg, N.seg, N.segw_g, {q.beta[0], q.beta[1]}};
-    // targets a pass: 16 (8), fewer while that leaves fewer than 4 blocks per SM (small trees)
+    // targets a pass: TG or, where a leaf holds more and they fill 4 blocks per SM, 2 TG (a pass stages every
+    // near source: 200k uniform points with 19 a leaf, 1 vector 531 us with 16, 458 us with 32; gradient of 2
+    // 1.93 and 1.83 ms with 8 and 16; adaptive 100k, whose leaves hold fewer, 797 and 849 us); fewer while
+    // that leaves fewer than 4 blocks per SM (small trees)
     const int64_t per = std::max<int64_t>(1, (t->n + nleaf - 1) / nleaf);
-    int tb = nd_tgt(NV, GRAD);
+    constexpr int TG = nd_tgt(NV, GRAD), TW = NV <= 2 && std::is_same<Geo, GridLeaves>::value ? 2 * TG : TG;
+    const bool wide = TW > TG && per > TG && nleaf * ((per + TW - 1) / TW) >= 608;
+    int tb = wide ? TW : TG;
     while (tb > 4 && nleaf * ((per + tb - 1) / tb) < 608) tb >>= 1;
     const unsigned gy = (unsigned)std::min<int64_t>(64, (per + tb - 1) / tb);
     const size_t shm = (size_t)(GRAD ? 32 : ND_SRC) * NV * sizeof(float4);
@@ -800,8 +807,8 @@ static void launch_near(lm_tree_s *t, Geo geo, int64_t nleaf, int nvq, int nv, c
                                                                  N.hgt, t->ustart, t->usrc, t->uterm, nq, N.q, nvq, t->qexp,
                                                                  t->n, nv, tb, free_on, t->us, go);
     };
-    if (N.zmax <= 1.0 / 16.0) run(k_near_df<NV, 4, 7, GRAD, Geo>);
-    else run(k_near_df<NV, 7, 12, GRAD, Geo>);
+    if (N.zmax <= 1.0 / 16.0) wide ? run(k_near_df<NV, 4, 7, GRAD, TW, Geo>) : run(k_near_df<NV, 4, 7, GRAD, TG, Geo>);
+    else wide ? run(k_near_df<NV, 7, 12, GRAD, TW, Geo>) : run(k_near_df<NV, 7, 12, GRAD, TG, Geo>);
 }
 template <int NV, class Geo>
 static void launch_pw(lm_tree_s *t, Geo geo, int64_t npw, int nv, cudaStream_t st)
