@@ -165,6 +165,11 @@ struct AdaptTree {
     int32_t *parent = nullptr, *pos = nullptr;         // [nbox] parent id (-1 for roots), child position
     int32_t *child = nullptr;                          // [nbox][4] (-1 for leaves)
     int32_t *leaves = nullptr, *nonleaf = nullptr, *pwleaves = nullptr; // box id lists
+    // mixed form, one vector: V entries sorted by class (lmfmm_few32.cu)
+    void *cls_tiles = nullptr;
+    int32_t *cls_src = nullptr, *cls_pos = nullptr; // [nv] source box, place in the slice's products
+    zf *cls_C = nullptr, *cls_M = nullptr;          // products of a slice [entries][2p+1]; multipoles [nbox][2p+1]
+    std::vector<int64_t> cls_slices;                // 5 numbers each (ClsSlice); empty: not used
     std::vector<int32_t> hpw;                          // host copy of pwleaves
     int64_t nv = 0;
     std::vector<int64_t> lev_nv;                       // [L + 1] V entries of the targets of level l
@@ -389,7 +394,7 @@ lm_status lm_run_apply_mixed(lm_tree_s *t, const void *q, int nvec, void *u, boo
 struct NearQuadF;
 lm_status lm_setup_few32(lm_tree_s *t, cudaStream_t st);
 void lm_few32_s2m(lm_tree_s *t, int nv, cudaStream_t st);
-void lm_few32_m2l(lm_tree_s *t, int nv, cudaStream_t st);
+int lm_few32_m2l(lm_tree_s *t, int nv, cudaStream_t st);
 int lm_few32_leaf(lm_tree_s *t, const NearQuadF &nq, int nv, cudaStream_t st);
 // tensor-core M2L (lmfmm_tc.cu)
 lm_status lm_setup_tc(lm_tree_s *t, cudaStream_t st);

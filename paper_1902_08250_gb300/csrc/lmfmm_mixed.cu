@@ -1364,8 +1364,7 @@ static lm_status run_mixed_adaptive(lm_tree_s *t, const void *q, int nvec, void 
         if (L > 0) lm_phase_end(t, PH_M2M, st, L);
         if (few) { // M2L of every level at once, then L2L adds
             lm_phase_begin(t, PH_M2L, st);
-            lm_few32_m2l(t, nv, st);
-            lm_phase_end(t, PH_M2L, st, 1);
+            lm_phase_end(t, PH_M2L, st, lm_few32_m2l(t, nv, st));
             if (L > 0) lm_phase_begin(t, PH_L2L, st);
             for (int l = 1; l <= L; ++l) MX_DISPATCH(P, launch_l2l_list_acc, A, t->lev[l], l, st);
             if (L > 0) lm_phase_end(t, PH_L2L, st, L);

@@ -170,8 +170,10 @@ __global__ void __launch_bounds__(256) k_oz_mmax(const OzLevel *lvs, int np, int
     __syncthreads();
     if ((int)threadIdx.x < nv && s[threadIdx.x]) atomicMax(&lv.mmax[threadIdx.x], s[threadIdx.x]);
 }
-// one thread per (plane, row of it, 8-wide K chunk): 8 orders of a (box, vector) into 5 digit
-// planes; the padding boxes and vectors beyond nv are written as zeros
+// one thread per (plane, row of it, 8-wide K chunk): 4 orders of a (box, vector) into 5 digit
+// planes; the padding boxes and vectors beyond nv are written as zeros.  Bound by memory: 250k strip,
+// 16 vectors, all levels 0.18 ms (0.27 ms with the real parts of all orders first, which reads each
+// component twice)
 __global__ void __launch_bounds__(256) k_oz_split(const OzLevel *lvs, int np, int nv, int nvs)
 {
     const OzLevel &lv = lvs[blockIdx.y];

@@ -154,6 +154,15 @@ def test_few_vector_mixed_kernels(lm, name, nvec):
     assert _rel(_apply(lm, t, q.astype(np.complex64)), ref) <= 1e-6
 
 
+@pytest.mark.parametrize("n, p", [(20_000, 14), (20_000, 24), (250_000, 8)])
+def test_adaptive_m2l_by_classes(lm, n, p):
+    """One vector (V entries by class; one slice and several) against two (a block per target box)."""
+    x, y, q = workloads.uniform_strip(n, 0.0, 9.9, -0.99, -0.01, nvec=2, seed=p)
+    q = q.astype(np.complex64)
+    t = _tree(lm, A, x, y, precision="mixed", p=p, adaptive=True, leaf_target=16)
+    assert _rel(_apply(lm, t, q[:1])[0], _apply(lm, t, q)[0]) <= 1e-6
+
+
 @pytest.mark.parametrize("n", [1, 40, 270, 1100, 2100, 4000])
 @pytest.mark.parametrize("band", [(-0.95, -0.05), (-1.0 + 1e-6, -1e-6)])
 def test_tensor_core_leaf_tiles(lm, n, band):
