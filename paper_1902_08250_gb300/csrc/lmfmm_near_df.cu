@@ -792,15 +792,17 @@ static void launch_near(lm_tree_s *t, Geo geo, int64_t nleaf, int nvq, int nv, c
     const NearDF nq{q.nray, GRAD ? q.ntail_g : q.ntail, imp ? 1 : 0, q.a_zero ? 1 : 0, GRAD ? N.node_g : N.node,
                     GRAD ? N.w_g : N.w, GRAD ? N.w2_g : N.w2, df{(float)(2.0 * t->med.d * kap), 0.f},
                     (float)(q.hray * kap), {q.rinf[0], q.rinf[1]}, q.nseg, N.seg, N.segw_g, {q.beta[0], q.beta[1]}};
-    // targets a pass: TG or, where a leaf holds more and they fill 4 blocks per SM, 2 TG (a pass stages every
-    // near source: 200k uniform points with 19 a leaf, 1 vector 531 us with 16, 458 us with 32; gradient of 2
-    // 1.93 and 1.83 ms with 8 and 16; adaptive 100k, whose leaves hold fewer, 797 and 849 us); fewer while
-    // that leaves fewer than 4 blocks per SM (small trees)
+    // targets a pass: TG or, where a leaf holds more and they leave 8 waves of 4 blocks per SM, 2 TG (a pass
+    // stages every near source: 200k uniform points with 19 a leaf, 1 vector 531 us with 16, 458 us with 32;
+    // gradient of 2 1.93 and 1.83 ms with 8 and 16; 30k points, 2.5 waves, 138 and 151 us; adaptive 100k, whose
+    // leaves hold fewer, 797 and 849 us); fewer while that leaves fewer than 4 blocks per SM (small trees), down
+    // to an item of kernel values a warp (2 rows x 2 halves of the sources, 4 rows for the gradient; 1000
+    // points 116 us with 4, 75 us with 2)
     const int64_t per = std::max<int64_t>(1, (t->n + nleaf - 1) / nleaf);
     constexpr int TG = nd_tgt(NV, GRAD), TW = NV <= 2 && std::is_same<Geo, GridLeaves>::value ? 2 * TG : TG;
-    const bool wide = TW > TG && per > TG && nleaf * ((per + TW - 1) / TW) >= 608;
+    const bool wide = TW > TG && per > TG && nleaf * ((per + TW - 1) / TW) >= 4864;
     int tb = wide ? TW : TG;
-    while (tb > 4 && nleaf * ((per + tb - 1) / tb) < 608) tb >>= 1;
+    while (tb > (GRAD ? 4 : 2) && nleaf * ((per + tb - 1) / tb) < 608) tb >>= 1;
     const unsigned gy = (unsigned)std::min<int64_t>(64, (per + tb - 1) / tb);
     const size_t shm = (size_t)(GRAD ? 32 : ND_SRC) * NV * sizeof(float4);
     const int free_on = t->med.opt.kernel == LM_KERNEL_G;

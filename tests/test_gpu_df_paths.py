@@ -53,8 +53,8 @@ NEAR = {
     "short_series": (A, 3000, 3.0, (-0.95, -0.05), 5, dict(p=20, depth=4)),     # z <= 1/16
     "leaf_of_17": (A, 17, 0.9, (-0.9, -0.1), 16, dict(p=20, depth=0)),          # one past a pass of targets
     "leaf_of_65": (A, 65, 0.9, (-0.9, -0.1), 8, dict(p=20, depth=0)),           # one past a round of sources
-    "wide_pass": (A, 30000, 3.0, (-0.95, -0.05), 1, dict(p=20, depth=4)),       # 39 points a leaf, passes of 32
-    "wide_pass_two": (A, 14000, 9.0, (-0.95, -0.05), 2, dict(p=20, depth=3)),
+    "wide_pass": (A, 100_000, 4.9, (-0.95, -0.05), 1, dict(p=20, depth=5)),     # 20 points a leaf, passes of 32
+    "wide_pass_two": (A, 180_000, 4.9, (-0.95, -0.05), 2, dict(p=20, depth=5)), # 35 points: two passes
     "low_order": (A, 500, 2.0, (-0.9, -0.1), 4, dict(p=1, depth=2)),
     "high_order": (A, 500, 2.0, (-0.9, -0.1), 16, dict(p=48, depth=1)),
     "interface": (A, 1500, 2.0, (-0.02, -1e-7), 11, dict(p=20, depth=3)),
