@@ -447,10 +447,13 @@ lm_status lm_misfit_grad(lm_tree t, lm_tree dtree, const void *q, const void *g,
  * FMM with two wave numbers: multipoles in k1 about the source boxes, local
  * expansions in k2 about the target boxes (Sec. 2.1), on a source and a target
  * tree sharing one lattice of d x d roots.  The medium must have kernel
- * LM_KERNEL_G and transmission interfaces.  Precision LM_FP64: every step in
- * FP64.  LM_MIXED: tables and near-field quadrature built in FP64; expansions,
+ * LM_KERNEL_G and transmission interfaces.  Tables and the near-field
+ * quadrature are built in FP64.  LM_FP64: every step of an apply in
+ * double-float (see lm_options.m2l_fp64; 3e-14 to 6e-14 relative l2 from the
+ * IEEE form), or in IEEE FP64 with m2l_fp64 = 1.  LM_MIXED: expansions,
  * translations and multiply-adds in FP32 (tables rounded once), near kernel
- * values evaluated in FP64 and rounded.
+ * values evaluated to about 1e-13 and rounded to FP32; results are FP32
+ * numbers, 2e-7 to 3e-7 relative l2 from the sum at p = 14 to 18.
  *   build_cross: xs, ys (device, [ns]) sources with 0 < ys < d; xt, yt
  *     (device, [nt]) targets with -d < yt < 0.  Copies what it needs.
  *   cross_apply: q device complex128 [nvec][ns]; u device complex128 [nvec][nt].

@@ -18,7 +18,8 @@
 // Precision: LM_FP64 builds tables and quadratures in FP64 and runs every step of an
 // apply in double-float on the FP32 pipes (lmfmm_exp_df.cu's expansions and
 // k_cross_near_df), or in IEEE FP64 with opt.m2l_fp64.  LM_MIXED keeps FP32 copies
-// of the tables; its expansions and translations are FP32, its near pairs as above.
+// of the tables; its expansions, translations and multiply-adds are FP32, its near kernel
+// values come from the double-float quadrature (about 1e-13) and are rounded to FP32.
 #include <algorithm>
 #include <map>
 #include <tuple>
@@ -86,7 +87,7 @@ struct lm_cross_s {
     zd *qs, *us; // [LM_MAXV][ns], [LM_MAXV][nt]
     // double-float near pairs (unless opt.m2l_fp64) and expansions (xdf)
     bool ndf, xdf;
-    float4 *qdf;                                       // [ns][nvec] densities scaled by 2^-qexp
+    float4 *qdf;                                       // [ns][nvec] densities scaled by 2^-qexp (FP64 form)
     int *qexp;
     float4 *seg_node, *seg_wdf, *tail_node, *tail_wdf; // quadrature of the near pairs (k_cross_tab)
     float4 *rel_s, *rel_t;                             // [n] offsets from the leaf centres times k1/2, k2/2
@@ -266,7 +267,15 @@ __device__ zd cross_near(const CrossNear &q, double k2, double X, double y, doub
 // 12.4 ms, of which the near pairs nearly all).
 // Node tables: lambda, s2 and s1 as (exponent, phase) coefficients in df_cexp's units; weights
 // of the two exponentials, complex (segment) or as P and iM of P Re(E) + i M Im(E) (tail).
+// The mixed form (F32) sums a pair's parts over the lanes, rounds the kernel value to FP32 and
+// multiplies in FP32, lane v for vector v: a source leaf summed on its own, then added to the
+// L2T value, so its results are FP32 numbers that do not depend on the split over the lanes.
 // ---------------------------------------------------------------------------
+__device__ __forceinline__ void cfma32(zf &a, zf b, zf c)
+{
+    a.re = fmaf(b.re, c.re, fmaf(-b.im, c.im, a.re));
+    a.im = fmaf(b.re, c.im, fmaf(b.im, c.re, a.im));
+}
 __global__ void k_cross_tab(int n, const zd *lam, const zd *s1, const zd *s2, const zd *w, int tail, float4 *node, float4 *wt)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -298,11 +307,12 @@ __device__ __forceinline__ df dot3(df a, df x, df b, df y, df c, df z)
     df_mac(s, c, z);
     return quick_two_sum(s.h, s.l);
 }
-template <int NV>
+template <int NV, bool F32>
 __global__ void __launch_bounds__(128) k_cross_near_df(double k2, const double *xt, const double *yt, const int64_t *lt,
                                                        const int64_t *ustart, const int32_t *usrc, const double *xs,
                                                        const double *ysm, const int64_t *lsrc, CrossNearDF nq,
-                                                       const float4 *qd, const int *qexp, int64_t nt, int nv, zd *us)
+                                                       const float4 *qd, const int *qexp, const zd *qs, int64_t ns,
+                                                       int64_t nt, int nv, zd *us)
 {
     __shared__ DfSmem tab;
     const int64_t b = blockIdx.x, lo = lt[b], hi = lt[b + 1];
@@ -317,8 +327,14 @@ __global__ void __launch_bounds__(128) k_cross_near_df(double k2, const double *
         float4 acc[NV];
 #pragma unroll
         for (int v = 0; v < NV; ++v) acc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
+        zf sum = {0.f, 0.f}; // F32, lane v < nv: the L2T value (FP32 numbers), then the leaves' sums
+        if (F32 && lane < nv) {
+            const zd o = us[(int64_t)lane * nt + i];
+            sum = zf{(float)o.re, (float)o.im};
+        }
         for (int64_t e = ustart[b]; e < ustart[b + 1]; ++e) {
             const int32_t s = usrc[e];
+            zf part = {0.f, 0.f};
             for (int64_t j0 = lsrc[s]; j0 < lsrc[s + 1]; j0 += 32) {
                 const int cnt = (int)min((int64_t)32, lsrc[s + 1] - j0);
                 // lane j: source j's offset, height and closed-form part (i/4) H0(k2 R)
@@ -366,11 +382,24 @@ __global__ void __launch_bounds__(128) k_cross_near_df(double k2, const double *
                         }
                     }
                     g = df_norm(g);
+                    if (F32) {
+                        const zf g32 = {df_warp_sum(df_re(g)).h, df_warp_sum(df_im(g)).h}; // hi + lo rounded to FP32
+                        if (lane < nv) {
+                            const zd q = qs[(int64_t)lane * ns + j0 + j];
+                            cfma32(part, g32, zf{(float)q.re, (float)q.im});
+                        }
+                        continue;
+                    }
 #pragma unroll
                     for (int v = 0; v < NV; ++v)
                         if (v < nv) dfc_mac(acc[v], g, qd[(j0 + j) * nv + v]);
                 }
             }
+            sum = sum + part;
+        }
+        if (F32) {
+            if (lane < nv) us[(int64_t)lane * nt + i] = zd{sum.re, sum.im};
+            continue;
         }
         const int ex = qexp_of(qexp);
 #pragma unroll
@@ -445,12 +474,6 @@ __global__ void k_cross_to32(const zd *a, int64_t n, zf *b)
 {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i < n) b[i] = zf{(float)a[i].re, (float)a[i].im};
-}
-
-__device__ __forceinline__ void cfma32(zf &a, zf b, zf c)
-{
-    a.re = fmaf(b.re, c.re, fmaf(-b.im, c.im, a.re));
-    a.im = fmaf(b.re, c.im, fmaf(b.im, c.re, a.im));
 }
 
 #define CROSS32_CHUNK 32
@@ -570,12 +593,9 @@ __global__ void k_cross_m2l32(int64_t nbox, int P, int nvec, const int64_t *vsta
     Lc[(b * np + p) * LM_MAXV + v] = Lc[(b * np + p) * LM_MAXV + v] + acc;
 }
 
-// L2T in k2 (FP32) and the near g_2^t pairs (kernel values from the FP64 quadrature,
-// multiply-adds in FP32), one thread per target of a leaf
+// L2T in k2 (FP32), one thread per target of a leaf; k_cross_near_df adds the near g_2^t pairs
 __global__ void k_cross_leaf32(LeafGeom g, int P, double k2, const double *xt, const double *yt, const int64_t *lt,
-                               const int64_t *ustart, const int32_t *usrc, const double *xs, const double *ysm,
-                               const int64_t *lsrc, CrossNear nq, const zf *Lc, const zd *qs, int64_t ns,
-                               int64_t nt, int nvec, int near, zd *us)
+                               const zf *Lc, int64_t nt, int nvec, zd *us)
 {
     const int np = 2 * P + 1;
     const int64_t b = blockIdx.x;
@@ -602,20 +622,6 @@ __global__ void k_cross_leaf32(LeafGeom g, int P, double k2, const double *xt, c
                     cfma32(acc[v], bn, Lb[(P - m) * LM_MAXV + v]);
                 }
             }
-        }
-        for (int64_t e = ustart[b]; near && e < ustart[b + 1]; ++e) {
-            const int32_t s = usrc[e];
-            zf part[LM_MAXV]; // one source leaf summed on its own
-            for (int v = 0; v < nvec; ++v) part[v] = zf{0.f, 0.f};
-            for (int64_t j = lsrc[s]; j < lsrc[s + 1]; ++j) {
-                const zd gd = cross_near(nq, k2, fabs(xi - xs[j]), yi, -ysm[j]);
-                const zf gij = {(float)gd.re, (float)gd.im};
-                for (int v = 0; v < nvec; ++v) {
-                    const zd qd = qs[(int64_t)v * ns + j];
-                    cfma32(part[v], gij, zf{(float)qd.re, (float)qd.im});
-                }
-            }
-            for (int v = 0; v < nvec; ++v) acc[v] = acc[v] + part[v];
         }
         for (int v = 0; v < nvec; ++v) us[(int64_t)v * nt + i] = zd{acc[v].re, acc[v].im};
     }
@@ -900,8 +906,10 @@ static lm_status cross_setup(lm_cross_s *c, const double *xs, const double *ys, 
     c->xdf = c->med.opt.precision == LM_FP64 && !c->med.opt.m2l_fp64 && lm_exp_df_fits(k1, wl) && lm_exp_df_fits(k2, wl);
     if (c->ndf) {
         const int nt = c->nray * c->ntail;
-        CTRY(calloc_dev(c, &c->qdf, (size_t)LM_MAXV * c->ns));
-        CTRY(calloc_dev(c, &c->qexp, 1));
+        if (c->med.opt.precision == LM_FP64) {
+            CTRY(calloc_dev(c, &c->qdf, (size_t)LM_MAXV * c->ns));
+            CTRY(calloc_dev(c, &c->qexp, 1));
+        }
         CTRY(calloc_dev(c, &c->seg_node, 3 * c->nseg));
         CTRY(calloc_dev(c, &c->seg_wdf, 2 * c->nseg));
         CTRY(calloc_dev(c, &c->tail_node, 3 * nt));
@@ -1036,12 +1044,13 @@ static void cross_near_df(lm_cross_s *c, int nv, cudaStream_t st)
     const dim3 g((unsigned)lv.ncol, (unsigned)std::max<int64_t>(1, std::min<int64_t>(16, 1216 / lv.ncol)));
     auto run = [&](auto kern) {
         kern<<<g, 128, 0, st>>>(c->med.k2, c->xs_t, c->ys_t, c->ls_t, c->ustart, c->usrc, c->xs_s, c->ys_s, c->ls_s, nq, c->qdf,
-                                c->qexp, c->nt, nv, c->us);
+                                c->qexp, c->qs, c->ns, c->nt, nv, c->us);
     };
-    if (nv == 1) run(k_cross_near_df<1>);
-    else if (nv == 2) run(k_cross_near_df<2>);
-    else if (nv <= 4) run(k_cross_near_df<4>);
-    else run(k_cross_near_df<16>);
+    if (c->med.opt.precision == LM_MIXED) run(k_cross_near_df<1, true>); // a lane per vector
+    else if (nv == 1) run(k_cross_near_df<1, false>);
+    else if (nv == 2) run(k_cross_near_df<2, false>);
+    else if (nv <= 4) run(k_cross_near_df<4, false>);
+    else run(k_cross_near_df<16, false>);
 }
 
 extern "C" lm_status lm_cross_apply(lm_cross c, const void *q, int nvec, void *u, void *stream)
@@ -1064,7 +1073,7 @@ extern "C" lm_status lm_cross_apply(lm_cross c, const void *q, int nvec, void *u
     for (int v0 = 0; v0 < nvec; v0 += LM_MAXV) {
         const int nv = std::min(LM_MAXV, nvec - v0);
         k_permute_in<<<gridc(c->ns, 256), 256, 0, st>>>(qd + (int64_t)v0 * c->ns, c->perm_s, c->ns, nv, 0, c->qs);
-        if (c->ndf || c->xdf) {
+        if (c->ndf && c->med.opt.precision == LM_FP64) {
             LM_CUDA(cudaMemsetAsync(c->qexp, 0x80, sizeof(int), st)); // below any exponent
             k_qexp<<<std::min(1024, gridc(c->ns * nv, 256)), 256, 0, st>>>(c->qs, c->ns, nv, c->qexp);
             k_q_df<<<gridc(c->ns * nv, 256), 256, 0, st>>>(c->qs, c->ns, nv, c->qexp, c->qdf);
@@ -1111,8 +1120,7 @@ extern "C" lm_status lm_cross_apply(lm_cross c, const void *q, int nvec, void *u
             }
             const CrossLevel &lv = c->lev[L];
             k_cross_leaf32<<<(unsigned)lv.nbox, 64, 0, st>>>(LeafGeom{lv.ncol, c->x0, lv.w}, P, c->med.k2, c->xs_t,
-                                                             c->ys_t, c->ls_t, c->ustart, c->usrc, c->xs_s, c->ys_s,
-                                                             c->ls_s, nq, lv.L32, c->qs, c->ns, c->nt, nv, !c->ndf, c->us);
+                                                             c->ys_t, c->ls_t, lv.L32, c->nt, nv, c->us);
             cross_near_df(c, nv, st);
             k_permute_out<<<gridc(c->nt, 256), 256, 0, st>>>(c->us, c->perm_t, c->nt, nv, 0, ud + (int64_t)v0 * c->nt);
             LM_CUDA(cudaGetLastError());
