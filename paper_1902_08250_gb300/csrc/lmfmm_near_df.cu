@@ -639,15 +639,16 @@ __global__ void __launch_bounds__(256) k_pw_src_df(Geo geo, int nseg, const floa
     }
 }
 
+#define PW_WARPS 8 // of a block of k_near_pw_df
 template <int NV, class Geo>
-__global__ void __launch_bounds__(256) k_near_pw_df(Geo geo, double kap, int nseg, const float4 *node, const float4 *wt,
+__global__ void __launch_bounds__(32 * PW_WARPS) k_near_pw_df(Geo geo, double kap, int nseg, const float4 *node, const float4 *wt,
                                                     const float4 *rel, const float4 *hgt, const int64_t *ls,
                                                     const int64_t *ustart, const int32_t *usrc, const int32_t *uterm,
                                                     const float4 *C, const int32_t *pwidx, const int *qexp, int64_t n,
                                                     int nv, zd *us)
 {
     __shared__ DfSmem tab;
-    __shared__ float4 ur[8][NV];
+    __shared__ float4 ur[PW_WARPS][NV];
     extern __shared__ float4 B[]; // [nk][nv]
     const int nk = 2 * nseg;
     const int64_t b = geo.id(blockIdx.x), lo = ls[b], hi = ls[b + 1];
@@ -768,9 +769,10 @@ lm_status lm_setup_near_df(lm_tree_s *t, cudaStream_t st)
         k_tail_tab_grad<<<gridn(tg, 64), 64, 0, st>>>(tg, q.tail_lam_g, q.tail_s2_g, q.tail_w2_g, nullptr, N.w2_g);
     k_seg_tab_grad<<<gridn(q.nseg, 64), 64, 0, st>>>(q.nseg, q.seg_lam, q.seg_s2, q.seg_w, q.seg_c, N.segw_g);
     LM_CUDA(cudaGetLastError());
-    // one limit for every tree: raised, never lowered under another tree's launch
+    // one limit for every tree: raised, never lowered under another tree's launch.  A launch asks for the
+    // dynamic part (largest at 16 vectors) and k_near_pw_df's own arrays; 48 KB need no attribute
     const int lim = 200 * 1024;
-    if (lm_near_pw64_smem(q.nseg) > 40 * 1024) {
+    if (lm_near_pw64_smem(q.nseg) + sizeof(DfSmem) + PW_WARPS * LM_MAXV * sizeof(float4) > 48 * 1024) {
         const void *f[] = {(const void *)k_near_pw_df<1, EdgeRowLeaves>, (const void *)k_near_pw_df<2, EdgeRowLeaves>,
                            (const void *)k_near_pw_df<4, EdgeRowLeaves>, (const void *)k_near_pw_df<8, EdgeRowLeaves>,
                            (const void *)k_near_pw_df<16, EdgeRowLeaves>, (const void *)k_near_pw_df<1, ListBoxes>,
@@ -823,7 +825,7 @@ static void launch_pw(lm_tree_s *t, Geo geo, int64_t npw, int nv, cudaStream_t s
     k_pw_src_df<NV><<<(unsigned)npw, 256, 0, st>>>(geo, nseg, N.seg, N.rel, N.hgt, t->leaf_start, t->ustart, t->uterm, N.q,
                                                    nv, (float4 *)t->pwC);
     const size_t shm = (size_t)2 * nseg * nv * sizeof(float4);
-    k_near_pw_df<NV><<<(unsigned)npw, 256, shm, st>>>(geo, kap, nseg, N.seg, N.segw, N.rel, N.hgt, t->leaf_start, t->ustart,
+    k_near_pw_df<NV><<<(unsigned)npw, 32 * PW_WARPS, shm, st>>>(geo, kap, nseg, N.seg, N.segw, N.rel, N.hgt, t->leaf_start, t->ustart,
                                                       t->usrc, t->uterm, (const float4 *)t->pwC, t->pwidx, t->qexp, t->n,
                                                       nv, t->us);
 }
