@@ -192,11 +192,11 @@ struct NearTabDF {
     float4 *node, *w, *w2;  // tail nodes [ray][node][2], weights [term][ray][node][2] (w2: see NearQuad::split)
     float4 *seg, *segw;     // segment nodes [node][2], weights [term][node]
     float4 *rel, *hgt;      // [n] offset from the leaf centre; y and y + d
-    float4 *q;              // [n][nvec] densities of the apply, scaled by 2^-qexp
+    float4 *q;              // [n][nvec] densities of the apply, scaled by 2^-qexp[vector]
     float4 *node_g, *w_g, *w2_g, *segw_g; // target gradient: its tails and per-pair segment weights
 };
 // Double-float expansions of the FP64 form (lmfmm_exp_df.cu): the M and Lc arrays then hold float4
-// (re hi, re lo, im hi, im lo) scaled by 2^-qexp, [box][2p+1][nvec]
+// (re hi, re lo, im hi, im lo) scaled by 2^-qexp[vector], [box][2p+1][nvec]
 // Series and recurrence coefficients of the basis (device, double-floats): c[n] = 1/(n (n+1)), n = 1..N, at
 // [n]; then 1/(m (N+m)) and 1/(m (N+1+m)), m = 1..nt, at [N + m] and [N + nt + m]
 struct BesselDF {
@@ -306,7 +306,7 @@ struct lm_tree_s {
     ExpDF xdf;
     OzData oz;
     LmArena mem, tmp; // the tree's arrays; temporaries of its build
-    int *qexp;   // device: binary exponent of the largest |density| component of the apply
+    int *qexp;   // device [LM_MAXV]: binary exponent of each vector's largest |density| component of the apply
     int64_t bytes;
     // phase profiling
     int prof_max, prof_used;
@@ -360,7 +360,7 @@ lm_status lm_setup_pwsrc(lm_tree_s *t, cudaStream_t st); // interface-leaf slots
 lm_status lm_setup_pwidx(lm_tree_s *t, int64_t *npw, cudaStream_t st);
 lm_status lm_setup_df(lm_tree_s *t, cudaStream_t st); // the FP64 form's double-float data
 lm_status lm_setup_near_df(lm_tree_s *t, cudaStream_t st); // double-float near field (lmfmm_near_df.cu)
-void lm_launch_q_df(lm_tree_s *t, int nv, cudaStream_t st);
+lm_status lm_launch_q_df(const zd *qs, int64_t n, int nv, int *qexp, float4 *q, cudaStream_t st); // (lmfmm_apply.cu)
 lm_status lm_launch_near_df(lm_tree_s *t, int nv, cudaStream_t st, int *launches);
 lm_status lm_launch_near_grad_df(lm_tree_s *t, int nvq, int v0, int nv, zd *u, zd *ux, zd *uy, cudaStream_t st);
 lm_status lm_launch_near64(lm_tree_s *t, int v0, int nv, zd *u, zd *ux, zd *uy, cudaStream_t st);

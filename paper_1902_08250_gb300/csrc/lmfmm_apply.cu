@@ -205,11 +205,13 @@ __global__ void k_m2l64(int64_t nbox, int P, int nvec, const int64_t *vstart, co
     Lc[(b * np + p) * LM_MAXV + v] += acc;
 }
 
-// largest |re|, |im| of the densities [nvec][n] -> its binary exponent, max-reduced into *qexp
-__global__ void k_qexp(const zd *qs, int64_t n, int nvec, int *qexp)
+// largest |re|, |im| of each vector of the densities [nvec][n] -> its binary exponent, max-reduced into
+// qexp[vector]; gridDim.y = nvec
+__global__ void k_qexp(const zd *qs, int64_t n, int *qexp)
 {
+    qs += blockIdx.y * n;
     double mx = 0.0;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n * nvec; i += (int64_t)gridDim.x * blockDim.x) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const zd a = qs[i];
         mx = fmax(mx, fmax(fabs(a.re), fabs(a.im)));
     }
@@ -217,8 +219,17 @@ __global__ void k_qexp(const zd *qs, int64_t n, int nvec, int *qexp)
     if ((threadIdx.x & 31) == 0 && mx > 0.0) {
         int e;
         frexp(mx, &e);
-        atomicMax(qexp, e);
+        atomicMax(&qexp[blockIdx.y], e);
     }
+}
+// densities qs [nv][n] (tree order) -> qexp, and double-floats [n][nv] scaled by it
+__global__ void k_q_df(const zd *qs, int64_t n, int nvec, const int *qexp, float4 *q);
+lm_status lm_launch_q_df(const zd *qs, int64_t n, int nv, int *qexp, float4 *q, cudaStream_t st)
+{
+    LM_CUDA(cudaMemsetAsync(qexp, 0x80, LM_MAXV * sizeof(int), st)); // below any exponent
+    k_qexp<<<dim3(std::max(1, std::min(1024 / nv, gridn(n, 256))), nv), 256, 0, st>>>(qs, n, qexp);
+    k_q_df<<<gridn(n * nv, 256), 256, 0, st>>>(qs, n, nv, qexp, q);
+    return LM_OK;
 }
 // threads of an S2M block: the (order, vector) entries rounded up to warps, 64 to 256
 static int p2m_threads(int nent) { return std::max(64, std::min(256, (nent + 31) / 32 * 32)); }
@@ -950,7 +961,7 @@ lm_status lm_setup_df(lm_tree_s *t, cudaStream_t st)
         return LM_OK;
     }
     t->ndf.wmax = wmax;
-    lm_status s = lm_dalloc(t, &t->qexp, 1);
+    lm_status s = lm_dalloc(t, &t->qexp, LM_MAXV);
     if (s == LM_OK) s = lm_setup_near_df(t, st);
     if (s == LM_OK) s = lm_setup_oz(t, st);
     if (s == LM_OK) s = lm_setup_exp_df(t, st);

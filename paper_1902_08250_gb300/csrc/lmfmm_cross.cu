@@ -50,8 +50,6 @@ __global__ void k_m2l64(int64_t nbox, int P, int nvec, const int64_t *vstart, co
                         const int32_t *vslot, const zd *tab, const zd *M, zd *Lc);
 __global__ void k_permute_in(const zd *q, const int64_t *perm, int64_t n, int nvec, int conjugate, zd *qs);
 __global__ void k_permute_out(const zd *us, const int64_t *perm, int64_t n, int nvec, int conjugate, zd *u);
-__global__ void k_qexp(const zd *qs, int64_t n, int nvec, int *qexp);
-__global__ void k_q_df(const zd *qs, int64_t n, int nvec, const int *qexp, float4 *q);
 #define CROSS_P2M_CHUNK 16 // points staged per round by k_p2m64
 
 struct CrossLevel {
@@ -401,12 +399,12 @@ __global__ void __launch_bounds__(128) k_cross_near_df(double k2, const double *
             if (lane < nv) us[(int64_t)lane * nt + i] = zd{sum.re, sum.im};
             continue;
         }
-        const int ex = qexp_of(qexp);
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
             const float4 a = df_norm(acc[v]);
             const df re = df_warp_sum(df_re(a)), im = df_warp_sum(df_im(a));
             if (lane == v && v < nv) {
+                const int ex = qexp_of(qexp, v);
                 zd &o = us[(int64_t)v * nt + i];
                 o = o + zd{ldexp(df_double(re), ex), ldexp(df_double(im), ex)};
             }
@@ -908,7 +906,7 @@ static lm_status cross_setup(lm_cross_s *c, const double *xs, const double *ys, 
         const int nt = c->nray * c->ntail;
         if (c->med.opt.precision == LM_FP64) {
             CTRY(calloc_dev(c, &c->qdf, (size_t)LM_MAXV * c->ns));
-            CTRY(calloc_dev(c, &c->qexp, 1));
+            CTRY(calloc_dev(c, &c->qexp, LM_MAXV));
         }
         CTRY(calloc_dev(c, &c->seg_node, 3 * c->nseg));
         CTRY(calloc_dev(c, &c->seg_wdf, 2 * c->nseg));
@@ -1073,11 +1071,8 @@ extern "C" lm_status lm_cross_apply(lm_cross c, const void *q, int nvec, void *u
     for (int v0 = 0; v0 < nvec; v0 += LM_MAXV) {
         const int nv = std::min(LM_MAXV, nvec - v0);
         k_permute_in<<<gridc(c->ns, 256), 256, 0, st>>>(qd + (int64_t)v0 * c->ns, c->perm_s, c->ns, nv, 0, c->qs);
-        if (c->ndf && c->med.opt.precision == LM_FP64) {
-            LM_CUDA(cudaMemsetAsync(c->qexp, 0x80, sizeof(int), st)); // below any exponent
-            k_qexp<<<std::min(1024, gridc(c->ns * nv, 256)), 256, 0, st>>>(c->qs, c->ns, nv, c->qexp);
-            k_q_df<<<gridc(c->ns * nv, 256), 256, 0, st>>>(c->qs, c->ns, nv, c->qexp, c->qdf);
-        }
+        if (c->ndf && c->med.opt.precision == LM_FP64)
+            CTRY(lm_launch_q_df(c->qs, c->ns, nv, c->qexp, c->qdf, st));
         if (c->xdf) {
             auto M = [&](int l) { return (float4 *)c->lev[l].M; };
             auto Lx = [&](int l) { return (float4 *)c->lev[l].Lc; };

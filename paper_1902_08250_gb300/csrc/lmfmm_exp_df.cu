@@ -1,6 +1,6 @@
 // lmfmm_exp_df.cu -- expansions of the FP64 form in double-float on the FP32
 // pipes: S2M, M2M, M2L, L2L and L2T.  Multipoles and local expansions are kept as
-// float4 (re hi, re lo, im hi, im lo), scaled by 2^-qexp, [box][2p+1][nvec]: an FP64
+// float4 (re hi, re lo, im hi, im lo), scaled by 2^-qexp[vector], [box][2p+1][nvec]: an FP64
 // value takes the same 16 bytes, but converting it costs FP64 instructions (64 issue
 // slots each), and with nvec instead of 16 slots per order the one-vector apply
 // reads whole lines.
@@ -187,7 +187,6 @@ __global__ void __launch_bounds__(128) k_l2t_df(Geo geo, int P, double k, Bessel
             put(2, m, v, y[0], y[1]);
         }
     }
-    const int ex = qexp_of(qexp);
     for (int64_t p0 = lo; p0 < hi; p0 += XD_PTS) {
         const int cnt = (int)min((int64_t)XD_PTS, hi - p0);
         __syncthreads();
@@ -204,6 +203,7 @@ __global__ void __launch_bounds__(128) k_l2t_df(Geo geo, int P, double k, Bessel
                 df_mac(a.x, a.y, c[1].x, c[1].y, bb.z, bb.w);
                 df_mac(a.z, a.w, c[1].z, c[1].w, bb.z, bb.w);
             }
+            const int ex = qexp_of(qexp, v0 + v);
             const zd r = {ldexp(df_double(df_re(a)), ex), ldexp(df_double(df_im(a)), ex)};
             if (GRAD) {
                 zd *o = set == 0 ? out.u : set == 1 ? out.ux : out.uy;
@@ -572,7 +572,6 @@ void lm_df_m2l(const M2LLevelDF *lev, int nlev, int64_t nblk, int P, int nv, cud
 
 __global__ void k_permute_in(const zd *q, const int64_t *perm, int64_t n, int nvec, int conjugate, zd *qs);
 __global__ void k_permute_out(const zd *us, const int64_t *perm, int64_t n, int nvec, int conjugate, zd *u);
-__global__ void k_qexp(const zd *qs, int64_t n, int nvec, int *qexp);
 
 // FP64 form in double-float, both tree kinds; with ux set, step 4 also evaluates the target gradient
 // and writes u (or null), ux, uy
@@ -594,9 +593,7 @@ lm_status lm_run_df(lm_tree_s *t, const zd *q, int nvec, zd *u, bool adjoint, zd
         const int nv = std::min(LM_MAXV, nvec - v0);
         lm_phase_begin(t, PH_PERMUTE, st);
         k_permute_in<<<gridn(n, 256), 256, 0, st>>>(q + (int64_t)v0 * n, t->perm, n, nv, adjoint, t->qs);
-        LM_CUDA(cudaMemsetAsync(t->qexp, 0x80, sizeof(int), st)); // below any exponent
-        k_qexp<<<std::min(1024, gridn(n * nv, 256)), 256, 0, st>>>(t->qs, n, nv, t->qexp);
-        lm_launch_q_df(t, nv, st);
+        TRY_X(lm_launch_q_df(t->qs, n, nv, t->qexp, t->ndf.q, st));
         lm_phase_end(t, PH_PERMUTE, st, 3);
         // step 2: S2M at every leaf, M2M up the levels
         lm_phase_begin(t, PH_S2M, st);

@@ -10,7 +10,8 @@
 // truncation (1e-13 to 1e-10 for p = 24 to 18).
 //
 // Units: coordinates are scaled by k2/2, so that z = dx^2 + dy^2 = (k2 r / 2)^2 is
-// the argument of the ascending series; densities by 2^-qexp (as the multipoles).
+// the argument of the ascending series; densities by 2^-qexp, an exponent per vector
+// (as the multipoles).
 // A kernel value g = g_re + i g_im is kept as (A, J), g_re = -A/(4 pi), g_im = J/4:
 // for the free pair A = (ln z + 2 gamma) J + 2 V, J = J0, so the constants are
 // applied once per target.  A pair closer than 2^-10 leaf widths takes its offset from the
@@ -168,13 +169,13 @@ __global__ void k_near_pts(Geo geo, double kap, double d, const double *xs, cons
     }
 }
 
-// densities in tree order [nvec][n] -> double-float [n][nvec], scaled by 2^-qexp
+// densities in tree order [nvec][n] -> double-float [n][nvec], scaled by 2^-qexp[vector]
 __global__ void k_q_df(const zd *qs, int64_t n, int nvec, const int *qexp, float4 *q)
 {
     const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (idx >= n * nvec) return;
     const int64_t i = idx / nvec;
-    const int v = (int)(idx % nvec), e = -qexp_of(qexp);
+    const int v = (int)(idx % nvec), e = -qexp_of(qexp, v);
     const zd a = qs[(int64_t)v * n + i];
     q[idx] = df_split(zd{ldexp(a.re, e), ldexp(a.im, e)});
 }
@@ -560,7 +561,6 @@ __global__ void __launch_bounds__(nd_threads(NV, GRAD), GRAD ? 3 : 512 / nd_thre
             }
         }
         __syncthreads();
-        const int ex = qexp_of(qexp);
         for (int i = tid; i < nt * nv * SETS; i += THR) {
             const int row = i % nt, vc = i / nt, vv = vc % nv, c = vc / nv;
             float4 a, j;
@@ -574,6 +574,7 @@ __global__ void __launch_bounds__(nd_threads(NV, GRAD), GRAD ? 3 : 512 / nd_thre
             }
             const double f = -1.0 / (4.0 * M_PI);
             zd r = {f * df_double(df_re(a)) - 0.25 * df_double(df_im(j)), f * df_double(df_im(a)) + 0.25 * df_double(df_re(j))};
+            const int ex = qexp_of(qexp, go.v0 + vv);
             r = zd{ldexp(r.re, ex), ldexp(r.im, ex)};
             if (GRAD) {
                 zd *o = c == 0 ? go.u : c == 1 ? go.ux : go.uy;
@@ -701,9 +702,10 @@ __global__ void __launch_bounds__(32 * PW_WARPS) k_near_pw_df(Geo geo, double ka
                 }
             }
             __syncthreads();
-            const int cnt = (int)min((int64_t)nwarp, hi - i0), ex = qexp_of(qexp);
+            const int cnt = (int)min((int64_t)nwarp, hi - i0);
             for (int t = threadIdx.x; t < cnt * nv; t += blockDim.x) {
                 const float4 a = ur[t % cnt][t / cnt];
+                const int ex = qexp_of(qexp, t / cnt);
                 zd &o = us[(int64_t)(t / cnt) * n + i0 + t % cnt];
                 o = o + zd{ldexp(df_double(df_re(a)), ex), ldexp(df_double(df_im(a)), ex)};
             }
@@ -828,12 +830,6 @@ static void launch_pw(lm_tree_s *t, Geo geo, int64_t npw, int nv, cudaStream_t s
     k_near_pw_df<NV><<<(unsigned)npw, 32 * PW_WARPS, shm, st>>>(geo, kap, nseg, N.seg, N.segw, N.rel, N.hgt, t->leaf_start, t->ustart,
                                                       t->usrc, t->uterm, (const float4 *)t->pwC, t->pwidx, t->qexp, t->n,
                                                       nv, t->us);
-}
-
-// densities of the apply (t->qs, tree order) as double-floats scaled by 2^-qexp
-void lm_launch_q_df(lm_tree_s *t, int nv, cudaStream_t st)
-{
-    k_q_df<<<gridn(t->n * nv, 256), 256, 0, st>>>(t->qs, t->n, nv, t->qexp, t->ndf.q);
 }
 
 // the direct interactions of nv vectors (t->ndf.q), added to t->us

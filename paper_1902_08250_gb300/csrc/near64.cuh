@@ -54,10 +54,12 @@ struct ListParents { // adaptive tree: parent ids[i], children from the box link
 };
 
 
-__device__ __forceinline__ int qexp_of(const int *qexp)
+// binary exponent of a vector's densities: each vector is scaled by its own, so that its result does not
+// depend on the others of the call (one exponent for all flushed a vector 2^-126 of the largest to zero)
+__device__ __forceinline__ int qexp_of(const int *qexp, int v)
 {
-    const int e = *qexp;
-    return e < -1000 ? 0 : e; // all densities zero: no scaling
+    const int e = qexp[v];
+    return e < -2000 ? 0 : e; // all densities zero: no scaling
 }
 
 // ---------------------------------------------------------------------------
