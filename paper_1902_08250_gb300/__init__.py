@@ -149,7 +149,7 @@ def create_medium(k1, k2, k3, d, *, p=20, depth=-1, leaf_target=48, precision=FP
     adaptive = True builds adaptive trees (either precision): a box with more than leaf_target points is
     split while its level is below depth (-1 -> 14).
     m2l_fp64 = True runs the whole FP64 apply in IEEE FP64 instead of double-float (on the FP32
-    pipes, the large contractions of uniform trees by exact digits on the tensor cores).
+    pipes, the large contractions of uniform trees by fixed-point digits on the tensor cores).
     tensor_leaf = 0 keeps the mixed leaf step (S2T and L2T) of 16-vector applies on the CUDA cores."""
     if isinstance(precision, str):
         precision = {"fp64": FP64, "mixed": MIXED}[precision]

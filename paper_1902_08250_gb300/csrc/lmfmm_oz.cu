@@ -1,12 +1,26 @@
 // lmfmm_oz.cu -- the FP64 form's M2L on the tensor cores (tcgen05, kind::f16) by
 // error-free slicing (Ozaki, Ogita, Oishi and Rump, Numer. Algorithms 59, 2012;
 // Mukunoki et al., ISC 2020): tables and multipoles are scaled to fixed point and cut
-// into 5 signed digits of 10 bits, held exactly in FP16.  A product of two digits has
-// at most 18 bits, so a sum over the 2(2p+1) <= 128 input orders is an integer that
-// the FP32 accumulator holds exactly; the digit pairs i + j <= 4 are kept, those of one
-// weight 2^{-10 (i + j)} in one accumulator, and the 5 integers of an output are
-// combined in double-float (50 bits against the 48 of the double-float contraction it
-// replaces).  Levels of at least OZ_MINBOX boxes of uniform trees, their M2M and L2L
+// into 5 signed digits of 10 bits, held exactly in FP16.  The digit pairs i + j <= 4 are
+// kept, those of one weight 2^{-10 w}, w = i + j, in one FP32 accumulator, and the 5 sums of
+// an output are combined in double-float.
+//
+// Exactness.  Digits are at most 2^9, so an entry adds at most 2^9 (A_0 + .. + A_w) to accumulator w, A_j
+// the sum of the magnitudes of the j-th digits of its table row.  That is 2^25 and more for 128 orders of
+// any size, but a table's rows decay (offsets of two widths and more, M2M and L2L triangular): the set-up
+// finds the largest A_0 + A_1 of the level's rows, and so many entries G <= OZ_GRP are summed before a
+// reading that 2^9 (A_0 + A_1) G <= 2^24: accumulators 0 and 1 hold their integers exactly whatever the
+// multipoles are (2^9 (A_0 + A_1) is 0.19 to 0.33 x 2^24 for box widths k w up to 2 and any p, so G is 3 to
+// 4; 0.47 at 4, 0.87 at 16, one entry).  Accumulator 2 stays below 2.8 x 2^24: it rounds, in units of
+// 2^-40 of the product of the scales, where the second digits of several sources are near their largest and match a
+// row's in sign.  For digits that do not know of each other its sum is 10 standard deviations below
+// 2^24.  Those of w = 3 and 4 round in units of 2^-50 and 2^-60.
+//
+// Accuracy is that of fixed point: a power of two scales a level's tables, another each vector's sources of a
+// level, and what is left out is 2^-50 of their product.  Double-float keeps 48 bits of every box; here a
+// box whose multipole is 10^-k of the level's largest keeps k digits fewer than the 15 of the largest.
+//
+// Levels of at least OZ_MINBOX boxes of uniform trees, their M2M and L2L
 // from OZ_MINSHIFT; the others run on the CUDA cores (lmfmm_exp_df.cu).
 //
 // A tile is 128 columns: 128 / nvs target boxes of one row and parity class, nvs vectors
@@ -26,9 +40,9 @@
 // 8-row groups), a stage of a table is one bulk copy, and any run of boxes one per digit and
 // chunk, whatever its offset.  Stages of up to 48 K (107 KB), two in flight.  Roles as in lmfmm_tc_tiles.cu:
 // a producer warp (a lane per copy), an MMA warp, 8 epilogue warps that read the 5
-// accumulators once per 4 entries: there is room for one set of accumulators, so that
-// reading them (about 50 FP32 instructions an element) and the MMAs take turns (with a
-// reading per entry 6.25 ms where 4.86 ms).  A lane of an epilogue warp holds a column,
+// accumulators once per G entries: there is room for one set of accumulators, so that
+// reading them (about 50 FP32 instructions an element) and the MMAs take turns (250k strip, 16
+// vectors, the apply with G = 4, 3, 2 and 1: 6.95, 7.06, 7.37 and 8.14 ms).  A lane of an epilogue warp holds a column,
 // so that it writes whole components, neighbouring vectors beside each other.
 // Bound by the copies from L2 (215 KB an entry and 128 columns at p = 22) and the
 // shared-memory reads of the MMAs' operands (7 KB each at 128 B per clock).
@@ -64,7 +78,7 @@
 // with its levels of 256 boxes here.
 #define OZ_MINSHIFT 4096
 #define OZ_PADL 2
-#define OZ_GRP 4 // entries summed in the accumulators before they are read
+#define OZ_GRP 4 // most entries summed in the accumulators before they are read
 
 // One level of a contraction: M2L (sources and targets a level's boxes), M2M (sources the children,
 // targets a level) or L2L (sources the parents).  Sources lie in planes of consecutive boxes: (row, column
@@ -79,7 +93,8 @@ struct OzLevel {
     const RowEnt *ents;     // (pad: rs is the source plane itself, its run starts at the tile's first box)
     const unsigned char *A; // split tables
     unsigned char *B;       // split sources
-    const uint32_t *tmax;   // [2] largest table component and row sum of the level (float bits)
+    const uint32_t *tmax;   // [3] largest table component and row sum of the level (float bits), largest sum of the
+                            // magnitudes of a row's first and second digits (integer)
     uint32_t *mmax;         // [LM_MAXV] largest source component per vector
     uint32_t *omax;         // the same of the result, or null
     const float4 *M;        // sources
@@ -87,9 +102,10 @@ struct OzLevel {
 };
 
 __device__ __forceinline__ int oz_exp(uint32_t bits) { return bits ? (int)((bits >> 23) & 0xff) - 127 : -126; }
-// the level's table exponent: components below 2^(e-1), row sums at most 2^(e+2), so that the leading
-// digits' sum over K and OZ_GRP = 4 entries stays below 2^24 (|digit| <= 512 on either side)
+// the level's table exponent: components below 2^(e-1), row sums at most 2^(e+2)
 __device__ __forceinline__ int oz_ea(const uint32_t *t) { return max(oz_exp(t[0]) + 2, oz_exp(t[1]) - 1); }
+// entries a reading: 2^9 tmax[2] G <= 2^24
+__device__ __forceinline__ int oz_grp(const uint32_t *t) { return max(1, min(OZ_GRP, (int)((1u << 15) / max(1u, t[2])))); }
 __device__ __forceinline__ float oz_pow2(int e) { return __int_as_float((max(-126, min(127, e)) + 127) << 23); }
 // table rows (2 p + re / im) in sweeps of oz_rows(np), a multiple of 16, at most OZ_RN
 __host__ __device__ __forceinline__ int oz_sweeps(int np) { return 2 * np <= OZ_RN ? 1 : 2; }
@@ -115,6 +131,23 @@ __global__ void __launch_bounds__(256) k_oz_tmax(const zd *tab, int np, uint32_t
     }
     if (mx > 0.f) atomicMax(tmax, __float_as_uint(mx));
     if (l1 > 0.f) atomicMax(tmax + 1, __float_as_uint(l1));
+}
+// the first two digits' magnitudes of each row (as k_oz_tsplit cuts them), one thread per row
+__global__ void __launch_bounds__(256) k_oz_tsum(const zd *tab, int np, uint32_t *tmax)
+{
+    const zd *T = tab + (int64_t)blockIdx.x * np * np;
+    const double sc = ldexp(1.0, OZ_BITS - oz_ea(tmax));
+    double mx = 0.0;
+    for (int r = threadIdx.x; r < 2 * np; r += blockDim.x) { // row 2 p + im: the same components for both
+        double s = 0.0;
+        for (int k = 0; k < 2 * np; ++k) {
+            const zd a = T[(r >> 1) * np + (k >> 1)];
+            const double x = sc * (((r ^ k) & 1) ? a.im : a.re), d = rint(x);
+            s += fabs(d) + fabs(rint((x - d) * 1024.0));
+        }
+        mx = fmax(mx, s);
+    }
+    atomicMax(tmax + 2, (uint32_t)mx);
 }
 // one thread per (class, 8-wide K chunk, row): 8 components into 5 digit planes
 __global__ void __launch_bounds__(256) k_oz_tsplit(const zd *tab, int64_t ncls, int np, const uint32_t *tmax,
@@ -364,8 +397,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_m2l_oz(const OzLevel *lvs, in
             for (int64_t tile = blockIdx.x; tile < ntiles && !stop && !*abort_s; tile += gridDim.x) {
                 int cls, i0, sw;
                 const OzLevel &lv = oz_tile(lvs, nlev, tile, ns, &cls, &i0, &sw, tb);
-                const int ne = lv.e0[cls + 1] - lv.e0[cls];
-                for (int e = 0; e < ne && !stop; e += OZ_GRP, ++item) {
+                const int ne = lv.e0[cls + 1] - lv.e0[cls], grp = oz_grp(lv.tmax);
+                for (int e = 0; e < ne && !stop; e += grp, ++item) {
                     if (!mbar_wait_lim(btempty, (item & 1) ^ 1, TC_WAIT_LIMIT, abort_s, err)) {
                         oz_fail(abort_s, err);
                         stop = true;
@@ -373,7 +406,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_m2l_oz(const OzLevel *lvs, in
                     }
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     int issued = 0;
-                    const int nstg = nst * min(OZ_GRP, ne - e);
+                    const int nstg = nst * min(grp, ne - e);
                     for (int q = 0, st = 0; q < nstg; ++q, ++it, st = st + 1 == nst ? 0 : st + 1) {
                         const int s = (int)(it % OZ_NST), kc = min(OZ_KC, KC - st * OZ_KC), ks = kc / 2;
                         if (!mbar_wait_lim(bfull + 8 * s, (it / OZ_NST) & 1, TC_WAIT_LIMIT, abort_s, err)) {
@@ -413,11 +446,11 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_m2l_oz(const OzLevel *lvs, in
         for (int64_t tile = blockIdx.x; tile < ntiles && !bad; tile += gridDim.x) {
             int cls, i0, sw;
             const OzLevel &lv = oz_tile(lvs, nlev, tile, ns, &cls, &i0, &sw, tb);
-            const int ne = lv.e0[cls + 1] - lv.e0[cls];
+            const int ne = lv.e0[cls + 1] - lv.e0[cls], grp = oz_grp(lv.tmax);
             df acc[OZ_RN / 2];
 #pragma unroll
             for (int r = 0; r < OZ_RN / 2; ++r) acc[r] = df{0.f, 0.f};
-            for (int e = 0; e < ne; e += OZ_GRP, ++item) {
+            for (int e = 0; e < ne; e += grp, ++item) {
                 if (!mbar_wait_lim(btfull, item & 1, TC_WAIT_LIMIT, abort_s, err)) {
                     oz_fail(abort_s, err);
                     bad = true;
@@ -546,11 +579,12 @@ static lm_status oz_setup_op(lm_tree_s *t, const zd *tab, size_t ncls, const std
     x.ents = de;
     TRY_O(lm_dalloc(t, &x.e0, e0.size()));
     TRY_O(lm_dalloc(t, &x.A, ncls * OZ_S * KC * rows * 16));
-    TRY_O(lm_dalloc(t, &x.tmax, 2));
+    TRY_O(lm_dalloc(t, &x.tmax, 3));
     LM_CUDA(cudaMemcpyAsync(de, ents.data(), ents.size() * sizeof(RowEnt), cudaMemcpyHostToDevice, st));
     LM_CUDA(cudaMemcpyAsync(x.e0, e0.data(), e0.size() * sizeof(int32_t), cudaMemcpyHostToDevice, st));
-    LM_CUDA(cudaMemsetAsync(x.tmax, 0, 2 * sizeof(uint32_t), st));
+    LM_CUDA(cudaMemsetAsync(x.tmax, 0, 3 * sizeof(uint32_t), st));
     k_oz_tmax<<<(unsigned)ncls, 256, 0, st>>>(tab, np, x.tmax);
+    k_oz_tsum<<<(unsigned)ncls, 128, 0, st>>>(tab, np, x.tmax);
     const int64_t nt = (int64_t)ncls * KC * rows;
     k_oz_tsplit<<<(unsigned)((nt + 255) / 256), 256, 0, st>>>(tab, (int64_t)ncls, np, x.tmax, x.A);
     LM_CUDA(cudaGetLastError());
