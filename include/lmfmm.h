@@ -199,6 +199,9 @@ lm_status lm_build_tree(lm_medium m, const double *x, const double *y, int64_t n
  *   u: device, complex128 [nvec][n] output (overwritten), input order; must
  *      not overlap q.
  *   nvec >= 1.
+ * The tensor-core kernels (LM_MIXED trees; LM_FP64 uniform trees with a level of
+ * 256 boxes or more, unless m2l_fp64 is 1) bound every wait inside them.  A wait that
+ * gives up does not fail the call: lm_sync_status reports it.
  * Errors: LM_EINVAL (nvec < 1, NULL or overlapping buffers), LM_ECUDA.
  */
 lm_status lm_apply(lm_tree t, const void *q, int nvec, void *u, void *stream);
@@ -471,7 +474,8 @@ void lm_destroy_cross(lm_cross c);
 /*
  * sync_status -- synchronise `stream` and report device-side failures of the
  * applies enqueued so far on tree t: LM_ETIMEOUT if a bounded wait inside a
- * tensor-core kernel gave up (the result of that apply is invalid), LM_OK
+ * tensor-core kernel gave up (the result of that apply is invalid, and so are
+ * those enqueued after it: their tensor-core kernels do no work), LM_OK
  * otherwise.  Clears the recorded failure.
  */
 lm_status lm_sync_status(lm_tree t, void *stream);
@@ -479,7 +483,8 @@ lm_status lm_sync_status(lm_tree t, void *stream);
 /*
  * set_poll_limit -- failure-path check of the bounded waits (no counterpart
  * in the paper).  For the next 16-vector apply of an LM_MIXED tree that runs
- * the tile-form tensor-core M2L, the MMA issuer's first wait for its operands
+ * the tile-form tensor-core M2L, or the next group of up to 16 vectors of an
+ * LM_FP64 tree that runs its M2L there, the MMA issuer's first wait for its operands
  * polls at most `limit` times (0: gives up at once) before it reports a
  * timeout; every other wait, including the waits that let copies and MMAs in
  * flight finish before tensor memory is freed, keeps the library's limit.

@@ -327,7 +327,7 @@ def sync_status(tree: Tree, stream=None):
 
 def set_poll_limit(tree: Tree, limit):
     """Limit the polls of the tensor-core M2L's first operand wait in the tree's next
-    16-vector apply (lm_set_poll_limit; 0 gives up at once, < 0 clears)."""
+    apply (16 vectors on mixed trees; lm_set_poll_limit; 0 gives up at once, < 0 clears)."""
     _check(_lib.lm_set_poll_limit(tree._h, int(limit)))
 
 

@@ -282,7 +282,7 @@ struct lm_tree_s {
     uint32_t *tt_mmax;          // per level: largest multipole component of the apply (float bits)
     std::vector<int64_t> tt_tbase, tt_mbase; // per level: first table, first box
     int tt_grid;                // persistent CTAs (one per SM)
-    int tt_poll_limit;          // polls of the first operand wait (-1: the library default)
+    int tt_poll_limit;          // polls of the first operand wait, FP64 form: of k_m2l_oz (-1: the library default)
     // tensor-core leaf step (16-vector applies on uniform trees)
     bool lf_ready;
     void *lf_pts;               // [n] float4 (x, y relative to the leaf centre, absolute y, 0)

@@ -178,6 +178,7 @@ extern "C" lm_status lm_build_tree(lm_medium m, const double *x, const double *y
     t->precision = m->opt.precision;
     t->max_nvec = m->opt.max_nvec;
     t->m2l_df = t->precision == LM_FP64 && m->opt.m2l_fp64 == 0;
+    t->tt_poll_limit = -1;
     lm_status s;
     if (m->opt.adaptive) {
         s = lm_setup_adaptive(t, x, y, st);
@@ -316,7 +317,7 @@ extern "C" lm_status lm_sync_status(lm_tree t, void *stream)
     if (f) {
         LM_CUDA(cudaMemsetAsync(t->dflag + 1, 0, sizeof(int), st));
         LM_CUDA(cudaStreamSynchronize(st));
-        lm_set_error("a bounded wait in the tensor-core M2L gave up; the apply result is invalid");
+        lm_set_error("a bounded wait in a tensor-core kernel gave up; the applies since the last sync_status are invalid");
         return LM_ETIMEOUT;
     }
     return LM_OK;

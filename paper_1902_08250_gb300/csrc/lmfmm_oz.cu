@@ -301,8 +301,9 @@ __device__ __forceinline__ void oz_fail(volatile int *abort_s, int *err)
     atomicOr(err, 1);
 }
 
+// first_limit >= 0: poll limit of the MMA issuer's first wait for operands (the timeout path's test)
 __global__ void __launch_bounds__(OZ_THREADS, 1) k_m2l_oz(const OzLevel *lvs, int nlev, int64_t ntiles, int np, int nv, int nvs,
-                                                          int *err)
+                                                          int *err, int first_limit)
 {
     extern __shared__ __align__(1024) unsigned char smem[];
     uint64_t *bars = (uint64_t *)(smem + OZ_NST * OZ_STAGE);
@@ -409,7 +410,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_m2l_oz(const OzLevel *lvs, in
                     const int nstg = nst * min(grp, ne - e);
                     for (int q = 0, st = 0; q < nstg; ++q, ++it, st = st + 1 == nst ? 0 : st + 1) {
                         const int s = (int)(it % OZ_NST), kc = min(OZ_KC, KC - st * OZ_KC), ks = kc / 2;
-                        if (!mbar_wait_lim(bfull + 8 * s, (it / OZ_NST) & 1, TC_WAIT_LIMIT, abort_s, err)) {
+                        const int lim = it == 0 && first_limit >= 0 ? first_limit : TC_WAIT_LIMIT;
+                        if (!mbar_wait_lim(bfull + 8 * s, (it / OZ_NST) & 1, lim, abort_s, err)) {
                             oz_fail(abort_s, err);
                             stop = true;
                             break;
@@ -670,7 +672,7 @@ static int oz_step(lm_tree_s *t, int op, size_t i, bool mmax, int nv, cudaStream
     if (mmax) k_oz_mmax<<<2 * (unsigned)Z.nsm, 256, 0, st>>>(d, t->np, nv);
     k_oz_split<<<(unsigned)std::min<int64_t>(8 * Z.nsm, (work + 255) / 256), 256, 0, st>>>(d, t->np, nv, nvs);
     const int64_t tiles = (op == OZ_M2M ? lv.nrow / 2 : 2 * lv.nrow) * ((ncl + tb - 1) / tb) * oz_sweeps(t->np);
-    k_m2l_oz<<<(unsigned)std::min<int64_t>(Z.nsm, tiles), OZ_THREADS, OZ_SMEM, st>>>(d, 1, tiles, t->np, nv, nvs, t->dflag + 1);
+    k_m2l_oz<<<(unsigned)std::min<int64_t>(Z.nsm, tiles), OZ_THREADS, OZ_SMEM, st>>>(d, 1, tiles, t->np, nv, nvs, t->dflag + 1, -1);
     return 2 + mmax;
 }
 
@@ -711,7 +713,8 @@ lm_status lm_launch_m2l_oz(lm_tree_s *t, int nv, cudaStream_t st, int *launches)
         k_oz_split<<<dim3(8 * (unsigned)Z.nsm, nl - n0), 256, 0, st>>>(d + n0, t->np, nv, 1 << f);
     }
     k_m2l_oz<<<(unsigned)std::min<int64_t>(Z.nsm, Z.ntile[f]), OZ_THREADS, OZ_SMEM, st>>>(
-        d, nl, Z.ntile[f], t->np, nv, 1 << f, t->dflag + 1);
+        d, nl, Z.ntile[f], t->np, nv, 1 << f, t->dflag + 1, t->tt_poll_limit);
+    t->tt_poll_limit = -1; // a test limit applies to one launch
     *launches = n0 < nl ? 3 : 1;
     LM_CUDA(cudaGetLastError());
     return LM_OK;
