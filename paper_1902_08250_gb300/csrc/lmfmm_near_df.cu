@@ -14,8 +14,11 @@
 // (as the multipoles).
 // A kernel value g = g_re + i g_im is kept as (A, J), g_re = -A/(4 pi), g_im = J/4:
 // for the free pair A = (ln z + 2 gamma) J + 2 V, J = J0, so the constants are
-// applied once per target.  A pair closer than 2^-10 leaf widths takes its offset from the
-// FP64 coordinates (the leaf-relative ones are good to 2^-49 of the leaf); pairs outside the
+// applied once per target.  A pair closer than 2^-6 leaf widths takes its offset from the
+// FP64 coordinates: the leaf-relative ones are good to 2^-49 of the leaf, an offset of s leaf widths to
+// 2^-48 / s, which the gradient shows (with 2^-10 the y-derivative of 3000 points within 0.02 of an interface was 4.5e-13 from
+// the IEEE form's, 4.8e-14 now, that of 100k clustered points 8.2e-14, 2.6e-14 now; times the same;
+// 2^-4 costs the gradient step 2 %).  Pairs outside the
 // series' range (z > 1, or closer than 2^-45 in these units) take the FP64 functions.
 #include <algorithm>
 #include <type_traits>
@@ -312,7 +315,7 @@ __global__ void __launch_bounds__(nd_threads(NV, GRAD), GRAD ? 3 : 512 / nd_thre
     tab.load();
     double cx, cy, bw;
     geo.centre(b, &cx, &cy, &bw);
-    const float zclose = (float)(kap * kap * bw * bw) * 0x1p-20f;
+    const float zclose = (float)(kap * kap * bw * bw) * 0x1p-12f; // pairs closer than 2^-6 leaf widths
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t u0 = ustart[b], u1 = ustart[b + 1];
     constexpr int ROWS = TG / (THR / 32), HALF = SRC / 32;
