@@ -135,7 +135,7 @@ __global__ void __launch_bounds__(256) k_image_expand(int P, const ImgInt *ints,
 {
     const int np = 2 * P + 1, nn = 4 * P + 1;
     __shared__ zd In[4 * LM_MAXP + 1];
-    __shared__ double fact[2 * LM_MAXP + 1], pw[2 * LM_MAXP + 1], rt[LM_MAXP + 1], rs[LM_MAXP + 1];
+    __shared__ double fact[2 * LM_MAXP + 1], pw[LM_MAXP + 1], rt[LM_MAXP + 1], rs[LM_MAXP + 1];
     const ImgCls c = cls[blockIdx.x];
     const ImgInt &I = ints[c.u];
     for (int n = threadIdx.x; n < nn; n += blockDim.x) {
@@ -146,7 +146,7 @@ __global__ void __launch_bounds__(256) k_image_expand(int P, const ImgInt *ints,
     }
     if (threadIdx.x < 4) {
         double v = 1.0;
-        const int lim = threadIdx.x < 2 ? 2 * P : P;
+        const int lim = threadIdx.x == 0 ? 2 * P : P;
         double *a = threadIdx.x == 0 ? fact : threadIdx.x == 1 ? pw : threadIdx.x == 2 ? rt : rs;
         for (int n = 0; n <= lim; ++n) {
             a[n] = v;
@@ -158,7 +158,9 @@ __global__ void __launch_bounds__(256) k_image_expand(int P, const ImgInt *ints,
     for (int idx = threadIdx.x; idx < np * np; idx += blockDim.x) {
         const int p = idx / np - P, q = idx % np - P, n = sum ? p + q : p - q;
         const int ap = abs(p), aq = abs(q), an = abs(n);
-        const double f = fact[an] / fact[ap] / fact[aq] * pw[ap + aq - an] * rt[ap] * rs[aq];
+        // (sc/2)^{|p|+|q|-|n|} as two equal powers beside their factorials: the whole power alone passes FP64's
+        // range for sc above 3235 at P = 48, where the entries do not
+        const double h = pw[(ap + aq - an) >> 1], f = fact[an] * (h / fact[ap] * rt[ap]) * (h / fact[aq] * rs[aq]);
         const zd v = f * In[n + 2 * P];
         const int ph = ((p - q) % 4 + 4) % 4; // i^{p-q}
         const zd r = ph == 0 ? v : ph == 1 ? zd{-v.im, v.re} : ph == 2 ? -v : zd{v.im, -v.re};
