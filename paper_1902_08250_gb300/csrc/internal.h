@@ -226,7 +226,7 @@ struct OzData {
         void *ents;
         int32_t *e0;
         unsigned char *A;
-        uint32_t *tmax;
+        int32_t *ea; // exponents of the orders, bounds of the readings (OzLevel)
     };
     struct Lv { // a level whose M2L (M2M to and L2L from the level above) runs on the tensor cores
         int l;
@@ -235,7 +235,7 @@ struct OzData {
     };
     std::vector<Lv> lv; // L, L - 1, ..
     size_t nshift = 0;  // of which the first take M2M and L2L too
-    uint32_t *mmax = nullptr;
+    uint32_t *mmax = nullptr, *bmax = nullptr;
     unsigned char *Btop = nullptr; // digits of the local expansions of the level above the last
     void *desc[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
     int64_t ntile[5] = {0, 0, 0, 0, 0}; // of the M2L

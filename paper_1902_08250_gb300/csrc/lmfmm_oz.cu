@@ -5,20 +5,26 @@
 // kept, those of one weight 2^{-10 w}, w = i + j, in one FP32 accumulator, and the 5 sums of
 // an output are combined in double-float.
 //
+// Scales.  Powers of two: one per order of a level's tables (rows), one per vector of a level's multipoles, one per
+// box and vector of L2L's sources, whose targets have one entry.  Components are below 1/2 then, row sums at most 4.
+// Accuracy is that of fixed point, 2^-50 of the scales: in M2L and M2M a box whose multipole is 10^-k of the level's
+// largest keeps k digits fewer than the 15 of the largest, where double-float keeps 48 bits of every box.  The orders'
+// and the boxes' scales are for the target gradient, which magnifies order p by |p| / w.  From the IEEE form, 250k
+// strip, 16 vectors, p = 20: potentials 4.8e-14, gradient 6.1e-14 (one scale a level: 5.1e-14, 2.7e-13; contractions in
+// double-float: 3.2e-13, 2.8e-13); 20k points on leaves of 1/64, sources 1e10 times weaker than those at the
+// strip's end, gradient 6 units from there 9.1e-13 (3.1e-12; 1.8e-13).
+//
 // Exactness.  Digits are at most 2^9, so an entry adds at most 2^9 (A_0 + .. + A_w) to accumulator w, A_j
 // the sum of the magnitudes of the j-th digits of its table row.  That is 2^25 and more for 128 orders of
-// any size, but a table's rows decay (offsets of two widths and more, M2M and L2L triangular): the set-up
-// finds the largest A_0 + A_1 of the level's rows, and so many entries G <= OZ_GRP are summed before a
-// reading that 2^9 (A_0 + A_1) G <= 2^24: accumulators 0 and 1 hold their integers exactly whatever the
-// multipoles are (2^9 (A_0 + A_1) is 0.19 to 0.33 x 2^24 for box widths k w up to 2 and any p, so G is 3 to
-// 4; 0.47 at 4, 0.87 at 16, one entry).  Accumulator 2 stays below 2.8 x 2^24: it rounds, in units of
-// 2^-40 of the product of the scales, where the second digits of several sources are near their largest and match a
-// row's in sign.  For digits that do not know of each other its sum is 10 standard deviations below
-// 2^24.  Those of w = 3 and 4 round in units of 2^-50 and 2^-60.
-//
-// Accuracy is that of fixed point: a power of two scales a level's tables, another each vector's sources of a
-// level, and what is left out is 2^-50 of their product.  Double-float keeps 48 bits of every box; here a
-// box whose multipole is 10^-k of the level's largest keeps k digits fewer than the 15 of the largest.
+// any size, but a table's rows decay: the set-up adds up A_0 + A_1 over the entries of every reading of the
+// level's lists, and so many entries G <= OZ_GRP are summed before a reading that 2^9 times the largest such sum is
+// at most 2^24: accumulators 0 and 1 hold their integers exactly whatever the multipoles are.  (M2L with 3
+// entries a reading: 0.74 to 0.98 x 2^24 for box widths k w up to 1 and p up to 31; 2 entries 0.98 at k w = 2, one
+// 0.55 at 4, 0.87 at 16; M2M 2 or 3.)
+// Accumulator 2 stays below 3 x 2^24: it rounds, in units of 2^-40 of the product of the scales, where
+// the second digits of several sources are near their largest and match a row's in sign.  For digits that
+// do not know of each other its sum is 10 standard deviations below 2^24.  Those of w = 3 and 4 round in
+// units of 2^-50 and 2^-60.
 //
 // Levels of at least OZ_MINBOX boxes of uniform trees, their M2M and L2L
 // from OZ_MINSHIFT; the others run on the CUDA cores (lmfmm_exp_df.cu).
@@ -42,7 +48,7 @@
 // a producer warp (a lane per copy), an MMA warp, 8 epilogue warps that read the 5
 // accumulators once per G entries: there is room for one set of accumulators, so that
 // reading them (about 50 FP32 instructions an element) and the MMAs take turns (250k strip, 16
-// vectors, the apply with G = 4, 3, 2 and 1: 6.95, 7.06, 7.37 and 8.14 ms).  A lane of an epilogue warp holds a column,
+// vectors, the apply with G = 4, 3, 2 and 1 everywhere: 6.95, 7.06, 7.37 and 8.14 ms; 7.19 as chosen).  A lane of an epilogue warp holds a column,
 // so that it writes whole components, neighbouring vectors beside each other.
 // Bound by the copies from L2 (215 KB an entry and 128 columns at p = 22) and the
 // shared-memory reads of the MMAs' operands (7 KB each at 128 B per clock).
@@ -93,19 +99,22 @@ struct OzLevel {
     const RowEnt *ents;     // (pad: rs is the source plane itself, its run starts at the tile's first box)
     const unsigned char *A; // split tables
     unsigned char *B;       // split sources
-    const uint32_t *tmax;   // [3] largest table component and row sum of the level (float bits), largest sum of the
-                            // magnitudes of a row's first and second digits (integer)
-    uint32_t *mmax;         // [LM_MAXV] largest source component per vector
+    const int32_t *ea;      // [np] exponent of each order's table rows; [3] largest sum of the first and second digits'
+                            // magnitudes over 2, 3, 4 entries of a list
+    uint32_t *mmax;         // [LM_MAXV] largest source component per vector; L2L: [sources][LM_MAXV], of each box
     uint32_t *omax;         // the same of the result, or null
     const float4 *M;        // sources
     float4 *L;              // targets
 };
 
 __device__ __forceinline__ int oz_exp(uint32_t bits) { return bits ? (int)((bits >> 23) & 0xff) - 127 : -126; }
-// the level's table exponent: components below 2^(e-1), row sums at most 2^(e+2)
-__device__ __forceinline__ int oz_ea(const uint32_t *t) { return max(oz_exp(t[0]) + 2, oz_exp(t[1]) - 1); }
-// entries a reading: 2^9 tmax[2] G <= 2^24
-__device__ __forceinline__ int oz_grp(const uint32_t *t) { return max(1, min(OZ_GRP, (int)((1u << 15) / max(1u, t[2])))); }
+// entries a reading: 2^9 (their A_0 + A_1) <= 2^24
+__device__ __forceinline__ int oz_grp(const int32_t *ea, int np)
+{
+    for (int g = OZ_GRP; g > 1; --g)
+        if (ea[np + g - 2] <= 1 << 15) return g;
+    return 1;
+}
 __device__ __forceinline__ float oz_pow2(int e) { return __int_as_float((max(-126, min(127, e)) + 127) << 23); }
 // table rows (2 p + re / im) in sweeps of oz_rows(np), a multiple of 16, at most OZ_RN
 __host__ __device__ __forceinline__ int oz_sweeps(int np) { return 2 * np <= OZ_RN ? 1 : 2; }
@@ -116,41 +125,61 @@ __host__ __device__ __forceinline__ int64_t oz_prow(int ncl, int tb, int nvs) { 
 // ---------------------------------------------------------------------------
 // operands
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_oz_tmax(const zd *tab, int np, uint32_t *tmax)
+// largest component and row sum (float bits) of each order over a level's tables
+__global__ void __launch_bounds__(128) k_oz_tmax(const zd *tab, int np, uint32_t *tmax)
 {
     const zd *T = tab + (int64_t)blockIdx.x * np * np;
-    float mx = 0.f, l1 = 0.f;
     for (int p = threadIdx.x; p < np; p += blockDim.x) {
+        float mx = 0.f;
         double s = 0.0;
         for (int q = 0; q < np; ++q) {
             const zd a = T[p * np + q];
             mx = fmaxf(mx, (float)fmax(fabs(a.re), fabs(a.im)));
             s += fabs(a.re) + fabs(a.im);
         }
-        l1 = fmaxf(l1, (float)s);
+        if (mx > 0.f) atomicMax(tmax + p, __float_as_uint(mx));
+        if (s > 0.0) atomicMax(tmax + np + p, __float_as_uint((float)s));
     }
-    if (mx > 0.f) atomicMax(tmax, __float_as_uint(mx));
-    if (l1 > 0.f) atomicMax(tmax + 1, __float_as_uint(l1));
 }
-// the first two digits' magnitudes of each row (as k_oz_tsplit cuts them), one thread per row
-__global__ void __launch_bounds__(256) k_oz_tsum(const zd *tab, int np, uint32_t *tmax)
+// the orders' exponents: components below 2^(e-1), row sums at most 2^(e+2)
+__global__ void k_oz_texp(const uint32_t *tmax, int np, int32_t *ea)
+{
+    const int p = threadIdx.x;
+    if (p < np) ea[p] = max(oz_exp(tmax[p]) + 2, oz_exp(tmax[np + p]) - 1);
+}
+// W[class][p]: the magnitudes of the first two digits of a row of order p (as k_oz_tsplit cuts them; the rows of the
+// real and the imaginary part hold the same components)
+__global__ void __launch_bounds__(128) k_oz_tsum(const zd *tab, int np, const int32_t *ea, int32_t *W)
 {
     const zd *T = tab + (int64_t)blockIdx.x * np * np;
-    const double sc = ldexp(1.0, OZ_BITS - oz_ea(tmax));
-    double mx = 0.0;
-    for (int r = threadIdx.x; r < 2 * np; r += blockDim.x) { // row 2 p + im: the same components for both
+    for (int p = threadIdx.x; p < np; p += blockDim.x) {
+        const double sc = ldexp(1.0, OZ_BITS - ea[p]);
         double s = 0.0;
         for (int k = 0; k < 2 * np; ++k) {
-            const zd a = T[(r >> 1) * np + (k >> 1)];
-            const double x = sc * (((r ^ k) & 1) ? a.im : a.re), d = rint(x);
+            const zd a = T[p * np + (k >> 1)];
+            const double x = sc * ((k & 1) ? a.im : a.re), d = rint(x);
             s += fabs(d) + fabs(rint((x - d) * 1024.0));
         }
-        mx = fmax(mx, s);
+        W[(int64_t)blockIdx.x * np + p] = (int32_t)s;
     }
-    atomicMax(tmax + 2, (uint32_t)mx);
+}
+// one block per list: its readings' sums of W, for 2, 3 and 4 entries a reading
+__global__ void __launch_bounds__(128) k_oz_gsum(const RowEnt *ents, const int32_t *e0, int np, const int32_t *W, int32_t *ea)
+{
+    const int b = e0[blockIdx.x], e = e0[blockIdx.x + 1];
+    for (int g = 2; g <= OZ_GRP; ++g) {
+        int mx = 0;
+        for (int p = threadIdx.x; p < np; p += blockDim.x)
+            for (int i = b; i < e; i += g) {
+                int s = 0;
+                for (int j = i; j < min(i + g, e); ++j) s += W[(int64_t)ents[j].slot * np + p];
+                mx = max(mx, s);
+            }
+        if (mx) atomicMax(ea + np + g - 2, mx);
+    }
 }
 // one thread per (class, 8-wide K chunk, row): 8 components into 5 digit planes
-__global__ void __launch_bounds__(256) k_oz_tsplit(const zd *tab, int64_t ncls, int np, const uint32_t *tmax,
+__global__ void __launch_bounds__(256) k_oz_tsplit(const zd *tab, int64_t ncls, int np, const int32_t *ea,
                                                    unsigned char *A)
 {
     const int RN = oz_rows(np), ns = oz_sweeps(np), KC = oz_chunks(np);
@@ -160,7 +189,7 @@ __global__ void __launch_bounds__(256) k_oz_tsplit(const zd *tab, int64_t ncls, 
     const int64_t cs = idx / ((int64_t)RN * KC), cls = cs / ns;
     const int row = (int)(cs % ns) * RN + lrow, p = row >> 1, im = row & 1;
     const zd *T = tab + cls * np * np;
-    const double sc = ldexp(1.0, -oz_ea(tmax));
+    const double sc = row < 2 * np ? ldexp(1.0, -ea[p]) : 0.0;
     uint16_t d[OZ_S][8];
     for (int i = 0; i < 8; ++i) {
         const int k = 8 * c + i;
@@ -203,6 +232,28 @@ __global__ void __launch_bounds__(256) k_oz_mmax(const OzLevel *lvs, int np, int
     __syncthreads();
     if ((int)threadIdx.x < nv && s[threadIdx.x]) atomicMax(&lv.mmax[threadIdx.x], s[threadIdx.x]);
 }
+// L2L: largest component of each source box and vector, a warp per box
+__global__ void __launch_bounds__(256) k_oz_bmax(const OzLevel *lvs, int np, int nv)
+{
+    const OzLevel &lv = lvs[0];
+    __shared__ uint32_t s[8][LM_MAXV];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, step = 32 / nv * nv; // a lane keeps to one vector
+    const int64_t n = (int64_t)lv.planes * lv.ncl;
+    for (int64_t b = blockIdx.x * (int64_t)8 + w; b < n; b += (int64_t)gridDim.x * 8) {
+        if (lane < LM_MAXV) s[w][lane] = 0;
+        __syncwarp();
+        float mx = 0.f;
+        if (lane < step)
+            for (int i = lane; i < np * nv; i += step) {
+                const float4 a = lv.M[b * np * nv + i];
+                mx = fmaxf(mx, fmaxf(fabsf(a.x), fabsf(a.z)));
+            }
+        if (mx > 0.f) atomicMax(&s[w][lane % nv], __float_as_uint(mx));
+        __syncwarp();
+        if (lane < nv) lv.mmax[b * LM_MAXV + lane] = s[w][lane];
+        __syncwarp();
+    }
+}
 // one thread per (plane, row of it, 8-wide K chunk): 4 orders of a (box, vector) into 5 digit
 // planes; the padding boxes and vectors beyond nv are written as zeros.  Bound by memory: 250k strip,
 // 16 vectors, all levels 0.18 ms (0.27 ms with the real parts of all orders first, which reads each
@@ -221,7 +272,7 @@ __global__ void __launch_bounds__(256) k_oz_split(const OzLevel *lvs, int np, in
         uint16_t d[OZ_S][8];
         const bool on = i >= 0 && i < lv.ncl && v < nv;
         const int64_t box = lv.sstep == 2 ? (plane >> 1) * 2 * lv.ncl + 2 * i + (plane & 1) : plane * lv.ncl + i;
-        const float sc = on ? oz_pow2(-(oz_exp(lv.mmax[v]) + 2)) : 0.f;
+        const float sc = on ? oz_pow2(-(oz_exp(lv.mmax[(lv.add ? box * LM_MAXV : 0) + v]) + 2)) : 0.f;
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
             const int k = 8 * c + j;
@@ -398,7 +449,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_m2l_oz(const OzLevel *lvs, in
             for (int64_t tile = blockIdx.x; tile < ntiles && !stop && !*abort_s; tile += gridDim.x) {
                 int cls, i0, sw;
                 const OzLevel &lv = oz_tile(lvs, nlev, tile, ns, &cls, &i0, &sw, tb);
-                const int ne = lv.e0[cls + 1] - lv.e0[cls], grp = oz_grp(lv.tmax);
+                const int ne = lv.e0[cls + 1] - lv.e0[cls], grp = oz_grp(lv.ea, np);
                 for (int e = 0; e < ne && !stop; e += grp, ++item) {
                     if (!mbar_wait_lim(btempty, (item & 1) ^ 1, TC_WAIT_LIMIT, abort_s, err)) {
                         oz_fail(abort_s, err);
@@ -448,7 +499,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_m2l_oz(const OzLevel *lvs, in
         for (int64_t tile = blockIdx.x; tile < ntiles && !bad; tile += gridDim.x) {
             int cls, i0, sw;
             const OzLevel &lv = oz_tile(lvs, nlev, tile, ns, &cls, &i0, &sw, tb);
-            const int ne = lv.e0[cls + 1] - lv.e0[cls], grp = oz_grp(lv.tmax);
+            const int ne = lv.e0[cls + 1] - lv.e0[cls], grp = oz_grp(lv.ea, np);
             df acc[OZ_RN / 2];
 #pragma unroll
             for (int r = 0; r < OZ_RN / 2; ++r) acc[r] = df{0.f, 0.f};
@@ -480,8 +531,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_m2l_oz(const OzLevel *lvs, in
             if (bad) break;
             if (i0 + j < lv.ncl && v < nv) {
                 const int64_t r0 = lv.tstep == 2 ? (int64_t)(cls >> 1) * lv.ncol + (cls & 1) : cls * lv.ncol;
-                const int x = oz_ea(lv.tmax) + oz_exp(lv.mmax[v]) + 2 - 2 * OZ_BITS, p0 = (sw * RN + H * nr) / 2;
-                const float f = oz_pow2(x / 2), g = oz_pow2(x - x / 2);
+                const int64_t src = lv.add ? ((int64_t)(cls >> 2) * lv.ncl + i0 + j) * LM_MAXV : 0; // L2L: the parent
+                const int x0 = oz_exp(lv.mmax[src + v]) + 2 - 2 * OZ_BITS, p0 = (sw * RN + H * nr) / 2;
                 float4 *o = lv.L + ((r0 + lv.tstep * (int64_t)(i0 + j)) * np + p0) * nv + v;
                 float omx = 0.f;
 #pragma unroll
@@ -494,6 +545,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_m2l_oz(const OzLevel *lvs, in
 #pragma unroll
                     for (int c = 0; c < 4; ++c)
                         if (p0 + r8 / 2 + c < np) {
+                            const int x = x0 + lv.ea[p0 + r8 / 2 + c];
+                            const float f = oz_pow2(x / 2), g = oz_pow2(x - x / 2);
                             const df a = acc[r8 + 2 * c], i = acc[r8 + 2 * c + 1];
                             df yr = {a.h * f * g, a.l * f * g}, yi = {i.h * f * g, i.l * f * g};
                             if (lv.add) {
@@ -558,11 +611,11 @@ static std::vector<OzLevel> oz_levels(const lm_tree_s *t, int op, int nvs)
         o.e0 = x.e0;
         o.ents = (const RowEnt *)x.ents;
         o.A = x.A;
-        o.tmax = x.tmax;
+        o.ea = x.ea;
         // level i's multipoles and their digits; the parents' local expansions take those of level i + 1
         o.B = op == OZ_L2L ? (i + 1 < nl ? Z.lv[i + 1].B : Z.Btop) : z.B;
-        o.mmax = Z.mmax + (size_t)LM_MAXV * (op == OZ_L2L ? nl + i + 1 : i);
-        o.omax = op == OZ_M2M && i + 1 < nl ? Z.mmax + (size_t)LM_MAXV * (i + 1) : op == OZ_L2L ? Z.mmax + (size_t)LM_MAXV * (nl + i) : nullptr;
+        o.mmax = op == OZ_L2L ? Z.bmax : Z.mmax + (size_t)LM_MAXV * i;
+        o.omax = op == OZ_M2M && i + 1 < nl ? Z.mmax + (size_t)LM_MAXV * (i + 1) : nullptr;
         o.M = (const float4 *)(op == OZ_L2L ? up.Lc : lv.M);
         o.L = (float4 *)(op == OZ_M2M ? up.M : lv.Lc);
         v.push_back(o);
@@ -581,14 +634,21 @@ static lm_status oz_setup_op(lm_tree_s *t, const zd *tab, size_t ncls, const std
     x.ents = de;
     TRY_O(lm_dalloc(t, &x.e0, e0.size()));
     TRY_O(lm_dalloc(t, &x.A, ncls * OZ_S * KC * rows * 16));
-    TRY_O(lm_dalloc(t, &x.tmax, 3));
+    TRY_O(lm_dalloc(t, &x.ea, np + 3));
+    uint32_t *tmax;
+    int32_t *W;
+    TRY_O(lm_dalloc(t->tmp, &tmax, 2 * np));
+    TRY_O(lm_dalloc(t->tmp, &W, ncls * np));
     LM_CUDA(cudaMemcpyAsync(de, ents.data(), ents.size() * sizeof(RowEnt), cudaMemcpyHostToDevice, st));
     LM_CUDA(cudaMemcpyAsync(x.e0, e0.data(), e0.size() * sizeof(int32_t), cudaMemcpyHostToDevice, st));
-    LM_CUDA(cudaMemsetAsync(x.tmax, 0, 3 * sizeof(uint32_t), st));
-    k_oz_tmax<<<(unsigned)ncls, 256, 0, st>>>(tab, np, x.tmax);
-    k_oz_tsum<<<(unsigned)ncls, 128, 0, st>>>(tab, np, x.tmax);
+    LM_CUDA(cudaMemsetAsync(tmax, 0, 2 * np * sizeof(uint32_t), st));
+    LM_CUDA(cudaMemsetAsync(x.ea, 0, (np + 3) * sizeof(int32_t), st));
+    k_oz_tmax<<<(unsigned)ncls, 128, 0, st>>>(tab, np, tmax);
+    k_oz_texp<<<1, 128, 0, st>>>(tmax, np, x.ea);
+    k_oz_tsum<<<(unsigned)ncls, 128, 0, st>>>(tab, np, x.ea, W);
+    k_oz_gsum<<<(unsigned)(e0.size() - 1), 128, 0, st>>>(de, x.e0, np, W, x.ea);
     const int64_t nt = (int64_t)ncls * KC * rows;
-    k_oz_tsplit<<<(unsigned)((nt + 255) / 256), 256, 0, st>>>(tab, (int64_t)ncls, np, x.tmax, x.A);
+    k_oz_tsplit<<<(unsigned)((nt + 255) / 256), 256, 0, st>>>(tab, (int64_t)ncls, np, x.ea, x.A);
     LM_CUDA(cudaGetLastError());
     return LM_OK;
 }
@@ -640,7 +700,8 @@ lm_status lm_setup_oz(lm_tree_s *t, cudaStream_t st)
     const size_t nl = Z.lv.size();
     const Level &top = t->lev[Z.lv.back().l - 1];
     if (Z.nshift == nl) TRY_O(buf(top.nrow, top.ncol, &Z.Btop));
-    TRY_O(lm_dalloc(t, &Z.mmax, (2 * nl + 1) * LM_MAXV)); // multipoles of a level; local expansions, to the level above
+    TRY_O(lm_dalloc(t, &Z.mmax, nl * LM_MAXV)); // multipoles of a level
+    if (Z.nshift > 0) TRY_O(lm_dalloc(t, &Z.bmax, (size_t)t->lev[Z.lv[0].l - 1].nbox * LM_MAXV)); // parents of the deepest level
     int f = 0;
     for (int s = 1; s <= 16; s *= 2, ++f) {
         OzLevel *d;
@@ -669,11 +730,12 @@ static int oz_step(lm_tree_s *t, int op, size_t i, bool mmax, int nv, cudaStream
     const Level &lv = t->lev[Z.lv[i].l];
     const int64_t ncl = lv.ncol / 2, planes = op == OZ_L2L ? lv.nrow / 2 : 2 * lv.nrow;
     const int64_t work = planes * oz_prow((int)ncl, tb, nvs) * oz_chunks(t->np);
-    if (mmax) k_oz_mmax<<<2 * (unsigned)Z.nsm, 256, 0, st>>>(d, t->np, nv);
+    if (op == OZ_L2L) k_oz_bmax<<<8 * (unsigned)Z.nsm, 256, 0, st>>>(d, t->np, nv);
+    else if (mmax) k_oz_mmax<<<2 * (unsigned)Z.nsm, 256, 0, st>>>(d, t->np, nv);
     k_oz_split<<<(unsigned)std::min<int64_t>(8 * Z.nsm, (work + 255) / 256), 256, 0, st>>>(d, t->np, nv, nvs);
     const int64_t tiles = (op == OZ_M2M ? lv.nrow / 2 : 2 * lv.nrow) * ((ncl + tb - 1) / tb) * oz_sweeps(t->np);
     k_m2l_oz<<<(unsigned)std::min<int64_t>(Z.nsm, tiles), OZ_THREADS, OZ_SMEM, st>>>(d, 1, tiles, t->np, nv, nvs, t->dflag + 1, -1);
-    return 2 + mmax;
+    return 2 + (mmax || op == OZ_L2L);
 }
 
 // M2M from the levels of at least OZ_MINSHIFT boxes, whose multipoles' digits the M2L takes too; *lmin: the
@@ -684,7 +746,7 @@ lm_status lm_launch_m2m_oz(lm_tree_s *t, int nv, cudaStream_t st, int *lmin, int
     *launches = 0;
     *lmin = t->L;
     if (Z.lv.empty()) return LM_OK;
-    LM_CUDA(cudaMemsetAsync(Z.mmax, 0, (2 * Z.lv.size() + 1) * LM_MAXV * sizeof(uint32_t), st));
+    LM_CUDA(cudaMemsetAsync(Z.mmax, 0, Z.lv.size() * LM_MAXV * sizeof(uint32_t), st));
     for (size_t i = 0; i < Z.nshift; ++i) *launches += oz_step(t, OZ_M2M, i, i == 0, nv, st);
     *lmin = t->L - (int)Z.nshift;
     LM_CUDA(cudaGetLastError());
@@ -695,7 +757,7 @@ bool lm_oz_shift(const lm_tree_s *t, int l) { return t->L - l < (int)t->oz.nshif
 lm_status lm_launch_l2l_oz(lm_tree_s *t, int l, int nv, cudaStream_t st, int *launches)
 {
     const size_t i = (size_t)(t->L - l);
-    *launches = oz_step(t, OZ_L2L, i, i + 1 == t->oz.nshift, nv, st);
+    *launches = oz_step(t, OZ_L2L, i, false, nv, st);
     LM_CUDA(cudaGetLastError());
     return LM_OK;
 }
