@@ -284,6 +284,21 @@ __device__ __noinline__ void seg_df_grad(const DfSmem &tab, const NearDF &q, int
     }
 }
 
+// A pair of points at the same place: the kernel is infinite, which no double-float sum holds (inf - inf in its error
+// terms).  What FP64 gives, an infinity with the density's sign (not a number for the derivatives), goes to the output
+// at once; the block adds its finite sums to it later.
+__device__ __noinline__ void add_coincident(const float4 *q, int nv, int64_t n, int64_t i, zd *u, zd *ux, zd *uy)
+{
+    for (int v = 0; v < nv; ++v) {
+        const int64_t k = (int64_t)v * n + i;
+        if (u) {
+            atomicAdd(&u[k].re, INFINITY * df_double(df_re(q[v])));
+            atomicAdd(&u[k].im, INFINITY * df_double(df_im(q[v])));
+        }
+        if (ux) ux[k] = uy[k] = zd{NAN, NAN};
+    }
+}
+
 // One block: up to tb targets of a leaf at a time against the leaf's flattened near
 // sources.  Round: 64 sources staged (coordinates in the target leaf's frame,
 // densities), the kernel values of all (target, source) pairs evaluated a lane per
@@ -416,7 +431,10 @@ __global__ void __launch_bounds__(nd_threads(NV, GRAD), GRAD ? 3 : 512 / nd_thre
                                 z = df_add(df_sq(dx), df_sq(dy));
                             }
                             const bool slow = z.h > 1.0f || z.h < ND_TINY;
-                            if (GRAD) {
+                            if (slow && xs[t0 + row] == xs[sj[s]] && ys[t0 + row] == ys[sj[s]])
+                                add_coincident(qd + sj[s] * nvq + go.v0, nv, n, GRAD ? go.perm[t0 + row] : t0 + row,
+                                               GRAD ? go.u : us, GRAD ? go.ux : nullptr, GRAD ? go.uy : nullptr);
+                            else if (GRAD) {
                                 HVal H;
                                 if (slow) h0_slow_grad(k * hypot(xs[t0 + row] - xs[sj[s]], ys[t0 + row] - ys[sj[s]]), &H);
                                 else h0_df_grad<D, T>(tab, z, &H);
@@ -583,11 +601,11 @@ __global__ void __launch_bounds__(nd_threads(NV, GRAD), GRAD ? 3 : 512 / nd_thre
                 zd *o = c == 0 ? go.u : c == 1 ? go.ux : go.uy;
                 if (o) {
                     zd &w = o[(int64_t)vv * n + go.perm[t0 + row]];
-                    w = w + r;
+                    w = zd{__ldcg(&w.re), __ldcg(&w.im)} + r;
                 }
-            } else {
+            } else { // (past L1, for add_coincident's atomics)
                 zd &o = us[(int64_t)vv * n + t0 + row];
-                o = o + r;
+                o = zd{__ldcg(&o.re), __ldcg(&o.im)} + r;
             }
         }
     }
