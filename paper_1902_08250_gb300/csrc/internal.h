@@ -260,7 +260,7 @@ struct lm_tree_s {
     int32_t *uterm;   // [nu]
     std::vector<Level> lev;
     NearQuad nq;
-    zd *qs, *us; // [LM_MAXV][n] tree-order scratch
+    zd *qs, *us; // [LM_MAXV][n] tree-order scratch (qs: where FP64 kernels read the densities)
     // mixed path
     float *xl32, *yl32, *y32; // leaf-local coordinates and absolute y, FP32 [n]
     int64_t *iperm;            // [n] input index -> tree position

@@ -459,10 +459,9 @@ lm_status lm_setup_adaptive(lm_tree_s *t, const double *x, const double *y, cuda
                             t->lev[clt[j]].scale, t->lev[cls[j]].scale, A.tab + (size_t)j * np * np});
         TRY_A(lm_build_m2l_tables(md, P, tcls, t->dflag, t->tmp, st));
     }
-    if (t->precision == LM_FP64) { // expansions and tree-order scratch
+    if (t->precision == LM_FP64) { // expansions and tree-order potentials
         TRY_A(lm_dalloc(t, &A.M, (size_t)nbox * np * LM_MAXV));
         TRY_A(lm_dalloc(t, &A.Lc, (size_t)nbox * np * LM_MAXV));
-        TRY_A(lm_dalloc(t, &t->qs, (size_t)LM_MAXV * n));
         TRY_A(lm_dalloc(t, &t->us, (size_t)LM_MAXV * n));
     }
     int hflag = 0;

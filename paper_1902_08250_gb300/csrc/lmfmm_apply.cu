@@ -948,20 +948,24 @@ lm_status lm_near_pw64_attr(size_t bytes)
 }
 
 // the double-float form's own data (FP64 form, unless opt.m2l_fp64 asks for IEEE FP64 throughout);
-// leaves t->m2l_df false where the form does not apply
+// leaves t->m2l_df false where the form does not apply.  FP64 kernels read the tree-order densities until the
+// potentials are written and have a buffer of their own for them; the double-float form has read them by then
+// (k_q_df) and permutes them into that of the potentials: 256 bytes a point.
 lm_status lm_setup_df(lm_tree_s *t, cudaStream_t st)
 {
-    if (!t->m2l_df) return LM_OK;
+    lm_status s = LM_OK;
+    if (!t->m2l_df) return lm_dalloc(t, &t->qs, (size_t)LM_MAXV * t->n);
     double wmax = t->adaptive ? 0.0 : t->lev[t->L].w; // the widest leaf
     if (t->adaptive)
         for (int64_t b = 0; b < t->at.nbox; ++b)
             if (t->at.hbox[4 * b + 3]) wmax = std::max(wmax, ldexp(t->med.d, -(int)t->at.hbox[4 * b]));
     if (!lm_exp_df_fits(t->med.k2, wmax)) {
         t->m2l_df = false;
-        return LM_OK;
+        return lm_dalloc(t, &t->qs, (size_t)LM_MAXV * t->n);
     }
     t->ndf.wmax = wmax;
-    lm_status s = lm_dalloc(t, &t->qexp, LM_MAXV);
+    if (!t->near_pw64) s = lm_dalloc(t, &t->qs, (size_t)LM_MAXV * t->n); // lm_launch_near64 reads them
+    if (s == LM_OK) s = lm_dalloc(t, &t->qexp, LM_MAXV);
     if (s == LM_OK) s = lm_setup_near_df(t, st);
     if (s == LM_OK) s = lm_setup_oz(t, st);
     if (s == LM_OK) s = lm_setup_exp_df(t, st);

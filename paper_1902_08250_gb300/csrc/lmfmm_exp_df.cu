@@ -587,13 +587,14 @@ lm_status lm_run_df(lm_tree_s *t, const zd *q, int nvec, zd *u, bool adjoint, zd
     const BesselDF B{t->xdf.bes, t->xdf.N, t->xdf.nt};
     const int P = t->p;
     const double k2 = t->med.k2;
+    zd *qs = t->qs ? t->qs : t->us; // (lm_setup_df)
     auto Mof = [&](int l) { return (float4 *)(ad ? A.M : t->lev[l].M); };
     auto Lof = [&](int l) { return (float4 *)(ad ? A.Lc : t->lev[l].Lc); };
     for (int v0 = 0; v0 < nvec; v0 += LM_MAXV) {
         const int nv = std::min(LM_MAXV, nvec - v0);
         lm_phase_begin(t, PH_PERMUTE, st);
-        k_permute_in<<<gridn(n, 256), 256, 0, st>>>(q + (int64_t)v0 * n, t->perm, n, nv, adjoint, t->qs);
-        TRY_X(lm_launch_q_df(t->qs, n, nv, t->qexp, t->ndf.q, st));
+        k_permute_in<<<gridn(n, 256), 256, 0, st>>>(q + (int64_t)v0 * n, t->perm, n, nv, adjoint, qs);
+        TRY_X(lm_launch_q_df(qs, n, nv, t->qexp, t->ndf.q, st));
         lm_phase_end(t, PH_PERMUTE, st, 3);
         // step 2: S2M at every leaf, M2M up the levels
         lm_phase_begin(t, PH_S2M, st);

@@ -773,8 +773,7 @@ lm_status lm_setup_tables(lm_tree_s *t, cudaStream_t st)
     if (mixed) {
         TRY(lm_setup_mixed(t, st));
     } else {
-        // tree-order scratch for densities and potentials
-        TRY(lm_dalloc(t, &t->qs, (size_t)LM_MAXV * t->n));
+        // tree-order potentials
         TRY(lm_dalloc(t, &t->us, (size_t)LM_MAXV * t->n));
     }
     LM_CUDA(cudaMemcpyAsync(&hflag, t->dflag, sizeof(int), cudaMemcpyDeviceToHost, st));
