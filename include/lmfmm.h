@@ -93,10 +93,18 @@ typedef struct {
                         expansions and the direct interactions in double-float on the FP32
                         pipes -- each value a pair of FP32 numbers (48-bit significand), exact
                         products by fma and error-free sums, densities scaled by a power of two
-                        per apply so the values stay inside FP32's exponent range; about 1e-14
-                        relative, and many times the FP64 pipe's rate on GB300.  Tables,
-                        quadratures and potentials are FP64 either way.  Trees whose leaves are
-                        wider than 140 / k2 take FP64 throughout. */
+                        per vector so the values stay inside FP32's exponent range --, the
+                        contractions of uniform trees' levels of 256 boxes and more by fixed-point
+                        digits on the tensor cores (2^-50 of a level's scales: boxes whose sources
+                        are 1e10 times weaker than a level's strongest keep about 1e-12).  Tables,
+                        quadratures and potentials are FP64 either way.  Measured from the IEEE
+                        form, relative l2: potentials 8e-15 to 2.4e-13, target gradients 1e-14 to
+                        1.2e-13, cross-layer operator 3e-14 to 5e-14; central differences of steps
+                        like 1e-6 need 1.  IEEE FP64 is taken by the direct pairs beyond k2 r = 2
+                        (each on its own), by all direct pairs where max(k1, k2, k3) is above
+                        about 15 at the default seg_order (segment coefficients beyond 200 KB of
+                        shared memory), and throughout by trees whose leaves are wider than
+                        140 / k2. */
     int tensor_leaf; /* LM_MIXED uniform trees, p <= 14, applies of 5-16 vectors: the leaf step's
                         multiply-adds over the vectors (direct S2T pairs and L2T) on the tcgen05
                         tensor cores, the kernel values on the CUDA cores (FP16 hi/lo split of both

@@ -201,8 +201,8 @@ struct DfSmem {
 
 // e^{x + i y} with x in units of ln 2 / 64 and y in units of 2 pi / 256 (the
 // callers' tables carry the factors): x and y split into the table index and a
-// remainder of at most half a unit, exact by construction.  Relative error about
-// 1e-13 (checked against FP64 in the tests through the kernels that use it).
+// remainder of at most half a unit, exact by construction.  Relative error below
+// 1e-13 (the exponential's series ends at t^4: 5e-14 at most).
 __device__ __forceinline__ float4 df_cexp(const DfSmem &T, df x, df y)
 {
     // 2^(n/64) (1 + t + t^2/2 + t^3/6 + t^4/24), t = r ln 2 / 64, |t| < 0.0055

@@ -6,8 +6,8 @@
 // for FP32, so the FP64 leaf kernel spent its time in H0 (28 DFMAs, a log, a
 // hypot) and in the tails (48 complex exponentials a pair, about 75 DFMAs each).
 // In double-float a free pair takes about 250 FP32 instructions and a tail node
-// about 170.  The kernel values carry about 47 bits: 1e-14 beside the FMM's own
-// truncation (1e-13 to 1e-10 for p = 24 to 18).
+// about 170.  The kernel values carry about 47 bits: one leaf of 60 points is 8e-15 from the IEEE
+// form, its gradient 1.3e-14, beside the FMM's own truncation (1e-13 to 1e-10 for p = 24 to 18).
 //
 // Units: coordinates are scaled by k2/2, so that z = dx^2 + dy^2 = (k2 r / 2)^2 is
 // the argument of the ascending series; densities by 2^-qexp, an exponent per vector
