@@ -37,8 +37,9 @@ def test_digits_largest_and_aligned():
     import paper_1902_08250_gb300 as lm
 
     tab = {(c, r): _table(special, c, r) for c in range(-3, 4) for r in range(-3, 4) if max(abs(c), abs(r)) >= 2}
-    ex = lambda v: math.floor(math.log2(v))
-    scale = 2.0 ** -max(ex(max(np.abs(a).max() for a in tab.values())) + 2, ex(max(np.abs(a).sum(1).max() for a in tab.values())) - 1)
+    ex = lambda v: np.floor(np.log2(v))
+    mags = np.abs(np.array(list(tab.values())))  # [offset][row][column]; a scale per row: components below 1/2, row sums at most 4
+    scale = 2.0 ** -np.maximum(ex(mags.max((0, 2))) + 2, ex(mags.sum(2).max(0)) - 1)[:, None]
     # the first entries of the list of a target box of even row and column: two rows up
     offs = [(2, 2), (1, 2), (0, 2), (-1, 2)]
     d0 = [np.rint(tab[o] * scale * 1024.0) for o in offs]
